@@ -63,12 +63,12 @@ def _load(path: str = _LIB_PATH) -> C.CDLL:
     lib = C.CDLL(path)
     vp, i32p, u8p = C.c_void_p, C.POINTER(C.c_int32), C.POINTER(C.c_uint8)
     cfgp = C.POINTER(hkv_config)
-    lib.hkv_plan.argtypes = [cfgp, i32p, u8p, i32p, C.POINTER(C.c_size_t), C.POINTER(C.c_size_t)]
-    lib.hkv_compress.argtypes = [cfgp, vp, vp, vp, vp, vp, i32p, u8p, i32p, vp, C.c_size_t, vp, C.c_size_t, vp,
+    lib.hkv_plan.argtypes = [cfgp, vp, vp, vp, C.POINTER(C.c_size_t), C.POINTER(C.c_size_t)]
+    lib.hkv_compress.argtypes = [cfgp, vp, vp, vp, vp, vp, vp, vp, vp, vp, C.c_size_t, vp, C.c_size_t, vp,
                                  C.POINTER(vp)]
-    lib.hkv_plan_offload.argtypes = [cfgp, i32p, u8p, i32p, C.POINTER(C.c_size_t), C.POINTER(C.c_size_t),
+    lib.hkv_plan_offload.argtypes = [cfgp, vp, vp, vp, C.POINTER(C.c_size_t), C.POINTER(C.c_size_t),
                                      C.POINTER(C.c_size_t)]
-    lib.hkv_compress_offload.argtypes = [cfgp, vp, vp, vp, vp, vp, i32p, u8p, i32p, vp, C.c_size_t, vp, C.c_size_t,
+    lib.hkv_compress_offload.argtypes = [cfgp, vp, vp, vp, vp, vp, vp, vp, vp, vp, C.c_size_t, vp, C.c_size_t,
                                          vp, C.c_size_t, vp, C.POINTER(vp)]
     lib.hkv_decode_attn.argtypes = [vp, vp, vp, vp]
     lib.hkv_decode_attn_multi.argtypes = [C.POINTER(vp), C.POINTER(vp), C.POINTER(vp), C.c_int32, vp]
@@ -91,7 +91,7 @@ def _load(path: str = _LIB_PATH) -> C.CDLL:
                                          C.c_uint32, i32p]
     lib.hkv_classify_workspace.argtypes = [C.POINTER(hkv_config), C.c_int32, C.POINTER(C.c_size_t),
                                            C.POINTER(C.c_size_t)]
-    lib.hkv_classify_heads.argtypes = [C.POINTER(hkv_config), vp, vp, C.c_int32, i32p, i32p, C.c_double, C.c_double,
+    lib.hkv_classify_heads.argtypes = [C.POINTER(hkv_config), vp, vp, C.c_int32, vp, vp, C.c_double, C.c_double,
                                        vp, C.c_size_t, vp, vp, vp]
     lib.hkv_status_string.argtypes = [C.c_int]
     lib.hkv_status_string.restype = C.c_char_p
@@ -134,6 +134,11 @@ def _ptr(a: np.ndarray, ctype):
     return a.ctypes.data_as(C.POINTER(ctype))
 
 
+def _host(a: np.ndarray) -> int:
+    """Host address of an array's first element (a typed ctypes pointer costs 1.5 us to make)."""
+    return a.ctypes.data
+
+
 def _dev(t) -> Optional[int]:
     """Device address of a torch CUDA tensor (None stays NULL)."""
     if t is None:
@@ -143,10 +148,24 @@ def _dev(t) -> Optional[int]:
     return t.data_ptr()
 
 
+_raw_current_stream = None   # () -> address of the current device's current stream, resolved at the first call
+
+
+def _current_stream() -> Optional[int]:
+    """The address alone: torch.cuda.current_stream() builds a Stream object around it, which took 3.6 us per call,
+    as much as the launch that follows."""
+    global _raw_current_stream
+    if _raw_current_stream is None:
+        import torch
+        torch.cuda.init()
+        get_stream, get_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+        _raw_current_stream = lambda: get_stream(get_device())  # noqa: E731
+    return _raw_current_stream() or None
+
+
 def _stream(stream) -> Optional[int]:
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream or None
+        return _current_stream()
     if hasattr(stream, "cuda_stream"):
         return stream.cuda_stream or None
     return int(stream) or None
@@ -162,7 +181,7 @@ def hkv_plan(cfg: hkv_config, seq_lens, head_type, budgets):
     """-> (cache_bytes, workspace_bytes); host arithmetic only."""
     sl, ht, bu = _i32(seq_lens), _u8(head_type), _i32(budgets)
     cb, wb = C.c_size_t(0), C.c_size_t(0)
-    _check(lib.hkv_plan(C.byref(cfg), _ptr(sl, C.c_int32), _ptr(ht, C.c_uint8), _ptr(bu, C.c_int32),
+    _check(lib.hkv_plan(C.byref(cfg), _host(sl), _host(ht), _host(bu),
                         C.byref(cb), C.byref(wb)), "hkv_plan")
     return int(cb.value), int(wb.value)
 
@@ -174,7 +193,7 @@ def hkv_compress(cfg: hkv_config, k, v, q_obs, token_scores, is_text, seq_lens, 
     sl, ht, bu = _i32(seq_lens), _u8(head_type), _i32(budgets)
     handle = C.c_void_p(None)
     _check(lib.hkv_compress(C.byref(cfg), _dev(k), _dev(v), _dev(q_obs), _dev(token_scores), _dev(is_text),
-                            _ptr(sl, C.c_int32), _ptr(ht, C.c_uint8), _ptr(bu, C.c_int32),
+                            _host(sl), _host(ht), _host(bu),
                             _dev(cache_mem), cache_mem.numel() * cache_mem.element_size(),
                             _dev(workspace), workspace.numel() * workspace.element_size(),
                             _stream(stream), C.byref(handle)), "hkv_compress")
@@ -185,7 +204,7 @@ def hkv_plan_offload(cfg: hkv_config, seq_lens, head_type, budgets):
     """-> (cache_bytes, workspace_bytes, host_bytes) for the variant with the dynamic heads' K/V in host memory."""
     sl, ht, bu = _i32(seq_lens), _u8(head_type), _i32(budgets)
     cb, wb, hb = C.c_size_t(0), C.c_size_t(0), C.c_size_t(0)
-    _check(lib.hkv_plan_offload(C.byref(cfg), _ptr(sl, C.c_int32), _ptr(ht, C.c_uint8), _ptr(bu, C.c_int32),
+    _check(lib.hkv_plan_offload(C.byref(cfg), _host(sl), _host(ht), _host(bu),
                                 C.byref(cb), C.byref(wb), C.byref(hb)), "hkv_plan_offload")
     return int(cb.value), int(wb.value), int(hb.value)
 
@@ -201,7 +220,7 @@ def hkv_compress_offload(cfg: hkv_config, k, v, q_obs, token_scores, is_text, se
     hp = host_mem.data_ptr() if host_mem is not None else None
     hn = host_mem.numel() * host_mem.element_size() if host_mem is not None else 0
     _check(lib.hkv_compress_offload(C.byref(cfg), _dev(k), _dev(v), _dev(q_obs), _dev(token_scores), _dev(is_text),
-                                    _ptr(sl, C.c_int32), _ptr(ht, C.c_uint8), _ptr(bu, C.c_int32),
+                                    _host(sl), _host(ht), _host(bu),
                                     _dev(cache_mem), cache_mem.numel() * cache_mem.element_size(), hp, hn,
                                     _dev(workspace), workspace.numel() * workspace.element_size(),
                                     _stream(stream), C.byref(handle)), "hkv_compress_offload")
@@ -341,7 +360,7 @@ def hkv_classify_heads(cfg: hkv_config, k, q_text, seq_lens, n_text, topk_fracti
     k, q_text, workspace, scores_out (float64) and head_type_out (uint8) are CUDA tensors."""
     sl, nt = _i32(seq_lens), _i32(n_text)
     _check(lib.hkv_classify_heads(C.byref(cfg), k.data_ptr(), q_text.data_ptr(), int(q_text.shape[1]),
-                                  _ptr(sl, C.c_int32), _ptr(nt, C.c_int32), float(topk_fraction), float(theta),
+                                  _host(sl), _host(nt), float(topk_fraction), float(theta),
                                   workspace.data_ptr(), workspace.numel() * workspace.element_size(),
                                   scores_out.data_ptr(), head_type_out.data_ptr(), _stream(stream)),
            "hkv_classify_heads")
