@@ -3,18 +3,22 @@
 // entries, their mean over the rows (the text-centric sparsity score) and the comparison with the
 // threshold theta.  Runs once per prompt and layer, before the budgets and the compression.
 //
-// Three kernels per pass over a block of rows:
-//   cls_logits_tc_kernel  base-2 logits of 256 rows x a range of 128-key tiles, tcgen05 tensor cores,
-//                      float32 into the workspace (rows padded to a multiple of 128 floats);
-//   cls_row_kernel     one CTA per row: the row in shared memory, max, p = 2^(l - max), normaliser,
-//                      the exact k-th largest p (histogram over the float bits, then exact ranking
-//                      of the threshold bin), the sum of the entries above it plus the tied share
-//                      (cls_row_regs_kernel when no row of the group is longer than 32768 entries:
-//                      the row in registers, the next row's copy in flight meanwhile);
-//   cls_finish_kernel  (after the last pass) mean of the rows' sums in double, fixed order, and
-//                      the label.
+// The logits are never stored.  Per pass over a block of rows (normally one pass):
+//   cls_gather_kernel, cls_sample_kernel
+//                      logits of up to 4096 keys per row, drawn at random from the context, on the tensor
+//                      cores; a histogram per row gives two bounds [lo, hi] that hold the row's k-th largest
+//                      logit with a miss probability of about 2e-6, and a reference for the exponent;
+//   cls_scan_kernel    all logits, drained from tensor memory straight into the row's sums: the normaliser over
+//                      everything, sum and number of the entries above hi; the few per cent of entries between lo
+//                      and hi are appended to the row's list;
+//   cls_select_kernel  a warp per row: the exact k-th largest among the listed entries, the row's sum.  A row whose
+//                      bounds missed, whose list overflowed or that holds a non-finite value is flagged instead;
+//   cls_fix_kernel     flagged rows one by one: all logits in one buffer and an exact selection over them;
+//   cls_finish_kernel  (after the last pass) mean of the rows' sums in double, fixed order, and the label.
+// The result is exact: sampling only decides how much has to be looked at twice.
 #include <algorithm>
 #include <cmath>
+#include <mutex>
 
 #include "hkv_device.cuh"
 #include "hkv_internal.h"
@@ -26,84 +30,590 @@ namespace {
 
 constexpr float kLog2e = 1.4426950408889634f;
 constexpr int kClsBatch = 64;          // sequences one group of launches takes
-constexpr int kClsRowThreads = 1024;
-constexpr int kClsSmemCols = 49152;    // longest row the row kernel keeps in shared memory
+constexpr int kClsSample = 4096;       // keys sampled per row (32 tiles)
+constexpr int kClsGroupMax = 8;        // most sampled keys that share a histogram entry (their largest logit)
+constexpr int kClsSampleBins = 112;    // histogram of the sample, six standard deviations wide
+constexpr double kClsSigmas = 4.75;    // margin of the bounds in standard deviations of the sample's rank
+constexpr int kClsSlack = 256;         // list entries per segment beyond its share: half of a video frame whose keys all lie between the bounds
+constexpr int kClsFixThreads = 1024;
+constexpr int kClsSmemCols = 49152;    // longest row the fix kernel keeps in shared memory
 constexpr int kClsRank = 256;          // largest threshold bin that is sorted directly
-constexpr int kClsBins = 4096;          // bits 30..18 of a float in [0, 1]: 32 bins per octave
+constexpr int kClsBins = 4096;         // bits 30..18 of a float in [0, 1]: 32 bins per octave
 constexpr int kClsShift = 18;
-constexpr int kClsLoadParts = 4;       // pieces a row arrives in, so that the maximum overlaps the copy
-constexpr int kClsRegVecs = 8;         // float4s of a row a thread keeps in registers (rows up to 32768 floats)
-constexpr int kClsRowScratch = (kClsBins + kClsRank + 32 + 8 + 32) * 4 + kClsLoadParts * 8;   // histogram, candidates, reduction slots, control words, warp sums, mbarriers
+constexpr int kClsFixScratch = (kClsBins + kClsRank + 32 + 8 + 32) * 4 + kHeadDim * 2;   // histogram, candidates, reduction slots, control words, warp sums, query row
+
+constexpr float kClsOpen = -3.0e38f;   // lower bound that takes every finite logit
 
 struct ClsParams {
   int32_t C[kClsBatch];   // context length of each sequence
   int32_t T[kClsBatch];   // text tokens (query rows / group) of each sequence
   int32_t k[kClsBatch];   // entries summed per row
-  int32_t n_kv_heads, n_q_heads, group, max_seq_len, t_stride;
+  int32_t n_sample[kClsBatch];                        // sampled keys
+  int32_t rank_hi[kClsBatch], rank_lo[kClsBatch];     // ranks among the sample's group maxima that bound the k-th largest
+  int64_t w_prefix[kClsBatch + 1];   // (row block, key tile) pairs of the sequences before each
+  int32_t n_batch, n_kv_heads, n_q_heads, group, max_seq_len, t_stride;
   int32_t row_begin, row_block;   // this pass covers rows [row_begin, row_begin + row_block) of every unit
-  int32_t c_stride;               // floats between two rows of the logits workspace (multiple of 128)
   int32_t r_stride;               // floats between two units of the row-sum array
-  int32_t smem_cols;              // rows up to this length are staged in shared memory
+  int32_t n_cta;                  // CTAs of the scan: CTA i takes pairs [i W / n_cta, (i + 1) W / n_cta), W = w_prefix[n_batch]
+  int32_t small;                  // W * n_cta fits 31 bits: 32-bit divisions
+  int32_t seg_max;                // most CTAs that share one row block
+  int32_t per_tile;               // list entries per half tile
+  int32_t list_stride;            // entries of one half row's list
+  int32_t sample_stride;          // rows of a unit in the sample buffer
+  float bins_at;                  // centre of the sample histogram in standard deviations above the mean
   float scale_log2e;
 };
 
-// ---------------------------------------------------------------------------------------------
-// Logits (tcgen05 tensor cores, accumulators in tensor memory).  One CTA = 256 rows of one unit x a range of
-// 128-key tiles; the tile's keys are the accumulator's rows (lanes) and the 256 query rows its columns, so a
-// draining warp owns 32 consecutive keys and 64 rows and writes, per row, one 128-byte line.
-// grid (key ranges, 256-row blocks of the pass, units).
-// ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(tc::kThreads, 1)
-    cls_logits_tc_kernel(const ClsParams P, const __nv_bfloat16* kin, const __nv_bfloat16* q_text, float* logits,
-                         int tiles_per_cta, int32_t* err) {
-  extern __shared__ __align__(16) uint8_t tc_smem[];
-  const int unit = blockIdx.z, b = unit / P.n_kv_heads, h = unit - b * P.n_kv_heads;
-  const int C = P.C[b], G = P.group, R = P.T[b] * G;
-  const int r_end = min(R, P.row_begin + P.row_block);
-  const int row0 = P.row_begin + blockIdx.y * tc::kQRows;
-  const int n_tiles = (C + tc::kKeysPerTile - 1) / tc::kKeysPerTile;
-  const int tile_begin = blockIdx.x * tiles_per_cta, tile_end = min(n_tiles, tile_begin + tiles_per_cta);
-  if (row0 >= r_end || tile_begin >= tile_end) return;
+// rows of sequence b in this pass, its 256-row blocks and its key tiles
+__device__ __forceinline__ int cls_rows(const ClsParams& P, int b) {
+  return max(0, min(P.row_block, P.T[b] * P.group - P.row_begin));
+}
+__device__ __forceinline__ int cls_blocks(const ClsParams& P, int b) { return (cls_rows(P, b) + tc::kQRows - 1) / tc::kQRows; }
+__device__ __forceinline__ int cls_tiles(const ClsParams& P, int b) { return (P.C[b] + tc::kKeysPerTile - 1) / tc::kKeysPerTile; }
+__device__ __forceinline__ int cls_sample_tiles(const ClsParams& P, int b) { return (P.n_sample[b] + tc::kKeysPerTile - 1) / tc::kKeysPerTile; }
+// first pair of CTA i, and the CTA that holds pair w
+__device__ __forceinline__ int64_t cls_cta_begin(const ClsParams& P, int i) {
+  if (P.small) return static_cast<uint32_t>(i) * static_cast<uint32_t>(P.w_prefix[P.n_batch]) / static_cast<uint32_t>(P.n_cta);
+  return static_cast<int64_t>(i) * P.w_prefix[P.n_batch] / P.n_cta;
+}
+__device__ __forceinline__ int cls_cta_of(const ClsParams& P, int64_t w) {
+  if (P.small) return static_cast<int>(((static_cast<uint32_t>(w) + 1u) * static_cast<uint32_t>(P.n_cta) - 1u) / static_cast<uint32_t>(P.w_prefix[P.n_batch]));
+  return static_cast<int>(((w + 1) * P.n_cta - 1) / P.w_prefix[P.n_batch]);
+}
 
-  auto q_row = [&](int row) -> const __nv_bfloat16* {
-    const int r = row0 + row;
-    if (r >= r_end) return nullptr;
-    const int i = r / G;
-    return q_text + ((static_cast<size_t>(b) * P.t_stride + i) * P.n_q_heads + h * G + (r - i * G)) * kHeadDim;
+// Where a segment's entries lie in a half row's list: a share for every tile before it, slack for every segment.
+__device__ __forceinline__ int cls_list_at(const ClsParams& P, int tile_begin, int index) {
+  return (tile_begin * P.per_tile & ~3) + index * kClsSlack;
+}
+
+// A row's bounds; without a sample (a workspace too small for one) every entry is listed.
+__device__ __forceinline__ float4 cls_bounds(const float4* bounds, size_t row) {
+  return bounds ? __ldcg(bounds + row) : make_float4(kClsOpen, INFINITY, 0.f, 0.f);
+}
+
+// A run of key tiles of one 256-row block of one unit.
+struct ClsSeg {
+  int key_row0, C, tile_begin, tile_end;
+  int b, unit, row0, n_rows;   // first row of the block within the pass, rows of it that exist
+  int index;                   // which of the block's segments
+  int64_t next;                // pair behind the segment
+};
+
+__device__ __forceinline__ const __nv_bfloat16* cls_q_row(const ClsParams& P, const __nv_bfloat16* q_text, int b, int h, int r) {
+  const int i = r / P.group;
+  return q_text + ((static_cast<size_t>(b) * P.t_stride + i) * P.n_q_heads + h * P.group + (r - i * P.group)) * kHeadDim;
+}
+__device__ __forceinline__ const __nv_bfloat16* cls_keys(const ClsParams& P, const __nv_bfloat16* kin, int unit) {
+  return kin + static_cast<size_t>(unit) * P.max_seq_len * kHeadDim;
+}
+
+// ---------------------------------------------------------------------------------------------
+// The keys sampled from every unit, as rows the tensor core can be fed with: row j holds the key at a pseudo-random
+// place of the context (with replacement, the same places for every unit of one length), so that neither a drift along
+// the context nor a period in it can bias the sample, and any eight rows are as good as independent.
+// grid (row groups of 16, units); samples: bf16 [unit][sample_stride][128].
+// ---------------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(256)
+    cls_gather_kernel(const __grid_constant__ ClsParams P, const uint4* kin, uint4* samples) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int unit = blockIdx.y, b = unit / P.n_kv_heads;
+  const int j = blockIdx.x * 16 + (threadIdx.x >> 4), piece = threadIdx.x & 15;
+  if (j >= (cls_sample_tiles(P, b) + 1) * tc::kKeysPerTile) return;
+  uint32_t x = static_cast<uint32_t>(j) * 0x9E3779B1u + 0x7F4A7C15u;   // any mixing will do
+  x ^= x >> 16; x *= 0x85EBCA6Bu; x ^= x >> 13; x *= 0xC2B2AE35u; x ^= x >> 16;
+  const size_t key = static_cast<size_t>(unit) * P.max_seq_len + __umulhi(x, static_cast<uint32_t>(P.C[b]));
+  samples[(static_cast<size_t>(unit) * P.sample_stride + j) * 16 + piece] = __ldg(kin + key * 16 + piece);
+}
+
+// ---------------------------------------------------------------------------------------------
+// Bounds of every row's k-th largest logit from the sample.  A CTA = one 256-row block; accumulator lanes = rows, two
+// threads per row (halves of each tile).  Tile 0 gives every row's mean and standard deviation, the others the
+// histogram (two rows share a 32-bit word).  What is counted is the largest logit of every group of up to eight
+// samples: a share q of the entries is a share 1 - (1 - q)^8 of the group maxima, which fixes a 5 % quantile as closely
+// as single samples do with an eighth of the shared-memory atomics (one atomic per sample: 5 us per tile).
+// grid: row blocks of the pass.  bounds: float4 [unit][row_block] = (lo, hi, scaled reference, -).
+// ---------------------------------------------------------------------------------------------
+constexpr int kClsHistBytes = kClsSampleBins * tc::kQRows * 2;
+constexpr int kClsSampleSmem = tc::seg_smem_fixed(tc::kStages) + kClsHistBytes;
+static_assert(kClsSampleSmem + 4096 <= 232448, "one CTA's shared memory");
+
+template <int kGroup>
+__global__ void __launch_bounds__(tc::kSegThreads, 1)
+    cls_sample_kernel(const __grid_constant__ ClsParams P, const __grid_constant__ CUtensorMap samples, const __nv_bfloat16* q_text,
+                      float4* bounds, int32_t* err) {
+  extern __shared__ __align__(16) uint8_t tc_smem[];
+  __shared__ float2 stat[2][tc::kQRows];   // (sum, sum of squares) of each half, then the running maxima
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  int b = 0, blk = blockIdx.x;
+  while (blk >= cls_blocks(P, b) * P.n_kv_heads) { blk -= cls_blocks(P, b) * P.n_kv_heads; ++b; }
+  const int n_blk = cls_blocks(P, b), h = blk / n_blk, row0 = (blk - h * n_blk) * tc::kQRows;
+  const int n_s = P.n_sample[b], rows = cls_rows(P, b);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+
+  auto segment = [&](int s, ClsSeg& seg) {
+    seg.key_row0 = (b * P.n_kv_heads + h) * P.sample_stride;
+    seg.tile_begin = 0;
+    seg.tile_end = cls_sample_tiles(P, b) + 1;
+    return s == 0;
   };
-  const __nv_bfloat16* keys =
-      kin + (static_cast<size_t>(b) * P.n_kv_heads + h) * static_cast<size_t>(P.max_seq_len) * kHeadDim;
-  float* out = logits + static_cast<size_t>(unit) * P.row_block * P.c_stride;
-  const float sc = P.scale_log2e;
-  auto epilogue = [&](int tile, int lane_row, int part, auto groups, float*, auto, uint64_t*) {
-    // accumulator lane = key lane_row of the tile, columns 64 part .. + 63 = rows row0 + 64 part + (0..63): for one
-    // row the 32 lanes of a warp hold 32 consecutive keys, so every store instruction writes one 128-byte line of
-    // that row and nothing has to be transposed
-    const int rb = row0 + 64 * part;   // the warp's first row (the same in every lane)
-    if (rb >= r_end) return;           // 64 padding rows
-    float* dst = out + static_cast<size_t>(rb - P.row_begin) * P.c_stride + static_cast<size_t>(tile) * tc::kKeysPerTile +
-                 lane_row;
-    const size_t stride = static_cast<size_t>(P.c_stride);
-    groups([&](int g, float (&v)[32]) {
-      const int nv = r_end - (rb + 32 * g);   // rows of this group that exist (the same in every lane)
-      float* p = dst + static_cast<size_t>(32 * g) * stride;
-      if (nv >= 32) {
+  auto q_row = [&](const ClsSeg&, int row) -> const __nv_bfloat16* {
+    return row0 + row < rows ? cls_q_row(P, q_text, b, h, P.row_begin + row0 + row) : nullptr;
+  };
+  uint8_t* user = nullptr;
+  float a_bin = 0.f, inv_w = 0.f, width = 0.f, vmax = -INFINITY;
+  uint32_t hist_row = 0, inc = 0;
+  uint32_t* hist = nullptr;
+  auto begin = [&](const ClsSeg&, int lane_row, int part) {
+    hist = reinterpret_cast<uint32_t*>(user);
+    const int dtid = threadIdx.x - 32, row = 128 * (part >> 1) + lane_row;
+    for (int i = dtid; i < kClsHistBytes / 16; i += tc::kDrainWarps * 32) reinterpret_cast<uint4*>(hist)[i] = make_uint4(0u, 0u, 0u, 0u);
+    hist_row = smem_u32(hist) + (row >> 1) * 4;
+    inc = (row & 1) ? 0x10000u : 1u;
+    tc::named_sync(tc::kBarDrain, tc::kDrainWarps * 32);
+  };
+  auto tile_fn = [&](const ClsSeg&, int tile, int lane_row, int part, uint32_t taddr) {
+    const int row = 128 * (part >> 1) + lane_row, half = part & 1;
+    if (tile == 0) {
+      float s1 = 0.f, s2 = 0.f;
+      tc::drain_raw(taddr, [&](int, uint32_t (&r)[16]) {
 #pragma unroll
-        for (int i = 0; i < 32; ++i) { *p = v[i] * sc; p += stride; }
-      } else {
-#pragma unroll
-        for (int i = 0; i < 32; ++i) {
-          if (i < nv) *p = v[i] * sc;
-          p += stride;
+        for (int c = 0; c < 16; ++c) {
+          const float v = __uint_as_float(r[c]);
+          s1 += v;
+          s2 = fmaf(v, v, s2);
         }
+      });
+      stat[half][row] = make_float2(s1, s2);
+      tc::named_sync(tc::kBarDrain, tc::kDrainWarps * 32);
+      const float2 x = stat[0][row], y = stat[1][row];
+      const float mean = (x.x + y.x) * (1.f / tc::kKeysPerTile), var = fmaxf((x.y + y.y) * (1.f / tc::kKeysPerTile) - mean * mean, 0.f);
+      const float sd = fmaxf(sqrtf(var), fmaxf(1e-5f * fabsf(mean), 1e-20f));
+      width = sd * (6.f / kClsSampleBins);
+      inv_w = 1.f / width;
+      a_bin = mean + (P.bins_at - 3.f) * sd;
+      return;
+    }
+    if (row0 + (row & ~31) >= rows) return;   // the warp's rows are all padding
+    const int left = n_s - (tile - 1) * tc::kKeysPerTile - 64 * half;   // samples in the thread's 64 columns
+    const bool all = left >= 64;
+    const float shift = -a_bin * inv_w;
+    // the largest of every group of kGroup samples (-inf for columns that hold none)
+    float top[64 / kGroup];
+    tc::drain_raw(taddr, [&](int g, uint32_t (&r)[16]) {
+      if (!all) {
+#pragma unroll
+        for (int c = 0; c < 16; ++c)
+          if (16 * g + c >= left) r[c] = 0xFF800000u;
+      }
+#pragma unroll
+      for (int c = 0; c < 16; c += kGroup) {
+        float m = __uint_as_float(r[c]);
+#pragma unroll
+        for (int e = 1; e < kGroup; ++e) m = fmaxf(m, __uint_as_float(r[c + e]));
+        top[(16 * g + c) / kGroup] = m;
       }
     });
+#pragma unroll
+    for (int j = 0; j < 64 / kGroup; ++j) {
+      vmax = fmaxf(vmax, top[j]);
+      const float u = fminf(fmaxf(fmaf(top[j], inv_w, shift), 0.f), static_cast<float>(kClsSampleBins - 1));
+      const uint32_t addr = hist_row + static_cast<uint32_t>(__float2int_rz(u)) * (tc::kQRows * 2);
+      if (all || j * kGroup < left) asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(addr), "r"(inc) : "memory");   // the group has a sample
+    }
   };
-  if (!tc::scores_cta<true>(tc_smem, q_row, keys, C, tile_begin, tile_end, epilogue) && threadIdx.x == 0)
+  auto end = [&](const ClsSeg&, int lane_row, int part, bool) {
+    const int row = 128 * (part >> 1) + lane_row, half = part & 1;
+    stat[half][row].x = vmax;
+    tc::named_sync(tc::kBarDrain, tc::kDrainWarps * 32);
+    if (half != 0 || row0 + row >= rows) return;
+    int cum = 0;
+    float lo = kClsOpen, hi = INFINITY;
+    bool have_lo = false;
+    for (int i = kClsSampleBins - 1; i >= 1; --i) {
+      cum += static_cast<int>((hist[i * (tc::kQRows / 2) + (row >> 1)] >> ((row & 1) * 16)) & 0xFFFFu);
+      const float edge = a_bin + static_cast<float>(i) * width;
+      if (cum <= P.rank_hi[b]) hi = edge;
+      if (!have_lo && cum >= P.rank_lo[b]) { lo = edge; have_lo = true; }
+    }
+    const float ref = fmaxf(stat[0][row].x, stat[1][row].x) * P.scale_log2e;
+    bounds[static_cast<size_t>(b * P.n_kv_heads + h) * P.row_block + row0 + row] = make_float4(lo, hi, ref, 0.f);
+  };
+  if (!tc::segments_cta<false, tc::kStages, ClsSeg>(tc_smem, &samples, segment, q_row, begin, tile_fn, end, &user) && threadIdx.x == 0)
     atomicCAS(&err[0], 0, HKV_ERR_TIMEOUT);
 }
 
-// Whole block (kClsRowThreads threads, every one calls): the highest bin b of hist[0, nbins) with
+// ---------------------------------------------------------------------------------------------
+// Every logit of the pass.  The (row block, key tile) pairs of the whole pass are cut into one equal run per CTA;
+// accumulator lanes = rows, so a draining thread owns one row and half of every tile's keys, with the row's bounds,
+// sums and list position in registers.  An entry above the upper bound joins sum and count; one between the bounds is
+// appended, by predicated instructions, to the thread's own column of shared memory, which goes to the row's list in
+// groups of four.
+// Bound: issue slots (ten per warp and entry at 72 % of the scheduler's cycles; four warps per scheduler is all the
+// registers allow).  One context of 32768 keys against 7168 rows: 132 us = 2.8 us per 256 x 128 tile; with only the lower
+// bound tested here 133 us and lists twice as long, with slots advanced by sign arithmetic instead of predicates 158 us.
+// grid: P.n_cta.  partial: float4 [unit][row_block][seg_max][2] = (normaliser, sum above hi, number above hi, listed
+// entries; the sign bit of the last = the list was full), list: float [unit][row_block][2][list_stride].
+// ---------------------------------------------------------------------------------------------
+constexpr int kClsSlots = 48;          // listed entries a draining thread stages in shared memory
+constexpr int kClsScanRing = 2;          // key tiles in shared memory (the slots need the room of a third)
+constexpr int kClsScanSmem = tc::seg_smem_fixed(kClsScanRing) + tc::kDrainWarps * kClsSlots * 128;
+static_assert(kClsScanSmem <= 232448, "one CTA's shared memory");
+
+__device__ __forceinline__ float lds_f32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
+// entry v with weight p: above hi -> sum and count; between lo and hi -> stored at shared address `at`, which moves on (a
+// lane's slots are 128 bytes apart)
+__device__ __forceinline__ void cls_take(float v, float p, float lo, float hi, float& sum, int& cnt, uint32_t& at) {
+  asm volatile(
+      "{\n"
+      ".reg .pred up, in;\n"
+      "setp.gt.f32 up, %3, %6;\n"
+      "@up add.f32 %0, %0, %4;\n"
+      "@up add.s32 %1, %1, 1;\n"
+      "setp.ge.and.f32 in, %3, %5, !up;\n"
+      "@in st.shared.f32 [%2], %3;\n"
+      "@in add.u32 %2, %2, 128;\n"
+      "}\n"
+      : "+f"(sum), "+r"(cnt), "+r"(at)
+      : "f"(v), "f"(p), "f"(lo), "f"(hi)
+      : "memory");
+}
+
+__global__ void __launch_bounds__(tc::kSegThreads, 1)
+    cls_scan_kernel(const __grid_constant__ ClsParams P, const __grid_constant__ CUtensorMap keys, const __nv_bfloat16* q_text, const float4* bounds,
+                    float4* partial, float* list, int32_t* err) {
+  extern __shared__ __align__(16) uint8_t tc_smem[];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const int64_t w_begin = cls_cta_begin(P, blockIdx.x), w_end = cls_cta_begin(P, blockIdx.x + 1);
+
+  auto segment = [&](int s, ClsSeg& seg) {
+    const int64_t w = s == 0 ? w_begin : seg.next;
+    if (w >= w_end) return false;
+    int b = 0;
+    while (w >= P.w_prefix[b + 1]) ++b;
+    const int n_tiles = cls_tiles(P, b), n_blk = cls_blocks(P, b);
+    const int64_t in_b = w - P.w_prefix[b];
+    const int ub = static_cast<int>(in_b / n_tiles);          // row block within the sequence's heads
+    const int h = ub / n_blk;
+    const int64_t block_begin = P.w_prefix[b] + static_cast<int64_t>(ub) * n_tiles;
+    seg.b = b;
+    seg.unit = b * P.n_kv_heads + h;
+    seg.row0 = (ub - h * n_blk) * tc::kQRows;
+    seg.n_rows = min(tc::kQRows, cls_rows(P, b) - seg.row0);
+    seg.key_row0 = seg.unit * P.max_seq_len;
+    seg.C = P.C[b];
+    seg.tile_begin = static_cast<int>(w - block_begin);
+    seg.next = min(w_end, block_begin + n_tiles);
+    seg.tile_end = static_cast<int>(seg.next - block_begin);
+    seg.index = static_cast<int>(blockIdx.x) - cls_cta_of(P, block_begin);
+    return true;
+  };
+  auto q_row = [&](const ClsSeg& seg, int row) -> const __nv_bfloat16* {
+    return row < seg.n_rows ? cls_q_row(P, q_text, seg.b, seg.unit - seg.b * P.n_kv_heads, P.row_begin + seg.row0 + row) : nullptr;
+  };
+
+  const float sc = P.scale_log2e;
+  const uint64_t sc2 = tc::pack_f32x2(sc, sc);
+  uint64_t nref2 = 0;
+  float lo = 0.f, hi = 0.f, z = 0.f, zc = 0.f, top = 0.f, topc = 0.f;
+  int cnt = 0;
+  bool full = false, idle = false;
+  float4 *ptr = nullptr, *limit = nullptr, *first = nullptr;
+  uint32_t slots = 0, at = 0;      // the thread's staging slots and the next free one
+  uint8_t* user = nullptr;
+  auto begin = [&](const ClsSeg& seg, int lane_row, int part) {
+    const int row = 128 * (part >> 1) + lane_row;
+    const size_t rg = static_cast<size_t>(seg.unit) * P.row_block + seg.row0 + row;
+    idle = (row & ~31) >= seg.n_rows;          // the warp's rows are all padding
+    float4 bd = make_float4(INFINITY, INFINITY, 0.f, 0.f);   // a padding row takes nothing
+    if (row < seg.n_rows) bd = cls_bounds(bounds, rg);
+    lo = bd.x;
+    hi = bd.y;
+    nref2 = tc::pack_f32x2(-bd.z, -bd.z);
+    z = zc = top = topc = 0.f;
+    cnt = 0;
+    full = false;
+    first = ptr = reinterpret_cast<float4*>(list + (rg * 2 + (part & 1)) * P.list_stride + cls_list_at(P, seg.tile_begin, seg.index));
+    limit = first + ((seg.tile_end - seg.tile_begin) * P.per_tile + kClsSlack) / 4 - 2;
+    at = slots = smem_u32(user) + ((threadIdx.x >> 5) - 1) * (kClsSlots * 128) + (threadIdx.x & 31) * 4;
+  };
+  // whole groups of four staged entries go to the row's list, the newest first; up to three stay
+  auto flush = [&]() {
+    const int n4 = static_cast<int>((at - slots) / 512u);
+    if (ptr + n4 > limit) {   // the row is done otherwise
+      full = true;
+      lo = INFINITY;
+      at = slots;
+      return;
+    }
+    for (const uint32_t end = at - 512u * n4; at != end;) {
+      at -= 512u;
+      __stcg(ptr++, make_float4(lds_f32(at), lds_f32(at + 128), lds_f32(at + 256), lds_f32(at + 384)));
+    }
+  };
+  auto tile_fn = [&](const ClsSeg& seg, int tile, int, int part, uint32_t taddr) {
+    if (idle) return;
+    const int left = seg.C - (tile * tc::kKeysPerTile + 64 * (part & 1));   // keys of the thread's 64 columns that exist
+    tc::drain_raw(taddr, [&](int g, uint32_t (&r)[16]) {
+      if (left < 64) {
+#pragma unroll
+        for (int c = 0; c < 16; ++c)
+          if (16 * g + c >= left) r[c] = 0xFF800000u;   // -inf: no weight, below every bound
+      }
+      if (__any_sync(0xffffffffu, at - slots > (kClsSlots - 16) * 128u)) flush();   // room for 16 more in every lane
+      uint64_t z2 = 0;
+      float t0 = 0.f, t1 = 0.f;
+#pragma unroll
+      for (int c = 0; c < 16; c += 2) {
+        const float v0 = __uint_as_float(r[c]), v1 = __uint_as_float(r[c + 1]);
+        float e0, e1;
+        tc::unpack_f32x2(tc::fma_f32x2(tc::pack_f32x2(v0, v1), sc2, nref2), e0, e1);
+        const float p0 = fast_exp2(e0), p1 = fast_exp2(e1);
+        z2 = tc::add_f32x2(z2, tc::pack_f32x2(p0, p1));
+        cls_take(v0, p0, lo, hi, t0, cnt, at);
+        cls_take(v1, p1, lo, hi, t1, cnt, at);
+      }
+      float a, b2;
+      tc::unpack_f32x2(z2, a, b2);
+      tc::add_compensated(z, zc, a + b2);
+      tc::add_compensated(top, topc, t0 + t1);
+    });
+  };
+  auto end = [&](const ClsSeg& seg, int lane_row, int part, bool) {
+    const int row = 128 * (part >> 1) + lane_row;
+    if (row >= seg.n_rows) return;
+    const size_t rg = static_cast<size_t>(seg.unit) * P.row_block + seg.row0 + row;
+    flush();
+    const uint32_t rest = (at - slots) / 128u;
+    if (rest) {
+      const float4 v = make_float4(lds_f32(slots), lds_f32(slots + 128), lds_f32(slots + 256), 0.f);
+      __stcg(ptr, v);   // limit leaves room for it
+    }
+    const uint32_t n = (static_cast<uint32_t>(ptr - first) * 4 + rest) | (full ? 0x80000000u : 0u);
+    partial[(rg * P.seg_max + seg.index) * 2 + (part & 1)] = make_float4(z, top, __int_as_float(cnt), __uint_as_float(n));
+  };
+  if (!tc::segments_cta<false, kClsScanRing, ClsSeg>(tc_smem, &keys, segment, q_row, begin, tile_fn, end, &user) &&
+      threadIdx.x == 0)
+    atomicCAS(&err[0], 0, HKV_ERR_TIMEOUT);
+}
+
+// ---------------------------------------------------------------------------------------------
+// Per row: the sums' parts in a fixed order, then the exact sum of the largest listed entries that are still missing from
+// the k.  A warp owns a row; its entries (a few per cent of the context) are gathered into shared memory.  Pass 1 counts them against four
+// thresholds around the place where the k-th largest should lie (interpolated between the bounds), which leaves about a
+// hundred entries undecided; pass 2 adds up what lies above and moves the undecided to the front of each lane's part,
+// where the threshold is closed in on exactly, interpolating and halving the order-preserving keys in turn.
+// Bound: instructions, about 1500 per warp and row.  cap: float4s of shared memory per warp (a longer list is walked in
+// global memory).
+// ---------------------------------------------------------------------------------------------
+constexpr int kClsUndecided = 256;   // entries the last stage takes over (eight per lane)
+__device__ __forceinline__ float cls_key_float(uint32_t key) {   // inverse of float_key
+  return __uint_as_float((key & 0x80000000u) ? (key ^ 0x80000000u) : ~key);
+}
+
+__global__ void __launch_bounds__(256, 3)
+    cls_select_kernel(const __grid_constant__ ClsParams P, const float4* bounds, const float4* partial, const float* list, float* rowsum,
+                      int32_t* n_flag, int32_t* flagged, int total_rows, int cap) {
+  extern __shared__ __align__(16) float4 sel_smem[];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  float4* buf = sel_smem + warp * cap;
+  const int idx = blockIdx.x * (blockDim.x >> 5) + warp;
+  const int unit = idx / P.row_block, row = idx - unit * P.row_block, b = min(unit / P.n_kv_heads, P.n_batch - 1);
+  const bool exists = idx < total_rows && row < cls_rows(P, b);
+  const int n_tiles = cls_tiles(P, b), blk = row / tc::kQRows;
+  const int64_t w0 = P.w_prefix[b] + (static_cast<int64_t>(unit - b * P.n_kv_heads) * cls_blocks(P, b) + blk) * n_tiles;
+  const int i0 = cls_cta_of(P, w0), n_rec = 2 * (cls_cta_of(P, w0 + n_tiles - 1) - i0 + 1);
+  const size_t rg = static_cast<size_t>(unit) * P.row_block + row;
+  const float4* part = partial + rg * P.seg_max * 2;
+  // offset of a record's entries, in float4s
+  auto rec_at = [&](int rec) {
+    const int sg = rec >> 1;
+    const int tile0 = sg == 0 ? 0 : static_cast<int>(cls_cta_begin(P, i0 + sg) - w0);
+    return ((rec & 1) * P.list_stride + cls_list_at(P, tile0, sg)) >> 2;
+  };
+  const float4* row_list = reinterpret_cast<const float4*>(list + rg * 2 * P.list_stride);
+  int my_at = rec_at(min(lane, n_rec - 1));   // record `lane`, before the wait
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (!exists) return;
+
+  const float4 bd = cls_bounds(bounds, rg);
+  float z = 0.f, s = 0.f;
+  int above = 0, n = 0, n4 = 0;
+  bool bad = false;
+  for (int r0 = 0; r0 < n_rec; r0 += 32) {
+    float4 rec = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (r0 + lane < n_rec) rec = __ldcg(part + r0 + lane);
+    if (r0 > 0) my_at = rec_at(min(r0 + lane, n_rec - 1));
+    z += rec.x;
+    s += rec.y;
+    above += __float_as_int(rec.z);
+    const uint32_t m = __float_as_uint(rec.w);
+    bad = bad || (m >> 31);
+    const int cnt = static_cast<int>(m & 0x7FFFFFFFu), cnt4 = (cnt + 3) >> 2;
+    n += __reduce_add_sync(0xffffffffu, cnt);
+    int incl = cnt4;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, incl, off);
+      if (lane >= off) incl += x;
+    }
+    const int to = n4 + incl - cnt4;
+    n4 += __shfl_sync(0xffffffffu, incl, 31);
+    if (n4 <= cap) {
+      // eight lanes per record, four records at a time; what the last float4 holds behind the end becomes -inf, which
+      // no comparison below takes
+      for (int r = lane >> 3; r < 32 && r0 + (r & ~3) < n_rec; r += 4) {
+        const int c = __shfl_sync(0xffffffffu, cnt, r), o = __shfl_sync(0xffffffffu, to, r), at = __shfl_sync(0xffffffffu, my_at, r);
+#pragma unroll 4
+        for (int e = lane & 7; 4 * e < c; e += 8) {
+          float4 v = __ldcg(row_list + at + e);
+          if (4 * e + 4 > c) {
+            if (4 * e + 1 >= c) v.y = -INFINITY;
+            if (4 * e + 2 >= c) v.z = -INFINITY;
+            v.w = -INFINITY;
+          }
+          buf[o + e] = v;
+        }
+        __syncwarp();
+      }
+    }
+  }
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) z += __shfl_xor_sync(0xffffffffu, z, off);
+  above = __reduce_add_sync(0xffffffffu, above);
+  __syncwarp();
+  const int need = P.k[b] - above;
+  bad = __any_sync(0xffffffffu, bad) || need < 0 || need > n || !(z > 0.f && z < INFINITY);
+  if (bad) {
+    if (lane == 0) flagged[atomicAdd(n_flag, 1)] = idx;
+    return;
+  }
+  const bool in_smem = n4 <= cap;
+  // fn(four entries) on this lane's share of the list, the same number of times in every lane; absent ones are -inf
+  auto each4 = [&](auto fn) {
+    const float4 none = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+    if (in_smem) {
+#pragma unroll 2
+      for (int e = 0; e < n4; e += 32) fn(e + lane < n4 ? buf[e + lane] : none);
+    } else {
+      for (int r = 0; r < n_rec; ++r) {
+        const int c = static_cast<int>(__float_as_uint(__ldcg(&part[r].w)) & 0x7FFFFFFFu);
+        const float4* src = row_list + rec_at(r);
+        for (int e0 = 0; 4 * e0 < c; e0 += 32) {
+          const int e = e0 + lane;
+          float4 v = 4 * e < c ? __ldcg(src + e) : none;
+          if (4 * e + 1 >= c) v.y = -INFINITY;
+          if (4 * e + 2 >= c) v.z = -INFINITY;
+          if (4 * e + 3 >= c) v.w = -INFINITY;
+          fn(v);
+        }
+      }
+    }
+  };
+  const float ref = bd.z, sc = P.scale_log2e;
+  auto weight = [&](float v) { return fast_exp2(fmaf(v, sc, -ref)); };   // as the scan computes it
+
+  // The bracket: ca entries are >= a (ca >= need), cb < need are > bb.
+  float a = bd.x, bb = bd.y;
+  int ca = n, cb = 0;
+  auto narrow = [&](float x, int c) {   // c entries are >= x
+    if (!(x > a && x <= bb)) return;
+    if (c >= need) { a = x; ca = c; }
+    else { bb = cls_key_float(float_key(x) - 1u); cb = c; }
+  };
+  auto count2 = [&](float x0, float x1) {
+    int c0 = 0, c1 = 0;
+    each4([&](const float4& v) {
+      c0 += v.x >= x0; c1 += v.x >= x1;
+      c0 += v.y >= x0; c1 += v.y >= x1;
+      c0 += v.z >= x0; c1 += v.z >= x1;
+      c0 += v.w >= x0; c1 += v.w >= x1;
+    });
+    narrow(x0, __reduce_add_sync(0xffffffffu, c0));
+    narrow(x1, __reduce_add_sync(0xffffffffu, c1));
+  };
+  if (need > 0 && need < n && (bb == INFINITY || !(a > kClsOpen))) {   // open on a side: the list's own range
+    float mn = INFINITY, mx = -INFINITY;
+    each4([&](const float4& v) {
+      if (v.x > -INFINITY) mn = fminf(mn, v.x);
+      if (v.y > -INFINITY) mn = fminf(mn, v.y);
+      if (v.z > -INFINITY) mn = fminf(mn, v.z);
+      if (v.w > -INFINITY) mn = fminf(mn, v.w);
+      mx = fmaxf(mx, fmaxf(fmaxf(v.x, v.y), fmaxf(v.z, v.w)));
+    });
+#pragma unroll
+    for (int off = 16; off >= 1; off >>= 1) {
+      mn = fminf(mn, __shfl_xor_sync(0xffffffffu, mn, off));
+      mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
+    }
+    a = fmaxf(a, mn);
+    bb = fminf(bb, mx);
+  }
+  auto place = [&]() { return a + (bb - a) * (static_cast<float>(ca - need) / static_cast<float>(ca - cb)); };
+  auto middle = [&](uint32_t num) {   // num quarters of the way up the keys, always inside (a, bb]
+    const uint32_t ka = float_key(a), kd = float_key(bb) - ka;
+    return cls_key_float(ka + kd / 4u * num + (num < 4u ? 1u : kd % 4u));
+  };
+  for (int it = 0; need > 0 && ca != need && a < bb && (!in_smem || ca - cb > kClsUndecided); ++it) {
+    const float x = place(), w = bb - a;
+    if (it < 3) count2(x - 0.07f * w, x + 0.07f * w);
+    else count2(middle(2), x);
+  }
+  // everything above the bracket; its own entries, if they still have to be ranked, move to the front of the buffer, a
+  // column per lane: after e iterations a column holds at most 4 e entries, the 32 e float4s that have been read (cap is
+  // a multiple of 32)
+  const bool ranked = need > 0 && ca != need && a < bb;
+  const float from = need == 0 ? INFINITY : ca == need ? a : cls_key_float(float_key(bb) + 1u);
+  if (!ranked) {
+    each4([&](const float4& v) {
+      s += (v.x >= from ? weight(v.x) : 0.f) + (v.y >= from ? weight(v.y) : 0.f);
+      s += (v.z >= from ? weight(v.z) : 0.f) + (v.w >= from ? weight(v.w) : 0.f);
+    });
+  } else {
+    const uint32_t column = smem_u32(buf) + lane * 4;
+    uint32_t at = column;
+    int unused = 0;
+    for (int e = 0; e < n4; e += 32) {
+      const float4 v = e + lane < n4 ? buf[e + lane] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+      __syncwarp();
+      cls_take(v.x, weight(v.x), a, bb, s, unused, at);
+      cls_take(v.y, weight(v.y), a, bb, s, unused, at);
+      cls_take(v.z, weight(v.z), a, bb, s, unused, at);
+      cls_take(v.w, weight(v.w), a, bb, s, unused, at);
+    }
+    const int mine = static_cast<int>((at - column) / 128u), base = cb;
+    float own[8];                    // the usual number in registers, more stay where they are
+#pragma unroll
+    for (int j = 0; j < 8; ++j) own[j] = j < mine ? lds_f32(column + 128u * j) : -INFINITY;
+    for (int it = 0; ca != need && a < bb; ++it) {
+      float x = place();
+      if ((it & 1) || !(x > a && x <= bb)) x = middle(2);
+      int c = 0;
+#pragma unroll
+      for (int j = 0; j < 8; ++j) c += own[j] >= x;
+      for (int j = 8; j < mine; ++j) c += lds_f32(column + 128u * j) >= x;
+      narrow(x, base + __reduce_add_sync(0xffffffffu, c));
+    }
+    const float rest = ca == need ? a : cls_key_float(float_key(bb) + 1u);
+#pragma unroll
+    for (int j = 0; j < 8; ++j) s += own[j] >= rest ? weight(own[j]) : 0.f;
+    for (int j = 8; j < mine; ++j) {
+      const float v = lds_f32(column + 128u * j);
+      s += v >= rest ? weight(v) : 0.f;
+    }
+  }
+  if (need > 0 && ca != need && lane == 0) s += static_cast<float>(need - cb) * weight(a);   // copies of one value: need - cb of them count
+#pragma unroll
+  for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+  if (lane == 0) rowsum[static_cast<size_t>(unit) * P.r_stride + P.row_begin + row] = s / z;
+}
+
+// Whole block (kClsFixThreads threads, every one calls): the highest bin b of hist[0, nbins) with
 // count(bins > b) < need <= count(bins >= b).  ctl[0] = b, ctl[1] = need - count(bins > b),
 // ctl[2] = count(b); visible after the caller's next barrier.  nbins is 4096, 1024 or 256; wsum is
 // scratch for 32 ints.
@@ -148,32 +658,28 @@ __device__ __forceinline__ void cls_find_bin(const int* hist, int nbins, int nee
 }
 
 // ---------------------------------------------------------------------------------------------
-// Sum of the k largest softmax entries of every row; a persistent CTA takes one row at a time.
-// The row's logits arrive in shared memory by bulk copy (the next row is meanwhile prefetched into
-// L2) and are replaced by p = 2^(l - max) in [0, 1], whose float bits order like the values.  The
-// k-th largest p is found exactly: a histogram over bits 30..18 of p (32 bins per octave, so the
-// lanes of a warp rarely meet in a bin), then the threshold bin's entries are sorted outright (four
-// threads per entry) and the first `need` of them join the sum of everything above the bin; a
-// crowded bin is first narrowed by histograms over bits 17..8 and 7..0.  Sums run in a fixed
-// order, so the result is deterministic.
-// rowsum: float [unit][r_stride]
+// Flagged rows, a CTA each: every logit of the row into one buffer (shared memory, or the lists' memory for rows beyond
+// kClsSmemCols), then p = 2^(l - max) in [0, 1], whose float bits order like the values.  The k-th largest p is found
+// exactly: a histogram over bits 30..18 of p (32 bins per octave, so the lanes of a warp rarely meet in a bin), then the
+// threshold bin's entries are sorted outright (four threads per entry) and the first `need` of them join the sum of
+// everything above the bin; a crowded bin is first narrowed by histograms over bits 17..8 and 7..0.  Sums run in a
+// fixed order, so the result is deterministic.  The logits come from 16-key x 8-column tensor-core tiles of which one
+// column is used: 16 bytes of a key's row per load, the products' order of summation permuted alike on both operands.
 // ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(kClsRowThreads)
-    cls_row_kernel(const ClsParams P, float* logits, float* rowsum, int rows_pass, int total_rows) {
+__global__ void __launch_bounds__(kClsFixThreads)
+    cls_fix_kernel(const __grid_constant__ ClsParams P, const __nv_bfloat16* kin, const __nv_bfloat16* q_text, float* rowsum,
+                   const int32_t* n_flag, const int32_t* flagged, float* rows_mem, int row_pitch, int smem_cols) {
   extern __shared__ __align__(16) uint8_t cls_smem[];
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   int* hist = reinterpret_cast<int*>(cls_smem);                   // [kClsBins]
   uint32_t* cand = reinterpret_cast<uint32_t*>(hist + kClsBins);  // [kClsRank]
   float* red = reinterpret_cast<float*>(cand + kClsRank);         // [32]
   int* ctl = reinterpret_cast<int*>(red + 32);                    // [8]
   int* wsum = ctl + 8;                                            // [32]
-  uint64_t* bar = reinterpret_cast<uint64_t*>(wsum + 32);         // [kClsLoadParts]
-  float* srow = reinterpret_cast<float*>(cls_smem + kClsRowScratch);
+  uint4* qs = reinterpret_cast<uint4*>(wsum + 32);                // the row's query, 16 pieces
+  float* srow = reinterpret_cast<float*>(cls_smem + kClsFixScratch);
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) {
-    for (int i = 0; i < kClsLoadParts; ++i) mbar_init(bar + i, 1);
-    mbar_fence_init();
-  }
-  uint32_t phases = 0;   // bit i: parity the next wait on barrier i looks for
 
   // block-wide reductions in a fixed order; every thread gets the result
   auto block_sum = [&](float v) {
@@ -198,70 +704,54 @@ __global__ void __launch_bounds__(kClsRowThreads)
     for (int off = 16; off >= 1; off >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, off));
     return v;
   };
-  // row `idx` of the pass: its unit, length and place; false for the rows a short sequence does not have
-  auto locate = [&](int idx, int* unit, int* C, int* r, size_t* off) {
-    if (idx >= total_rows) return false;
-    *unit = idx / rows_pass;
-    const int rr = idx - *unit * rows_pass, b = *unit / P.n_kv_heads;
-    *C = P.C[b];
-    *r = P.row_begin + rr;
-    *off = (static_cast<size_t>(*unit) * P.row_block + rr) * P.c_stride;
-    return *r < P.T[b] * P.group;
-  };
 
-  for (int idx = blockIdx.x; idx < total_rows; idx += gridDim.x) {
-    int unit, C, r;
-    size_t row_off;
-    if (!locate(idx, &unit, &C, &r, &row_off)) continue;
-    const int k = P.k[unit / P.n_kv_heads];
-    const bool staged = C <= P.smem_cols;
-    // p overwrites the logits: in shared memory, or for longer rows in place in the workspace
-    float* row = staged ? srow : logits + row_off;
+  const int n_rows = *n_flag;
+  for (int f = blockIdx.x; f < n_rows; f += gridDim.x) {
+    const int idx = flagged[f];
+    const int unit = idx / P.row_block, r = P.row_begin + (idx - unit * P.row_block), b = unit / P.n_kv_heads;
+    const int C = P.C[b], k = P.k[b];
+    float* row = C <= smem_cols ? srow : rows_mem + static_cast<size_t>(blockIdx.x) * row_pitch;
     float4* row4 = reinterpret_cast<float4*>(row);
     const int n4 = (C + 3) >> 2;
-    // the row arrives in kClsLoadParts pieces of part4 float4s (a multiple of the block size), each on its own barrier
-    const int part4 = ((n4 + kClsLoadParts - 1) / kClsLoadParts + kClsRowThreads - 1) / kClsRowThreads * kClsRowThreads;
-
     __syncthreads();   // the previous row's readers are done with the buffers
-    if (tid == 0 && staged) {
-      // whole 16-byte pieces: rows start 256-byte aligned and are padded to a multiple of 128 floats
-      fence_proxy_async();
-      for (int part = 0; part < kClsLoadParts; ++part) {
-        const int beg = part * part4, end = min(n4, beg + part4);
-        if (beg >= end) break;
-        mbar_arrive_expect_tx(bar + part, static_cast<uint32_t>(end - beg) * 16u);
-        for (int o = beg; o < end; o += 2048)
-          bulk_g2s(row4 + o, reinterpret_cast<const float4*>(logits + row_off) + o,
-                   static_cast<uint32_t>(min(2048, end - o)) * 16u, bar + part);
-      }
-      // start the next row's trip from HBM to L2 meanwhile
-      int u2, C2, r2;
-      size_t off2;
-      if (locate(idx + gridDim.x, &u2, &C2, &r2, &off2) && C2 <= P.smem_cols) {
-        const uint32_t b2 = static_cast<uint32_t>((C2 + 3) / 4 * 16);
-        for (uint32_t o = 0; o < b2; o += 32768u)
-          bulk_prefetch_l2(reinterpret_cast<const char*>(logits + off2) + o, min(32768u, b2 - o));
+    if (tid < 16) qs[tid] = reinterpret_cast<const uint4*>(cls_q_row(P, q_text, b, unit - b * P.n_kv_heads, r))[tid];
+    for (int i = tid; i < kClsBins; i += kClsFixThreads) hist[i] = 0;
+    if (tid == 0) ctl[3] = 0;
+    // floats between C and the next multiple of four: -inf, that is p = 0, which no top-k sum can feel
+    if (tid < 4 * n4 - C) row[C + tid] = -INFINITY;
+    __syncthreads();
+    float mx = -INFINITY;
+    {
+      const uint4* kp = reinterpret_cast<const uint4*>(cls_keys(P, kin, unit));
+      const int g = lane >> 2, t = lane & 3;
+      uint4 q[4];
+#pragma unroll
+      for (int kb = 0; kb < 4; ++kb) q[kb] = g == 0 ? qs[kb * 4 + t] : make_uint4(0u, 0u, 0u, 0u);
+      for (int j0 = warp * 16; j0 < C; j0 += kClsFixThreads / 32 * 16) {
+        const uint4* k0 = kp + static_cast<size_t>(min(j0 + g, C - 1)) * 16 + t;
+        const uint4* k1 = kp + static_cast<size_t>(min(j0 + g + 8, C - 1)) * 16 + t;
+        uint4 x[4], y[4];
+#pragma unroll
+        for (int kb = 0; kb < 4; ++kb) { x[kb] = __ldg(k0 + kb * 4); y[kb] = __ldg(k1 + kb * 4); }
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int kb = 0; kb < 4; ++kb) {
+          mma_bf16(acc, x[kb].x, y[kb].x, x[kb].y, y[kb].y, q[kb].x, q[kb].y);
+          mma_bf16(acc, x[kb].z, y[kb].z, x[kb].w, y[kb].w, q[kb].z, q[kb].w);
+        }
+        if (t == 0) {
+          const float l0 = acc[0] * P.scale_log2e, l1 = acc[2] * P.scale_log2e;
+          if (j0 + g < C) { row[j0 + g] = l0; mx = fmaxf(mx, l0); }
+          if (j0 + g + 8 < C) { row[j0 + g + 8] = l1; mx = fmaxf(mx, l1); }
+        }
       }
     }
-    for (int i = tid; i < kClsBins; i += kClsRowThreads) hist[i] = 0;
-    if (tid == 0) ctl[3] = 0;
+    const float M = block_max(mx);   // its barriers also publish the row
 
-    // Rows of up to kClsRegItems floats per thread stay in REGISTERS from the moment they land: the maximum, the
-    // probabilities, the histogram and the final sum are then computed without another trip through shared memory.
-    // Longer rows keep p in the row buffer (shared memory, or the workspace) and are walked again per pass.
-    const bool regs = staged && n4 <= kClsRegVecs * kClsRowThreads;
-    float4 rv[kClsRegVecs];
     // visits every float4 this thread owns (p once the probabilities exist)
     auto each4 = [&](auto fn) {
-      if (regs) {
-#pragma unroll
-        for (int q = 0; q < kClsRegVecs; ++q) {
-          if (q * kClsRowThreads + tid < n4) fn(rv[q]);
-        }
-      } else {
 #pragma unroll 4
-        for (int i = tid; i < n4; i += kClsRowThreads) fn(row4[i]);
-      }
+      for (int i = tid; i < n4; i += kClsFixThreads) fn(row4[i]);
     };
     auto each = [&](auto fn) {
       each4([&](const float4& v) { fn(v.x); fn(v.y); fn(v.z); fn(v.w); });
@@ -279,99 +769,22 @@ __global__ void __launch_bounds__(kClsRowThreads)
       return (t0 + t1) + (t2 + t3);
     };
 
-    // maximum, piece by piece as the row lands; the up to three floats between C and the next
-    // multiple of four become -inf, that is p = 0: zeros below every real entry, which no top-k
-    // sum can feel
-    float mx = -INFINITY;
-    bool landed = true;
-    auto tail_fix = [&](float4& v, int i) {
-      if (i == n4 - 1 && (C & 3)) {
-        if ((C & 3) < 2) v.y = -INFINITY;
-        if ((C & 3) < 3) v.z = -INFINITY;
-        v.w = -INFINITY;
-      }
-    };
-    if (regs) {
-      static_assert(kClsLoadParts == 4, "piece index by three comparisons");
-      const int m4 = part4 / kClsRowThreads;   // blocks of kClsRowThreads vectors per piece
-      uint32_t waited = 0u;
-#pragma unroll
-      for (int q = 0; q < kClsRegVecs; ++q) {
-        rv[q] = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
-        if (q * kClsRowThreads < n4) {                       // the whole block of 1024 vectors lies in one piece
-          const int part = (q >= m4) + (q >= 2 * m4) + (q >= 3 * m4);   // = q * kClsRowThreads / part4
-          if (landed && !((waited >> part) & 1u)) {
-            landed = mbar_wait_bounded(bar + part, (phases >> part) & 1u);
-            phases ^= 1u << part;
-            waited |= 1u << part;
-          }
-          const int i = q * kClsRowThreads + tid;
-          if (landed && i < n4) {
-            float4 v = row4[i];
-            tail_fix(v, i);
-            rv[q] = v;
-            mx = fmaxf(fmaxf(mx, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));
-          }
-        }
-      }
-      // pieces past the row's end were never armed; pieces armed but not visited cannot exist (every armed piece
-      // holds at least one block of vectors)
-    } else {
-      for (int part = 0; part < kClsLoadParts; ++part) {
-        const int beg = part * part4, end = min(n4, beg + part4);
-        if (beg >= end) break;
-        if (staged && landed) {
-          landed = mbar_wait_bounded(bar + part, (phases >> part) & 1u);
-          phases ^= 1u << part;
-        }
-        if (!landed) continue;
-        for (int i = beg + tid; i < end; i += kClsRowThreads) {
-          float4 v = row4[i];
-          if (i == n4 - 1 && (C & 3)) {
-            tail_fix(v, i);
-            row4[i] = v;
-          }
-          mx = fmaxf(fmaxf(mx, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));
-        }
-      }
-    }
-    if (__syncthreads_or(!landed)) {   // never seen; the whole CTA leaves, the row's sum and the score become NaN
-      if (tid == 0) rowsum[static_cast<size_t>(unit) * P.r_stride + r] = __int_as_float(0x7FC00000);
-      return;
-    }
-    const float M = block_max(mx);
-
     // p, normaliser, histogram
     auto prob = [&](float l) {
       // a NaN logit counts as no attention (fmaxf returns its other operand); every bit pattern stays in [0, bits(1)]
       return fminf(fmaxf(fast_exp2(l - M), 0.f), 1.f);
     };
     float z = 0.f;
-    if (regs) {
-#pragma unroll
-      for (int q = 0; q < kClsRegVecs; ++q) {
-        if (q * kClsRowThreads + tid < n4) {
-          const float4 pq = make_float4(prob(rv[q].x), prob(rv[q].y), prob(rv[q].z), prob(rv[q].w));
-          rv[q] = pq;
-          z += (pq.x + pq.y) + (pq.z + pq.w);
-          atomicAdd(&hist[__float_as_uint(pq.x) >> kClsShift], 1);
-          atomicAdd(&hist[__float_as_uint(pq.y) >> kClsShift], 1);
-          atomicAdd(&hist[__float_as_uint(pq.z) >> kClsShift], 1);
-          atomicAdd(&hist[__float_as_uint(pq.w) >> kClsShift], 1);
-        }
-      }
-    } else {
 #pragma unroll 4
-      for (int i = tid; i < n4; i += kClsRowThreads) {
-        const float4 v = row4[i];
-        const float4 q = make_float4(prob(v.x), prob(v.y), prob(v.z), prob(v.w));
-        row4[i] = q;
-        z += (q.x + q.y) + (q.z + q.w);
-        atomicAdd(&hist[__float_as_uint(q.x) >> kClsShift], 1);
-        atomicAdd(&hist[__float_as_uint(q.y) >> kClsShift], 1);
-        atomicAdd(&hist[__float_as_uint(q.z) >> kClsShift], 1);
-        atomicAdd(&hist[__float_as_uint(q.w) >> kClsShift], 1);
-      }
+    for (int i = tid; i < n4; i += kClsFixThreads) {
+      const float4 v = row4[i];
+      const float4 q = make_float4(prob(v.x), prob(v.y), prob(v.z), prob(v.w));
+      row4[i] = q;
+      z += (q.x + q.y) + (q.z + q.w);
+      atomicAdd(&hist[__float_as_uint(q.x) >> kClsShift], 1);
+      atomicAdd(&hist[__float_as_uint(q.y) >> kClsShift], 1);
+      atomicAdd(&hist[__float_as_uint(q.z) >> kClsShift], 1);
+      atomicAdd(&hist[__float_as_uint(q.w) >> kClsShift], 1);
     }
     const float Z = block_sum(z);   // its barriers also publish the histogram
     cls_find_bin(hist, kClsBins, k, ctl, wsum);
@@ -437,7 +850,7 @@ __global__ void __launch_bounds__(kClsRowThreads)
       const int width = shift == kClsShift ? 10 : 8;
       const int nshift = shift - width;
       const uint32_t mask = (1u << width) - 1u;
-      for (int i = tid; i < (1 << width); i += kClsRowThreads) hist[i] = 0;
+      for (int i = tid; i < (1 << width); i += kClsFixThreads) hist[i] = 0;
       __syncthreads();
       each([&](float e) {
         const uint32_t u = __float_as_uint(e);
@@ -456,321 +869,12 @@ __global__ void __launch_bounds__(kClsRowThreads)
   }
 }
 
-// ---------------------------------------------------------------------------------------------
-// The same row sums for rows of up to kClsRegCols entries, every entry in a register of the CTA
-// (kClsRegThreads threads x 32 entries), as a two-row pipeline: a row lands in shared memory in
-// pieces of one vector per thread, each on its own mbarrier; once every thread has taken its
-// entries into registers (the first block barrier of the row) one thread starts the NEXT row's
-// copies into the same buffer, so they travel while this row's probabilities, histogram,
-// threshold and sums are computed.  That thread also works out where the next row lies and hands
-// it over through a two-slot descriptor in shared memory.  Arithmetic as in cls_row_kernel; sums in
-// a fixed order.  (Measured and dropped: 512 threads of 64 entries -- a sixth fewer instructions,
-// but a quarter slower with half the warps to hide latency; the threshold bin ranked by one warp
-// after the last barrier -- slower than ranking it with the whole block between two barriers.)
-// ---------------------------------------------------------------------------------------------
-constexpr int kClsRegCols = 32768;
-constexpr int kClsRegThreads = 1024;   // 512 threads x 128 entries issue a sixth fewer instructions but hide less latency: slower
-constexpr int kClsRegWarps = kClsRegThreads / 32;
-constexpr int kClsRegVecsT = kClsRegCols / 4 / kClsRegThreads;   // float4s per thread: 16
-// histogram, candidates, their sorted copy, three reduction slots, control words, warp sums, two row descriptors,
-// piece barriers
-constexpr int kClsRegScratch = (kClsBins + 2 * kClsRank + 3 * 32 + 8 + 32 + 2 * 8) * 4 + kClsRegVecsT * 8;
-static_assert(kClsRegScratch % 16 == 0, "the row buffer is 16-byte aligned");
-constexpr int kClsRegBinsPer = kClsBins / kClsRegThreads;   // bins a thread sums in the threshold search
-static_assert((kClsRegBinsPer == 4 || kClsRegBinsPer == 8) && kClsRegVecsT <= 32, "whole int4s of bins per thread; one phase bit per piece");
-
-// cls_find_bin for a block of kClsRegThreads threads (nbins 4096, 1024 or 256).
-__device__ __forceinline__ void cls_find_bin_regs(const int* hist, int nbins, int need, int* ctl, int* wsum) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int per = nbins == kClsBins ? kClsRegBinsPer : nbins > kClsRegThreads ? nbins / kClsRegThreads : 1;   // 4 or 8; 2 or 1; 1
-  int loc[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-  if (nbins == kClsBins) {
-    const int4 u = reinterpret_cast<const int4*>(hist)[tid * (kClsRegBinsPer / 4)];
-    loc[0] = u.x; loc[1] = u.y; loc[2] = u.z; loc[3] = u.w;
-    if (kClsRegBinsPer == 8) {
-      const int4 v = reinterpret_cast<const int4*>(hist)[tid * 2 + 1];
-      loc[4] = v.x; loc[5] = v.y; loc[6] = v.z; loc[7] = v.w;
-    }
-  } else if (per == 2) {
-    const int2 u = reinterpret_cast<const int2*>(hist)[tid];
-    loc[0] = u.x; loc[1] = u.y;
-  } else if (tid < nbins) {
-    loc[0] = hist[tid];
-  }
-  const int tot = ((loc[0] + loc[1]) + (loc[2] + loc[3])) + ((loc[4] + loc[5]) + (loc[6] + loc[7]));
-  int run = tot;   // becomes the sum over this and the higher lanes of the warp
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const int v = __shfl_down_sync(0xffffffffu, run, off);
-    if (lane + off < 32) run += v;
-  }
-  if (lane == 0) wsum[warp] = run;
-  __syncthreads();
-  const int wt = lane < kClsRegWarps ? wsum[lane] : 0;
-  int wrun = wt;   // sum over warps >= lane
-#pragma unroll
-  for (int off = 1; off < 32; off <<= 1) {
-    const int v = __shfl_down_sync(0xffffffffu, wrun, off);
-    if (lane + off < 32) wrun += v;
-  }
-  int acc = __shfl_sync(0xffffffffu, wrun - wt, warp) + run - tot;   // items in the bins above this thread's
-  if (acc < need && need <= acc + tot) {
-#pragma unroll
-    for (int j = 7; j >= 0; --j) {
-      if (j < per && acc < need && need <= acc + loc[j]) {
-        ctl[0] = tid * per + j;
-        ctl[1] = need - acc;
-        ctl[2] = loc[j];
-      }
-      if (j < per) acc += loc[j];
-    }
-  }
-}
-
-__global__ void __launch_bounds__(kClsRegThreads)
-    cls_row_regs_kernel(const ClsParams P, const float* logits, float* rowsum, int rows_pass, int total_rows) {
-  extern __shared__ __align__(16) uint8_t cls_smem[];
-  int* hist = reinterpret_cast<int*>(cls_smem);                   // [kClsBins]
-  uint32_t* cand = reinterpret_cast<uint32_t*>(hist + kClsBins);  // [kClsRank]
-  float* sorted = reinterpret_cast<float*>(cand + kClsRank);      // [kClsRank]: the threshold bin in descending order
-  float* red = sorted + kClsRank;                                 // [3][32]: one slot per reduction of a row
-  int* ctl = reinterpret_cast<int*>(red + 3 * 32);                // [8]
-  int* wsum = ctl + 8;                                            // [32]
-  int* desc = wsum + 32;                                          // [2][8]: idx (-1: none), unit, C, r, k, offset lo, hi
-  uint64_t* bar = reinterpret_cast<uint64_t*>(desc + 16);         // [kClsRegVecsT]
-  float4* srow4 = reinterpret_cast<float4*>(cls_smem + kClsRegScratch);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-
-  // thread 0 only: the first row at or after `idx` (stride gridDim.x) that exists -> descriptor slot, and its copies
-  auto post_row = [&](int idx, int slot) {
-    int* d = desc + slot * 8;
-    for (; idx < total_rows; idx += gridDim.x) {
-      const int unit = idx / rows_pass, rr = idx - unit * rows_pass, b = unit / P.n_kv_heads;
-      const int r = P.row_begin + rr;
-      if (r >= P.T[b] * P.group) continue;      // a short sequence does not have this row
-      const int C = P.C[b];
-      const size_t off = (static_cast<size_t>(unit) * P.row_block + rr) * P.c_stride;
-      d[0] = idx; d[1] = unit; d[2] = C; d[3] = r; d[4] = P.k[b];
-      const int n4 = (C + 3) >> 2;
-      // whole 16-byte pieces: rows start 256-byte aligned and are padded to a multiple of 128 floats
-      fence_proxy_async();
-      const float4* src = reinterpret_cast<const float4*>(logits + off);
-      for (int q = 0; q * kClsRegThreads < n4; ++q) {
-        const uint32_t bytes = static_cast<uint32_t>(min(kClsRegThreads, n4 - q * kClsRegThreads)) * 16u;
-        mbar_arrive_expect_tx(bar + q, bytes);
-        bulk_g2s(srow4 + q * kClsRegThreads, src + q * kClsRegThreads, bytes, bar + q);
-      }
-      return;
-    }
-    d[0] = -1;
-  };
-
-  if (tid == 0) {
-    for (int i = 0; i < kClsRegVecsT; ++i) mbar_init(bar + i, 1);
-    mbar_fence_init();
-    ctl[3] = 0;
-    post_row(blockIdx.x, 0);
-  }
-  for (int i = tid; i < kClsBins; i += kClsRegThreads) hist[i] = 0;
-  __syncthreads();
-  uint32_t phases = 0;   // bit q: parity the next wait on barrier q looks for
-
-  for (int it = 0;; ++it) {
-    const int* d = desc + (it & 1) * 8;
-    const int idx = d[0];
-    if (idx < 0) break;
-    const int unit = d[1], C = d[2], r = d[3], k = d[4];
-    const int n4 = (C + 3) >> 2;
-
-    // the row's entries into registers, piece by piece as they land, with the running maximum; the up to three
-    // floats between C and the next multiple of four become -inf, that is p = 0: zeros below every real entry,
-    // which no top-k sum can feel
-    float4 rv[kClsRegVecsT];   // rv[q] is used only where q * kClsRegThreads + tid < n4
-    float mx = -INFINITY;
-    bool landed = true;
-    const int i_fix = (C & 3) ? n4 - 1 : -1;   // the vector with floats past the row's end
-#pragma unroll
-    for (int q = 0; q < kClsRegVecsT; ++q) {
-      if (q * kClsRegThreads < n4) {
-        if (landed) landed = mbar_wait_bounded(bar + q, (phases >> q) & 1u);
-        phases ^= 1u << q;
-        const int i = q * kClsRegThreads + tid;
-        if (landed && i < n4) {
-          float4 v = srow4[i];
-          if (i == i_fix) {
-            if ((C & 3) < 2) v.y = -INFINITY;
-            if ((C & 3) < 3) v.z = -INFINITY;
-            v.w = -INFINITY;
-          }
-          rv[q] = v;
-          mx = fmaxf(fmaxf(mx, fmaxf(v.x, v.y)), fmaxf(v.z, v.w));
-        }
-      }
-    }
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, off));
-    if (lane == 0) red[warp] = mx;
-    // every thread holds its entries: the buffer is free.  A wait that ran out (never seen): the whole CTA
-    // leaves, the row's sum and with it the unit's score become NaN
-    if (__syncthreads_or(!landed)) {
-      if (tid == 0) rowsum[static_cast<size_t>(unit) * P.r_stride + r] = __int_as_float(0x7FC00000);
-      return;
-    }
-    if (tid == 0) post_row(idx + gridDim.x, (it + 1) & 1);   // the next row travels during the rest of this one
-    float M = lane < kClsRegWarps ? red[lane] : -INFINITY;
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
-
-    // p = 2^(l - max) in [0, 1] (a NaN logit counts as no attention: fmaxf returns its other operand), the
-    // normaliser, and the histogram over bits 30..18 of p
-    float z = 0.f;
-#pragma unroll
-    for (int q = 0; q < kClsRegVecsT; ++q) {
-      if (q * kClsRegThreads + tid < n4) {
-        float4 pq;
-        pq.x = fminf(fmaxf(fast_exp2(rv[q].x - M), 0.f), 1.f);
-        pq.y = fminf(fmaxf(fast_exp2(rv[q].y - M), 0.f), 1.f);
-        pq.z = fminf(fmaxf(fast_exp2(rv[q].z - M), 0.f), 1.f);
-        pq.w = fminf(fmaxf(fast_exp2(rv[q].w - M), 0.f), 1.f);
-        rv[q] = pq;
-        z += (pq.x + pq.y) + (pq.z + pq.w);
-        atomicAdd(&hist[__float_as_uint(pq.x) >> kClsShift], 1);
-        atomicAdd(&hist[__float_as_uint(pq.y) >> kClsShift], 1);
-        atomicAdd(&hist[__float_as_uint(pq.z) >> kClsShift], 1);
-        atomicAdd(&hist[__float_as_uint(pq.w) >> kClsShift], 1);
-      }
-    }
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) z += __shfl_xor_sync(0xffffffffu, z, off);
-    if (lane == 0) red[32 + warp] = z;
-    __syncthreads();   // publishes the warp sums and the histogram
-    float Z = lane < kClsRegWarps ? red[32 + lane] : 0.f;
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, off);
-    cls_find_bin_regs(hist, kClsBins, k, ctl, wsum);
-    __syncthreads();
-    auto each4 = [&](auto fn) {
-#pragma unroll
-      for (int q = 0; q < kClsRegVecsT; ++q) {
-        if (q * kClsRegThreads + tid < n4) fn(rv[q]);
-      }
-    };
-    // the sum of every entry whose bit pattern is at least `from`; four partial sums added in a fixed order
-    auto add_from = [&](uint32_t from) {
-      float t0 = 0.f, t1 = 0.f, t2 = 0.f, t3 = 0.f;
-      each4([&](const float4& v) {
-        t0 += __float_as_uint(v.x) >= from ? v.x : 0.f;
-        t1 += __float_as_uint(v.y) >= from ? v.y : 0.f;
-        t2 += __float_as_uint(v.z) >= from ? v.z : 0.f;
-        t3 += __float_as_uint(v.w) >= from ? v.w : 0.f;
-      });
-      return (t0 + t1) + (t2 + t3);
-    };
-    // the entries with bit patterns in [lo, lo + span) each reserve a slot of cand[] (the caller knows their number)
-    auto collect = [&](uint32_t lo, uint32_t span) {
-      each4([&](const float4& v) {
-        const uint32_t a = __float_as_uint(v.x) - lo, b = __float_as_uint(v.y) - lo, c = __float_as_uint(v.z) - lo,
-                       e = __float_as_uint(v.w) - lo;
-        if (min(min(a, b), min(c, e)) < span) {
-          if (a < span) cand[atomicAdd(&ctl[3], 1)] = a + lo;
-          if (b < span) cand[atomicAdd(&ctl[3], 1)] = b + lo;
-          if (c < span) cand[atomicAdd(&ctl[3], 1)] = c + lo;
-          if (e < span) cand[atomicAdd(&ctl[3], 1)] = e + lo;
-        }
-      });
-    };
-    uint32_t prefix = static_cast<uint32_t>(ctl[0]);
-    int shift = kClsShift, need = ctl[1], cnt = ctl[2];
-    float top = 0.f;
-    int n_sorted = 0;   // entries of sorted[] that belong to the sum
-    for (;;) {
-      const uint32_t bin_lo = prefix << shift, bin_span = 1u << shift;   // the bin = bit patterns [bin_lo, bin_lo + bin_span)
-      if (need == cnt) {                      // the whole bin is inside the top k
-        top = add_from(bin_lo);
-        break;
-      }
-      // A sharply peaked row: all `need` entries taken from the bin add up to less than 2^-26 while the sum holds
-      // the row's maximum p = 1, so they cannot move it by half a unit in the last place
-      if (static_cast<float>(need) * __uint_as_float(bin_lo + bin_span) < 1.4901161e-8f) {
-        top = add_from(bin_lo + bin_span);
-        break;
-      }
-      if (cnt <= kClsRank) {
-        // up to kClsRank entries: ranked exactly (descending; equal values in an arbitrary but complete order) by
-        // several threads per entry; warp 0 adds the first `need` in that order after the row's last barrier
-        top = add_from(bin_lo + bin_span);
-        collect(bin_lo, bin_span);
-        __syncthreads();
-        constexpr int kSh = kClsRegThreads == 1024 ? 2 : 1;   // log2 of threads per entry when all kClsRank slots are in use
-        const int sh = cnt <= kClsRank / 2 ? kSh + 1 : kSh;
-        const int c = tid >> sh, part = tid & ((1 << sh) - 1);
-        const uint32_t mk = c < cnt ? cand[c] : 0u;
-        int rank = 0;   // entries that come before this one
-        if (c < cnt) {
-          for (int j = part; j < cnt; j += 1 << sh) {
-            const uint32_t o = cand[j];
-            rank += (o > mk) || (o == mk && j < c);
-          }
-        }
-        for (int off = 1; off < (1 << sh); off <<= 1) rank += __shfl_xor_sync(0xffffffffu, rank, off);
-        if (c < cnt && part == 0) sorted[rank] = __uint_as_float(mk);
-        n_sorted = need;
-        break;
-      }
-      if (shift == 0) {                       // more than kClsRank copies of one value: `need` of them count
-        top = add_from(prefix + 1u);
-        if (tid == 0) top += static_cast<float>(need) * __uint_as_float(prefix);
-        break;
-      }
-      // a crowded bin: histogram of the next bits of its entries (17..8, then 7..0)
-      const int width = shift == kClsShift ? 10 : 8;
-      const int nshift = shift - width;
-      const uint32_t mask = (1u << width) - 1u;
-      for (int i = tid; i < (1 << width); i += kClsRegThreads) hist[i] = 0;
-      __syncthreads();
-      each4([&](const float4& v) {
-        const uint32_t u[4] = {__float_as_uint(v.x), __float_as_uint(v.y), __float_as_uint(v.z), __float_as_uint(v.w)};
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-          if ((u[e] >> shift) == prefix) atomicAdd(&hist[(u[e] >> nshift) & mask], 1);
-      });
-      __syncthreads();
-      cls_find_bin_regs(hist, 1 << width, need, ctl, wsum);
-      __syncthreads();
-      prefix = (prefix << width) | static_cast<uint32_t>(ctl[0]);
-      shift = nshift;
-      need = ctl[1];
-      cnt = ctl[2];
-    }
-#pragma unroll
-    for (int off = 16; off >= 1; off >>= 1) top += __shfl_xor_sync(0xffffffffu, top, off);
-    if (lane == 0) red[64 + warp] = top;
-    __syncthreads();   // every reader of the histogram area and of the control words is done
-    if (warp == 0) {
-      float t = lane < kClsRegWarps ? red[64 + lane] : 0.f;
-#pragma unroll
-      for (int off = 16; off >= 1; off >>= 1) t += __shfl_xor_sync(0xffffffffu, t, off);
-      if (n_sorted > 0) {   // the threshold bin's share, largest first, in a fixed order
-        float s = 0.f;
-        for (int j = lane; j < n_sorted; j += 32) s += sorted[j];
-#pragma unroll
-        for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-        t += s;
-      }
-      if (lane == 0) {
-        rowsum[static_cast<size_t>(unit) * P.r_stride + r] = t / Z;
-        ctl[3] = 0;
-      }
-    }
-    for (int i = tid; i < kClsBins; i += kClsRegThreads) hist[i] = 0;   // for the next row; its first barrier orders it
-  }
-}
-
 // Mean of a unit's row sums (double, fixed order) and its label: 0 static if score >= theta, else 1.
 __global__ void __launch_bounds__(256)
-    cls_finish_kernel(const ClsParams P, const float* rowsum, const int32_t* err, double theta, double* scores_out,
+    cls_finish_kernel(const __grid_constant__ ClsParams P, const float* rowsum, const int32_t* err, double theta, double* scores_out,
                       uint8_t* type_out, int unit0) {
   __shared__ double part[256];
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const int unit = blockIdx.x, b = unit / P.n_kv_heads;
   const int R = P.T[b] * P.group;
   const float* rs = rowsum + static_cast<size_t>(unit) * P.r_stride;
@@ -791,6 +895,61 @@ __global__ void __launch_bounds__(256)
 }
 
 inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
+
+// x with P(Z > x) = q for a standard normal Z, by bisection of the complementary error function
+double cls_normal_quantile(double q) {
+  double lo = -3.0, hi = 6.0;   // outside, the sample's range would be empty anyway
+  for (int i = 0; i < 40; ++i) {
+    const double x = 0.5 * (lo + hi);
+    (0.5 * std::erfc(x * 0.7071067811865476) > q ? lo : hi) = x;
+  }
+  return 0.5 * (lo + hi);
+}
+
+// Shared-memory limits of the kernels and the number of SMs, once per device.
+cudaError_t cls_configure(int* n_sm) {
+  constexpr int kMaxDevices = 64;
+  static std::mutex mutex;
+  static int sms[kMaxDevices] = {};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lock(mutex);
+  if (sms[dev] == 0) {
+    constexpr auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    int n = 0;
+    if ((e = cudaFuncSetAttribute(cls_sample_kernel<8>, attr, kClsSampleSmem)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(cls_sample_kernel<4>, attr, kClsSampleSmem)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(cls_sample_kernel<2>, attr, kClsSampleSmem)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(cls_sample_kernel<1>, attr, kClsSampleSmem)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(cls_scan_kernel, attr, kClsScanSmem)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(cls_select_kernel, attr, 200 * 1024)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(cls_fix_kernel, attr, kClsFixScratch + kClsSmemCols * 4)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+      return e;
+    sms[dev] = n;
+  }
+  *n_sm = sms[dev];
+  return cudaSuccess;
+}
+
+// One launch; `dependent`: it may be set up while its predecessor on the stream still runs (every kernel here that is
+// launched so waits for the predecessor before it touches memory).
+template <class... Params, class... Args>
+cudaError_t launch_cls(void (*kernel)(Params...), int grid, int threads, size_t smem, cudaStream_t stream, bool dependent, Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr{};
+  cfg.gridDim = dim3(static_cast<unsigned>(grid));
+  cfg.blockDim = dim3(static_cast<unsigned>(threads));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
 
 hkv_status cls_check(const hkv_config* cfg, int32_t n_text_max) {
   if (!cfg) return HKV_ERR_INVALID_ARG;
@@ -863,37 +1022,29 @@ extern "C" hkv_status hkv_classify_heads(const hkv_config* cfg, const void* k, c
   const size_t c_stride = round_up(c_max, tc::kKeysPerTile);
   const size_t row_bytes = c_stride * sizeof(float) * s.group_units;
   if (workspace_bytes < s.head_bytes + 16 * row_bytes) return HKV_ERR_WORKSPACE;
-  const int row_block = static_cast<int>(
-      std::min<size_t>(round_up(s.r_max, 16), (workspace_bytes - s.head_bytes) / row_bytes / 16 * 16));
+  const size_t room = workspace_bytes - s.head_bytes;
 
   const int smem_cols = static_cast<int>(round_up(std::min(c_max, kClsSmemCols), 64));
-  const size_t row_smem = kClsRowScratch + static_cast<size_t>(smem_cols) * sizeof(float);
-  if (cudaFuncSetAttribute(cls_row_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(row_smem)) != cudaSuccess)
-    return HKV_ERR_CUDA;
-  const size_t regs_smem = kClsRegScratch + static_cast<size_t>(kClsRegCols) * sizeof(float);
-  if (cudaFuncSetAttribute(cls_row_regs_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(regs_smem)) != cudaSuccess)
-    return HKV_ERR_CUDA;
-
-  int dev = 0, n_sm = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n_sm < 1)
-    return HKV_ERR_CUDA;
+  int n_sm = 0;
+  if (cls_configure(&n_sm) != cudaSuccess) { cudaGetLastError(); return HKV_ERR_CUDA; }
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
-  int32_t* err = static_cast<int32_t*>(workspace);
+  int32_t* err = static_cast<int32_t*>(workspace);   // [0] error word, [1] flagged rows of the pass
   float* rowsum = reinterpret_cast<float*>(static_cast<char*>(workspace) + kAlign);
   if (cudaMemsetAsync(err, 0, kAlign, cs) != cudaSuccess) return HKV_ERR_CUDA;
-  if (cudaFuncSetAttribute(cls_logits_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::kSmemBytes) !=
-      cudaSuccess)
-    return HKV_ERR_CUDA;
-  float* logits = reinterpret_cast<float*>(static_cast<char*>(workspace) + s.head_bytes);
   const float scale =
       cfg->softmax_scale > 0.f ? cfg->softmax_scale : 1.0f / std::sqrt(static_cast<float>(cfg->head_dim));
   for (int b0 = 0; b0 < cfg->batch; b0 += s.group_batch) {
     const int nb = std::min(s.group_batch, cfg->batch - b0);
+    const int units = nb * cfg->n_kv_heads;
     ClsParams P{};
     int r_max = 0, cg_max = 0;
+    const double at_sigma = cls_normal_quantile(topk_fraction);
+    // the sampled keys may take an eighth of the workspace (they do where the caller gives the preferred size)
+    const int sample_max = static_cast<int>(std::max<size_t>(16, std::min<size_t>(kClsSample, room / 8 / (static_cast<size_t>(units) * kRowBytes) / tc::kKeysPerTile * tc::kKeysPerTile)));
+    int n_sample_max = 0;
+    int group = kClsGroupMax;   // about half of the groups should hold an entry of the top share at most
+    while (group > 1 && group * topk_fraction > 0.5) group /= 2;
+    double share = 0.0;   // expected part of a row that lies between the bounds
     for (int i = 0; i < nb; ++i) {
       const int C = seq_lens[b0 + i];
       P.C[i] = C;
@@ -902,41 +1053,124 @@ extern "C" hkv_status hkv_classify_heads(const hkv_config* cfg, const void* k, c
       P.k[i] = static_cast<int32_t>(std::max(1.0, std::min(static_cast<double>(C), kk)));
       r_max = std::max(r_max, P.T[i] * G);
       cg_max = std::max(cg_max, C);
+      // ranks among the sample's group maxima that hold the k-th largest between them
+      const int ns = std::min(C, sample_max);
+      const int groups = ns / tc::kKeysPerTile * (tc::kKeysPerTile / group) + (ns % tc::kKeysPerTile + group - 1) / group;
+      const double q = static_cast<double>(P.k[i]) / C, f = 1.0 - std::pow(1.0 - q, group), at = f * groups;
+      const double margin = kClsSigmas * std::sqrt(at * (1.0 - f)) + 2.0;
+      P.n_sample[i] = ns;
+      n_sample_max = std::max(n_sample_max, ns);
+      P.rank_hi[i] = static_cast<int32_t>(std::floor(at - margin));   // negative: no upper bound
+      P.rank_lo[i] = static_cast<int32_t>(std::ceil(at + margin));    // above the sample: no lower bound
+      auto entries = [&](double rank) { return 1.0 - std::pow(1.0 - std::max(0.0, std::min(1.0, rank / groups)), 1.0 / group); };
+      const double bin = (6.0 / kClsSampleBins) * 0.4 * std::exp(-0.5 * at_sigma * at_sigma);   // the histogram bin at each bound
+      share = std::max(share, std::min(1.0, entries(at + margin) - entries(at - margin) + 2.0 * bin));
     }
+    P.n_batch = nb;
     P.n_kv_heads = cfg->n_kv_heads;
     P.n_q_heads = cfg->n_q_heads;
     P.group = G;
     P.max_seq_len = cfg->max_seq_len;
     P.t_stride = n_text_max;
-    P.row_block = row_block;
-    P.c_stride = static_cast<int32_t>(c_stride);
     P.r_stride = s.r_max;
-    P.smem_cols = smem_cols;
+    P.bins_at = static_cast<float>(at_sigma);
     P.scale_log2e = scale * kLog2e;
+    // Rows per pass and list room.  A row takes its bounds, two partial records per CTA that shares its block, its entry
+    // in the flag list and two lists of `per_tile` entries per key tile plus kClsSlack per segment.  The lists get at
+    // least 1.3 times their (generously) expected length, and up to six times where the workspace allows it in one pass:
+    // keys of a video frame are correlated, so a stretch of the context may hold several times its share.
+    const int n_tiles = (cg_max + tc::kKeysPerTile - 1) / tc::kKeysPerTile;
+    auto tiles_of = [&](int rows) {
+      int64_t w = 0;
+      for (int i = 0; i < nb; ++i)
+        w += static_cast<int64_t>(cfg->n_kv_heads) * ((std::min(rows, P.T[i] * G) + tc::kQRows - 1) / tc::kQRows) *
+             ((P.C[i] + tc::kKeysPerTile - 1) / tc::kKeysPerTile);
+      return w;
+    };
+    auto ctas_of = [&](int64_t w) { return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(n_sm, w / 2))); };
+    auto segs_of = [&](int64_t w) { return static_cast<int>(std::min<int64_t>(n_tiles, n_tiles / std::max<int64_t>(1, w / ctas_of(w)) + 2)); };
+    auto bytes_of = [&](int seg_max, int per_tile) {
+      return static_cast<size_t>(8) * (static_cast<size_t>(n_tiles) * per_tile + static_cast<size_t>(seg_max) * kClsSlack) + 32u * seg_max + 20u;
+    };
+    auto per_tile_of = [&](double times) { return std::min(64, static_cast<int>(std::ceil(times * share * 64.0))); };
+    P.sample_stride = static_cast<int32_t>(round_up(n_sample_max, tc::kKeysPerTile) + tc::kKeysPerTile);
+    size_t sample_bytes = static_cast<size_t>(units) * P.sample_stride * kRowBytes;
+    const bool sampled = sample_bytes <= room / 2;   // no room (the smallest workspace of a short context): list every entry
+    if (!sampled) { sample_bytes = 0; share = 1.0; }
+    const size_t fixed = 4 * kAlign + sample_bytes;
+    int row_block = r_max, seg_max = segs_of(tiles_of(r_max)), per_tile = per_tile_of(1.3);
+    while (row_block > 1 && bytes_of(seg_max, per_tile) * row_block * units + fixed > room) {
+      const size_t fit = (room - fixed) / units / bytes_of(seg_max, per_tile);
+      row_block = static_cast<int>(std::max<size_t>(1, std::min<size_t>(row_block - 1, fit)));
+      if (row_block > tc::kQRows) row_block = row_block / tc::kQRows * tc::kQRows;
+      seg_max = segs_of(tiles_of(row_block));
+    }
+    if (row_block == r_max)
+      while (per_tile < per_tile_of(6.0) && bytes_of(seg_max, per_tile + 1) * row_block * units + fixed <= room) ++per_tile;
+    const size_t rows_all = static_cast<size_t>(row_block) * units;
+    if (bytes_of(seg_max, per_tile) * rows_all + fixed > room) return HKV_ERR_WORKSPACE;
+    P.row_block = row_block;
+    P.seg_max = seg_max;
+    P.per_tile = per_tile;
+    P.list_stride = (n_tiles * per_tile & ~3) + seg_max * kClsSlack;
+    char* at = static_cast<char*>(workspace) + s.head_bytes;
+    char* samples = at;                               at += sample_bytes;
+    float4* bounds = reinterpret_cast<float4*>(at);   at += round_up(rows_all * sizeof(float4), kAlign);
+    float4* partial = reinterpret_cast<float4*>(at);  at += round_up(rows_all * seg_max * 2 * sizeof(float4), kAlign);
+    int32_t* flagged = reinterpret_cast<int32_t*>(at); at += round_up(rows_all * sizeof(int32_t), kAlign);
+    float* list = reinterpret_cast<float*>(at);
+    // rows the fix kernel cannot hold in shared memory take the lists' memory (their content is dead by then)
+    const int fix_ctas = cg_max <= smem_cols
+                             ? n_sm
+                             : static_cast<int>(std::max<size_t>(1, std::min<size_t>(n_sm, (workspace_bytes - (at - static_cast<char*>(workspace))) / (c_stride * sizeof(float)))));
     const __nv_bfloat16* kg = static_cast<const __nv_bfloat16*>(k) +
                               static_cast<size_t>(b0) * cfg->n_kv_heads * cfg->max_seq_len * kHeadDim;
     const __nv_bfloat16* qg = static_cast<const __nv_bfloat16*>(q_text) +
                               static_cast<size_t>(b0) * n_text_max * cfg->n_q_heads * kHeadDim;
-    const int units = nb * cfg->n_kv_heads;
-    for (int rb = 0; rb < r_max; rb += row_block) {
-      P.row_begin = rb;
-      const int rows = std::min(row_block, r_max - rb);
-      // key ranges sized so that the launch is about one wave of CTAs
-      const int row_blocks = (rows + tc::kQRows - 1) / tc::kQRows;
-      const int n_tiles = (cg_max + tc::kKeysPerTile - 1) / tc::kKeysPerTile;
-      const int splits = std::max(1, std::min(n_tiles, n_sm / std::max(1, units * row_blocks)));
-      const int tiles_per_cta = (n_tiles + splits - 1) / splits;
-      cls_logits_tc_kernel<<<dim3((n_tiles + tiles_per_cta - 1) / tiles_per_cta, row_blocks, units), tc::kThreads,
-                             tc::kSmemBytes, cs>>>(P, kg, qg, logits, tiles_per_cta, err);
-      const int total_rows = rows * units;
-      if (cg_max <= kClsRegCols)   // every row of the group fits the threads' registers: the pipelined kernel
-        cls_row_regs_kernel<<<std::min(total_rows, n_sm), kClsRegThreads, regs_smem, cs>>>(P, logits, rowsum, rows,
-                                                                                           total_rows);
-      else
-        cls_row_kernel<<<std::min(total_rows, n_sm), kClsRowThreads, row_smem, cs>>>(P, logits, rowsum, rows, total_rows);
+    // a warp of the selection holds a third more entries than expected, as far as shared memory goes
+    // (whole iterations of a warp: the undecided entries' columns overwrite the iterations already read)
+    const int sel_cap = static_cast<int>(round_up(static_cast<size_t>(std::min(12.0 * 1024 - 32, std::ceil(1.35 * share * cg_max / 4.0) + 2.0 * seg_max + 16.0)), 32));
+    const int sel_warps = std::max(1, std::min(8, static_cast<int>(200 * 1024 / (sel_cap * sizeof(float4)))));
+    const auto sample_kernel = group == 8 ? cls_sample_kernel<8> : group == 4 ? cls_sample_kernel<4> : group == 2 ? cls_sample_kernel<2> : cls_sample_kernel<1>;
+    CUtensorMap map, sample_map;
+    cudaError_t e = tc::key_map(&map, kg, static_cast<uint64_t>(units) * cfg->max_seq_len);
+    if (!sampled) bounds = nullptr;
+    if (e == cudaSuccess && sampled) e = tc::key_map(&sample_map, samples, static_cast<uint64_t>(units) * P.sample_stride);
+    if (e == cudaSuccess && sampled) {
+      cls_gather_kernel<<<dim3(static_cast<unsigned>(P.sample_stride / 16), static_cast<unsigned>(units)), 256, 0, cs>>>(
+          P, reinterpret_cast<const uint4*>(kg), reinterpret_cast<uint4*>(samples));
+      e = cudaGetLastError();
     }
-    cls_finish_kernel<<<units, 256, 0, cs>>>(P, rowsum, err, theta, scores_out, head_type_out, b0 * cfg->n_kv_heads);
-    if (cudaGetLastError() != cudaSuccess) return HKV_ERR_CUDA;
+    for (int rb = 0; rb < r_max && e == cudaSuccess; rb += row_block) {
+      P.row_begin = rb;
+      int blocks = 0;
+      P.w_prefix[0] = 0;
+      for (int i = 0; i < nb; ++i) {
+        const int rows = std::max(0, std::min(row_block, P.T[i] * G - rb)), blk = (rows + tc::kQRows - 1) / tc::kQRows;
+        blocks += blk * cfg->n_kv_heads;
+        P.w_prefix[i + 1] = P.w_prefix[i] + static_cast<int64_t>(cfg->n_kv_heads) * blk * ((P.C[i] + tc::kKeysPerTile - 1) / tc::kKeysPerTile);
+      }
+      // fewer pairs than in the first pass never mean more CTAs per block than it was sized for
+      P.n_cta = ctas_of(P.w_prefix[nb]);
+      if (rb > 0) {
+        while (P.n_cta > 1 && segs_of(P.w_prefix[nb]) > seg_max && n_tiles / std::max<int64_t>(1, P.w_prefix[nb] / P.n_cta) + 2 > seg_max) --P.n_cta;
+      }
+      P.small = (P.w_prefix[nb] + 1) * P.n_cta < (1ll << 31);
+      if (rb > 0 && cudaMemsetAsync(err + 1, 0, sizeof(int32_t), cs) != cudaSuccess) return HKV_ERR_CUDA;
+      if (sampled) e = launch_cls(sample_kernel, blocks, tc::kSegThreads, kClsSampleSmem, cs, rb == 0, P, sample_map, qg, bounds, err);
+      if (e == cudaSuccess) e = launch_cls(cls_scan_kernel, P.n_cta, tc::kSegThreads, kClsScanSmem, cs, sampled, P, map, qg,
+                                           static_cast<const float4*>(bounds), partial, list, err);
+      if (e == cudaSuccess) e = launch_cls(cls_select_kernel, static_cast<int>((rows_all + sel_warps - 1) / sel_warps), sel_warps * 32,
+                                           static_cast<size_t>(sel_warps) * sel_cap * sizeof(float4), cs, true, P, static_cast<const float4*>(bounds),
+                                           static_cast<const float4*>(partial), static_cast<const float*>(list), rowsum, err + 1, flagged,
+                                           static_cast<int>(rows_all), sel_cap);
+      if (e == cudaSuccess) e = launch_cls(cls_fix_kernel, fix_ctas, kClsFixThreads, kClsFixScratch + static_cast<size_t>(smem_cols) * sizeof(float), cs, true,
+                                           P, kg, qg, rowsum, static_cast<const int32_t*>(err + 1), static_cast<const int32_t*>(flagged), list,
+                                           static_cast<int>(c_stride), smem_cols);
+    }
+    if (e == cudaSuccess) e = launch_cls(cls_finish_kernel, units, 256, 0, cs, true, P, static_cast<const float*>(rowsum), static_cast<const int32_t*>(err),
+                                         theta, scores_out, head_type_out, b0 * cfg->n_kv_heads);
+    if (e != cudaSuccess) { cudaGetLastError(); return HKV_ERR_CUDA; }
   }
   return HKV_OK;
 }

@@ -15,6 +15,8 @@
 // in bits 24..28.  An M = 128 accumulator puts row i in tensor-memory lane i and column j in column
 // base + j; warp w of the CTA may read lanes 32 * (w % 4) .. + 31.
 #pragma once
+#include <cuda.h>
+
 #include "hkv_device.cuh"
 
 namespace hkv {
@@ -314,6 +316,264 @@ __device__ bool scores_cta(uint8_t* smem_raw, QRowFn q_row, const __nv_bfloat16*
   fence_after_sync();
   if (warp == 1) tmem_dealloc(tmem_base, kTmemCols);
   return all_ok;
+}
+
+
+// ---- packed pairs of floats (one instruction for two elements) ----
+__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ void unpack_f32x2(uint64_t v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+// sum += x with the rounding error carried in comp (compensated summation; no fast-math in this library)
+__device__ __forceinline__ void add_compensated(float& sum, float& comp, float x) {
+  const float y = x - comp, t = sum + y;
+  comp = (t - sum) - y;
+  sum = t;
+}
+
+// ---------------------------------------------------------------------------------------------
+// The segment engine.  A CTA walks a list of SEGMENTS -- a block of up to kQRows query rows against a run of key tiles
+// of the same head -- so that work can be cut into equal shares of the whole launch's tiles whatever the heads'
+// lengths, with one tensor-memory allocation and one pipeline per CTA: the key tiles of the next segment are already
+// arriving while the last ones of the current are drained, and only the 64 KB of query rows are exchanged between two
+// segments (by the draining warps, behind a named barrier they share with the issuer).
+// Warp 0 brings in key tiles (TMA, two boxes of 64 elements x 128 keys in the operands' swizzled layout) and feeds the
+// tensor core; sixteen warps drain.  The hand-back of an accumulator buffer is a named barrier (arrive / sync): a warp
+// that polls an mbarrier meanwhile took half of its scheduler's issue slots from the draining warps.
+//   map               tensor map over all keys as rows of 128 bf16, boxes of 64 x 128 (key_map below)
+//   segment(s, seg)   the CTA's s-th segment; false behind the last.  Seg has tile_begin, tile_end and key_row0, the row
+//                     of tile 0's first key in the map.  Rows behind the head's last key hold whatever the tensor holds
+//                     there (zero behind its end): the caller masks them
+//   q_row(seg, row)   pointer to a query row's 128 bf16, or nullptr for a zero row
+//   begin(seg, lane_row, part), tile(seg, tile, lane_row, part, taddr), end(seg, lane_row, part, ok): called by the
+//                     draining threads as in scores_cta; taddr is the tensor-memory address of the thread's
+//                     64 columns (drain_raw); ok: no wait has run out so far
+// kKeysAsRows as in scores_cta; kRing: key tiles of shared memory.  *user: shared memory behind the barriers' page, the caller's.  kSegThreads threads.
+// ---------------------------------------------------------------------------------------------
+constexpr int kSegThreads = (1 + kDrainWarps) * 32;
+constexpr int kBarDrainIssue = 1, kBarDrain = 2, kBarAcc = 3;   // named barriers (kBarAcc + accumulator buffer)
+__device__ __forceinline__ void named_sync(int id, int threads) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ void named_arrive(int id, int threads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+constexpr int seg_smem_fixed(int stages) { return kQBytes + stages * kStageBytes + kBarBytes + 1024; }   // + the caller's bytes
+
+// 32 lanes x 16 columns, waited for: the four warps of a scheduler hide each other's latency, and the values need no copy
+// between the read and its wait.
+__device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr)
+      : "memory");
+}
+// A draining thread's 64 columns as four groups of 16: fn(group, r) with columns 16 group ..
+template <class Fn>
+__device__ __forceinline__ void drain_raw(uint32_t taddr, Fn fn) {
+#pragma unroll
+  for (int g = 0; g < 4; ++g) {
+    uint32_t r[16];
+    tmem_ld16(taddr + 16u * g, r);
+    fn(g, r);
+  }
+}
+
+// Loads the box at (x, y) of a two-dimensional tensor map into shared memory; bytes are credited to `bar`.
+__device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(dst),
+      "l"(map), "r"(x), "r"(y), "r"(smem_u32(bar))
+      : "memory");
+}
+
+template <bool kKeysAsRows, int kRing, class Seg, class SegmentFn, class QRowFn, class BeginFn, class TileFn, class EndFn>
+__device__ bool segments_cta(uint8_t* smem_raw, const CUtensorMap* map, SegmentFn segment, QRowFn q_row, BeginFn begin,
+                             TileFn tile_fn, EndFn end, uint8_t** user) {
+  uint8_t* smem = smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u);   // operand planes are 1024-byte aligned
+  uint8_t* qs = smem;
+  uint8_t* ks = smem + kQBytes;
+  uint64_t* full = reinterpret_cast<uint64_t*>(ks + kRing * kStageBytes);
+  uint64_t* empty = full + kRing;
+  uint64_t* acc_full = empty + kRing;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 2);
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  *user = ks + kRing * kStageBytes + kBarBytes;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+
+  if (tid == 0) {
+    for (int s = 0; s < kRing; ++s) {
+      mbar_init(full + s, 1);
+      mbar_init(empty + s, 1);
+    }
+    for (int b = 0; b < 2; ++b) mbar_init(acc_full + b, 1);
+    mbar_fence_init();
+    *abort_flag = 0;
+  }
+  if (warp == 0) {
+    tmem_alloc(tmem_slot, kTmemCols);
+    tmem_relinquish();
+  }
+  fence_before_sync();
+  __syncthreads();
+  fence_after_sync();
+  const uint32_t tmem_base = *tmem_slot;
+  // a wait that runs out makes every role go on without waiting or working, so that all still meet at the barriers
+  bool ok = true;
+  auto wait = [&](uint64_t* bar, uint32_t parity) {
+    if (ok && !mbar_try_wait(bar, parity)) {
+      const long long start = clock64();
+      for (uint32_t it = 1; ok && !mbar_try_wait(bar, parity); ++it) {
+        if ((it & 255u) == 0u && (*abort_flag || clock64() - start > HKV_WAIT_CYCLES)) ok = false;
+      }
+      if (!ok) *abort_flag = 1;
+    }
+  };
+
+  if (warp == 0) {
+    constexpr uint32_t idesc = kKeysAsRows ? InstrDesc<128, 256>::value : InstrDesc<128, 128>::value;
+    const uint32_t q_addr = smem_u32(qs), k_addr0 = smem_u32(ks);
+    // the tiles to load run kRing - 1 ahead of the tiles to compute, through the same list of segments
+    Seg ld, seg;
+    int ld_sg = 0, ld_tile = 0, n_ld = 0;
+    bool ld_more = segment(0, ld);
+    if (ld_more) ld_tile = ld.tile_begin;
+    auto load_next = [&]() {
+      if (!ld_more) return;
+      const int s = n_ld % kRing;
+      if (n_ld >= kRing) wait(empty + s, ((n_ld / kRing) - 1) & 1);
+      if (ok && lane == 0) {
+        const uint32_t dst = k_addr0 + static_cast<uint32_t>(s * kStageBytes);
+        mbar_arrive_expect_tx(full + s, kStageBytes);
+        tma_load_2d(dst, map, 0, ld.key_row0 + ld_tile * kKeysPerTile, full + s);
+        tma_load_2d(dst + kPlaneBytesK, map, 64, ld.key_row0 + ld_tile * kKeysPerTile, full + s);
+      }
+      __syncwarp();
+      ++n_ld;
+      if (++ld_tile == ld.tile_end) {
+        ld_more = segment(++ld_sg, ld);
+        if (ld_more) ld_tile = ld.tile_begin;
+      }
+    };
+    for (int j = 0; j < kRing - 1; ++j) load_next();
+    int i = 0;
+    for (int sg = 0; segment(sg, seg); ++sg) {
+      named_sync(kBarDrainIssue, (kDrainWarps + 1) * 32);   // the segment's query rows are in place
+      fence_after_sync();
+      for (int tile = seg.tile_begin; tile < seg.tile_end; ++tile, ++i) {
+        const int s = i % kRing, buf = i & 1;
+        if (i >= 2) named_sync(kBarAcc + buf, (kDrainWarps + 1) * 32);   // tile i - 2 has been drained
+        wait(full + s, (i / kRing) & 1);
+        fence_after_sync();
+        if (ok && lane == 0) {
+          const uint32_t k_addr = k_addr0 + static_cast<uint32_t>(s * kStageBytes);
+          const uint32_t d = tmem_base + static_cast<uint32_t>(buf * 256);
+#pragma unroll
+          for (int kk = 0; kk < 8; ++kk) {   // K = 16 elements = 32 bytes per instruction; 4 per half-plane
+            const uint32_t koff = static_cast<uint32_t>((kk >> 2) * kPlaneBytesK + (kk & 3) * 32);
+            const uint32_t qoff = static_cast<uint32_t>((kk >> 2) * kPlaneBytesQ + (kk & 3) * 32);
+            if (kKeysAsRows) {
+              umma_bf16(d, smem_desc(k_addr + koff), smem_desc(q_addr + qoff), idesc, kk != 0);
+            } else {
+              umma_bf16(d, smem_desc(q_addr + qoff), smem_desc(k_addr + koff), idesc, kk != 0);
+              umma_bf16(d + 128u, smem_desc(q_addr + qoff + 128u * 128u), smem_desc(k_addr + koff), idesc, kk != 0);
+            }
+          }
+          umma_commit(empty + s);        // the stage may be refilled once these instructions have read it
+          umma_commit(acc_full + buf);   // and the accumulator is complete
+        }
+        __syncwarp();
+        load_next();   // into the stage of tile i - 1, whose instructions have had a tile's time to finish
+      }
+    }
+    // arrivals on the barriers of the last tiles must land before the CTA may leave
+    for (int t = max(0, i - 2); t < i; ++t) named_sync(kBarAcc + (t & 1), (kDrainWarps + 1) * 32);
+    for (int t = max(0, i - kRing); t < i; ++t) wait(empty + t % kRing, (t / kRing) & 1);
+  } else {
+    // ---- drain: warp w owns lane quarter w % 4 (the hardware's rule) and column part (w - 1) / 4 ----
+    const int quarter = warp & 3, part = (warp - 1) >> 2;
+    const int row = quarter * 32 + lane;
+    const int dtid = tid - 32;
+    int i = 0;
+    Seg seg;
+    for (int sg = 0; segment(sg, seg); ++sg) {
+      // the query block, four loads in flight per thread; every instruction that read the previous block has
+      // completed, because this thread has seen the segment's last accumulator
+#pragma unroll 1
+      for (int base = dtid; base < kQRows * 16; base += 4 * kDrainWarps * 32) {
+        uint4 v[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int idx = base + u * kDrainWarps * 32;
+          const __nv_bfloat16* src = q_row(seg, idx >> 4);
+          v[u] = src ? __ldg(reinterpret_cast<const uint4*>(src) + (idx & 15)) : make_uint4(0u, 0u, 0u, 0u);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int idx = base + u * kDrainWarps * 32;
+          *reinterpret_cast<uint4*>(qs + piece_offset(idx >> 4, idx & 15, kPlaneBytesQ)) = v[u];
+        }
+      }
+      fence_proxy_async();   // written by ordinary stores, read by the tensor core
+      fence_before_sync();
+      named_sync(kBarDrainIssue, (kDrainWarps + 1) * 32);
+      begin(seg, row, part);
+      for (int tile = seg.tile_begin; tile < seg.tile_end; ++tile, ++i) {
+        const int buf = i & 1;
+        wait(acc_full + buf, (i >> 1) & 1);
+        fence_after_sync();
+        const uint32_t taddr =
+            tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(buf * 256 + part * 64);
+        tile_fn(seg, tile, row, part, taddr);
+        fence_before_sync();
+        named_arrive(kBarAcc + buf, (kDrainWarps + 1) * 32);
+      }
+      end(seg, row, part, ok);
+    }
+  }
+  const bool all_ok = !__syncthreads_or(!ok);
+  fence_after_sync();
+  if (warp == 0) tmem_dealloc(tmem_base, kTmemCols);
+  return all_ok;
+}
+
+// Host: the tensor map segments_cta takes, over `rows` keys of 128 bf16 from `keys` on.
+inline cudaError_t key_map(CUtensorMap* map, const void* keys, uint64_t rows) {
+  using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*,
+                              const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
+                              CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+  static Encode encode = [] {
+    void* fn = nullptr;
+    cudaDriverEntryPointQueryResult found;
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+        found != cudaDriverEntryPointSuccess)
+      fn = nullptr;
+    return reinterpret_cast<Encode>(fn);
+  }();
+  if (!encode) return cudaErrorNotSupported;
+  const cuuint64_t dims[2] = {128, rows}, strides[1] = {256};
+  const cuuint32_t box[2] = {64, kKeysPerTile}, step[2] = {1, 1};
+  const CUresult r = encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(keys), dims, strides, box, step,
+                            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
 }  // namespace tc

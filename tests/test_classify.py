@@ -208,3 +208,28 @@ def test_gpu_classify_random_shapes(case):
     L = hi.tiny(seed=7100 + case, B=B, C=C, chunk_size=32, w=8, Hq=G * Hkv, Hkv=Hkv, d=128,
                 ragged=bool(rng.integers(0, 2)) and C > 5 * B + 16)
     _check_case(L, T, fraction, workspace=str(rng.choice(["preferred", "min"])), seed=case)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("C,T,G,fraction,kind", [
+    (127, 9, 4, 0.05, ""), (129, 64, 4, 0.05, ""), (4096, 37, 7, 0.05, ""), (4097, 65, 4, 0.2, ""), (8200, 256, 1, 0.05, ""),
+    (9000, 40, 7, 0.05, "ties"), (9000, 40, 7, 0.3, "ties"), (6000, 33, 8, 0.05, "clustered"), (5000, 7, 4, 0.001, "nan")])
+def test_gpu_classify_edges_of_the_sampled_bounds(C, T, G, fraction, kind):
+    """Contexts around the sample's and a tile's size, row blocks of 256 rows and one more, and inputs whose threshold the
+    sample cannot bound closely: a value shared by a third of the keys at the threshold, keys near the threshold
+    packed into one stretch of the context (the list of that stretch overflows), keys that are not finite."""
+    L = hi.tiny(seed=51, B=1, C=C, chunk_size=32, w=8, Hq=2 * G, Hkv=2, d=128, ragged=False)
+    rng = np.random.default_rng(C)
+    if kind == "ties":        # one key repeated: its logit lies at or near the threshold for many rows
+        L.k[0, :, rng.permutation(C)[:C // 3]] = L.k[0, :, 5][None]
+    elif kind == "clustered":
+        L.k[0, :, 1000:1900] = hi.f32_to_bf16_bits(hi.bf16_bits_to_f32(L.k[0, :, 1000:1001]) +
+                                                   0.2 * rng.standard_normal((2, 900, 128)).astype(np.float32))
+    if kind != "nan":
+        _check_case(L, T, fraction)
+        return
+    q_text, counts = hi.text_queries(L, T, seed=5)
+    ref = _oracle_scores(L, q_text, counts, fraction)
+    L.k[0, 1, 4321] = 0x7FC0   # the head without it must not notice; the other one still answers
+    got, _ = _gpu_scores(L, q_text, counts, fraction, 0.9)
+    assert abs(got[0, 0] - ref[0, 0]) <= SCORE_TOL and 0.0 < got[0, 1] <= 1.0 + 1e-6
