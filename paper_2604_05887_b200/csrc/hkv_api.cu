@@ -180,7 +180,9 @@ StepSide* step_side() {
   std::lock_guard<std::mutex> lock(g_step_mutex);
   StepSide& s = g_step_side[dev];
   if (!s.ready) {
-    bool ok = cudaStreamCreateWithFlags(&s.stream, cudaStreamNonBlocking) == cudaSuccess;
+    int least = 0, greatest = 0;
+    bool ok = cudaDeviceGetStreamPriorityRange(&least, &greatest) == cudaSuccess &&
+              cudaStreamCreateWithPriority(&s.stream, cudaStreamNonBlocking, greatest) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&s.fork, cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&s.q_done, cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&s.q_done2, cudaEventDisableTiming) == cudaSuccess;
@@ -280,27 +282,43 @@ static hkv_status compress_common(const hkv_config* cfg, const void* k, const vo
     for (int i = 0; i < H.n_units; ++i) {
       if (c->units[i].type) *dl++ = i; else *sl++ = i;
     }
-    bool ok = cudaMemcpyAsync(c->dev_base, img.data(), tables, cudaMemcpyHostToDevice, s) == cudaSuccess;
-    // n_valid and the error word start at zero
-    ok = ok && cudaMemsetAsync(c->dev_base + H.n_valid_off, 0, static_cast<size_t>(H.err_off + 8 - H.n_valid_off), s) ==
-                   cudaSuccess;
-    // dynamic heads beside the static ones, on the library's second stream (forked from and joined to `s`)
+    // the running tile counts lie behind the row statistics (see build_plan)
+    const bool window = H.n_static > 0 && !token_scores;
+    const int R_pad = (H.obs_window * H.group + 15) / 16 * 16;
+    int32_t* tile_prefix = window ? reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + ws_rowstat_off +
+                                                               8ll * H.n_static * tiles_max * R_pad)
+                                  : nullptr;
+    int64_t total_tiles = 0;
+    for (const auto& u : c->units) total_tiles += u.type == 0 ? (u.C + 127) / 128 : 0;
+    bool ok = launch_setup(c->dev_base, img.data(), static_cast<int>(tables), static_cast<int>(H.n_valid_off),
+                           static_cast<int>(H.err_off + 8 - H.n_valid_off), tile_prefix, s) == cudaSuccess;
+    // Static heads beside the dynamic ones, on the library's second stream (forked from and joined to `s`): it has the
+    // higher priority, so that the long chain of the static heads' kernels never queues behind the dynamic heads' blocks.
     StepSide* side = (H.n_static > 0 && H.n_dynamic > 0) ? step_side() : nullptr;
     std::unique_lock<std::mutex> side_lock;
     if (side) side_lock = std::unique_lock<std::mutex>(side->enqueue);
-    if (ok && side) {
-      ok = cudaEventRecord(side->fork, s) == cudaSuccess && cudaStreamWaitEvent(side->stream, side->fork, 0) == cudaSuccess;
-      ok = ok && launch_build_dynamic(c->dev_base, k, v, H, c->max_dyn_rows, c->max_chunks, side->stream) == cudaSuccess;
-      ok = ok && cudaEventRecord(side->join, side->stream) == cudaSuccess;
+    cudaStream_t ss = side ? side->stream : s;
+    if (ok && side) ok = cudaEventRecord(side->fork, s) == cudaSuccess && cudaStreamWaitEvent(ss, side->fork, 0) == cudaSuccess;
+    // The dynamic heads' copies slow the window scores down where both run (HBM).  If they are short enough to be done
+    // while the second pass, the selection and the gather run (~2.1 us per tile of a CTA + 30 us; the copies at about
+    // 6 TB/s), they start after the first pass; else at once.  (10 static + 6 dynamic units of 24-32 K tokens: 131 us
+    // against 141; 13 + 19 of 50 K: 277 against 291.)
+    bool later = false;
+    if (side && window) {
+      int64_t build_bytes = 0;
+      for (const auto& u : c->units) build_bytes += u.type == 0 ? 0 : 4ll * kRowBytes * u.C;
+      later = static_cast<double>(build_bytes) / 6.0e6 < 2.1 * static_cast<double>(total_tiles) / 148.0 + 30.0;
     }
     if (ok && H.n_static > 0) {
-      if (!token_scores)
-        ok = launch_window_scores(c->dev_base, static_cast<char*>(workspace), k, q_obs, H, c->units, ws_rowstat_off,
-                                  tiles_max, s) == cudaSuccess;
-      ok = ok && launch_static_select(c->dev_base, static_cast<char*>(workspace), token_scores, is_text, H, s) == cudaSuccess;
-      ok = ok && launch_gather_static(c->dev_base, k, v, H, c->max_static_rows, s) == cudaSuccess;
+      if (window)
+        ok = launch_window_scores(c->dev_base, static_cast<char*>(workspace), k, q_obs, H, total_tiles, ws_rowstat_off,
+                                  tiles_max, tile_prefix, later ? side->q_done : nullptr, ss) == cudaSuccess;
+      ok = ok && launch_static_select(c->dev_base, static_cast<char*>(workspace), token_scores, is_text, H, ss) == cudaSuccess;
+      ok = ok && launch_gather_static(c->dev_base, k, v, H, c->max_static_rows, ss) == cudaSuccess;
+      if (side) ok = ok && cudaEventRecord(side->join, ss) == cudaSuccess;
     }
-    if (ok && H.n_dynamic > 0 && !side)
+    if (ok && later) ok = cudaStreamWaitEvent(s, side->q_done, 0) == cudaSuccess;
+    if (ok && H.n_dynamic > 0)
       ok = launch_build_dynamic(c->dev_base, k, v, H, c->max_dyn_rows, c->max_chunks, s) == cudaSuccess;
     if (ok && side) ok = cudaStreamWaitEvent(s, side->join, 0) == cudaSuccess;
     if (!ok) { cudaGetLastError(); delete c; return HKV_ERR_CUDA; }

@@ -4,6 +4,8 @@
 // 16-byte pieces XOR-permuted by (row & 7), the layout the flash-decode kernel stages with plain
 // bulk copies and reads with bank-conflict-free ldmatrix.
 #include <algorithm>
+#include <cstring>
+#include <mutex>
 
 #include "hkv_device.cuh"
 #include "hkv_internal.h"
@@ -24,198 +26,298 @@ __device__ __forceinline__ const Unit* unit_of(const char* cache, const Header* 
 }
 
 // ---------------------------------------------------------------------------------------------
+// The cache's tables (header, unit records, unit lists) written, the counters behind them cleared, and the running sum
+// of the static units' key tiles, by which the window-score kernels share out their work, left in the workspace.
+// Tables of up to N bytes travel in the launch itself (one launch instead of a staged copy and a fill: 4 us less before
+// the first kernel may start); larger ones have been copied before (N = 0).  One block.
+// ---------------------------------------------------------------------------------------------
+template <int N>
+struct alignas(16) TableImage { uint8_t bytes[N]; };
+template <>
+struct TableImage<0> {};
+constexpr int kSetupThreads = 512;
+template <int N>
+__global__ void __launch_bounds__(kSetupThreads)
+    setup_kernel(const __grid_constant__ TableImage<N> image, char* cache, int table_bytes, int zero_begin, int zero_bytes,
+                 int32_t* tile_prefix) {
+  __shared__ int warp_sum[kSetupThreads / 32];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const char* src = cache;
+  if constexpr (N > 0) {
+    src = reinterpret_cast<const char*>(image.bytes);
+    for (int i = tid * 16; i < table_bytes; i += kSetupThreads * 16)
+      *reinterpret_cast<uint4*>(cache + i) = *reinterpret_cast<const uint4*>(src + i);
+  }
+  for (int i = tid * 4; i < zero_bytes; i += kSetupThreads * 4) *reinterpret_cast<int32_t*>(cache + zero_begin + i) = 0;
+  if (!tile_prefix) return;
+  const Header* hdr = reinterpret_cast<const Header*>(src);
+  const int32_t* list = reinterpret_cast<const int32_t*>(src + hdr->sta_list_off);
+  const Unit* units = reinterpret_cast<const Unit*>(src + kUnitsOff);
+  int before = 0;
+  for (int base = 0; base < hdr->n_static; base += kSetupThreads) {
+    const int i = base + tid;
+    const int mine = i < hdr->n_static ? (units[list[i]].C + tc::kKeysPerTile - 1) / tc::kKeysPerTile : 0;
+    int incl = mine;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+      const int x = __shfl_up_sync(0xffffffffu, incl, off);
+      if (lane >= off) incl += x;
+    }
+    __syncthreads();
+    if (lane == 31) warp_sum[warp] = incl;
+    __syncthreads();
+    int total = 0;
+    for (int w2 = 0; w2 < kSetupThreads / 32; ++w2) {
+      if (w2 < warp) incl += warp_sum[w2];
+      total += warp_sum[w2];
+    }
+    if (i < hdr->n_static) tile_prefix[i] = before + incl - mine;
+    before += total;
+  }
+  if (tid == 0) tile_prefix[hdr->n_static] = before;
+}
+
+// ---------------------------------------------------------------------------------------------
 // Window scores.  S_w = softmax over ALL tokens of the w*G window rows' logits, s_w = mean of rows
 // (row r = window position r / G, query head r % G of the group).  The logits run on the tcgen05
-// tensor cores: one CTA = one static unit x one range of 128-key tiles x one block of up to 256
-// rows; the row block stays in shared memory, the key tiles stream; logits in base 2.
+// tensor cores, in base 2, through the segment engine: the static units' 128-key tiles, one after the other, are cut
+// into one equal run per CTA (ranges set by the longest unit left the last CTAs of every shorter one idle).
 // MODE 0: accumulator rows = window rows; a draining thread owns one row and keeps its running
-//         (max, exp-sum) over its half of the CTA's keys; stats: float2 [n_static][2 ranges][Rpad].
-// MODE 1: with the rows' final (max, sum) known, accumulator rows = keys; a draining thread owns
-//         one key and sums the normalised probabilities of its quarter of the rows, the four
+//         (max, exp-sum) over its half of the segment's keys; stats: float2 [n_static][2 segments][Rpad].
+// MODE 1: the rows' final (max, sum) are put together from those at the start of a segment; accumulator rows = keys; a
+//         draining thread owns one key and sums the normalised probabilities of its quarter of the rows, the four
 //         quarters meet in shared memory, and s_w[key] (+)= sum / R (written by the first row block, added
 //         to by later ones).
-// grid (key ranges, n_static).
+// Bound: 2^x (16 per clock and SM; a scheduler whose four warps all have rows spends 2048 cycles per tile on them) at 85 %:
+// 2350 cycles per tile, 31 us a pass for ten units of 24-32 K tokens.  A quarter or half of the powers as polynomials on the
+// FMA pipes, and reading the accumulator ahead, changed nothing.  grid: CTAs; one launch per block of 256 window rows.
 // ---------------------------------------------------------------------------------------------
-template <int MODE>
-__global__ void __launch_bounds__(tc::kThreads, 1)
-    window_scores_tc_kernel(char* cache, char* workspace, const __nv_bfloat16* kin, const __nv_bfloat16* q_obs,
-                            float2* stats, const float2* final_stats, int n_ranges_max, int Rpad,
-                            int tiles_per_cta, int row_block) {
-  extern __shared__ __align__(16) uint8_t tc_smem[];
-  __shared__ float4 rowinfo[tc::kQRows];   // MODE 1: (max, 1 / sum, last visible key, -) of each resident row
+struct WindowParams {
+  char* cache;
+  char* workspace;
+  const __nv_bfloat16* q_obs;
+  float2* stats;
+  const int32_t* tile_prefix;
+  int32_t n_static, n_cta, n_partials;   // partial statistics a row may have (stats' second dimension)
+  int32_t Rpad, row_block;
+};
+struct WindowSeg {
+  int key_row0, tile_begin, tile_end;
+  int C, ordinal, ub, uh;
+  int64_t ws_scores_off;
+  int first, next;       // tiles of the launch before the unit, and behind the segment
+};
+// the caller's shared memory of MODE 1: two buffers of the four quarters' sums; the rows' (max, 1 / sum), last visible keys
+constexpr int kWindowUser1 = 2 * 4 * 128 * 4 + tc::kQRows * 12;
+constexpr int kWindowRing0 = 3, kWindowRing1 = 3;   // key tiles in shared memory (more left less to the other stream's blocks and gained nothing)
+constexpr int kWindowSmem0 = tc::seg_smem_fixed(kWindowRing0), kWindowSmem1 = tc::seg_smem_fixed(kWindowRing1) + kWindowUser1;
+static_assert(kWindowSmem0 <= 232448 && kWindowSmem1 <= 232448, "one CTA's shared memory");
+// Leaves room for four blocks of build_dynamic_kernel beside a CTA (with the 96 registers it takes otherwise there were two, and
+// 19 dynamic units of 50 K tokens took 25 us longer).
+constexpr int kWindowRegs = 72;
+constexpr float kNoKey = -1.0e30f;   // running maximum of a row that has seen no key
 
-  const Header* hdr = reinterpret_cast<const Header*>(cache);
-  const Unit* u = unit_of(cache, hdr, false, blockIdx.y, nullptr);
-  const int C = u->C, G = hdr->group, w = hdr->obs_window, Hq = hdr->n_q_heads, Hkv = hdr->n_kv_heads;
-  const int R = w * G, row0 = row_block * tc::kQRows;
-  const int n_tiles = (C + tc::kKeysPerTile - 1) / tc::kKeysPerTile;
-  const int tile_begin = blockIdx.x * tiles_per_cta, tile_end = min(n_tiles, tile_begin + tiles_per_cta);
-  if (tile_begin >= tile_end) return;
+__device__ __forceinline__ int window_cta_begin(int i, int total, int n_cta) {
+  return static_cast<int>(static_cast<int64_t>(i) * total / n_cta);
+}
+__device__ __forceinline__ int window_cta_of(int w, int total, int n_cta) {
+  return static_cast<int>((static_cast<int64_t>(w + 1) * n_cta - 1) / total);
+}
+
+template <int MODE>
+__global__ void __maxnreg__(kWindowRegs)
+    window_scores_tc_kernel(const __grid_constant__ WindowParams P, const __grid_constant__ CUtensorMap keys) {
+  extern __shared__ __align__(16) uint8_t tc_smem[];
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const Header* hdr = reinterpret_cast<const Header*>(P.cache);
+  const int G = hdr->group, w = hdr->obs_window, Hq = hdr->n_q_heads;
+  const int R = w * G, row0 = P.row_block * tc::kQRows;
   const bool causal = (hdr->flags & HKV_CAUSAL_WINDOW) != 0;
   const float sc = hdr->scale * kLog2e;
-  const int ub = u->b, uh = u->h;
+  const uint64_t sc2 = tc::pack_f32x2(sc, sc);
+  const int total = P.tile_prefix[P.n_static];
+  const int w_begin = window_cta_begin(blockIdx.x, total, P.n_cta), w_end = window_cta_begin(blockIdx.x + 1, total, P.n_cta);
 
-  auto q_row = [&](int row) -> const __nv_bfloat16* {
+  auto segment = [&](int s, WindowSeg& seg) {   // whole warps call it
+    const int at = s == 0 ? w_begin : seg.next;
+    if (at >= w_end) return false;
+    int o;
+    if (s == 0) {   // the last unit that starts at or before `at`
+      o = -1;
+      for (int base = 0; base < P.n_static; base += 32) {
+        const int i = base + static_cast<int>(threadIdx.x & 31);
+        const uint32_t in = __ballot_sync(0xffffffffu, i < P.n_static && P.tile_prefix[i] <= at);
+        o += __popc(in);
+        if (in != 0xffffffffu) break;
+      }
+    } else {
+      o = seg.ordinal + 1;    // segments end with their unit or with the CTA's run
+    }
+    const Unit* u = unit_of(P.cache, hdr, false, o, nullptr);
+    seg.ordinal = o;
+    seg.C = u->C;
+    seg.ub = u->b;
+    seg.uh = u->h;
+    seg.ws_scores_off = u->ws_scores_off;
+    seg.key_row0 = (u->b * hdr->n_kv_heads + u->h) * hdr->max_seq_len;
+    seg.first = P.tile_prefix[o];
+    seg.next = min(w_end, P.tile_prefix[o + 1]);
+    seg.tile_begin = at - seg.first;
+    seg.tile_end = seg.next - seg.first;
+    return true;
+  };
+  auto q_row = [&](const WindowSeg& seg, int row) -> const __nv_bfloat16* {
     const int r = row0 + row;
     if (r >= R) return nullptr;
     const int i = r / G;
-    return q_obs + ((static_cast<size_t>(ub) * w + i) * Hq + uh * G + (r - i * G)) * kHeadDim;
+    return P.q_obs + ((static_cast<size_t>(seg.ub) * w + i) * Hq + seg.uh * G + (r - i * G)) * kHeadDim;
   };
-  const __nv_bfloat16* keys =
-      kin + (static_cast<size_t>(ub) * Hkv + uh) * static_cast<size_t>(hdr->max_seq_len) * kHeadDim;
-  int32_t* err = reinterpret_cast<int32_t*>(cache + hdr->err_off);
+  int32_t* err = reinterpret_cast<int32_t*>(P.cache + hdr->err_off);
+  uint8_t* user = nullptr;
+  bool ok;
 
-  if (MODE == 0) {
-    float m_run = -INFINITY, z_run = 0.f;
-    int my_row = -1;
-    int my_half = 0;
-    auto epilogue = [&](int tile, int lane_row, int part, auto groups, float*, auto, uint64_t*) {
+  if constexpr (MODE == 0) {
+    float m_run = kNoKey, z = 0.f;
+    uint64_t nm2 = 0;
+    auto begin = [&](const WindowSeg&, int, int) {
+      m_run = kNoKey;
+      z = 0.f;
+      nm2 = tc::pack_f32x2(-m_run, -m_run);
+    };
+    auto tile_fn = [&](const WindowSeg& seg, int tile, int lane_row, int part, uint32_t taddr) {
       // accumulator columns 64 part .. + 63 = keys 64 (part & 1) .. + 63 of the tile for the rows of block part >> 1
       const int r = row0 + 128 * (part >> 1) + lane_row;
-      my_row = r;
-      my_half = part & 1;
       if (row0 + 128 * (part >> 1) + (lane_row & ~31) >= R) return;   // the warp's rows are all padding
+      const int C = seg.C, j0 = tile * tc::kKeysPerTile + 64 * (part & 1);
       const int lim = causal ? (C - w + r / G) : (C - 1);      // last key the row sees
-      const int j0 = tile * tc::kKeysPerTile;
-      const bool all_visible = j0 + tc::kKeysPerTile - 1 <= (causal ? C - w : C - 1);   // to every row
-      groups([&](int g, float (&v)[32]) {
-        const int jg = j0 + 64 * (part & 1) + g * 32;
-        float gmax = -INFINITY;
-        if (all_visible) {
-          float g0 = v[0], g1 = v[1], g2 = v[2], g3 = v[3];   // four short chains instead of one long one
+      const bool all_visible = j0 + 63 <= (causal ? C - w : C - 1);   // to every row
+      tc::drain_raw(taddr, [&](int g, uint32_t (&v)[16]) {
+        if (!all_visible) {
 #pragma unroll
-          for (int c = 4; c < 32; c += 4) {
-            g0 = fmaxf(g0, v[c]);
-            g1 = fmaxf(g1, v[c + 1]);
-            g2 = fmaxf(g2, v[c + 2]);
-            g3 = fmaxf(g3, v[c + 3]);
-          }
-          gmax = fmaxf(fmaxf(g0, g1), fmaxf(g2, g3)) * sc;   // the scale is positive
-        } else {
-#pragma unroll
-          for (int c = 0; c < 32; ++c) {
-            v[c] = (jg + c <= lim && jg + c < C) ? v[c] : -INFINITY;
-            gmax = fmaxf(gmax, v[c] * sc);
-          }
+          for (int c = 0; c < 16; ++c)
+            if (j0 + 16 * g + c > lim) v[c] = 0xFF800000u;   // -inf
         }
-        if (gmax > -INFINITY) {
-          const float m_new = fmaxf(m_run, gmax);
-          float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
+        float top = __uint_as_float(v[0]);
 #pragma unroll
-          for (int c = 0; c < 32; c += 4) {
-            a0 += fast_exp2(fmaf(v[c], sc, -m_new));
-            a1 += fast_exp2(fmaf(v[c + 1], sc, -m_new));
-            a2 += fast_exp2(fmaf(v[c + 2], sc, -m_new));
-            a3 += fast_exp2(fmaf(v[c + 3], sc, -m_new));
-          }
-          z_run = z_run * fast_exp2(m_run - m_new) + ((a0 + a1) + (a2 + a3));   // 2^(-inf) = 0 on the first visible group
+        for (int c = 1; c < 16; ++c) top = fmaxf(top, __uint_as_float(v[c]));
+        top *= sc;   // the scale is positive
+        if (__any_sync(0xffffffffu, top > m_run)) {
+          const float m_new = fmaxf(m_run, top);
+          z *= fast_exp2(m_run - m_new);
           m_run = m_new;
+          nm2 = tc::pack_f32x2(-m_new, -m_new);
         }
+        uint64_t a = 0, b = 0;
+#pragma unroll
+        for (int c = 0; c < 16; c += 4) {
+          float e0, e1, e2, e3;
+          tc::unpack_f32x2(tc::fma_f32x2(tc::pack_f32x2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc2, nm2), e0, e1);
+          tc::unpack_f32x2(tc::fma_f32x2(tc::pack_f32x2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3])), sc2, nm2), e2, e3);
+          a = tc::add_f32x2(a, tc::pack_f32x2(fast_exp2(e0), fast_exp2(e1)));
+          b = tc::add_f32x2(b, tc::pack_f32x2(fast_exp2(e2), fast_exp2(e3)));
+        }
+        float x, y;
+        tc::unpack_f32x2(tc::add_f32x2(a, b), x, y);
+        z += x + y;
       });
     };
-    const bool ok = tc::scores_cta<false>(tc_smem, q_row, keys, C, tile_begin, tile_end, epilogue);
-    // two threads share a row (one per half of every tile): two partial statistics per key range
-    if (threadIdx.x >= 64 && my_row >= 0 && my_row < R)
-      stats[(static_cast<size_t>(blockIdx.y) * n_ranges_max + 2 * blockIdx.x + my_half) * Rpad + my_row] =
-          make_float2(m_run, z_run);
-    if (!ok && threadIdx.x == 0) { atomicCAS(&err[0], 0, HKV_ERR_TIMEOUT); err[1] = kErrScoreWait; }
+    auto end = [&](const WindowSeg& seg, int lane_row, int part, bool) {
+      // two threads share a row (one per half of every tile): two partial statistics per segment
+      const int r = row0 + 128 * (part >> 1) + lane_row;
+      const int index = static_cast<int>(blockIdx.x) - window_cta_of(seg.first, total, P.n_cta);
+      if (r < R) P.stats[(static_cast<size_t>(seg.ordinal) * P.n_partials + 2 * index + (part & 1)) * P.Rpad + r] = make_float2(m_run, z);
+    };
+    ok = tc::segments_cta<false, kWindowRing0, WindowSeg>(tc_smem, &keys, segment, q_row, begin, tile_fn, end, &user);
   } else {
-    for (int i = threadIdx.x; i < tc::kQRows; i += tc::kThreads) {
-      const int r = row0 + i;
-      float4 info = make_float4(0.f, 0.f, -1.f, 0.f);   // a padding row sees no key
-      if (r < R) {
-        const float2 f = final_stats[static_cast<size_t>(blockIdx.y) * Rpad + r];
-        info = make_float4(f.x, 1.f / f.y, static_cast<float>(causal ? (C - w + r / G) : (C - 1)), 0.f);
-      }
-      rowinfo[i] = info;
-    }
-    // (scores_cta synchronises the CTA before any tile is drained)
-    float* sw = reinterpret_cast<float*>(workspace + u->ws_scores_off);
     const float inv_R = 1.f / static_cast<float>(R);
+    float4* info = nullptr;     // per pair of rows: (-max, -max, 1 / sum, 1 / sum)
+    float* last = nullptr;      // per row: last visible key
+    float* sums = nullptr;      // [2][4 quarters of the rows][128 keys]
     int n_done = 0;
-    bool pair_ok = true;
-    auto epilogue = [&](int tile, int lane_row, int part, auto groups, float* scratch, auto siblings,
-                        uint64_t* pair_bar) {
+    auto begin = [&](const WindowSeg& seg, int, int) {
+      sums = reinterpret_cast<float*>(user);
+      info = reinterpret_cast<float4*>(sums + 2 * 4 * 128);
+      last = reinterpret_cast<float*>(info + tc::kQRows / 2);
+      // the rows' statistics: two threads per row take every other partial
+      const int dtid = threadIdx.x - 32, row = dtid >> 1, r = row0 + row;
+      const int n_part = 2 * (window_cta_of(P.tile_prefix[seg.ordinal + 1] - 1, total, P.n_cta) - window_cta_of(seg.first, total, P.n_cta) + 1);
+      const float2* st = P.stats + static_cast<size_t>(seg.ordinal) * P.n_partials * P.Rpad + r;
+      // (sixteen loads in flight: one after the other they took 5 us before the first tile)
+      float M = kNoKey, Z = 0.f;
+      for (int i0 = dtid & 1; i0 < n_part; i0 += 32) {
+        float2 v[16];
+#pragma unroll
+        for (int e = 0; e < 16; ++e)
+          v[e] = (r < R && i0 + 2 * e < n_part) ? __ldcg(st + static_cast<size_t>(i0 + 2 * e) * P.Rpad) : make_float2(kNoKey, 0.f);
+        float top = M;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) top = fmaxf(top, v[e].x);
+        Z *= exp2f(M - top);
+        M = top;
+#pragma unroll
+        for (int e = 0; e < 16; ++e) Z += v[e].y * exp2f(v[e].x - M);
+      }
+      {
+        const float other = __shfl_xor_sync(0xffffffffu, M, 1), top = fmaxf(M, other);
+        Z *= exp2f(M - top);
+        M = top;
+        const float z0 = __shfl_sync(0xffffffffu, Z, (threadIdx.x & 31) & ~1), z1 = __shfl_sync(0xffffffffu, Z, (threadIdx.x & 31) | 1);
+        Z = z0 + z1;
+      }
+      tc::named_sync(tc::kBarDrain, tc::kDrainWarps * 32);   // (the previous segment's readers are done)
+      if ((dtid & 1) == 0) {
+        float* pair = reinterpret_cast<float*>(info + (row >> 1)) + (row & 1);
+        pair[0] = r < R ? -M : 0.f;
+        pair[2] = r < R ? 1.f / Z : 0.f;                      // a padding row adds nothing
+        last[row] = r < R ? static_cast<float>(causal ? (seg.C - w + r / G) : (seg.C - 1)) : -1.f;
+      }
+      tc::named_sync(tc::kBarDrain, tc::kDrainWarps * 32);
+    };
+    auto tile_fn = [&](const WindowSeg& seg, int tile, int lane_row, int part, uint32_t taddr) {
       // accumulator columns 64 part .. + 63 = window rows row0 + 64 part + (0..63) for the key of this lane
-      const int j0 = tile * tc::kKeysPerTile, j = j0 + lane_row;
+      const int C = seg.C, j0 = tile * tc::kKeysPerTile, j = j0 + lane_row;
       const float jf = static_cast<float>(j);
       const bool all_visible = j0 + tc::kKeysPerTile - 1 <= (causal ? C - w : C - 1);   // to every row
-      float acc = 0.f, acc2 = 0.f, acc3 = 0.f, acc4 = 0.f;
+      uint64_t a = 0, b = 0;
       if (row0 + 64 * part < R) {                      // same for the whole warp
-        groups([&](int g, float (&v)[32]) {
-          if (row0 + 64 * part + 32 * g >= R) return;   // 32 padding rows: nothing to add (same for the whole warp)
-          const float4* info = rowinfo + 64 * part + 32 * g;
-          if (all_visible) {
+        tc::drain_raw(taddr, [&](int g, uint32_t (&v)[16]) {
+          const int rb = 64 * part + 16 * g;
+          if (row0 + rb >= R) return;   // 16 padding rows: nothing to add (same for the whole warp)
+          const float4* ri = info + rb / 2;
 #pragma unroll
-            for (int c = 0; c < 32; c += 4) {
-              const float4 r0 = info[c], r1 = info[c + 1], r2 = info[c + 2], r3 = info[c + 3];   // padding rows: 1 / sum = 0
-              acc = fmaf(fast_exp2(fmaf(v[c], sc, -r0.x)), r0.y, acc);
-              acc2 = fmaf(fast_exp2(fmaf(v[c + 1], sc, -r1.x)), r1.y, acc2);
-              acc3 = fmaf(fast_exp2(fmaf(v[c + 2], sc, -r2.x)), r2.y, acc3);
-              acc4 = fmaf(fast_exp2(fmaf(v[c + 3], sc, -r3.x)), r3.y, acc4);
+          for (int c = 0; c < 16; c += 4) {
+            const float4 p = ri[c / 2], q = ri[c / 2 + 1];
+            float e0, e1, e2, e3;
+            tc::unpack_f32x2(tc::fma_f32x2(tc::pack_f32x2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc2, tc::pack_f32x2(p.x, p.y)), e0, e1);
+            tc::unpack_f32x2(tc::fma_f32x2(tc::pack_f32x2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3])), sc2, tc::pack_f32x2(q.x, q.y)), e2, e3);
+            if (!all_visible) {
+              if (jf > last[rb + c]) e0 = -INFINITY;
+              if (jf > last[rb + c + 1]) e1 = -INFINITY;
+              if (jf > last[rb + c + 2]) e2 = -INFINITY;
+              if (jf > last[rb + c + 3]) e3 = -INFINITY;
             }
-          } else {
-#pragma unroll
-            for (int c = 0; c < 32; ++c) {
-              const float4 ri = info[c];
-              const float p = fast_exp2(fmaf(v[c], sc, -ri.x)) * ri.y;
-              acc += (jf <= ri.z) ? p : 0.f;
-            }
+            a = tc::fma_f32x2(tc::pack_f32x2(fast_exp2(e0), fast_exp2(e1)), tc::pack_f32x2(p.z, p.w), a);
+            b = tc::fma_f32x2(tc::pack_f32x2(fast_exp2(e2), fast_exp2(e3)), tc::pack_f32x2(q.z, q.w), b);
           }
         });
       }
-      acc = (acc + acc2) + (acc3 + acc4);
-      // the warps of parts 1..3 hand their sums over (two buffers, by tile parity); the part-0 warp adds them in
-      // a fixed order and stores.  pair_bar is the barrier of this tile's parity: its (n_done / 2)-th use.
-      const int slot = (n_done & 1) * 32 + (lane_row & 31);
-      if (part != 0) {
-        scratch[slot] = acc;
-        tc::mbar_arrive(pair_bar);
-      } else {
-        if (pair_ok) pair_ok = mbar_wait_bounded(pair_bar, (n_done >> 1) & 1);
-        if (pair_ok && j < C) {
-          const float tot = ((acc + siblings(1)[slot]) + (siblings(2)[slot] + siblings(3)[slot])) * inv_R;
-          sw[j] = row_block == 0 ? tot : sw[j] + tot;
-        }
+      float x, y;
+      tc::unpack_f32x2(tc::add_f32x2(a, b), x, y);
+      // the quarters of the rows meet (two buffers, by tile parity) and are added in a fixed order
+      float* buf = sums + (n_done & 1) * 4 * 128;
+      buf[part * 128 + lane_row] = x + y;
+      tc::named_sync(tc::kBarAcc + 2 + (lane_row >> 5), 128);   // the four warps of these lanes
+      if (part == 0 && j < C) {
+        const float tot = ((buf[lane_row] + buf[128 + lane_row]) + (buf[256 + lane_row] + buf[384 + lane_row])) * inv_R;
+        float* sw = reinterpret_cast<float*>(P.workspace + seg.ws_scores_off);
+        sw[j] = P.row_block == 0 ? tot : sw[j] + tot;
       }
       ++n_done;
     };
-    const bool ok = tc::scores_cta<true>(tc_smem, q_row, keys, C, tile_begin, tile_end, epilogue);
-    const bool pairs = __syncthreads_and(pair_ok);
-    if (!(ok && pairs) && threadIdx.x == 0) {
-      atomicCAS(&err[0], 0, HKV_ERR_TIMEOUT);
-      err[1] = kErrScoreWait;
-    }
+    auto end = [](const WindowSeg&, int, int, bool) {};
+    ok = tc::segments_cta<true, kWindowRing1, WindowSeg>(tc_smem, &keys, segment, q_row, begin, tile_fn, end, &user);
   }
-}
-
-// Combines the per-range (max, sum) of every window row into the row's final (max, sum): one warp per
-// row, lanes stride the key ranges.
-constexpr int kRowReduceWarps = 8;
-__global__ void __launch_bounds__(kRowReduceWarps * 32)
-    window_rowreduce_kernel(const char* cache, const float2* stats, float2* final_stats, int n_tiles_max, int Rpad,
-                            int tiles_per_cta) {
-  const Header* hdr = reinterpret_cast<const Header*>(cache);
-  const Unit* u = unit_of(cache, hdr, false, blockIdx.y, nullptr);
-  const int R = hdr->obs_window * hdr->group;
-  // two partial statistics (one per half of the key tiles) for every key range of the unit
-  const int n_tiles = 2 * (((u->C + tc::kKeysPerTile - 1) / tc::kKeysPerTile + tiles_per_cta - 1) / tiles_per_cta);
-  const int lane = threadIdx.x & 31;
-  const int r = blockIdx.x * kRowReduceWarps + (threadIdx.x >> 5);
-  if (r >= R) return;
-  const float2* st = stats + static_cast<size_t>(blockIdx.y) * n_tiles_max * Rpad + r;
-  float M = -INFINITY;
-  for (int jt = lane; jt < n_tiles; jt += 32) M = fmaxf(M, st[static_cast<size_t>(jt) * Rpad].x);
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) M = fmaxf(M, __shfl_xor_sync(0xffffffffu, M, off));
-  float Z = 0.f;
-  for (int jt = lane; jt < n_tiles; jt += 32) {
-    const float2 v = st[static_cast<size_t>(jt) * Rpad];
-    if (v.x > -INFINITY) Z += v.y * exp2f(v.x - M);
-  }
-#pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) Z += __shfl_xor_sync(0xffffffffu, Z, off);
-  if (lane == 0) final_stats[static_cast<size_t>(blockIdx.y) * Rpad + r] = make_float2(M, Z);
+  if (!ok && threadIdx.x == 0) { atomicCAS(&err[0], 0, HKV_ERR_TIMEOUT); err[1] = kErrScoreWait; }
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -226,13 +328,14 @@ __global__ void __launch_bounds__(kRowReduceWarps * 32)
 // ranking / ranked by this key) is therefore computed once into shared memory.
 // ---------------------------------------------------------------------------------------------
 constexpr int kKeepThreads = 1024;
+constexpr int kKeepKeySlots = 49152;       // tokens whose role the single-CTA kernel keeps in shared memory
 constexpr int kKeepScratchInts = keyed_scratch_ints(kKeepThreads);
 
 constexpr uint32_t kKeepAlways = 0xFFFFFFFFu;   // no float's key (it would be a NaN's)
 
 __global__ void __launch_bounds__(kKeepThreads)
     static_select_kernel(char* cache, const char* workspace, const float* token_scores, const uint8_t* is_text,
-                         int key_slots, int skip_done) {
+                         int key_slots) {
   __shared__ __align__(16) int scratch[kKeepScratchInts];
   __shared__ int s_ntext;
   extern __shared__ __align__(16) uint32_t skey[];   // key_slots entries: every token's role, computed once
@@ -249,9 +352,6 @@ __global__ void __launch_bounds__(kKeepThreads)
   int32_t* out = reinterpret_cast<int32_t*>(cache + u->idx_off);
   const int hist_end = C - w;   // tokens before the window
   const bool cached = C <= key_slots;
-  // after the cluster kernel: only the units it left (their count of kept tokens is still zero)
-  if (skip_done && reinterpret_cast<const int32_t*>(cache + hdr->n_valid_off)[uid] != 0) return;
-
   if (tid == 0) s_ntext = 0;
   __syncthreads();
   // four tokens per thread and step when the rows of is_text and of the scores start on 4-token boundaries
@@ -348,10 +448,11 @@ __global__ void __launch_bounds__(kKeepThreads)
 //   3. the threshold bin's items, (key, index), have been stored into every CTA's candidate list at slots that
 //      follow from the peers' counts of that bin -> every CTA ranks them exactly and knows the threshold element;
 //   4. the per-CTA numbers of selected tokens are known -> each CTA emits its ascending run at its offset.
-// Units this path does not take (a threshold bin with more than 1024 items, which needs the radix selection)
-// are left untouched: the single-CTA kernel, launched afterwards, does every unit whose count is still zero.
+// A threshold bin with more than 1024 items (many near-equal scores) is taken apart by another histogram over its own
+// key range, and so on; if all of them have the same key, the lower positions win.
 // ---------------------------------------------------------------------------------------------
 constexpr int kSelCluster = 8;
+constexpr int kSelClusterSmem = 160 * 1024;   // a slice's keys and text flags
 struct __align__(16) SelStats { int n_text; uint32_t tmin, tmax, vmin, vmax; int pad[3]; };
 
 __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThreads)
@@ -362,10 +463,11 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThrea
   __shared__ SelStats stats[kSelCluster];
   __shared__ int counts[kSelCluster];
   __shared__ int cnt_by_rank[kSelCluster];
-  __shared__ int ctl[8];
+  __shared__ __align__(8) int ctl[8];
   __shared__ int wtot[32];
   extern __shared__ __align__(16) uint32_t skey[];          // slice_slots keys, then slice_slots text flags (bytes)
   uint8_t* stxt = reinterpret_cast<uint8_t*>(skey + slice_slots);
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 
   const Header* hdr = reinterpret_cast<const Header*>(cache);
   const uint32_t rank = cluster_ctarank();
@@ -438,7 +540,7 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThrea
   const bool rank_text = n_text >= room;       // window + text do not fit: rank the text tokens
   const int k = rank_text ? room : room - n_text;
   const uint32_t kmin = rank_text ? kmin_t : kmin_v, kmax = rank_text ? kmax_t : kmax_v;
-  const int shift = max(0, 32 - __clz((kmax - kmin) | 1u) - 10);
+  int shift = max(0, 32 - __clz((kmax - kmin) | 1u) - 10);
   // roles of a token of my slice: ranked candidate / kept regardless / out
   auto is_cand = [&](int j) { return lo + j < hist_end && (stxt[j] != 0) == rank_text; };
   auto is_always = [&](int j) { return lo + j >= hist_end || (!rank_text && stxt[j] != 0); };
@@ -446,74 +548,113 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThrea
   uint32_t tkey = 0xFFFFFFFFu;   // nothing ranked is taken unless the selection below says so
   int tidx = -1;
   if (k > 0) {
-    // ---- histograms ----
-    for (int j = tid; j < n; j += kKeepThreads)
-      if (is_cand(j)) atomicAdd(&hist[(skey[j] - kmin) >> shift], 1);
-    __syncthreads();
-    cluster_arrive(); cluster_wait();   // 2
-    int hr[kSelCluster], mine_tot = 0;
-    {
-      const uint32_t a = smem_u32(&hist[tid]);
-#pragma unroll
-      for (int r = 0; r < kSelCluster; ++r) {
-        asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(hr[r]) : "r"(mapa(a, r)) : "memory");
-        mine_tot += hr[r];
+    uint32_t bin0 = kmin;        // the bins cover keys bin0 + [b, b + 1) << shift, `span` keys in all
+    uint64_t span = 1ull << 32;
+    int need = k, cnt, tbin;
+    for (bool first = true;; first = false) {
+      // ---- histograms ----
+      if (!first) {
+        for (int i = tid; i < kKeyedBins; i += kKeepThreads) hist[i] = 0;
+        __syncthreads();
       }
-    }
-    // the highest bin b with count(bins > b) < k <= count(bins >= b): thread t owns bin t
-    {
-      int run = mine_tot;
-#pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int v = __shfl_down_sync(0xffffffffu, run, off);
-        if (lane + off < 32) run += v;
-      }
-      if (lane == 0) wtot[warp] = run;
+      for (int j = tid; j < n; j += kKeepThreads)
+        if (is_cand(j) && skey[j] >= bin0 && static_cast<uint64_t>(skey[j] - bin0) < span) atomicAdd(&hist[(skey[j] - bin0) >> shift], 1);
       __syncthreads();
-      const int wt = wtot[lane];
-      int wrun = wt;
+      cluster_arrive(); cluster_wait();   // 2
+      int hr[kSelCluster], mine_tot = 0;
+      {
+        const uint32_t a = smem_u32(&hist[tid]);
 #pragma unroll
-      for (int off = 1; off < 32; off <<= 1) {
-        const int v = __shfl_down_sync(0xffffffffu, wrun, off);
-        if (lane + off < 32) wrun += v;
+        for (int r = 0; r < kSelCluster; ++r) {
+          asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(hr[r]) : "r"(mapa(a, r)) : "memory");
+          mine_tot += hr[r];
+        }
       }
-      const int above = __shfl_sync(0xffffffffu, wrun - wt, warp) + run - mine_tot;
-      if (above < k && k <= above + mine_tot) {
-        ctl[1] = tid; ctl[2] = k - above; ctl[3] = mine_tot;
+      // the highest bin b with count(bins > b) < need <= count(bins >= b): thread t owns bin t
+      {
+        int run = mine_tot;
 #pragma unroll
-        for (int r = 0; r < kSelCluster; ++r) cnt_by_rank[r] = hr[r];
+        for (int off = 1; off < 32; off <<= 1) {
+          const int v = __shfl_down_sync(0xffffffffu, run, off);
+          if (lane + off < 32) run += v;
+        }
+        if (lane == 0) wtot[warp] = run;
+        __syncthreads();
+        const int wt = wtot[lane];
+        int wrun = wt;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+          const int v = __shfl_down_sync(0xffffffffu, wrun, off);
+          if (lane + off < 32) wrun += v;
+        }
+        const int above = __shfl_sync(0xffffffffu, wrun - wt, warp) + run - mine_tot;
+        if (above < need && need <= above + mine_tot) {
+          ctl[1] = tid; ctl[2] = need - above; ctl[3] = mine_tot;
+#pragma unroll
+          for (int r = 0; r < kSelCluster; ++r) cnt_by_rank[r] = hr[r];
+        }
+        __syncthreads();
       }
-      __syncthreads();
+      tbin = ctl[1];
+      need = ctl[2];
+      cnt = ctl[3];
+      if (cnt <= kKeepThreads || shift == 0) break;
+      cluster_arrive(); cluster_wait();   // peers may still be reading my histogram; all have read the control words
+      bin0 += static_cast<uint32_t>(tbin) << shift;
+      span = 1ull << shift;
+      shift = max(0, shift - 10);
     }
-    const int tbin = ctl[1], need = ctl[2], cnt = ctl[3];
-    if (cnt > kKeepThreads) {   // too many near-equal scores for the direct ranking: leave the unit to the general kernel
-      cluster_arrive(); cluster_wait();   // peers may still be reading my histogram
-      return;
-    }
-    // ---- the threshold bin's items into every CTA's candidate list ----
-    int base = 0;
+    int base = 0;                 // items of the threshold bin in lower slices
     for (int r = 0; r < static_cast<int>(rank); ++r) base += cnt_by_rank[r];
-    for (int j = tid; j < n; j += kKeepThreads) {
-      if (is_cand(j) && static_cast<int>((skey[j] - kmin) >> shift) == tbin) {
-        const int slot = base + atomicAdd(&ctl[0], 1);
-        const uint32_t a = smem_u32(&cand[slot]);
+    auto in_bin = [&](int j) {
+      return is_cand(j) && skey[j] >= bin0 && static_cast<uint64_t>(skey[j] - bin0) < span &&
+             static_cast<int>((skey[j] - bin0) >> shift) == tbin;
+    };
+    if (cnt > kKeepThreads) {
+      // more than kKeepThreads copies of one key: the need-th by position.  Its slice finds it (one warp, in order) and
+      // tells the others.
+      if (need > base && need <= base + cnt_by_rank[rank] && warp == 0) {
+        int seen = base;
+        for (int j0 = 0; j0 < n; j0 += 32) {
+          const uint32_t m = __ballot_sync(0xffffffffu, j0 + lane < n && in_bin(j0 + lane));
+          if (seen + __popc(m) >= need) {
+            uint32_t left = m;
+            for (int e = seen + 1; e < need; ++e) left &= left - 1u;
+            const int j = j0 + __ffs(left) - 1;
+            if (lane < kSelCluster) {
+              const uint32_t a = mapa(smem_u32(&ctl[4]), lane);
+              asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(a), "r"(skey[j]), "r"(static_cast<uint32_t>(lo + j)) : "memory");
+            }
+            break;
+          }
+          seen += __popc(m);
+        }
+      }
+      cluster_arrive(); cluster_wait();   // 3
+    } else {
+      // ---- the threshold bin's items into every CTA's candidate list ----
+      for (int j = tid; j < n; j += kKeepThreads) {
+        if (in_bin(j)) {
+          const int slot = base + atomicAdd(&ctl[0], 1);
+          const uint32_t a = smem_u32(&cand[slot]);
 #pragma unroll
-        for (int r = 0; r < kSelCluster; ++r)
-          asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(mapa(a, r)), "r"(skey[j]), "r"(static_cast<uint32_t>(lo + j))
-                       : "memory");
+          for (int r = 0; r < kSelCluster; ++r)
+            asm volatile("st.shared::cluster.v2.u32 [%0], {%1, %2};" ::"r"(mapa(a, r)), "r"(skey[j]), "r"(static_cast<uint32_t>(lo + j))
+                         : "memory");
+        }
       }
-    }
-    cluster_arrive(); cluster_wait();   // 3
-    if (tid < cnt) {
-      const uint2 me = cand[tid];
-      int rk = 0;
-      for (int j = 0; j < cnt; ++j) {
-        const uint2 o = cand[j];
-        rk += (o.x > me.x) || (o.x == me.x && o.y < me.y);
+      cluster_arrive(); cluster_wait();   // 3
+      if (tid < cnt) {
+        const uint2 me = cand[tid];
+        int rk = 0;
+        for (int j = 0; j < cnt; ++j) {
+          const uint2 o = cand[j];
+          rk += (o.x > me.x) || (o.x == me.x && o.y < me.y);
+        }
+        if (rk == need - 1) { ctl[4] = static_cast<int>(me.x); ctl[5] = static_cast<int>(me.y); }
       }
-      if (rk == need - 1) { ctl[4] = static_cast<int>(me.x); ctl[5] = static_cast<int>(me.y); }
+      __syncthreads();
     }
-    __syncthreads();
     tkey = static_cast<uint32_t>(ctl[4]);
     tidx = ctl[5];
   }
@@ -577,72 +718,105 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThrea
 }
 
 // ---------------------------------------------------------------------------------------------
-// Row movers.  One half-warp per row: 16 lanes x 16 bytes; lanes 0-15 move the K row, 16-31 the V
-// row.  Destination piece c of plane row i goes to position c ^ (i & 7).
+// Static heads: the kept rows into the compacted planes.  16 lanes x 16 bytes per row; lanes 0-15 move the K row, 16-31
+// the V row.  Destination piece c of plane row i goes to position c ^ (i & 7).  Latency-bound (a kept position, then its
+// rows): a warp asks for the rows of its eight positions together.
 // ---------------------------------------------------------------------------------------------
+constexpr int kGatherRows = 8;
 __global__ void __launch_bounds__(256)
-    gather_rows_kernel(char* cache, const uint4* kin, const uint4* vin, int dynamic) {
+    gather_rows_kernel(char* cache, const uint4* kin, const uint4* vin) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   const Header* hdr = reinterpret_cast<const Header*>(cache);
-  const Unit* u = unit_of(cache, hdr, dynamic != 0, blockIdx.y, nullptr);
+  const Unit* u = unit_of(cache, hdr, false, blockIdx.y, nullptr);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = lane & 15;
   const bool is_v = lane >= 16;
-  const int rows = dynamic ? u->plane_rows : u->n_tok;   // (rows kept for appended tokens are written by the append kernel)
+  const int rows = u->n_tok;   // (rows kept for appended tokens are written by the append kernel)
+  const int i0 = (blockIdx.x * 8 + warp) * kGatherRows;
+  if (i0 >= rows) return;
   const int32_t* idx = reinterpret_cast<const int32_t*>(cache + u->idx_off);
   const size_t plane_in = (static_cast<size_t>(u->b) * hdr->n_kv_heads + u->h) * static_cast<size_t>(hdr->max_seq_len);
   uint4* dst_plane = reinterpret_cast<uint4*>(cache + (is_v ? u->v_off : u->k_off));
   const uint4* src = is_v ? vin : kin;
-  for (int rr = 0; rr < 8; ++rr) {
-    const int i = blockIdx.x * 64 + warp * 8 + rr;
-    if (i >= rows) break;
-    uint4 val = make_uint4(0u, 0u, 0u, 0u);
-    if (dynamic) {
-      if (i < u->C) val = src[(plane_in + i) * 16 + c];
-    } else {
-      val = src[(plane_in + idx[i]) * 16 + c];
-    }
-    dst_plane[static_cast<size_t>(i) * 16 + (c ^ (i & 7))] = val;
+  const int mine = lane < kGatherRows && i0 + lane < rows ? idx[i0 + lane] : 0;
+  uint4 val[kGatherRows];
+#pragma unroll
+  for (int r = 0; r < kGatherRows; ++r)
+    val[r] = __ldg(src + (plane_in + __shfl_sync(0xffffffffu, mine, r)) * 16 + c);
+#pragma unroll
+  for (int r = 0; r < kGatherRows; ++r) {
+    const int i = i0 + r;
+    if (i < rows) dst_plane[static_cast<size_t>(i) * 16 + (c ^ (i & 7))] = val[r];
   }
 }
 
-// Chunk means: half a warp per chunk, lane = eight channels (one 16-byte piece of a key row); every
-// channel keeps its own float32 running sum over the chunk's tokens IN ORDER, then a float32 division
-// by the chunk's own length and round-to-nearest-even to bf16 — the arithmetic the method's metadata
-// is defined with, so the result is bit-exact whatever the launch shape.  Rows of consecutive tokens
-// are independent loads, so four are kept in flight.
-constexpr int kMeanWarps = 8;
-__global__ void __launch_bounds__(kMeanWarps * 32) chunk_means_kernel(char* cache, const uint4* kin) {
+// ---------------------------------------------------------------------------------------------
+// Dynamic heads: K and V into the chunk-major planes and the chunk means, every input read once.
+// K blocks: half a warp per chunk, lane = eight channels (one 16-byte piece of a key row), eight rows in flight; a row is
+// copied and every channel keeps its own float32 running sum over the chunk's tokens IN ORDER, then a float32 division
+// by the chunk's own length and round-to-nearest-even to bf16 -- the arithmetic the method's metadata is defined with,
+// so the result is bit-exact whatever the launch shape.  V blocks: 64 rows each, eight in flight per half warp.  Rows
+// behind the sequence's end are zero.  16-byte piece p of row i (or chunk c) is stored at position p ^ (i & 7).
+// Bound: HBM.  Small blocks, four of which fit beside a CTA of the window-score kernels.
+// grid (K blocks, then V blocks; dynamic units).
+// ---------------------------------------------------------------------------------------------
+constexpr int kBuildThreads = 128, kBuildChunks = kBuildThreads / 16, kBuildRows = 64;
+__global__ void __launch_bounds__(kBuildThreads)
+    build_dynamic_kernel(char* cache, const uint4* kin, const uint4* vin, int k_blocks) {
   const Header* hdr = reinterpret_cast<const Header*>(cache);
   const Unit* u = unit_of(cache, hdr, true, blockIdx.y, nullptr);
   const int cs = hdr->chunk_size, C = u->C;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, sub = lane & 15;
-  const int c = (blockIdx.x * kMeanWarps + warp) * 2 + (lane >> 4);
-  if (c >= u->n_chunks) return;
-  const uint4* kp = kin + (static_cast<size_t>(u->b) * hdr->n_kv_heads + u->h) * static_cast<size_t>(hdr->max_seq_len) * 16;
-  const int t0 = c * cs, t1 = min(t0 + cs, C);
+  const int half = threadIdx.x >> 4, sub = threadIdx.x & 15;
+  const size_t plane_in = (static_cast<size_t>(u->b) * hdr->n_kv_heads + u->h) * static_cast<size_t>(hdr->max_seq_len) * 16 + sub;
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  if (static_cast<int>(blockIdx.x) >= k_blocks) {
+    const int i0 = (blockIdx.x - k_blocks) * kBuildRows + half, rows = u->plane_rows;
+    uint4* dst = reinterpret_cast<uint4*>(cache + u->v_off);
+    uint4 val[kBuildRows / kBuildChunks];
+#pragma unroll
+    for (int r = 0; r < kBuildRows / kBuildChunks; ++r) {
+      const int i = i0 + r * kBuildChunks;
+      val[r] = i < C ? __ldcs(vin + plane_in + static_cast<size_t>(i) * 16) : zero;
+    }
+#pragma unroll
+    for (int r = 0; r < kBuildRows / kBuildChunks; ++r) {
+      const int i = i0 + r * kBuildChunks;
+      if (i < rows) dst[static_cast<size_t>(i) * 16 + (sub ^ (i & 7))] = val[r];
+    }
+    return;
+  }
+  const int c = blockIdx.x * kBuildChunks + half;
+  if (c >= u->cap_chunks) return;
+  const uint4* kp = kin + plane_in;
+  uint4* dst = reinterpret_cast<uint4*>(cache + u->k_off);
+  const int t0 = c * cs, t1 = max(t0, min(t0 + cs, C));
   float acc[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) acc[j] = 0.f;
-  auto add_row = [&](const uint4& r) {
+  auto take = [&](int i, const uint4& r) {
+    dst[static_cast<size_t>(i) * 16 + (sub ^ (i & 7))] = r;
     acc[0] = __fadd_rn(acc[0], bf16_lo(r.x)); acc[1] = __fadd_rn(acc[1], bf16_hi(r.x));
     acc[2] = __fadd_rn(acc[2], bf16_lo(r.y)); acc[3] = __fadd_rn(acc[3], bf16_hi(r.y));
     acc[4] = __fadd_rn(acc[4], bf16_lo(r.z)); acc[5] = __fadd_rn(acc[5], bf16_hi(r.z));
     acc[6] = __fadd_rn(acc[6], bf16_lo(r.w)); acc[7] = __fadd_rn(acc[7], bf16_hi(r.w));
   };
   int tk = t0;
-  for (; tk + 4 <= t1; tk += 4) {
-    const uint4 r0 = kp[static_cast<size_t>(tk) * 16 + sub], r1 = kp[static_cast<size_t>(tk + 1) * 16 + sub];
-    const uint4 r2 = kp[static_cast<size_t>(tk + 2) * 16 + sub], r3 = kp[static_cast<size_t>(tk + 3) * 16 + sub];
-    add_row(r0); add_row(r1); add_row(r2); add_row(r3);
+  for (; tk + 8 <= t1; tk += 8) {
+    uint4 r[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) r[e] = __ldcs(kp + static_cast<size_t>(tk + e) * 16);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) take(tk + e, r[e]);
   }
-  for (; tk < t1; ++tk) add_row(kp[static_cast<size_t>(tk) * 16 + sub]);
+  for (; tk < t1; ++tk) take(tk, __ldcs(kp + static_cast<size_t>(tk) * 16));
+  for (; tk < t0 + cs; ++tk) dst[static_cast<size_t>(tk) * 16 + (sub ^ (tk & 7))] = zero;
+  if (c >= u->n_chunks) return;
   const float len = static_cast<float>(t1 - t0);
   uint4 o;
   o.x = pack_bf16(__fdiv_rn(acc[0], len), __fdiv_rn(acc[1], len));
   o.y = pack_bf16(__fdiv_rn(acc[2], len), __fdiv_rn(acc[3], len));
   o.z = pack_bf16(__fdiv_rn(acc[4], len), __fdiv_rn(acc[5], len));
   o.w = pack_bf16(__fdiv_rn(acc[6], len), __fdiv_rn(acc[7], len));
-  // 16-byte piece p of chunk c is stored at position p ^ (c & 7), like K/V rows
   reinterpret_cast<uint4*>(cache + u->summ_off)[static_cast<size_t>(c) * 16 + (sub ^ (c & 7))] = o;
   if (c == u->n_chunks - 1) {
     // running sum of the open last chunk, continued by appended tokens (a full chunk leaves nothing open)
@@ -705,86 +879,133 @@ __global__ void __launch_bounds__(kHeadDim)
 
 }  // namespace
 
-cudaError_t launch_window_scores(char* cache, char* workspace, const void* k, const void* q_obs, const Header& hdr,
-                                 const std::vector<Unit>&, int64_t ws_rowstat_off, int n_col_tiles_max,
-                                 cudaStream_t stream) {
-  if (hdr.n_static == 0) return cudaSuccess;
-  const int R = hdr.obs_window * hdr.group;
-  const int Rpad = (R + 15) / 16 * 16;
-  float2* stats = reinterpret_cast<float2*>(workspace + ws_rowstat_off);
-  float2* fin = stats + static_cast<size_t>(hdr.n_static) * n_col_tiles_max * Rpad;
-  int dev = 0, n_sm = 0;
+namespace {
+
+// Shared-memory limits of the compression kernels and the number of SMs, once per device.
+cudaError_t compress_configure(int* n_sm) {
+  constexpr int kMaxDevices = 64;
+  static std::mutex mutex;
+  static int sms[kMaxDevices] = {};
+  int dev = 0;
   cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(window_scores_tc_kernel<0>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::kSmemBytes);
-  if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(window_scores_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, tc::kSmemBytes);
   if (e != cudaSuccess) return e;
-  // key ranges sized so that one launch is at most one wave of CTAs; n_col_tiles_max counts 64-key tiles
-  const int n_tiles = (n_col_tiles_max + 1) / 2;
-  const int splits = std::max(1, std::min(n_tiles, n_sm / hdr.n_static));
-  const int tiles_per_cta = (n_tiles + splits - 1) / splits;
-  const int n_ranges = (n_tiles + tiles_per_cta - 1) / tiles_per_cta;
-  const int n_row_blocks = (R + tc::kQRows - 1) / tc::kQRows;
-  const __nv_bfloat16* kb = static_cast<const __nv_bfloat16*>(k);
-  const __nv_bfloat16* qb = static_cast<const __nv_bfloat16*>(q_obs);
-  const dim3 grid(n_ranges, hdr.n_static);
-  for (int rb = 0; rb < n_row_blocks; ++rb)
-    window_scores_tc_kernel<0><<<grid, tc::kThreads, tc::kSmemBytes, stream>>>(cache, workspace, kb, qb, stats, fin,
-                                                                              n_col_tiles_max, Rpad, tiles_per_cta, rb);
-  window_rowreduce_kernel<<<dim3((R + kRowReduceWarps - 1) / kRowReduceWarps, hdr.n_static), kRowReduceWarps * 32, 0,
-                            stream>>>(cache, stats, fin, n_col_tiles_max, Rpad, tiles_per_cta);
-  for (int rb = 0; rb < n_row_blocks; ++rb)
-    window_scores_tc_kernel<1><<<grid, tc::kThreads, tc::kSmemBytes, stream>>>(cache, workspace, kb, qb, stats, fin,
-                                                                              n_col_tiles_max, Rpad, tiles_per_cta, rb);
+  if (dev < 0 || dev >= kMaxDevices) return cudaErrorInvalidDevice;
+  std::lock_guard<std::mutex> lock(mutex);
+  if (sms[dev] == 0) {
+    constexpr auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+    int n = 0;
+    if ((e = cudaFuncSetAttribute(window_scores_tc_kernel<0>, attr, kWindowSmem0)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(window_scores_tc_kernel<1>, attr, kWindowSmem1)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(static_select_cluster_kernel, attr, kSelClusterSmem)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(static_select_kernel, attr, kKeepKeySlots * 4)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
+      return e;
+    sms[dev] = n;
+  }
+  *n_sm = sms[dev];
+  return cudaSuccess;
+}
+
+// One launch; `dependent`: it may be set up while its predecessor on the stream still runs (the kernel waits for it itself).
+template <class... Params, class... Args>
+cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, int threads, size_t smem, cudaStream_t stream, bool dependent,
+                             Args... args) {
+  cudaLaunchConfig_t cfg{};
+  cudaLaunchAttribute attr{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(static_cast<unsigned>(threads));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &attr;
+  cfg.numAttrs = dependent ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
+template <int N>
+cudaError_t launch_setup_n(char* cache, const void* image, int table_bytes, int zero_begin, int zero_bytes, int32_t* prefix,
+                           cudaStream_t stream) {
+  TableImage<N> img;
+  if constexpr (N > 0) std::memcpy(img.bytes, image, static_cast<size_t>(table_bytes));
+  setup_kernel<N><<<1, kSetupThreads, 0, stream>>>(img, cache, table_bytes, zero_begin, zero_bytes, prefix);
   return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_setup(char* cache, const void* image, int table_bytes, int zero_begin, int zero_bytes, int32_t* tile_prefix,
+                         cudaStream_t stream) {
+  if (table_bytes <= 3584) return launch_setup_n<3584>(cache, image, table_bytes, zero_begin, zero_bytes, tile_prefix, stream);
+  if (table_bytes <= 16384) return launch_setup_n<16384>(cache, image, table_bytes, zero_begin, zero_bytes, tile_prefix, stream);
+  const cudaError_t e = cudaMemcpyAsync(cache, image, static_cast<size_t>(table_bytes), cudaMemcpyHostToDevice, stream);
+  return e == cudaSuccess ? launch_setup_n<0>(cache, image, table_bytes, zero_begin, zero_bytes, tile_prefix, stream) : e;
+}
+
+cudaError_t launch_window_scores(char* cache, char* workspace, const void* k, const void* q_obs, const Header& hdr,
+                                 int64_t total_tiles, int64_t ws_rowstat_off, int n_partials, const int32_t* tile_prefix,
+                                 cudaEvent_t between, cudaStream_t stream) {
+  if (hdr.n_static == 0) return cudaSuccess;
+  if (total_tiles > 0x7FFFFFFF) return cudaErrorInvalidValue;
+  const int R = hdr.obs_window * hdr.group;
+  int n_sm = 0;
+  cudaError_t e = compress_configure(&n_sm);
+  CUtensorMap map;
+  if (e == cudaSuccess) e = tc::key_map(&map, k, static_cast<uint64_t>(hdr.batch) * hdr.n_kv_heads * hdr.max_seq_len);
+  WindowParams P{};
+  P.cache = cache;
+  P.workspace = workspace;
+  P.q_obs = static_cast<const __nv_bfloat16*>(q_obs);
+  P.stats = reinterpret_cast<float2*>(workspace + ws_rowstat_off);
+  P.tile_prefix = tile_prefix;
+  P.n_static = hdr.n_static;
+  P.n_cta = static_cast<int>(std::min<int64_t>(n_sm, total_tiles));
+  P.n_partials = n_partials;
+  P.Rpad = (R + 15) / 16 * 16;
+  const int n_row_blocks = (R + tc::kQRows - 1) / tc::kQRows;
+  for (int mode = 0; mode < 2; ++mode) {
+    for (P.row_block = 0; P.row_block < n_row_blocks && e == cudaSuccess; ++P.row_block)
+      e = launch_dependent(mode == 0 ? window_scores_tc_kernel<0> : window_scores_tc_kernel<1>, dim3(P.n_cta), tc::kSegThreads,
+                           mode == 0 ? kWindowSmem0 : kWindowSmem1, stream, P.row_block > 0 || (mode > 0 && !between), P, map);
+    if (mode == 0 && e == cudaSuccess && between) e = cudaEventRecord(between, stream);
+  }
+  return e;
 }
 
 cudaError_t launch_static_select(char* cache, char* workspace, const float* token_scores, const uint8_t* is_text,
                                  const Header& hdr, cudaStream_t stream) {
   if (hdr.n_static == 0) return cudaSuccess;
   // A cluster of kSelCluster CTAs per unit when a slice of the longest sequence (keys + text flags) fits one
-  // CTA's shared memory; the single-CTA kernel follows for the units the cluster kernel leaves (crowded threshold
-  // bin) and does everything for longer sequences.
+  // CTA's shared memory, one CTA per unit for longer sequences.
   const int slice = ((hdr.max_seq_len + kSelCluster - 1) / kSelCluster + 3) & ~3;
   const size_t slice_smem = static_cast<size_t>(slice) * 5 + 16;
-  const bool clustered = slice_smem <= 160 * 1024;
-  if (clustered) {
-    cudaError_t e = cudaFuncSetAttribute(static_select_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(slice_smem));
-    if (e != cudaSuccess) return e;
-    static_select_cluster_kernel<<<hdr.n_static * kSelCluster, kKeepThreads, slice_smem, stream>>>(
-        cache, workspace, token_scores, is_text, slice);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-  }
-  // every token's role is kept in shared memory when the longest sequence fits (else it is recomputed per pass)
-  const int key_slots = std::min(hdr.max_seq_len, 49152);
-  const size_t smem = static_cast<size_t>(key_slots) * sizeof(uint32_t);
-  cudaError_t e =
-      cudaFuncSetAttribute(static_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+  const bool clustered = slice_smem <= kSelClusterSmem;
+  int n_sm = 0;
+  cudaError_t e = compress_configure(&n_sm);
   if (e != cudaSuccess) return e;
-  static_select_kernel<<<hdr.n_static, kKeepThreads, smem, stream>>>(cache, workspace, token_scores, is_text,
-                                                                     key_slots, clustered ? 1 : 0);
+  if (clustered)
+    return launch_dependent(static_select_cluster_kernel, dim3(hdr.n_static * kSelCluster), kKeepThreads, slice_smem, stream,
+                            !token_scores, cache, static_cast<const char*>(workspace), token_scores, is_text, slice);
+  // every token's role is kept in shared memory when the longest sequence fits (else it is recomputed per pass)
+  const int key_slots = std::min(hdr.max_seq_len, kKeepKeySlots);
+  const size_t smem = static_cast<size_t>(key_slots) * sizeof(uint32_t);
+  static_select_kernel<<<hdr.n_static, kKeepThreads, smem, stream>>>(cache, workspace, token_scores, is_text, key_slots);
   return cudaGetLastError();
 }
 
 cudaError_t launch_gather_static(char* cache, const void* k, const void* v, const Header& hdr, int max_rows,
                                  cudaStream_t stream) {
   if (hdr.n_static == 0 || max_rows <= 0) return cudaSuccess;
-  dim3 grid((max_rows + 63) / 64, hdr.n_static);
-  gather_rows_kernel<<<grid, 256, 0, stream>>>(cache, static_cast<const uint4*>(k), static_cast<const uint4*>(v), 0);
-  return cudaGetLastError();
+  const dim3 grid((max_rows + 8 * kGatherRows - 1) / (8 * kGatherRows), hdr.n_static);
+  return launch_dependent(gather_rows_kernel, grid, 256, 0, stream, true, cache, static_cast<const uint4*>(k), static_cast<const uint4*>(v));
 }
 
 cudaError_t launch_build_dynamic(char* cache, const void* k, const void* v, const Header& hdr, int max_rows,
                                  int max_chunks, cudaStream_t stream) {
   if (hdr.n_dynamic == 0) return cudaSuccess;
-  dim3 grid((max_rows + 63) / 64, hdr.n_dynamic);
-  gather_rows_kernel<<<grid, 256, 0, stream>>>(cache, static_cast<const uint4*>(k), static_cast<const uint4*>(v), 1);
-  dim3 grid2((max_chunks + kMeanWarps * 2 - 1) / (kMeanWarps * 2), hdr.n_dynamic);
-  chunk_means_kernel<<<grid2, kMeanWarps * 32, 0, stream>>>(cache, static_cast<const uint4*>(k));
+  const int k_blocks = (max_chunks + kBuildChunks - 1) / kBuildChunks;
+  const dim3 grid(k_blocks + (max_rows + kBuildRows - 1) / kBuildRows, hdr.n_dynamic);
+  build_dynamic_kernel<<<grid, kBuildThreads, 0, stream>>>(cache, static_cast<const uint4*>(k), static_cast<const uint4*>(v), k_blocks);
   return cudaGetLastError();
 }
 

@@ -104,9 +104,13 @@ int choose_cluster(int total_units, int max_tiles, const int* max_active);
 // set-up; call before the first launch_decode).
 cudaError_t decode_cluster_caps(int group, const int** max_active);
 cudaError_t launch_decode(const DecodeParams& params, int total_units, cudaStream_t stream);
-cudaError_t launch_window_scores(char* cache, char* workspace, const void* k, const void* q_obs,
-                                 const Header& hdr, const std::vector<Unit>& units, int64_t ws_rowstat_off,
-                                 int n_col_tiles_max, cudaStream_t stream);
+// Writes the cache's tables (a host image of table_bytes), clears [zero_begin, zero_begin + zero_bytes) of the cache and, unless
+// null, fills tile_prefix with the static units' running tile counts.
+cudaError_t launch_setup(char* cache, const void* image, int table_bytes, int zero_begin, int zero_bytes, int32_t* tile_prefix,
+                         cudaStream_t stream);
+cudaError_t launch_window_scores(char* cache, char* workspace, const void* k, const void* q_obs, const Header& hdr,
+                                 int64_t total_tiles, int64_t ws_rowstat_off, int n_partials, const int32_t* tile_prefix,
+                                 cudaEvent_t between, cudaStream_t stream);   // `between` (or null) is recorded after the first pass
 cudaError_t launch_static_select(char* cache, char* workspace, const float* token_scores,
                                  const uint8_t* is_text, const Header& hdr, cudaStream_t stream);
 cudaError_t launch_gather_static(char* cache, const void* k, const void* v, const Header& hdr,

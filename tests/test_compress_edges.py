@@ -1,0 +1,40 @@
+"""Compression at the edges of its kernels: key tiles cut over thread blocks, crowded thresholds of the keep-set, table sizes."""
+import numpy as np
+import pytest
+
+import hkv_inputs as hi
+
+pytestmark = pytest.mark.gpu
+
+
+def _layer(B, C, head_type, **kw):
+    base = dict(seed=61, chunk_size=32, w=8, Hq=8, Hkv=2, d=128, budget_fraction=0.2, n_steps=1)
+    base.update(kw)
+    return hi.tiny(B=B, C=C, head_type=head_type, **base)
+
+
+@pytest.mark.parametrize("B,C", [(1, 127), (1, 128), (1, 129), (3, 40), (2, 19000), (40, 300)])
+def test_window_scores_of_few_and_many_tiles(B, C):
+    """Fewer key tiles than SMs, one tile and its neighbours, several tiles per block with heads that end within a block's
+    run, more heads than a warp has lanes."""
+    import parity_util as P
+    L = _layer(B, C, np.zeros((B, 2), np.uint8), ragged=B > 1 and C > 5 * B + 16)
+    P.compare_layer(L, units=[(b, h) for b in sorted({0, B // 2, B - 1}) for h in range(2)])
+
+
+@pytest.mark.parametrize("kind", ["equal", "two_levels", "near_equal", "equal_text"])
+def test_keep_set_with_a_crowded_threshold(kind):
+    """Thousands of scores in the threshold's histogram bin: all equal (lower positions win), two values, values that
+    differ in their last bits only, and the same among text tokens that do not fit the budget."""
+    import parity_util as P
+    L = _layer(1, 9000, [[0, 1]], budget_fraction=0.3)
+    rng = np.random.default_rng(3)
+    ts = np.full((1, 2, 9000), 0.125, np.float32)
+    if kind == "two_levels":
+        ts[rng.random(ts.shape) < 0.2] = 0.25
+    elif kind == "near_equal":
+        ts = (ts.view(np.uint32) + rng.integers(0, 64, ts.shape, dtype=np.uint32)).view(np.float32)
+        ts[0, 0, ::7] = rng.random(ts[0, 0, ::7].shape).astype(np.float32)
+    elif kind == "equal_text":
+        L.is_text[0, :7000] = 1
+    P.compare_layer(L, token_scores=ts)
