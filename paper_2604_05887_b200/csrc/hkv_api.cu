@@ -106,8 +106,6 @@ hkv_status build_plan(const hkv_config* cfg, const int32_t* seq_lens, const uint
   // ---- cache_mem layout ----
   int64_t off = kUnitsOff;
   off = align_up(off + sizeof(Unit) * H.n_units);
-  H.dyn_list_off = off;  off = align_up(off + 4ll * std::max(1, H.n_dynamic));
-  H.sta_list_off = off;  off = align_up(off + 4ll * std::max(1, H.n_static));
   H.n_valid_off = off;   off = align_up(off + 4ll * H.n_units);   // tables end here; the rest starts at zero
   H.err_off = off;       off = align_up(off + 8);
   for (auto& u : c.units) {
@@ -276,11 +274,10 @@ static hkv_status compress_common(const hkv_config* cfg, const void* k, const vo
     const size_t tables = static_cast<size_t>(H.n_valid_off);
     std::vector<char> img(tables, 0);
     std::memcpy(img.data(), &H, sizeof(H));
-    std::memcpy(img.data() + kUnitsOff, c->units.data(), sizeof(Unit) * c->units.size());
-    int32_t* dl = reinterpret_cast<int32_t*>(img.data() + H.dyn_list_off);
-    int32_t* sl = reinterpret_cast<int32_t*>(img.data() + H.sta_list_off);
-    for (int i = 0; i < H.n_units; ++i) {
-      if (c->units[i].type) *dl++ = i; else *sl++ = i;
+    {
+      Unit* dyn = reinterpret_cast<Unit*>(img.data() + kUnitsOff);
+      Unit* sta = dyn + H.n_dynamic;
+      for (const auto& u : c->units) *(u.type ? dyn++ : sta++) = u;
     }
     // the running tile counts lie behind the row statistics (see build_plan)
     const bool window = H.n_static > 0 && !token_scores;
@@ -380,10 +377,12 @@ int hkv_profile_attach(void* dev_buffer, long long n_ctas) {
 }
 #endif
 
-static hkv_status decode_stages(hkv_cache* const* caches, const void* const* q, void* const* out, int32_t n,
-                                void* stream, bool do_select, bool do_attend) {
-  if (!caches || !q || n < 1 || n > kMaxMulti || (do_attend && !out)) return HKV_ERR_INVALID_ARG;
-  DecodeParams P;
+}  // extern "C"
+
+template <int N>
+static hkv_status decode_stages_n(hkv_cache* const* caches, const void* const* q, void* const* out, int32_t n,
+                                  void* stream, bool do_select, bool do_attend) {
+  DecodeParams<N> P;
   std::memset(&P, 0, sizeof(P));
   P.n = n;
   int max_tiles = 1, n_dynamic = 0;
@@ -402,8 +401,6 @@ static hkv_status decode_stages(hkv_cache* const* caches, const void* const* q, 
     P.out[i] = do_attend ? out[i] : nullptr;
     P.n_valid_off[i] = H.n_valid_off;
     P.err_off[i] = H.err_off;
-    P.dyn_list_off[i] = H.dyn_list_off;
-    P.sta_list_off[i] = H.sta_list_off;
     P.n_dynamic[i] = H.n_dynamic;
     P.unit_prefix[i + 1] = P.unit_prefix[i] + H.n_units;
     max_tiles = std::max(max_tiles, c->max_tiles);
@@ -432,12 +429,24 @@ static hkv_status decode_stages(hkv_cache* const* caches, const void* const* q, 
     const long long sta = static_cast<long long>(total_units - n_dynamic) * P.cluster;
     P.static_first = (2 * all > slots && sta <= slots - all) ? 1u : 0u;
   }
-  // The launch may overlap the tail of a preceding decode launch (it touches nothing that depends on
-  // earlier work before its dependency wait).  Right after hkv_compress the cache itself is what
-  // the preceding kernels are still writing, so that first launch is fully serialised.
+  // The launch may start beside the tail of its predecessor on the stream.  After another decode launch it then reads the
+  // cache's tables and first rows at once; right after hkv_compress or hkv_append, which write those, it waits first and
+  // gains the launch's own latency only.
   bool fresh = false;
   for (int i = 0; i < n; ++i) fresh = fresh || caches[i]->fresh;
-  P.pdl = fresh ? 0u : 1u;
+  P.late = fresh ? 1u : 0u;
+  {
+    const int total = P.group * kHeadDim;
+    auto magic = [](int d) { return d > 1 ? 0xFFFFFFFFu / static_cast<uint32_t>(d) + 1u : 0u; };
+    P.merge_per = (((total + P.cluster - 1) / P.cluster) + 3) & ~3;
+    P.cluster_magic = magic(P.cluster);
+    P.merge_magic = magic(P.merge_per);
+    P.chunk_magic = magic(P.chunk_size);
+  }
+  if constexpr (N == 1) {
+    if (!decode_step_instance(P, caches[0]->max_chunks, max_tiles))
+      return decode_stages_n<kMaxMulti>(caches, q, out, n, stream, do_select, do_attend);
+  }
 #ifdef HKV_PROFILE
   {
     const long long ctas = static_cast<long long>(total_units) * P.cluster;
@@ -448,13 +457,28 @@ static hkv_status decode_stages(hkv_cache* const* caches, const void* const* q, 
     }
   }
 #endif
-  if (launch_decode(P, total_units, static_cast<cudaStream_t>(stream)) != cudaSuccess) {
+  cudaError_t e;
+  if constexpr (N == 1) {
+    e = launch_decode_step(P, caches[0]->max_chunks, total_units, static_cast<cudaStream_t>(stream));
+  } else {
+    e = launch_decode(P, total_units, static_cast<cudaStream_t>(stream));
+  }
+  if (e != cudaSuccess) {
     cudaGetLastError();
     return HKV_ERR_CUDA;
   }
   for (int i = 0; i < n; ++i) caches[i]->fresh = false;
   return HKV_OK;
 }
+
+static hkv_status decode_stages(hkv_cache* const* caches, const void* const* q, void* const* out, int32_t n,
+                                void* stream, bool do_select, bool do_attend) {
+  if (!caches || !q || n < 1 || n > kMaxMulti || (do_attend && !out)) return HKV_ERR_INVALID_ARG;
+  return n == 1 ? decode_stages_n<1>(caches, q, out, n, stream, do_select, do_attend)
+                : decode_stages_n<kMaxMulti>(caches, q, out, n, stream, do_select, do_attend);
+}
+
+extern "C" {
 
 hkv_status hkv_decode_attn_multi(hkv_cache* const* caches, const void* const* q, void* const* out, int32_t n,
                                  void* stream) {

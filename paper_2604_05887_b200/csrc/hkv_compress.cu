@@ -19,14 +19,13 @@ constexpr float kLog2e = 1.4426950408889634f;
 
 __device__ __forceinline__ const Unit* unit_of(const char* cache, const Header* hdr, bool dynamic, int ordinal,
                                                int* uid_out) {
-  const int32_t* list = reinterpret_cast<const int32_t*>(cache + (dynamic ? hdr->dyn_list_off : hdr->sta_list_off));
-  const int uid = list[ordinal];
+  const int uid = dynamic ? ordinal : hdr->n_dynamic + ordinal;
   if (uid_out) *uid_out = uid;
   return reinterpret_cast<const Unit*>(cache + kUnitsOff) + uid;
 }
 
 // ---------------------------------------------------------------------------------------------
-// The cache's tables (header, unit records, unit lists) written, the counters behind them cleared, and the running sum
+// The cache's tables (header, unit records) written, the counters behind them cleared, and the running sum
 // of the static units' key tiles, by which the window-score kernels share out their work, left in the workspace.
 // Tables of up to N bytes travel in the launch itself (one launch instead of a staged copy and a fill: 4 us less before
 // the first kernel may start); larger ones have been copied before (N = 0).  One block.
@@ -51,12 +50,11 @@ __global__ void __launch_bounds__(kSetupThreads)
   for (int i = tid * 4; i < zero_bytes; i += kSetupThreads * 4) *reinterpret_cast<int32_t*>(cache + zero_begin + i) = 0;
   if (!tile_prefix) return;
   const Header* hdr = reinterpret_cast<const Header*>(src);
-  const int32_t* list = reinterpret_cast<const int32_t*>(src + hdr->sta_list_off);
-  const Unit* units = reinterpret_cast<const Unit*>(src + kUnitsOff);
+  const Unit* units = reinterpret_cast<const Unit*>(src + kUnitsOff) + hdr->n_dynamic;   // the static ones
   int before = 0;
   for (int base = 0; base < hdr->n_static; base += kSetupThreads) {
     const int i = base + tid;
-    const int mine = i < hdr->n_static ? (units[list[i]].C + tc::kKeysPerTile - 1) / tc::kKeysPerTile : 0;
+    const int mine = i < hdr->n_static ? (units[i].C + tc::kKeysPerTile - 1) / tc::kKeysPerTile : 0;
     int incl = mine;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
@@ -833,32 +831,40 @@ __global__ void __launch_bounds__(kBuildThreads)
 // unit's record is advanced.  One CTA of 128 threads per unit; thread = channel.
 __global__ void __launch_bounds__(kHeadDim)
     append_kernel(char* cache, const __nv_bfloat16* k_new, const __nv_bfloat16* v_new) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  // (what appends never change: read while the predecessor on the stream still runs)
   const Header* hdr = reinterpret_cast<const Header*>(cache);
   Unit* u = reinterpret_cast<Unit*>(cache + kUnitsOff) + blockIdx.x;
   const int d = threadIdx.x, cs = hdr->chunk_size;
-  const int C = u->C;
   const bool dynamic = u->type != 0;
-  const int row = dynamic ? C : u->n_tok;
-  if (row >= u->plane_rows) {   // no room left (the host refuses this before launching)
+  const size_t in = (static_cast<size_t>(u->b) * hdr->n_kv_heads + u->h) * kHeadDim + d;
+  float* tail = reinterpret_cast<float*>(cache + u->tail_sum_off);
+  const int plane_rows = u->plane_rows, budget_raw = u->budget_raw;
+  const int64_t k_off = u->k_off, v_off = u->v_off, summ_off = u->summ_off, idx_off = u->idx_off;
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // what they do change, and the new rows, in one round of loads
+  const volatile Unit* now = u;
+  const int C = now->C, n_tok = now->n_tok;
+  int n_chunks = now->n_chunks;
+  const __nv_bfloat16 kv = k_new[in], vv = v_new[in];
+  const float open_sum = dynamic ? __ldcg(tail + d) : 0.f;
+  const int row = dynamic ? C : n_tok;
+  if (row >= plane_rows) {   // no room left (the host refuses this before launching)
     if (d == 0) {
       int32_t* err = reinterpret_cast<int32_t*>(cache + hdr->err_off);
       if (atomicCAS(&err[0], 0, HKV_ERR_INDEX) == 0) err[1] = kErrIndex;
     }
     return;
   }
-  const size_t in = (static_cast<size_t>(u->b) * hdr->n_kv_heads + u->h) * kHeadDim + d;
-  const __nv_bfloat16 kv = k_new[in], vv = v_new[in];
   const size_t out = static_cast<size_t>(row) * kHeadDim + ((((d >> 3) ^ (row & 7)) << 3) | (d & 7));
-  reinterpret_cast<__nv_bfloat16*>(cache + u->k_off)[out] = kv;
-  reinterpret_cast<__nv_bfloat16*>(cache + u->v_off)[out] = vv;
-  int n_chunks = u->n_chunks;
+  reinterpret_cast<__nv_bfloat16*>(cache + k_off)[out] = kv;
+  reinterpret_cast<__nv_bfloat16*>(cache + v_off)[out] = vv;
   if (dynamic) {
     const int c = C / cs;                       // chunk the new token falls into
     const int len = C - c * cs + 1;
-    float* tail = reinterpret_cast<float*>(cache + u->tail_sum_off);
-    const float sum = __fadd_rn(len == 1 ? 0.f : tail[d], __bfloat162float(kv));
+    const float sum = __fadd_rn(len == 1 ? 0.f : open_sum, __bfloat162float(kv));
     tail[d] = (len == cs) ? 0.f : sum;          // a chunk that just filled up leaves nothing open
-    reinterpret_cast<__nv_bfloat16*>(cache + u->summ_off)[static_cast<size_t>(c) * kHeadDim + ((((d >> 3) ^ (c & 7)) << 3) | (d & 7))] =
+    reinterpret_cast<__nv_bfloat16*>(cache + summ_off)[static_cast<size_t>(c) * kHeadDim + ((((d >> 3) ^ (c & 7)) << 3) | (d & 7))] =
         __float2bfloat16_rn(__fdiv_rn(sum, static_cast<float>(len)));
     n_chunks = c + 1;
   }
@@ -867,12 +873,12 @@ __global__ void __launch_bounds__(kHeadDim)
     u->C = C + 1;
     if (dynamic) {
       u->n_chunks = n_chunks;
-      const int k_sel = min(n_chunks, (min(u->budget_raw, C + 1) + cs - 1) / cs);
+      const int k_sel = min(n_chunks, (min(budget_raw, C + 1) + cs - 1) / cs);
       u->k_sel = k_sel;
       u->n_tok = k_sel * cs;
     } else {
-      reinterpret_cast<int32_t*>(cache + u->idx_off)[u->n_tok] = C;   // position of the new token
-      u->n_tok = u->n_tok + 1;
+      reinterpret_cast<int32_t*>(cache + idx_off)[n_tok] = C;   // position of the new token
+      u->n_tok = n_tok + 1;
     }
   }
 }
@@ -1010,9 +1016,8 @@ cudaError_t launch_build_dynamic(char* cache, const void* k, const void* v, cons
 }
 
 cudaError_t launch_append(char* cache, const void* k_new, const void* v_new, const Header& hdr, cudaStream_t stream) {
-  append_kernel<<<hdr.n_units, kHeadDim, 0, stream>>>(cache, static_cast<const __nv_bfloat16*>(k_new),
-                                                      static_cast<const __nv_bfloat16*>(v_new));
-  return cudaGetLastError();
+  return launch_dependent(append_kernel, dim3(hdr.n_units), kHeadDim, 0, stream, true, cache,
+                          static_cast<const __nv_bfloat16*>(k_new), static_cast<const __nv_bfloat16*>(v_new));
 }
 
 }  // namespace hkv

@@ -134,8 +134,25 @@ __device__ __forceinline__ unsigned long long phase_stamp() {
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-template <int NT, int W>   // NT: 8-wide column tiles of query heads (1 for groups up to 8, 2 up to 16); W: warps
-__global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __grid_constant__ DecodeParams P) {
+// The two rarely taken selections, out of line: the kernel's instructions are read once per launch and CTA, so what a step
+// does not execute must not lie between what it does.
+template <int W>
+__device__ __noinline__ int select_crowded(const float* scores, int n_chunks, int k_sel, uint16_t* out, int* scratch) {
+  return block_topk_smem<W>(scores, n_chunks, k_sel, [&](int pos, int i) { out[pos] = static_cast<uint16_t>(i); }, scratch);
+}
+__device__ __noinline__ int select_global(const float* gscores, int n_chunks, int k_sel, int32_t* gsel, int* scratch) {
+  return block_select_emit(
+      n_chunks, k_sel, [&](int i) { return float_key(__ldcg(&gscores[i])); }, [](int) { return false; },
+      [&](int pos, int i) { gsel[pos] = i; }, scratch, scratch + 256, scratch + 256 + 96);
+}
+
+// NT: 8-wide column tiles of query heads (1 for groups up to 8, 2 up to 16); W: warps; N: caches the arguments have room for.
+// IPT > 0: a whole step of one cache (selection and attention) whose units have at most 256 IPT chunks of a multiple of eight
+// tokens (of kTile, if ONE); IPT = 0: anything.  The general kernel has 160 KB of instructions, more than an SM caches, of which
+// a step executes a fifth: an instance for what nearly every step is made the 28-layer step of four sequences 287 -> 255 us.
+template <int NT, int W, int N, int IPT, bool ONE>
+__global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __grid_constant__ DecodeParams<N> P) {
+  constexpr bool FULL = IPT > 0;
   extern __shared__ __align__(1024) uint8_t smem[];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -144,10 +161,13 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
   const bool clustered = csize > 1;
   const uint32_t crank = clustered ? cluster_ctarank() : 0u;
   HKV_STAMP(0)
+  // A launch whose caches have just been written waits before it reads anything and lets its successor start only then: what
+  // starts before its predecessors are done may rely on every write but those of the last decode launches.
+  if (P.late) pdl_wait();
   pdl_launch_dependents();
 
-  const int cid = blockIdx.x / csize;
-  const int li = find_slot(P.unit_prefix, P.n, cid);
+  const int cid = static_cast<int>(cluster_id());
+  const int li = N == 1 ? 0 : find_slot(P.unit_prefix, P.n, cid);
   char* base = P.cache[li];
   int uid;
   {
@@ -155,19 +175,16 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
     // device has room for while its predecessor still runs: the unit type that gains most from that early
     // start (see decode_stages) takes the cache's first clusters.
     const int c = cid - P.unit_prefix[li], nd = P.n_dynamic[li], ns = P.unit_prefix[li + 1] - P.unit_prefix[li] - nd;
-    const int32_t* dl = reinterpret_cast<const int32_t*>(base + P.dyn_list_off[li]);
-    const int32_t* sl = reinterpret_cast<const int32_t*>(base + P.sta_list_off[li]);
-    if (P.static_first) uid = c < ns ? sl[c] : dl[c - ns];
-    else uid = c < nd ? dl[c] : sl[c - nd];
+    uid = P.static_first ? (c < ns ? nd + c : c - ns) : c;   // (the table holds the dynamic units first)
   }
   const Unit* up = reinterpret_cast<const Unit*>(base + kUnitsOff) + uid;
   const int G = P.group, Hq = P.n_q_heads, cs = P.chunk_size;
-  const int ub = uid / P.n_kv_heads, uh = uid - ub * P.n_kv_heads;
-  const bool do_select = (P.phase & kPhaseSelect) != 0, do_attend = (P.phase & kPhaseAttend) != 0;
+  const bool do_select = FULL || (P.phase & kPhaseSelect) != 0, do_attend = FULL || (P.phase & kPhaseAttend) != 0;
   constexpr bool kPushMerge = NT == 1;   // wider groups do not fit the receive area and use the pull merge
 
   // the unit's record (uniform loads, issued together)
   const int utype = up->type, C = up->C, n_tok = up->n_tok, n_chunks = up->n_chunks, k_sel = up->k_sel;
+  const int ub = up->b, uh = up->h;
 #ifdef HKV_CHECKED
   const int plane_rows = up->plane_rows;
 #endif
@@ -183,18 +200,16 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
   // merge geometry (push merge): the output's G*128 elements are dealt to the cluster's CTAs in slices of
   // `per`; CTA r owns elements [r * per, r * per + own_cnt(r))
   const int total = G * kHeadDim;
-  const int per = (((total + csize - 1) / csize) + 3) & ~3;
-  // divisions by the cluster size, the slice length and the chunk size sit on the step's critical path
-  // further down: their multipliers are worked out here, before the dependency wait
-  const uint32_t csize_magic = clustered ? fastdiv_magic(static_cast<uint32_t>(csize)) : 0u;
-  const uint32_t per_magic = fastdiv_magic(static_cast<uint32_t>(per));
-  const bool cs_fast = cs > 1 && static_cast<uint64_t>(n_tok) * static_cast<uint64_t>(cs) < (1ull << 32);
-  const uint32_t cs_magic = cs > 1 ? fastdiv_magic(static_cast<uint32_t>(cs)) : 0u;
+  const int per = P.merge_per;
+  // divisions by the cluster size, the slice length and the chunk size by the host's multipliers: here they delay the first
+  // copies wherever the launch cannot start beside its predecessor, further down they sit on the step's chain
+  const uint32_t csize_magic = P.cluster_magic, per_magic = P.merge_magic, cs_magic = P.chunk_magic;
+  const bool cs_fast = FULL || (cs > 1 && static_cast<uint64_t>(n_tok) * static_cast<uint64_t>(cs) < (1ull << 32));
   auto div_cs = [&](int x) { return cs_fast ? fastdiv(x, cs_magic) : x / cs; };
   auto own_cnt = [&](int r) { return max(0, min(total, (r + 1) * per) - r * per); };
 
   const bool identity = dynamic && k_sel >= n_chunks;          // every chunk is loaded: no list needed
-  const bool fits = n_chunks <= kSelSmemChunks;                // scores and ids fit shared memory
+  const bool fits = FULL || n_chunks <= kSelSmemChunks;                // scores and ids fit shared memory
   const bool scoring = dynamic && do_select;
   // scores travel through shared memory (and the exchange between the cluster's CTAs) only when a selection
   // needs them there; otherwise they go straight to global memory
@@ -272,15 +287,15 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
   // every tile inside one chunk (one copy pair, issued by lane 0); any other size lets up to 32
   // chunks touch a tile (one lane per chunk).  Row keys differ from (row & 7) only when the chunk
   // size is not a multiple of 8.
-  const bool one_chunk = !contiguous && (cs % kTile) == 0;
-  const bool need_keys = !contiguous && (cs & 7) != 0;
+  const bool one_chunk = !contiguous && (ONE || (!FULL && (cs % kTile) == 0));
+  const bool need_keys = !FULL && !contiguous && (cs & 7) != 0;
   auto issue_attn = [&](int j) {   // whole warp; arms stage (seq0 + j) % stages with CTA tile j
     const int stage = (seq0 + j) % kDecStages;
     uint8_t* st = smem + stage * kStageBytes;
     const int v0 = (at_tile0 + j) * kTile;
     const int v1 = min(v0 + kTile, n_valid);
     HKV_CHECK(v0 >= 0 && v0 < v1 && v1 - v0 <= kTile, 100);
-    if (contiguous || one_chunk) {
+    if (ONE || contiguous || one_chunk) {
       if (lane == 0) {
         size_t row = static_cast<size_t>(v0);
         if (one_chunk) {
@@ -347,7 +362,7 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
   int wb_lo = 0, wb_hi = 0;   // this CTA's share of the score write-back
   bool sc_fine = true;
   if (scoring) {
-    const int mt_per = (n_mt + csize - 1) / csize;
+    const int mt_per = clustered ? fastdiv(n_mt + csize - 1, csize_magic) : n_mt;
     sc_row0 = min(n_chunks, static_cast<int>(crank) * mt_per * 16);
     sc_row1 = min(n_chunks, sc_row0 + mt_per * 16);
     sc_n = (sc_row1 - sc_row0 + kScoreTile - 1) / kScoreTile;
@@ -375,8 +390,9 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
   // does not read).  Who asks for what is settled here, off the critical path.
   bool early_on = false;
   if (exchange && do_attend && !P.offload) {
-    const int my_tiles = ((k_sel * cs + kTile - 1) / kTile + csize - 1) / csize;
-    early_on = my_tiles <= kPrefetchMaxTiles && (tid % csize) == static_cast<int>(crank);
+    const int tiles = (k_sel * cs + kTile - 1) / kTile;
+    const int my_tiles = clustered ? fastdiv(tiles + csize - 1, csize_magic) : tiles;
+    early_on = my_tiles <= kPrefetchMaxTiles && (!clustered || tid - fastdiv(tid, csize_magic) * csize == static_cast<int>(crank));
   }
   auto early = [&](int ci) {
     if (!early_on) return;
@@ -567,34 +583,33 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
           hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, off));
         }
         uint2* cand = reinterpret_cast<uint2*>(smem + kCandOff);
-        const int ipt = (n_chunks + W * 32 - 1) / (W * 32);
+        [[maybe_unused]] const int ipt = (n_chunks + W * 32 - 1) / (W * 32);
         auto stamp = [&](int k2) { HKV_STAMP(20 + k2) };
         emitted = -1;
-        if (ipt <= 1) emitted = block_topk_blocked<W, 1, 256>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
-        else if (ipt <= 2) emitted = block_topk_blocked<W, 2, 256>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
-        else if (ipt <= 4) emitted = block_topk_blocked<W, 4, 512>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
-        else if (ipt <= 8) emitted = block_topk_blocked<W, 8, 512>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
+        if constexpr (FULL) {
+          emitted = block_topk_blocked<W, FULL ? IPT : 1, IPT <= 2 ? 256 : 512>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
+        } else {
+          if (ipt <= 1) emitted = block_topk_blocked<W, 1, 256>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
+          else if (ipt <= 2) emitted = block_topk_blocked<W, 2, 256>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
+          else if (ipt <= 4) emitted = block_topk_blocked<W, 4, 512>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
+          else if (ipt <= 8) emitted = block_topk_blocked<W, 8, 512>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
+        }
         if (emitted < 0) {
           // crowded threshold bin (or more scores than the fast path takes): the general selection, its
           // scratch in the idle ring
-          emitted = block_topk_smem<W>(
-              sc_smem, n_chunks, k_sel, [&](int pos, int i) { sel16[pos] = static_cast<uint16_t>(i); },
-              reinterpret_cast<int*>(smem));
+          emitted = select_crowded<W>(sc_smem, n_chunks, k_sel, sel16, reinterpret_cast<int*>(smem));
           fence_proxy_async();   // the ring goes back to the bulk copies
           __syncthreads();
         }
         sel_in_smem = true;
       }
-    } else {
+    } else if constexpr (!FULL) {
       // more chunks than shared memory holds: selection on the scores in global memory; every CTA of the
       // cluster writes the same list to the same place
       __threadfence();
       if (clustered) { cluster_arrive(); cluster_wait(); } else { __syncthreads(); }
       HKV_STAMP(5)
-      int* fb = reinterpret_cast<int*>(smem);
-      emitted = block_select_emit(
-          n_chunks, k_sel, [&](int i) { return float_key(__ldcg(&gscores[i])); }, [](int) { return false; },
-          [&](int pos, int i) { gsel[pos] = i; }, fb, fb + 256, fb + 256 + 96);
+      emitted = select_global(gscores, n_chunks, k_sel, gsel, reinterpret_cast<int*>(smem));
       fence_proxy_async();
       __syncthreads();
     }
@@ -622,7 +637,7 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
     if (!do_attend) return;
     // "my selection is done": from here on my score area is free to receive the peers' partial results
     if (clustered && kPushMerge && !bar_pending) { cluster_arrive_relaxed(); bar_pending = true; }
-  } else if (dynamic) {
+  } else if (!FULL && dynamic) {
     setup_attn(__ldcg(n_valid_g));   // attention only: the list of an earlier selection
   }
 
@@ -630,7 +645,7 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
   // flash-decoding over the unit's token list
   // =============================================================================================
   const float sc = P.scale_log2e;
-  if (!attn_armed && !dead) {
+  if (!FULL && !attn_armed && !dead) {
     for (int j = warp; j < min(at_n, kDecStages); j += W) issue_attn(j);
   }
 
@@ -790,7 +805,9 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
   }
 
   };
-  if (need_keys) run_tiles(std::true_type{}); else run_tiles(std::false_type{});
+  if constexpr (FULL) run_tiles(std::false_type{});
+  else if (need_keys) run_tiles(std::true_type{});
+  else run_tiles(std::false_type{});
 
   HKV_STAMP(8)
   // a warp that gave up tells the others, so that nobody parks results over copies still in flight
@@ -1046,16 +1063,24 @@ cudaError_t configure(const ClusterCaps** out) {
   std::lock_guard<std::mutex> lock(g_caps_mutex);
   ClusterCaps& caps = caps_of[dev];
   if (!caps.ready) {
-    e = cudaFuncSetAttribute(decode_kernel<NT, warps_of(NT)>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(decode_kernel<NT, warps_of(NT)>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    auto allow = [&](auto kernel) {
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+    };
+    allow(decode_kernel<NT, warps_of(NT), kMaxMulti, 0, false>);
+    if constexpr (NT == 1) {
+      allow(decode_kernel<1, warps_of(1), 1, 1, false>); allow(decode_kernel<1, warps_of(1), 1, 1, true>);
+      allow(decode_kernel<1, warps_of(1), 1, 2, false>); allow(decode_kernel<1, warps_of(1), 1, 2, true>);
+      allow(decode_kernel<1, warps_of(1), 1, 4, false>); allow(decode_kernel<1, warps_of(1), 1, 4, true>);
+      allow(decode_kernel<1, warps_of(1), 1, 8, false>); allow(decode_kernel<1, warps_of(1), 1, 8, true>);
+    }
     if (e != cudaSuccess) return e;
     for (int c = 1; c <= kMaxCluster; ++c) {
       cudaLaunchConfig_t cfg;
       cudaLaunchAttribute attr[2];
       fill_config<NT>(cfg, attr, 1, c, false, nullptr);
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, decode_kernel<NT, warps_of(NT)>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+      if (cudaOccupancyMaxActiveClusters(&n, decode_kernel<NT, warps_of(NT), kMaxMulti, 0, false>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
       caps.max_active[c] = n;
     }
     caps.ready = true;
@@ -1064,12 +1089,12 @@ cudaError_t configure(const ClusterCaps** out) {
   return cudaSuccess;
 }
 
-template <int NT>
-cudaError_t launch_nt(const DecodeParams& params, int total_units, cudaStream_t stream) {
+template <int NT, int N, int IPT, bool ONE>
+cudaError_t launch_nt(const DecodeParams<N>& params, int total_units, cudaStream_t stream) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
-  fill_config<NT>(cfg, attr, total_units, params.cluster, params.pdl != 0, stream);
-  return cudaLaunchKernelEx(&cfg, decode_kernel<NT, warps_of(NT)>, params);
+  fill_config<NT>(cfg, attr, total_units, params.cluster, true, stream);
+  return cudaLaunchKernelEx(&cfg, decode_kernel<NT, warps_of(NT), N, IPT, ONE>, params);
 }
 
 }  // namespace
@@ -1120,10 +1145,28 @@ cudaError_t launch_selftest_wait(int32_t* err_word, cudaStream_t stream) {
 }
 #endif
 
-cudaError_t launch_decode(const DecodeParams& params, int total_units, cudaStream_t stream) {
+cudaError_t launch_decode(const DecodeParams<kMaxMulti>& params, int total_units, cudaStream_t stream) {
   if (total_units <= 0) return cudaSuccess;
-  if (params.group > 8) return launch_nt<2>(params, total_units, stream);
-  return launch_nt<1>(params, total_units, stream);
+  return params.group > 8 ? launch_nt<2, kMaxMulti, 0, false>(params, total_units, stream)
+                          : launch_nt<1, kMaxMulti, 0, false>(params, total_units, stream);
+}
+
+bool decode_step_instance(const DecodeParams<1>& P, int max_chunks, int max_tiles) {
+  return P.phase == (kPhaseSelect | kPhaseAttend) && P.group <= 8 && P.chunk_size % 8 == 0 && max_chunks <= kSelSmemChunks &&
+         static_cast<uint64_t>(max_tiles + 1) * kTile * static_cast<uint64_t>(P.chunk_size) < (1ull << 32);
+}
+
+cudaError_t launch_decode_step(const DecodeParams<1>& params, int max_chunks, int total_units, cudaStream_t stream) {
+  if (total_units <= 0) return cudaSuccess;
+  const bool one = params.chunk_size % kTile == 0;
+  auto go = [&](auto ipt) {
+    return one ? launch_nt<1, 1, decltype(ipt)::value, true>(params, total_units, stream)
+               : launch_nt<1, 1, decltype(ipt)::value, false>(params, total_units, stream);
+  };
+  if (max_chunks <= 256) return go(std::integral_constant<int, 1>{});
+  if (max_chunks <= 512) return go(std::integral_constant<int, 2>{});
+  if (max_chunks <= 1024) return go(std::integral_constant<int, 4>{});
+  return go(std::integral_constant<int, 8>{});
 }
 
 }  // namespace hkv

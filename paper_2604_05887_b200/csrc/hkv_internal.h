@@ -23,7 +23,8 @@ constexpr int kStageBytes = kTile * kRowBytes * 2 + 256;   // K tile + V tile + 
 constexpr int kScoreTile = 2 * kTile;     // most chunk means one stage holds while chunks are scored
 constexpr int kSelSmemChunks = 2048;      // chunk scores / selected ids a CTA keeps in shared memory
 
-// One (sequence b, kv head h) pair of a layer; unit id = b * n_kv_heads + h.
+// One (sequence b, kv head h) pair of a layer.  On the device the dynamic units come first, then the static ones, so that a
+// kernel of one type finds its record without a list; the host keeps them by b * n_kv_heads + h.
 struct Unit {
   int32_t type;        // 0 static, 1 dynamic
   int32_t b, h;
@@ -53,17 +54,16 @@ struct Header {
   uint32_t flags;
   float scale;
   int32_t pad[3];
-  int64_t dyn_list_off;  // int32[n_dynamic] unit ids of dynamic units
-  int64_t sta_list_off;  // int32[n_static]
   int64_t n_valid_off;   // int32[n_units] attended tokens (dynamic: written by every selection)
   int64_t err_off;       // int32[2] device error word: code, detail
 };
 constexpr int64_t kUnitsOff = 256;
 static_assert(sizeof(Header) <= kUnitsOff, "Header layout");
 
-// Arguments of the decode kernel: up to kMaxMulti caches side by side.  A cluster of `cluster`
-// CTAs works on one unit; clusters [unit_prefix[i], unit_prefix[i+1]) belong to cache i.
+// Arguments of the decode kernel for up to N caches side by side (1, or kMaxMulti).  A cluster of `cluster` CTAs works on one unit; clusters
+// [unit_prefix[i], unit_prefix[i+1]) belong to cache i.
 enum DecodePhase : uint32_t { kPhaseSelect = 1u, kPhaseAttend = 2u };
+template <int N>
 struct DecodeParams {
   int32_t n;
   int32_t cluster;
@@ -71,19 +71,21 @@ struct DecodeParams {
   float scale_log2e;
   uint32_t phase;      // kPhaseSelect | kPhaseAttend
   uint32_t out_f32;
-  uint32_t pdl;        // launched with programmatic stream serialization
   uint32_t group_max;  // chunk score = max over the group's heads instead of their sum
   uint32_t offload;    // the dynamic units' K/V planes live in host memory: no L2 prefetch requests for them
-  int32_t unit_prefix[kMaxMulti + 1];
-  char* cache[kMaxMulti];
-  const void* q[kMaxMulti];
-  void* out[kMaxMulti];
-  int64_t n_valid_off[kMaxMulti];
-  int64_t err_off[kMaxMulti];
-  int64_t dyn_list_off[kMaxMulti];   // unit ids of each cache's dynamic / static units: a cache's clusters take one
-  int64_t sta_list_off[kMaxMulti];   // type first, then the other (static_first)
-  int32_t n_dynamic[kMaxMulti];
-  uint32_t static_first;
+  uint32_t static_first;             // a cache's clusters take its static units first, then the dynamic ones
+  uint32_t late;                     // a cache of this launch has just been written: nothing is read before the dependency wait
+  // multipliers of the divisions by the cluster size, a CTA's slice of the merge and the chunk size (device code divides by
+  // them where every instruction counts); 0 where the divisor is 1
+  int32_t merge_per;
+  uint32_t cluster_magic, merge_magic, chunk_magic;
+  int32_t unit_prefix[N + 1];
+  char* cache[N];
+  const void* q[N];
+  void* out[N];
+  int64_t n_valid_off[N];
+  int64_t err_off[N];
+  int32_t n_dynamic[N];
 #ifdef HKV_PROFILE
   unsigned long long* prof;   // kProfSlots time stamps (ns) per CTA, or null
 #endif
@@ -103,7 +105,11 @@ int choose_cluster(int total_units, int max_tiles, const int* max_active);
 // Cluster capacities of the decode kernel for this group size (also performs the kernel's one-time
 // set-up; call before the first launch_decode).
 cudaError_t decode_cluster_caps(int group, const int** max_active);
-cudaError_t launch_decode(const DecodeParams& params, int total_units, cudaStream_t stream);
+cudaError_t launch_decode(const DecodeParams<kMaxMulti>& params, int total_units, cudaStream_t stream);
+// The instances for a whole step of one cache (longest token list max_tiles tiles, at most max_chunks chunks per unit), and
+// whether they take it.
+bool decode_step_instance(const DecodeParams<1>& params, int max_chunks, int max_tiles);
+cudaError_t launch_decode_step(const DecodeParams<1>& params, int max_chunks, int total_units, cudaStream_t stream);
 // Writes the cache's tables (a host image of table_bytes), clears [zero_begin, zero_begin + zero_bytes) of the cache and, unless
 // null, fills tile_prefix with the static units' running tile counts.
 cudaError_t launch_setup(char* cache, const void* image, int table_bytes, int zero_begin, int zero_bytes, int32_t* tile_prefix,
