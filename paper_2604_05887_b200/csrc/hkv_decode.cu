@@ -252,14 +252,17 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
   // Waits until stage `stage` holds the tile with ring sequence number `q` (0-based over both
   // phases): first until it has been armed with that tile, then until the copies have landed.
   // Both waits are bounded; false = gave up.
-  auto wait_tile = [&](int stage, uint32_t q) -> bool {
+  auto wait_armed = [&](int stage, uint32_t q) -> bool {
     if (armed[stage] != q + 1u) {
       const long long start = clock64();
       for (uint32_t it = 1; armed[stage] != q + 1u; ++it) {
         if ((it & 255u) == 0u && clock64() - start > HKV_WAIT_CYCLES) return false;
       }
     }
-    return mbar_wait_bounded(&bars[stage], (q / kDecStages) & 1u);
+    return true;
+  };
+  auto wait_tile = [&](int stage, uint32_t q) -> bool {
+    return wait_armed(stage, q) && mbar_wait_bounded(&bars[stage], (q / kDecStages) & 1u);
   };
 
   bool dead = false;    // a bounded wait ran out: stop issuing, keep every hand-over
@@ -576,6 +579,7 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
       HKV_STAMP(5)
       if (!dead) {
         float lo = INFINITY, hi = -INFINITY;
+#pragma unroll 1   // (unrolled, it delayed the step by 0.1 us per layer)
         for (int i = lane; i < csize * W; i += 32) { const float2 b2 = bounds[i]; lo = fminf(lo, b2.x); hi = fmaxf(hi, b2.y); }
 #pragma unroll
         for (int off = 16; off >= 1; off >>= 1) {
@@ -669,7 +673,18 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
     uint8_t* st = smem + stage * kStageBytes;
     const int v0 = (at_tile0 + j) * kTile;
     const int nrow = min(kTile, n_valid - v0);
-    if (!wait_tile(stage, seq0 + static_cast<uint32_t>(j))) {
+    const bool partial = nrow < kTile;
+    bool there = wait_armed(stage, seq0 + static_cast<uint32_t>(j));
+    if (partial && there) {
+      // V rows past the end are not copied: cleared, while the others are still on their way, so that stale bits cannot
+      // poison P*V (their logits are masked, so stale K rows do no harm)
+      for (int r = nrow + (lane >> 4); r < kTile; r += 2)
+        reinterpret_cast<uint4*>(st + kTile * kRowBytes + r * kRowBytes)[lane & 15] = make_uint4(0u, 0u, 0u, 0u);
+      fence_proxy_async();
+      __syncwarp();
+    }
+    there = there && mbar_wait_bounded(&bars[stage], ((seq0 + static_cast<uint32_t>(j)) / kDecStages) & 1u);
+    if (!there) {
       if (lane == 0) { atomicCAS(&err[0], 0, HKV_ERR_TIMEOUT); err[1] = kErrDecodeWait; }
       dead = true;
       break;
@@ -685,16 +700,6 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
     dead = __any_sync(0xffffffffu, dead);
     if (dead) break;
 #endif
-    const bool partial = nrow < kTile;
-    if (partial) {
-      // rows past the end were not copied: clear them so that stale bits cannot poison P*V
-      for (int r = nrow; r < kTile; ++r) {
-        reinterpret_cast<uint2*>(st + r * kRowBytes)[lane] = make_uint2(0u, 0u);
-        reinterpret_cast<uint2*>(st + kTile * kRowBytes + r * kRowBytes)[lane] = make_uint2(0u, 0u);
-      }
-      fence_proxy_async();
-      __syncwarp();
-    }
     const uint32_t kbase = smem_u32(st), vbase = kbase + kTile * kRowBytes;
 
     // S^T = K Q^T : rows = tokens (two 16-row tiles), columns = query heads; the reduction over the
