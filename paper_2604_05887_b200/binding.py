@@ -134,9 +134,14 @@ def _ptr(a: np.ndarray, ctype):
     return a.ctypes.data_as(C.POINTER(ctype))
 
 
-def _host(a: np.ndarray) -> int:
-    """Host address of an array's first element (a typed ctypes pointer costs 1.5 us to make)."""
-    return a.ctypes.data
+_INT32, _UINT8 = np.dtype(np.int32), np.dtype(np.uint8)
+
+
+def _host(a, dtype) -> bytes:
+    """A host table as the bytes the library reads during the call (an array's ctypes address costs ten times as much)."""
+    if type(a) is not np.ndarray or a.dtype != dtype:
+        a = np.asarray(a).astype(dtype)
+    return a.tobytes()
 
 
 def _dev(t) -> Optional[int]:
@@ -148,19 +153,22 @@ def _dev(t) -> Optional[int]:
     return t.data_ptr()
 
 
-_raw_current_stream = None   # () -> address of the current device's current stream, resolved at the first call
+def _first_stream() -> Optional[int]:
+    """Address of the current device's current stream.  The address alone: torch.cuda.current_stream() builds a Stream
+    object around it, which took 3.6 us per call, as much as the launch that follows.  (The first call resolves the two
+    functions and replaces itself.)"""
+    global _current_stream
+    import torch
+    torch.cuda.init()
+    get_stream, get_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
+
+    def current() -> Optional[int]:
+        return get_stream(get_device()) or None
+    _current_stream = current
+    return current()
 
 
-def _current_stream() -> Optional[int]:
-    """The address alone: torch.cuda.current_stream() builds a Stream object around it, which took 3.6 us per call,
-    as much as the launch that follows."""
-    global _raw_current_stream
-    if _raw_current_stream is None:
-        import torch
-        torch.cuda.init()
-        get_stream, get_device = torch._C._cuda_getCurrentRawStream, torch._C._cuda_getDevice
-        _raw_current_stream = lambda: get_stream(get_device())  # noqa: E731
-    return _raw_current_stream() or None
+_current_stream = _first_stream
 
 
 def _stream(stream) -> Optional[int]:
@@ -179,9 +187,9 @@ def make_config(batch, n_q_heads, n_kv_heads, head_dim, max_seq_len, chunk_size,
 
 def hkv_plan(cfg: hkv_config, seq_lens, head_type, budgets):
     """-> (cache_bytes, workspace_bytes); host arithmetic only."""
-    sl, ht, bu = _i32(seq_lens), _u8(head_type), _i32(budgets)
+    sl, ht, bu = _host(seq_lens, _INT32), _host(head_type, _UINT8), _host(budgets, _INT32)
     cb, wb = C.c_size_t(0), C.c_size_t(0)
-    _check(lib.hkv_plan(C.byref(cfg), _host(sl), _host(ht), _host(bu),
+    _check(lib.hkv_plan(C.byref(cfg), sl, ht, bu,
                         C.byref(cb), C.byref(wb)), "hkv_plan")
     return int(cb.value), int(wb.value)
 
@@ -190,21 +198,21 @@ def hkv_compress(cfg: hkv_config, k, v, q_obs, token_scores, is_text, seq_lens, 
                  cache_mem, workspace, stream=None) -> int:
     """Enqueue the compression of one layer; returns the cache handle (an integer address).
     k, v, q_obs, token_scores, is_text, cache_mem, workspace: torch CUDA tensors (or None)."""
-    sl, ht, bu = _i32(seq_lens), _u8(head_type), _i32(budgets)
+    sl, ht, bu = _host(seq_lens, _INT32), _host(head_type, _UINT8), _host(budgets, _INT32)
     handle = C.c_void_p(None)
     _check(lib.hkv_compress(C.byref(cfg), _dev(k), _dev(v), _dev(q_obs), _dev(token_scores), _dev(is_text),
-                            _host(sl), _host(ht), _host(bu),
-                            _dev(cache_mem), cache_mem.numel() * cache_mem.element_size(),
-                            _dev(workspace), workspace.numel() * workspace.element_size(),
+                            sl, ht, bu,
+                            _dev(cache_mem), cache_mem.nbytes,
+                            _dev(workspace), workspace.nbytes,
                             _stream(stream), C.byref(handle)), "hkv_compress")
     return handle.value
 
 
 def hkv_plan_offload(cfg: hkv_config, seq_lens, head_type, budgets):
     """-> (cache_bytes, workspace_bytes, host_bytes) for the variant with the dynamic heads' K/V in host memory."""
-    sl, ht, bu = _i32(seq_lens), _u8(head_type), _i32(budgets)
+    sl, ht, bu = _host(seq_lens, _INT32), _host(head_type, _UINT8), _host(budgets, _INT32)
     cb, wb, hb = C.c_size_t(0), C.c_size_t(0), C.c_size_t(0)
-    _check(lib.hkv_plan_offload(C.byref(cfg), _host(sl), _host(ht), _host(bu),
+    _check(lib.hkv_plan_offload(C.byref(cfg), sl, ht, bu,
                                 C.byref(cb), C.byref(wb), C.byref(hb)), "hkv_plan_offload")
     return int(cb.value), int(wb.value), int(hb.value)
 
@@ -213,22 +221,27 @@ def hkv_compress_offload(cfg: hkv_config, k, v, q_obs, token_scores, is_text, se
                          cache_mem, host_mem, workspace, stream=None) -> int:
     """hkv_compress with the dynamic heads' K/V planes written to `host_mem`, a pinned CPU tensor (or None when
     the layer has no dynamic head)."""
-    sl, ht, bu = _i32(seq_lens), _u8(head_type), _i32(budgets)
+    sl, ht, bu = _host(seq_lens, _INT32), _host(head_type, _UINT8), _host(budgets, _INT32)
     handle = C.c_void_p(None)
     if host_mem is not None and (host_mem.is_cuda or not host_mem.is_pinned() or not host_mem.is_contiguous()):
         raise ValueError("expected a contiguous pinned CPU tensor")
     hp = host_mem.data_ptr() if host_mem is not None else None
-    hn = host_mem.numel() * host_mem.element_size() if host_mem is not None else 0
+    hn = host_mem.nbytes if host_mem is not None else 0
     _check(lib.hkv_compress_offload(C.byref(cfg), _dev(k), _dev(v), _dev(q_obs), _dev(token_scores), _dev(is_text),
-                                    _host(sl), _host(ht), _host(bu),
-                                    _dev(cache_mem), cache_mem.numel() * cache_mem.element_size(), hp, hn,
-                                    _dev(workspace), workspace.numel() * workspace.element_size(),
+                                    sl, ht, bu,
+                                    _dev(cache_mem), cache_mem.nbytes, hp, hn,
+                                    _dev(workspace), workspace.nbytes,
                                     _stream(stream), C.byref(handle)), "hkv_compress_offload")
     return handle.value
 
 
 def hkv_decode_attn(cache: int, q, out, stream=None) -> None:
-    _check(lib.hkv_decode_attn(cache, _dev(q), _dev(out), _stream(stream)), "hkv_decode_attn")
+    # (called once per layer and step: the helpers' bodies in line, half a microsecond of four)
+    if not (q.is_cuda and out.is_cuda and q.is_contiguous() and out.is_contiguous()):
+        raise ValueError("expected a contiguous CUDA tensor")
+    status = lib.hkv_decode_attn(cache, q.data_ptr(), out.data_ptr(), _current_stream() if stream is None else _stream(stream))
+    if status:
+        raise HkvError(status, "hkv_decode_attn")
 
 
 def hkv_decode_attn_multi(caches: Sequence[int], qs, outs, stream=None) -> None:
@@ -275,7 +288,11 @@ def hkv_topk_chunks_noalloc(q, means, k: int, out_ids, stream=None) -> None:
 
 def hkv_append(cache: int, k_new, v_new, stream=None) -> None:
     """k_new, v_new: bf16 CUDA [B, Hkv, d], the new token's key / value of every KV head."""
-    _check(lib.hkv_append(cache, _dev(k_new), _dev(v_new), _stream(stream)), "hkv_append")
+    if not (k_new.is_cuda and v_new.is_cuda and k_new.is_contiguous() and v_new.is_contiguous()):
+        raise ValueError("expected a contiguous CUDA tensor")
+    status = lib.hkv_append(cache, k_new.data_ptr(), v_new.data_ptr(), _current_stream() if stream is None else _stream(stream))
+    if status:
+        raise HkvError(status, "hkv_append")
 
 
 def hkv_cache_destroy(cache: int) -> None:
@@ -358,10 +375,10 @@ def hkv_classify_heads(cfg: hkv_config, k, q_text, seq_lens, n_text, topk_fracti
                        workspace, scores_out, head_type_out, stream=None):
     """Text-centric sparsity score and static / dynamic label of every (sequence, kv head); see hkv.h.
     k, q_text, workspace, scores_out (float64) and head_type_out (uint8) are CUDA tensors."""
-    sl, nt = _i32(seq_lens), _i32(n_text)
+    sl, nt = _host(seq_lens, _INT32), _host(n_text, _INT32)
     _check(lib.hkv_classify_heads(C.byref(cfg), k.data_ptr(), q_text.data_ptr(), int(q_text.shape[1]),
-                                  _host(sl), _host(nt), float(topk_fraction), float(theta),
-                                  workspace.data_ptr(), workspace.numel() * workspace.element_size(),
+                                  sl, nt, float(topk_fraction), float(theta),
+                                  workspace.data_ptr(), workspace.nbytes,
                                   scores_out.data_ptr(), head_type_out.data_ptr(), _stream(stream)),
            "hkv_classify_heads")
 
