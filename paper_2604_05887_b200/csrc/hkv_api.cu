@@ -289,9 +289,14 @@ static hkv_status compress_common(const hkv_config* cfg, const void* k, const vo
     for (const auto& u : c->units) total_tiles += u.type == 0 ? (u.C + 127) / 128 : 0;
     bool ok = launch_setup(c->dev_base, img.data(), static_cast<int>(tables), static_cast<int>(H.n_valid_off),
                            static_cast<int>(H.err_off + 8 - H.n_valid_off), tile_prefix, s) == cudaSuccess;
-    // Static heads beside the dynamic ones, on the library's second stream (forked from and joined to `s`): it has the
-    // higher priority, so that the long chain of the static heads' kernels never queues behind the dynamic heads' blocks.
-    StepSide* side = (H.n_static > 0 && H.n_dynamic > 0) ? step_side() : nullptr;
+    int64_t build_bytes = 0;
+    for (const auto& u : c->units) build_bytes += u.type == 0 ? 0 : 4ll * kRowBytes * u.C;
+    // A short prompt: few key tiles (they leave half of the SMs free) and copies of a few microseconds.  All kernels go on one
+    // stream, each set up beside its predecessors, the dynamic heads' last: it runs beside the selection and the gather.
+    const bool chain = window && total_tiles <= 74 && build_bytes <= (24ll << 20) && !c->host_bytes;
+    // Else the static heads run beside the dynamic ones, on the library's second stream (forked from and joined to `s`): it has
+    // the higher priority, so that the long chain of the static heads' kernels never queues behind the dynamic heads' blocks.
+    StepSide* side = (H.n_static > 0 && H.n_dynamic > 0 && !chain) ? step_side() : nullptr;
     std::unique_lock<std::mutex> side_lock;
     if (side) side_lock = std::unique_lock<std::mutex>(side->enqueue);
     cudaStream_t ss = side ? side->stream : s;
@@ -301,22 +306,18 @@ static hkv_status compress_common(const hkv_config* cfg, const void* k, const vo
     // 6 TB/s), they start after the first pass; else at once.  (10 static + 6 dynamic units of 24-32 K tokens: 131 us
     // against 141; 13 + 19 of 50 K: 277 against 291.)
     bool later = false;
-    if (side && window) {
-      int64_t build_bytes = 0;
-      for (const auto& u : c->units) build_bytes += u.type == 0 ? 0 : 4ll * kRowBytes * u.C;
-      later = static_cast<double>(build_bytes) / 6.0e6 < 2.1 * static_cast<double>(total_tiles) / 148.0 + 30.0;
-    }
+    if (side && window) later = static_cast<double>(build_bytes) / 6.0e6 < 2.1 * static_cast<double>(total_tiles) / 148.0 + 30.0;
     if (ok && H.n_static > 0) {
       if (window)
         ok = launch_window_scores(c->dev_base, static_cast<char*>(workspace), k, q_obs, H, total_tiles, ws_rowstat_off,
-                                  tiles_max, tile_prefix, later ? side->q_done : nullptr, ss) == cudaSuccess;
-      ok = ok && launch_static_select(c->dev_base, static_cast<char*>(workspace), token_scores, is_text, H, ss) == cudaSuccess;
-      ok = ok && launch_gather_static(c->dev_base, k, v, H, c->max_static_rows, ss) == cudaSuccess;
+                                  tiles_max, tile_prefix, later ? side->q_done : nullptr, chain, ss) == cudaSuccess;
+      ok = ok && launch_static_select(c->dev_base, static_cast<char*>(workspace), token_scores, is_text, H, chain, ss) == cudaSuccess;
+      ok = ok && launch_gather_static(c->dev_base, k, v, H, c->max_static_rows, chain, ss) == cudaSuccess;
       if (side) ok = ok && cudaEventRecord(side->join, ss) == cudaSuccess;
     }
     if (ok && later) ok = cudaStreamWaitEvent(s, side->q_done, 0) == cudaSuccess;
     if (ok && H.n_dynamic > 0)
-      ok = launch_build_dynamic(c->dev_base, k, v, H, c->max_dyn_rows, c->max_chunks, s) == cudaSuccess;
+      ok = launch_build_dynamic(c->dev_base, k, v, H, c->max_dyn_rows, c->max_chunks, chain, s) == cudaSuccess;
     if (ok && side) ok = cudaStreamWaitEvent(s, side->join, 0) == cudaSuccess;
     if (!ok) { cudaGetLastError(); delete c; return HKV_ERR_CUDA; }
     *out = c;

@@ -98,6 +98,7 @@ struct WindowParams {
   const int32_t* tile_prefix;
   int32_t n_static, n_cta, n_partials;   // partial statistics a row may have (stats' second dimension)
   int32_t Rpad, row_block;
+  int32_t early;         // let the next kernel of a short chain start (see launch_window_scores)
 };
 struct WindowSeg {
   int key_row0, tile_begin, tile_end;
@@ -126,7 +127,9 @@ template <int MODE>
 __global__ void __maxnreg__(kWindowRegs)
     window_scores_tc_kernel(const __grid_constant__ WindowParams P, const __grid_constant__ CUtensorMap keys) {
   extern __shared__ __align__(16) uint8_t tc_smem[];
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  // (in a short chain the tables are complete when the first pass has passed its wait, and the second one starts after that)
+  if (MODE == 0 || !P.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (P.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const Header* hdr = reinterpret_cast<const Header*>(P.cache);
   const int G = hdr->group, w = hdr->obs_window, Hq = hdr->n_q_heads;
   const int R = w * G, row0 = P.row_block * tc::kQRows;
@@ -236,6 +239,7 @@ __global__ void __maxnreg__(kWindowRegs)
       sums = reinterpret_cast<float*>(user);
       info = reinterpret_cast<float4*>(sums + 2 * 4 * 128);
       last = reinterpret_cast<float*>(info + tc::kQRows / 2);
+      if (P.early) asm volatile("griddepcontrol.wait;" ::: "memory");   // for the first pass's statistics
       // the rows' statistics: two threads per row take every other partial
       const int dtid = threadIdx.x - 32, row = dtid >> 1, r = row0 + row;
       const int n_part = 2 * (window_cta_of(P.tile_prefix[seg.ordinal + 1] - 1, total, P.n_cta) - window_cta_of(seg.first, total, P.n_cta) + 1);
@@ -455,7 +459,7 @@ struct __align__(16) SelStats { int n_text; uint32_t tmin, tmax, vmin, vmax; int
 
 __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThreads)
     static_select_cluster_kernel(char* cache, const char* workspace, const float* token_scores, const uint8_t* is_text,
-                                 int slice_slots) {
+                                 int slice_slots, int early) {
   __shared__ __align__(16) int hist[kKeyedBins];
   __shared__ __align__(16) uint2 cand[kKeepThreads];
   __shared__ SelStats stats[kSelCluster];
@@ -465,6 +469,7 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThrea
   __shared__ int wtot[32];
   extern __shared__ __align__(16) uint32_t skey[];          // slice_slots keys, then slice_slots text flags (bytes)
   uint8_t* stxt = reinterpret_cast<uint8_t*>(skey + slice_slots);
+  if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
   const Header* hdr = reinterpret_cast<const Header*>(cache);
@@ -722,7 +727,8 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThrea
 // ---------------------------------------------------------------------------------------------
 constexpr int kGatherRows = 8;
 __global__ void __launch_bounds__(256)
-    gather_rows_kernel(char* cache, const uint4* kin, const uint4* vin) {
+    gather_rows_kernel(char* cache, const uint4* kin, const uint4* vin, int early) {
+  if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const Header* hdr = reinterpret_cast<const Header*>(cache);
   const Unit* u = unit_of(cache, hdr, false, blockIdx.y, nullptr);
@@ -759,8 +765,7 @@ __global__ void __launch_bounds__(256)
 // grid (K blocks, then V blocks; dynamic units).
 // ---------------------------------------------------------------------------------------------
 constexpr int kBuildThreads = 128, kBuildChunks = kBuildThreads / 16, kBuildRows = 64;
-__global__ void __launch_bounds__(kBuildThreads)
-    build_dynamic_kernel(char* cache, const uint4* kin, const uint4* vin, int k_blocks) {
+__device__ __forceinline__ void build_dynamic(char* cache, const uint4* kin, const uint4* vin, int k_blocks) {
   const Header* hdr = reinterpret_cast<const Header*>(cache);
   const Unit* u = unit_of(cache, hdr, true, blockIdx.y, nullptr);
   const int cs = hdr->chunk_size, C = u->C;
@@ -823,6 +828,13 @@ __global__ void __launch_bounds__(kBuildThreads)
 #pragma unroll
     for (int j = 0; j < 8; ++j) tail[j] = open ? acc[j] : 0.f;
   }
+}
+
+__global__ void __launch_bounds__(kBuildThreads)
+    build_dynamic_kernel(char* cache, const uint4* kin, const uint4* vin, int k_blocks) {
+  build_dynamic(cache, kin, vin, k_blocks);
+  // (at the end of a short chain this kernel runs beside its predecessors; whoever waits for it waits for them too)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // Adds one token to every unit: the key / value rows go to the end of the unit's planes (static: the
@@ -950,7 +962,7 @@ cudaError_t launch_setup(char* cache, const void* image, int table_bytes, int ze
 
 cudaError_t launch_window_scores(char* cache, char* workspace, const void* k, const void* q_obs, const Header& hdr,
                                  int64_t total_tiles, int64_t ws_rowstat_off, int n_partials, const int32_t* tile_prefix,
-                                 cudaEvent_t between, cudaStream_t stream) {
+                                 cudaEvent_t between, bool chain, cudaStream_t stream) {
   if (hdr.n_static == 0) return cudaSuccess;
   if (total_tiles > 0x7FFFFFFF) return cudaErrorInvalidValue;
   const int R = hdr.obs_window * hdr.group;
@@ -967,19 +979,20 @@ cudaError_t launch_window_scores(char* cache, char* workspace, const void* k, co
   P.n_static = hdr.n_static;
   P.n_cta = static_cast<int>(std::min<int64_t>(n_sm, total_tiles));
   P.n_partials = n_partials;
+  P.early = chain ? 1 : 0;
   P.Rpad = (R + 15) / 16 * 16;
   const int n_row_blocks = (R + tc::kQRows - 1) / tc::kQRows;
   for (int mode = 0; mode < 2; ++mode) {
     for (P.row_block = 0; P.row_block < n_row_blocks && e == cudaSuccess; ++P.row_block)
       e = launch_dependent(mode == 0 ? window_scores_tc_kernel<0> : window_scores_tc_kernel<1>, dim3(P.n_cta), tc::kSegThreads,
-                           mode == 0 ? kWindowSmem0 : kWindowSmem1, stream, P.row_block > 0 || (mode > 0 && !between), P, map);
+                           mode == 0 ? kWindowSmem0 : kWindowSmem1, stream, chain || P.row_block > 0 || (mode > 0 && !between), P, map);
     if (mode == 0 && e == cudaSuccess && between) e = cudaEventRecord(between, stream);
   }
   return e;
 }
 
 cudaError_t launch_static_select(char* cache, char* workspace, const float* token_scores, const uint8_t* is_text,
-                                 const Header& hdr, cudaStream_t stream) {
+                                 const Header& hdr, bool chain, cudaStream_t stream) {
   if (hdr.n_static == 0) return cudaSuccess;
   // A cluster of kSelCluster CTAs per unit when a slice of the longest sequence (keys + text flags) fits one
   // CTA's shared memory, one CTA per unit for longer sequences.
@@ -991,7 +1004,7 @@ cudaError_t launch_static_select(char* cache, char* workspace, const float* toke
   if (e != cudaSuccess) return e;
   if (clustered)
     return launch_dependent(static_select_cluster_kernel, dim3(hdr.n_static * kSelCluster), kKeepThreads, slice_smem, stream,
-                            !token_scores, cache, static_cast<const char*>(workspace), token_scores, is_text, slice);
+                            !token_scores, cache, static_cast<const char*>(workspace), token_scores, is_text, slice, chain ? 1 : 0);
   // every token's role is kept in shared memory when the longest sequence fits (else it is recomputed per pass)
   const int key_slots = std::min(hdr.max_seq_len, kKeepKeySlots);
   const size_t smem = static_cast<size_t>(key_slots) * sizeof(uint32_t);
@@ -1000,19 +1013,20 @@ cudaError_t launch_static_select(char* cache, char* workspace, const float* toke
 }
 
 cudaError_t launch_gather_static(char* cache, const void* k, const void* v, const Header& hdr, int max_rows,
-                                 cudaStream_t stream) {
+                                 bool chain, cudaStream_t stream) {
   if (hdr.n_static == 0 || max_rows <= 0) return cudaSuccess;
   const dim3 grid((max_rows + 8 * kGatherRows - 1) / (8 * kGatherRows), hdr.n_static);
-  return launch_dependent(gather_rows_kernel, grid, 256, 0, stream, true, cache, static_cast<const uint4*>(k), static_cast<const uint4*>(v));
+  return launch_dependent(gather_rows_kernel, grid, 256, 0, stream, true, cache, static_cast<const uint4*>(k), static_cast<const uint4*>(v),
+                          chain ? 1 : 0);
 }
 
 cudaError_t launch_build_dynamic(char* cache, const void* k, const void* v, const Header& hdr, int max_rows,
-                                 int max_chunks, cudaStream_t stream) {
+                                 int max_chunks, bool chain, cudaStream_t stream) {
   if (hdr.n_dynamic == 0) return cudaSuccess;
   const int k_blocks = (max_chunks + kBuildChunks - 1) / kBuildChunks;
   const dim3 grid(k_blocks + (max_rows + kBuildRows - 1) / kBuildRows, hdr.n_dynamic);
-  build_dynamic_kernel<<<grid, kBuildThreads, 0, stream>>>(cache, static_cast<const uint4*>(k), static_cast<const uint4*>(v), k_blocks);
-  return cudaGetLastError();
+  return launch_dependent(build_dynamic_kernel, grid, kBuildThreads, 0, stream, chain, cache, static_cast<const uint4*>(k),
+                          static_cast<const uint4*>(v), k_blocks);
 }
 
 cudaError_t launch_append(char* cache, const void* k_new, const void* v_new, const Header& hdr, cudaStream_t stream) {

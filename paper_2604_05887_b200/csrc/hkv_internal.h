@@ -112,17 +112,19 @@ bool decode_step_instance(const DecodeParams<1>& params, int max_chunks, int max
 cudaError_t launch_decode_step(const DecodeParams<1>& params, int max_chunks, int total_units, cudaStream_t stream);
 // Writes the cache's tables (a host image of table_bytes), clears [zero_begin, zero_begin + zero_bytes) of the cache and, unless
 // null, fills tile_prefix with the static units' running tile counts.
+// chain (launch_window_scores .. launch_build_dynamic): the compression's kernels follow one another on one stream, each set up
+// beside its predecessors.
 cudaError_t launch_setup(char* cache, const void* image, int table_bytes, int zero_begin, int zero_bytes, int32_t* tile_prefix,
                          cudaStream_t stream);
 cudaError_t launch_window_scores(char* cache, char* workspace, const void* k, const void* q_obs, const Header& hdr,
                                  int64_t total_tiles, int64_t ws_rowstat_off, int n_partials, const int32_t* tile_prefix,
-                                 cudaEvent_t between, cudaStream_t stream);   // `between` (or null) is recorded after the first pass
+                                 cudaEvent_t between, bool chain, cudaStream_t stream);   // `between` (or null) is recorded after the first pass
 cudaError_t launch_static_select(char* cache, char* workspace, const float* token_scores,
-                                 const uint8_t* is_text, const Header& hdr, cudaStream_t stream);
+                                 const uint8_t* is_text, const Header& hdr, bool chain, cudaStream_t stream);
 cudaError_t launch_gather_static(char* cache, const void* k, const void* v, const Header& hdr,
-                                 int max_rows, cudaStream_t stream);
+                                 int max_rows, bool chain, cudaStream_t stream);
 cudaError_t launch_build_dynamic(char* cache, const void* k, const void* v, const Header& hdr,
-                                 int max_rows, int max_chunks, cudaStream_t stream);
+                                 int max_rows, int max_chunks, bool chain, cudaStream_t stream);
 cudaError_t launch_append(char* cache, const void* k_new, const void* v_new, const Header& hdr, cudaStream_t stream);
 size_t decode_smem_bytes();
 #ifdef HKV_CHECKED
