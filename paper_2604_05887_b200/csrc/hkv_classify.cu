@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(tc::kSegThreads, 1)
   auto tile_fn = [&](const ClsSeg& seg, int tile, int, int part, uint32_t taddr) {
     if (idle) return;
     const int left = seg.C - (tile * tc::kKeysPerTile + 64 * (part & 1));   // keys of the thread's 64 columns that exist
-    tc::drain_raw(taddr, [&](int g, uint32_t (&r)[16]) {
+    tc::drain_raw<1>(taddr, [&](int g, uint32_t (&r)[16]) {
       if (left < 64) {
 #pragma unroll
         for (int c = 0; c < 16; ++c)

@@ -308,7 +308,7 @@ __global__ void __maxnreg__(kWindowRegs)
       // the quarters of the rows meet (two buffers, by tile parity) and are added in a fixed order
       float* buf = sums + (n_done & 1) * 4 * 128;
       buf[part * 128 + lane_row] = x + y;
-      tc::named_sync(tc::kBarAcc + 2 + (lane_row >> 5), 128);   // the four warps of these lanes
+      tc::named_sync(tc::kBarUser + (lane_row >> 5), 128);   // the four warps of these lanes
       if (part == 0 && j < C) {
         const float tot = ((buf[lane_row] + buf[128 + lane_row]) + (buf[256 + lane_row] + buf[384 + lane_row])) * inv_R;
         float* sw = reinterpret_cast<float*>(P.workspace + seg.ws_scores_off);

@@ -111,9 +111,11 @@ __device__ __forceinline__ void add_compensated(float& sum, float& comp, float x
 // lengths, with one tensor-memory allocation and one pipeline per CTA: the key tiles of the next segment are already
 // arriving while the last ones of the current are drained, and only the 64 KB of query rows are exchanged between two
 // segments (by the draining warps, behind a named barrier they share with the issuer).
-// Warp 0 brings in key tiles (TMA, two boxes of 64 elements x 128 keys in the operands' swizzled layout) and feeds the
-// tensor core; sixteen warps drain.  The hand-back of an accumulator buffer is a named barrier (arrive / sync): a warp
-// that polls an mbarrier meanwhile took half of its scheduler's issue slots from the draining warps.
+// The last warp brings in key tiles (TMA, two boxes of 64 elements x 128 keys in the operands' swizzled layout), warp 0
+// feeds the tensor core; sixteen warps drain.  (With one warp for both, a tile's instructions held it for 1250 cycles and
+// the next tile's copies for 500 more: 2050 cycles per tile with a light drain, 1500 so.)  The hand-back of an
+// accumulator buffer or a stage is a named barrier (arrive / sync): a warp that polls an mbarrier meanwhile took half
+// of its scheduler's issue slots from the draining warps.
 //   map               tensor map over all keys as rows of 128 bf16, boxes of 64 x 128 (key_map below)
 //   segment(s, seg)   the CTA's s-th segment; false behind the last.  Seg has tile_begin, tile_end and key_row0, the row
 //                     of tile 0's first key in the map.  Rows behind the head's last key hold whatever the tensor holds
@@ -127,8 +129,9 @@ __device__ __forceinline__ void add_compensated(float& sum, float& comp, float x
 // 128 t + 127 = the tile's keys); true: accumulator rows = the tile's keys, columns = the 256 query rows.
 // kRing: key tiles of shared memory.  *user: shared memory behind the barriers' page, the caller's.  kSegThreads threads.
 // ---------------------------------------------------------------------------------------------
-constexpr int kSegThreads = (1 + kDrainWarps) * 32;
-constexpr int kBarDrainIssue = 1, kBarDrain = 2, kBarAcc = 3;   // named barriers (kBarAcc + accumulator buffer)
+constexpr int kSegThreads = (2 + kDrainWarps) * 32;
+// named barriers: kBarAcc + accumulator buffer, kBarLoad + stage; kBarUser and above are the caller's
+constexpr int kBarDrainIssue = 1, kBarDrain = 2, kBarAcc = 3, kBarLoad = 5, kBarUser = 9;
 __device__ __forceinline__ void named_sync(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
@@ -149,9 +152,9 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16]) {
       : "memory");
 }
 // A draining thread's 64 columns as four groups of 16: fn(group, r) with columns 16 group ..
-template <class Fn>
+template <int kUnroll = 4, class Fn>
 __device__ __forceinline__ void drain_raw(uint32_t taddr, Fn fn) {
-#pragma unroll
+#pragma unroll kUnroll
   for (int g = 0; g < 4; ++g) {
     uint32_t r[16];
     tmem_ld16(taddr + 16u * g, r);
@@ -174,18 +177,15 @@ __device__ bool segments_cta(uint8_t* smem_raw, const CUtensorMap* map, SegmentF
   uint8_t* qs = smem;
   uint8_t* ks = smem + kQBytes;
   uint64_t* full = reinterpret_cast<uint64_t*>(ks + kRing * kStageBytes);
-  uint64_t* empty = full + kRing;
-  uint64_t* acc_full = empty + kRing;
+  uint64_t* acc_full = full + kRing;
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   *user = ks + kRing * kStageBytes + kBarBytes;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  static_assert(kRing <= kBarUser - kBarLoad, "a named barrier per stage");
 
   if (tid == 0) {
-    for (int s = 0; s < kRing; ++s) {
-      mbar_init(full + s, 1);
-      mbar_init(empty + s, 1);
-    }
+    for (int s = 0; s < kRing; ++s) mbar_init(full + s, 1);
     for (int b = 0; b < 2; ++b) mbar_init(acc_full + b, 1);
     mbar_fence_init();
     *abort_flag = 0;
@@ -213,29 +213,7 @@ __device__ bool segments_cta(uint8_t* smem_raw, const CUtensorMap* map, SegmentF
   if (warp == 0) {
     constexpr uint32_t idesc = kKeysAsRows ? InstrDesc<128, 256>::value : InstrDesc<128, 128>::value;
     const uint32_t q_addr = smem_u32(qs), k_addr0 = smem_u32(ks);
-    // the tiles to load run kRing - 1 ahead of the tiles to compute, through the same list of segments
-    Seg ld, seg;
-    int ld_sg = 0, ld_tile = 0, n_ld = 0;
-    bool ld_more = segment(0, ld);
-    if (ld_more) ld_tile = ld.tile_begin;
-    auto load_next = [&]() {
-      if (!ld_more) return;
-      const int s = n_ld % kRing;
-      if (n_ld >= kRing) wait(empty + s, ((n_ld / kRing) - 1) & 1);
-      if (ok && lane == 0) {
-        const uint32_t dst = k_addr0 + static_cast<uint32_t>(s * kStageBytes);
-        mbar_arrive_expect_tx(full + s, kStageBytes);
-        tma_load_2d(dst, map, 0, ld.key_row0 + ld_tile * kKeysPerTile, full + s);
-        tma_load_2d(dst + kPlaneBytesK, map, 64, ld.key_row0 + ld_tile * kKeysPerTile, full + s);
-      }
-      __syncwarp();
-      ++n_ld;
-      if (++ld_tile == ld.tile_end) {
-        ld_more = segment(++ld_sg, ld);
-        if (ld_more) ld_tile = ld.tile_begin;
-      }
-    };
-    for (int j = 0; j < kRing - 1; ++j) load_next();
+    Seg seg;
     int i = 0;
     for (int sg = 0; segment(sg, seg); ++sg) {
       named_sync(kBarDrainIssue, (kDrainWarps + 1) * 32);   // the segment's query rows are in place
@@ -259,16 +237,43 @@ __device__ bool segments_cta(uint8_t* smem_raw, const CUtensorMap* map, SegmentF
               umma_bf16(d + 128u, smem_desc(q_addr + qoff + 128u * 128u), smem_desc(k_addr + koff), idesc, kk != 0);
             }
           }
-          umma_commit(empty + s);        // the stage may be refilled once these instructions have read it
-          umma_commit(acc_full + buf);   // and the accumulator is complete
+          umma_commit(acc_full + buf);   // the accumulator is complete, the stage may be refilled
         }
         __syncwarp();
-        load_next();   // into the stage of tile i - 1, whose instructions have had a tile's time to finish
       }
     }
     // arrivals on the barriers of the last tiles must land before the CTA may leave
     for (int t = max(0, i - 2); t < i; ++t) named_sync(kBarAcc + (t & 1), (kDrainWarps + 1) * 32);
-    for (int t = max(0, i - kRing); t < i; ++t) wait(empty + t % kRing, (t / kRing) & 1);
+  } else if (warp == kDrainWarps + 1) {
+    // ---- loads, kRing tiles ahead of the tensor core; the first draining warp passes on that a tile's instructions
+    // have completed, so that this warp never polls
+    Seg seg, done;
+    int n = 0, sg_ld = 0, tile = 0;
+    bool more = segment(0, seg);
+    if (more) tile = seg.tile_begin;
+    auto load_next = [&]() {
+      if (!more) return;
+      const int s = n++ % kRing;
+      if (ok && lane == 0) {
+        const uint32_t dst = smem_u32(ks) + static_cast<uint32_t>(s * kStageBytes);
+        mbar_arrive_expect_tx(full + s, kStageBytes);
+        tma_load_2d(dst, map, 0, seg.key_row0 + tile * kKeysPerTile, full + s);
+        tma_load_2d(dst + kPlaneBytesK, map, 64, seg.key_row0 + tile * kKeysPerTile, full + s);
+      }
+      __syncwarp();
+      if (++tile == seg.tile_end) {
+        more = segment(++sg_ld, seg);
+        if (more) tile = seg.tile_begin;
+      }
+    };
+    for (int j = 0; j < kRing; ++j) load_next();
+    int i = 0;
+    for (int sg = 0; segment(sg, done); ++sg)
+      for (int t = done.tile_begin; t < done.tile_end; ++t, ++i) {
+        named_sync(kBarLoad + i % kRing, 64);
+        if (*abort_flag) ok = false;   // no copy may start once the others have given up
+        load_next();
+      }
   } else {
     // ---- drain: warp w owns lane quarter w % 4 (the hardware's rule) and column part (w - 1) / 4 ----
     const int quarter = warp & 3, part = (warp - 1) >> 2;
@@ -301,6 +306,7 @@ __device__ bool segments_cta(uint8_t* smem_raw, const CUtensorMap* map, SegmentF
       for (int tile = seg.tile_begin; tile < seg.tile_end; ++tile, ++i) {
         const int buf = i & 1;
         wait(acc_full + buf, (i >> 1) & 1);
+        if (warp == 1) named_arrive(kBarLoad + i % kRing, 64);   // its stage is free
         fence_after_sync();
         const uint32_t taddr =
             tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(buf * 256 + part * 64);
