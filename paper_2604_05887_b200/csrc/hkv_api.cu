@@ -303,19 +303,20 @@ static hkv_status compress_common(const hkv_config* cfg, const void* k, const vo
     if (ok && side) ok = cudaEventRecord(side->fork, s) == cudaSuccess && cudaStreamWaitEvent(ss, side->fork, 0) == cudaSuccess;
     // The dynamic heads' copies slow the window scores down where both run (HBM).  If they are short enough to be done
     // while the second pass, the selection and the gather run (~2.1 us per tile of a CTA + 30 us; the copies at about
-    // 6 TB/s), they start after the first pass; else at once.  (10 static + 6 dynamic units of 24-32 K tokens: 131 us
-    // against 141; 13 + 19 of 50 K: 277 against 291.)
+    // 6 TB/s), they start once the second pass's blocks are running; else once the first one's are.  (Blocks of the copies
+    // that got onto the SMs before a pass's held it up by the length of one: 5 to 8 us.  10 static + 6 dynamic units of 24-32 K
+    // tokens: 131 us against 141; 13 + 19 of 50 K: 277 against 291.)
     bool later = false;
     if (side && window) later = static_cast<double>(build_bytes) / 6.0e6 < 2.1 * static_cast<double>(total_tiles) / 148.0 + 30.0;
     if (ok && H.n_static > 0) {
       if (window)
         ok = launch_window_scores(c->dev_base, static_cast<char*>(workspace), k, q_obs, H, total_tiles, ws_rowstat_off,
-                                  tiles_max, tile_prefix, later ? side->q_done : nullptr, chain, ss) == cudaSuccess;
+                                  tiles_max, tile_prefix, side ? side->q_done : nullptr, later ? 1 : 0, chain, ss) == cudaSuccess;
       ok = ok && launch_static_select(c->dev_base, static_cast<char*>(workspace), token_scores, is_text, H, chain, ss) == cudaSuccess;
       ok = ok && launch_gather_static(c->dev_base, k, v, H, c->max_static_rows, chain, ss) == cudaSuccess;
       if (side) ok = ok && cudaEventRecord(side->join, ss) == cudaSuccess;
     }
-    if (ok && later) ok = cudaStreamWaitEvent(s, side->q_done, 0) == cudaSuccess;
+    if (ok && side && window) ok = cudaStreamWaitEvent(s, side->q_done, 0) == cudaSuccess;
     if (ok && H.n_dynamic > 0)
       ok = launch_build_dynamic(c->dev_base, k, v, H, c->max_dyn_rows, c->max_chunks, chain, s) == cudaSuccess;
     if (ok && side) ok = cudaStreamWaitEvent(s, side->join, 0) == cudaSuccess;

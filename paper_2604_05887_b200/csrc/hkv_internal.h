@@ -118,7 +118,7 @@ cudaError_t launch_setup(char* cache, const void* image, int table_bytes, int ze
                          cudaStream_t stream);
 cudaError_t launch_window_scores(char* cache, char* workspace, const void* k, const void* q_obs, const Header& hdr,
                                  int64_t total_tiles, int64_t ws_rowstat_off, int n_partials, const int32_t* tile_prefix,
-                                 cudaEvent_t between, bool chain, cudaStream_t stream);   // `between` (or null) is recorded after the first pass
+                                 cudaEvent_t started, int started_pass, bool chain, cudaStream_t stream);   // `started` (or null): recorded once that pass's blocks run
 cudaError_t launch_static_select(char* cache, char* workspace, const float* token_scores,
                                  const uint8_t* is_text, const Header& hdr, bool chain, cudaStream_t stream);
 cudaError_t launch_gather_static(char* cache, const void* k, const void* v, const Header& hdr,
