@@ -50,16 +50,18 @@ struct ClsParams {
   int32_t k[kClsBatch];   // entries summed per row
   int32_t n_sample[kClsBatch];                        // sampled keys
   int32_t rank_hi[kClsBatch], rank_lo[kClsBatch];     // ranks among the sample's group maxima that bound the k-th largest
-  int64_t w_prefix[kClsBatch + 1];   // (row block, key tile) pairs of the sequences before each
+  int64_t w_prefix[kClsBatch + 1];   // work of the sequences before each: (row block, key tile) pairs, weighted (cls_weight)
   int32_t n_batch, n_kv_heads, n_q_heads, group, max_seq_len, t_stride;
   int32_t row_begin, row_block;   // this pass covers rows [row_begin, row_begin + row_block) of every unit
   int32_t r_stride;               // floats between two units of the row-sum array
-  int32_t n_cta;                  // CTAs of the scan: CTA i takes pairs [i W / n_cta, (i + 1) W / n_cta), W = w_prefix[n_batch]
+  int32_t n_cta;                  // CTAs of the scan: CTA i takes the pairs that start in [i W / n_cta, (i + 1) W / n_cta), W = w_prefix[n_batch]
+  int32_t weight, weight_half;    // of a pair with more than 128 rows, of any other
   int32_t small;                  // W * n_cta fits 31 bits: 32-bit divisions
   int32_t seg_max;                // most CTAs that share one row block
   int32_t per_tile;               // list entries per half tile
   int32_t list_stride;            // entries of one half row's list
   int32_t sample_stride;          // rows of a unit in the sample buffer
+  int32_t split;                  // CTAs (a cluster) that share a row block's samples
   float bins_at;                  // centre of the sample histogram in standard deviations above the mean
   float scale_log2e;
 };
@@ -71,7 +73,30 @@ __device__ __forceinline__ int cls_rows(const ClsParams& P, int b) {
 __device__ __forceinline__ int cls_blocks(const ClsParams& P, int b) { return (cls_rows(P, b) + tc::kQRows - 1) / tc::kQRows; }
 __device__ __forceinline__ int cls_tiles(const ClsParams& P, int b) { return (P.C[b] + tc::kKeysPerTile - 1) / tc::kKeysPerTile; }
 __device__ __forceinline__ int cls_sample_tiles(const ClsParams& P, int b) { return (P.n_sample[b] + tc::kKeysPerTile - 1) / tc::kKeysPerTile; }
-// first pair of CTA i, and the CTA that holds pair w
+// tiles of samples a CTA of the cluster takes; in the buffer every CTA's are preceded by a copy of the first tile
+__device__ __forceinline__ int cls_sample_per(const ClsParams& P, int b) { return (cls_sample_tiles(P, b) + P.split - 1) / P.split; }
+// A pair with up to 128 rows has half of the tensor-core instructions and two busy warps per scheduler instead of four:
+// 1.75 us against 2.6, so they count two and three where a pass has both.  (336 rows in one full and one partial block:
+// the scan took 60 us with equal weights, when CTAs with partial blocks were done after 42.)
+__device__ __forceinline__ int cls_weight(const ClsParams& P, int rows) { return rows > tc::kQRows / 2 ? P.weight : P.weight_half; }
+struct ClsBlock {        // a row block's place in the order of work
+  int64_t begin;
+  int weight, n_tiles;
+};
+__device__ __forceinline__ ClsBlock cls_block(const ClsParams& P, int b, int h, int blk) {
+  ClsBlock r;
+  const int n_blk = cls_blocks(P, b), rows = cls_rows(P, b);
+  r.n_tiles = cls_tiles(P, b);
+  const int last = cls_weight(P, rows - (n_blk - 1) * tc::kQRows);
+  r.weight = blk == n_blk - 1 ? last : P.weight;
+  r.begin = P.w_prefix[b] + (static_cast<int64_t>(h) * ((n_blk - 1) * P.weight + last) + blk * P.weight) * r.n_tiles;
+  return r;
+}
+// the first tile of a block that starts at or behind `w`
+__device__ __forceinline__ int cls_tile_from(const ClsBlock& k, int64_t w) {
+  return static_cast<int>(min(static_cast<int64_t>(k.n_tiles), (w - k.begin + k.weight - 1) / k.weight));
+}
+// where CTA i begins, and the CTA that holds what starts at w
 __device__ __forceinline__ int64_t cls_cta_begin(const ClsParams& P, int i) {
   if (P.small) return static_cast<uint32_t>(i) * static_cast<uint32_t>(P.w_prefix[P.n_batch]) / static_cast<uint32_t>(P.n_cta);
   return static_cast<int64_t>(i) * P.w_prefix[P.n_batch] / P.n_cta;
@@ -111,15 +136,22 @@ __device__ __forceinline__ const __nv_bfloat16* cls_keys(const ClsParams& P, con
 // The keys sampled from every unit, as rows the tensor core can be fed with: row j holds the key at a pseudo-random
 // place of the context (with replacement, the same places for every unit of one length), so that neither a drift along
 // the context nor a period in it can bias the sample, and any eight rows are as good as independent.
-// grid (row groups of 16, units); samples: bf16 [unit][sample_stride][128].
+// grid (row groups of 16, units); samples: bf16 [unit][sample_stride][128].  Also clears the error word (`first`) and the
+// number of flagged rows.
 // ---------------------------------------------------------------------------------------------
 __global__ void __launch_bounds__(256)
-    cls_gather_kernel(const __grid_constant__ ClsParams P, const uint4* kin, uint4* samples) {
+    cls_gather_kernel(const __grid_constant__ ClsParams P, const uint4* kin, uint4* samples, int32_t* err, int first) {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int unit = blockIdx.y, b = unit / P.n_kv_heads;
   const int j = blockIdx.x * 16 + (threadIdx.x >> 4), piece = threadIdx.x & 15;
-  if (j >= (cls_sample_tiles(P, b) + 1) * tc::kKeysPerTile) return;
-  uint32_t x = static_cast<uint32_t>(j) * 0x9E3779B1u + 0x7F4A7C15u;   // any mixing will do
+  if (blockIdx.x == 0 && unit == 0 && threadIdx.x == 0) {
+    if (first) err[0] = 0;
+    err[1] = 0;
+  }
+  const int per = cls_sample_per(P, b), slot = j / tc::kKeysPerTile, rank = slot / (per + 1), at = slot - rank * (per + 1);
+  const int tile = at == 0 ? 0 : rank * per + at;
+  if (rank >= P.split || tile > cls_sample_tiles(P, b)) return;
+  uint32_t x = static_cast<uint32_t>(tile * tc::kKeysPerTile + j % tc::kKeysPerTile) * 0x9E3779B1u + 0x7F4A7C15u;   // any mixing will do
   x ^= x >> 16; x *= 0x85EBCA6Bu; x ^= x >> 13; x *= 0xC2B2AE35u; x ^= x >> 16;
   const size_t key = static_cast<size_t>(unit) * P.max_seq_len + __umulhi(x, static_cast<uint32_t>(P.C[b]));
   samples[(static_cast<size_t>(unit) * P.sample_stride + j) * 16 + piece] = __ldg(kin + key * 16 + piece);
@@ -131,11 +163,14 @@ __global__ void __launch_bounds__(256)
 // histogram (two rows share a 32-bit word).  What is counted is the largest logit of every group of up to eight
 // samples: a share q of the entries is a share 1 - (1 - q)^8 of the group maxima, which fixes a 5 % quantile as closely
 // as single samples do with an eighth of the shared-memory atomics (one atomic per sample: 5 us per tile).
-// grid: row blocks of the pass.  bounds: float4 [unit][row_block] = (lo, hi, scaled reference, -).
+// Bound: a chain of copy, instructions and drain per tile, 33 tiles one after the other (37 us whatever the number of row
+// blocks).  Where SMs would stay empty a cluster of P.split CTAs shares a block's tiles, each with its own copy of tile 0
+// in front, and adds the histograms up over distributed shared memory: with eight, 8 row blocks take 15 us.
+// grid: row blocks of the pass x P.split.  bounds: float4 [unit][row_block] = (lo, hi, scaled reference, -).
 // ---------------------------------------------------------------------------------------------
 constexpr int kClsHistBytes = kClsSampleBins * tc::kQRows * 2;
 constexpr int kClsSampleSmem = tc::seg_smem_fixed(tc::kStages) + kClsHistBytes;
-static_assert(kClsSampleSmem + 4096 <= 232448, "one CTA's shared memory");
+static_assert(kClsSampleSmem + 6144 <= 232448, "one CTA's shared memory");
 
 template <int kGroup>
 __global__ void __launch_bounds__(tc::kSegThreads, 1)
@@ -143,17 +178,20 @@ __global__ void __launch_bounds__(tc::kSegThreads, 1)
                       float4* bounds, int32_t* err) {
   extern __shared__ __align__(16) uint8_t tc_smem[];
   __shared__ float2 stat[2][tc::kQRows];   // (sum, sum of squares) of each half, then the running maxima
+  __shared__ float2 place[tc::kQRows];     // where a row's histogram begins, width of an entry
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  int b = 0, blk = blockIdx.x;
+  const int rank = blockIdx.x % P.split;
+  int b = 0, blk = blockIdx.x / P.split;
   while (blk >= cls_blocks(P, b) * P.n_kv_heads) { blk -= cls_blocks(P, b) * P.n_kv_heads; ++b; }
   const int n_blk = cls_blocks(P, b), h = blk / n_blk, row0 = (blk - h * n_blk) * tc::kQRows;
-  const int n_s = P.n_sample[b], rows = cls_rows(P, b);
+  const int n_s = P.n_sample[b], rows = cls_rows(P, b), per = cls_sample_per(P, b);
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
   auto segment = [&](int s, ClsSeg& seg) {
-    seg.key_row0 = (b * P.n_kv_heads + h) * P.sample_stride;
+    seg.key_row0 = (b * P.n_kv_heads + h) * P.sample_stride + rank * (per + 1) * tc::kKeysPerTile;
+    seg.n_rows = min(tc::kQRows, rows - row0);
     seg.tile_begin = 0;
-    seg.tile_end = cls_sample_tiles(P, b) + 1;
+    seg.tile_end = 1 + max(0, min(per, cls_sample_tiles(P, b) - rank * per));
     return s == 0;
   };
   auto q_row = [&](const ClsSeg&, int row) -> const __nv_bfloat16* {
@@ -194,7 +232,7 @@ __global__ void __launch_bounds__(tc::kSegThreads, 1)
       return;
     }
     if (row0 + (row & ~31) >= rows) return;   // the warp's rows are all padding
-    const int left = n_s - (tile - 1) * tc::kKeysPerTile - 64 * half;   // samples in the thread's 64 columns
+    const int left = n_s - (rank * per + tile - 1) * tc::kKeysPerTile - 64 * half;   // samples in the thread's 64 columns
     const bool all = left >= 64;
     const float shift = -a_bin * inv_w;
     // the largest of every group of kGroup samples (-inf for columns that hold none)
@@ -224,22 +262,56 @@ __global__ void __launch_bounds__(tc::kSegThreads, 1)
   auto end = [&](const ClsSeg&, int lane_row, int part, bool) {
     const int row = 128 * (part >> 1) + lane_row, half = part & 1;
     stat[half][row].x = vmax;
-    tc::named_sync(tc::kBarDrain, tc::kDrainWarps * 32);
-    if (half != 0 || row0 + row >= rows) return;
-    int cum = 0;
-    float lo = kClsOpen, hi = INFINITY;
-    bool have_lo = false;
-    for (int i = kClsSampleBins - 1; i >= 1; --i) {
-      cum += static_cast<int>((hist[i * (tc::kQRows / 2) + (row >> 1)] >> ((row & 1) * 16)) & 0xFFFFu);
-      const float edge = a_bin + static_cast<float>(i) * width;
-      if (cum <= P.rank_hi[b]) hi = edge;
-      if (!have_lo && cum >= P.rank_lo[b]) { lo = edge; have_lo = true; }
-    }
-    const float ref = fmaxf(stat[0][row].x, stat[1][row].x) * P.scale_log2e;
-    bounds[static_cast<size_t>(b * P.n_kv_heads + h) * P.row_block + row0 + row] = make_float4(lo, hi, ref, 0.f);
+    if (half == 0) place[row] = make_float2(a_bin, width);
   };
   if (!tc::segments_cta<false, tc::kStages, ClsSeg>(tc_smem, &samples, segment, q_row, begin, tile_fn, end, &user) && threadIdx.x == 0)
     atomicCAS(&err[0], 0, HKV_ERR_TIMEOUT);
+
+  // a CTA finishes its share of the rows: the others' counts into its own histogram, the maxima, then the bounds
+  hist = reinterpret_cast<uint32_t*>(user);
+  const int share = tc::kQRows / P.split, first = rank * share;
+  float top = -INFINITY;
+  if (P.split > 1) {
+    cluster_arrive();
+    cluster_wait();
+    const int words = share / 2;
+    for (int i = threadIdx.x; i < kClsSampleBins * words; i += tc::kSegThreads) {
+      const int bin = i / words, at = bin * (tc::kQRows / 2) + first / 2 + i - bin * words;
+      float other[7];   // all loads in flight (bits, not numbers)
+#pragma unroll
+      for (int r = 1; r < 8; ++r) other[r - 1] = r < P.split ? ld_cluster_f32(mapa(smem_u32(hist + at), (rank + r) & (P.split - 1))) : 0.f;
+      uint32_t sum = hist[at];
+#pragma unroll
+      for (int r = 0; r < 7; ++r) sum += __float_as_uint(other[r]);
+      hist[at] = sum;   // (nobody else reads this CTA's share of its own histogram)
+    }
+    if (threadIdx.x < share) {
+      float other[16];
+#pragma unroll
+      for (int r = 0; r < 16; ++r)
+        other[r] = (r >> 1) < P.split ? ld_cluster_f32(mapa(smem_u32(&stat[r & 1][first + threadIdx.x].x), r >> 1)) : -INFINITY;
+#pragma unroll
+      for (int r = 0; r < 16; ++r) top = fmaxf(top, other[r]);
+    }
+    cluster_arrive();
+    cluster_wait();     // also: no CTA leaves while another reads it
+  } else if (threadIdx.x < share) {
+    top = fmaxf(stat[0][threadIdx.x].x, stat[1][threadIdx.x].x);
+  }
+  const int row = first + threadIdx.x;
+  if (threadIdx.x >= share || row0 + row >= rows) return;
+  int cum = 0;
+  float lo = kClsOpen, hi = INFINITY;
+  bool have_lo = false;
+  a_bin = place[row].x;
+  width = place[row].y;
+  for (int i = kClsSampleBins - 1; i >= 1; --i) {
+    cum += static_cast<int>((hist[i * (tc::kQRows / 2) + (row >> 1)] >> ((row & 1) * 16)) & 0xFFFFu);
+    const float edge = a_bin + static_cast<float>(i) * width;
+    if (cum <= P.rank_hi[b]) hi = edge;
+    if (!have_lo && cum >= P.rank_lo[b]) { lo = edge; have_lo = true; }
+  }
+  bounds[static_cast<size_t>(b * P.n_kv_heads + h) * P.row_block + row0 + row] = make_float4(lo, hi, top * P.scale_log2e, 0.f);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -291,25 +363,29 @@ __global__ void __launch_bounds__(tc::kSegThreads, 1)
   const int64_t w_begin = cls_cta_begin(P, blockIdx.x), w_end = cls_cta_begin(P, blockIdx.x + 1);
 
   auto segment = [&](int s, ClsSeg& seg) {
-    const int64_t w = s == 0 ? w_begin : seg.next;
-    if (w >= w_end) return false;
-    int b = 0;
-    while (w >= P.w_prefix[b + 1]) ++b;
-    const int n_tiles = cls_tiles(P, b), n_blk = cls_blocks(P, b);
-    const int64_t in_b = w - P.w_prefix[b];
-    const int ub = static_cast<int>(in_b / n_tiles);          // row block within the sequence's heads
-    const int h = ub / n_blk;
-    const int64_t block_begin = P.w_prefix[b] + static_cast<int64_t>(ub) * n_tiles;
-    seg.b = b;
-    seg.unit = b * P.n_kv_heads + h;
-    seg.row0 = (ub - h * n_blk) * tc::kQRows;
-    seg.n_rows = min(tc::kQRows, cls_rows(P, b) - seg.row0);
-    seg.key_row0 = seg.unit * P.max_seq_len;
-    seg.C = P.C[b];
-    seg.tile_begin = static_cast<int>(w - block_begin);
-    seg.next = min(w_end, block_begin + n_tiles);
-    seg.tile_end = static_cast<int>(seg.next - block_begin);
-    seg.index = static_cast<int>(blockIdx.x) - cls_cta_of(P, block_begin);
+    int64_t w = s == 0 ? w_begin : seg.next;
+    for (;;) {
+      if (w >= w_end) return false;
+      int b = 0;
+      while (w >= P.w_prefix[b + 1]) ++b;
+      const int n_blk = cls_blocks(P, b), n_tiles = cls_tiles(P, b);
+      const int64_t unit_work = (P.w_prefix[b + 1] - P.w_prefix[b]) / P.n_kv_heads, in_b = w - P.w_prefix[b];
+      const int h = static_cast<int>(in_b / unit_work);
+      const int blk = min(n_blk - 1, static_cast<int>((in_b - h * unit_work) / (static_cast<int64_t>(n_tiles) * P.weight)));
+      const ClsBlock k = cls_block(P, b, h, blk);
+      seg.b = b;
+      seg.unit = b * P.n_kv_heads + h;
+      seg.row0 = blk * tc::kQRows;
+      seg.n_rows = min(tc::kQRows, cls_rows(P, b) - seg.row0);
+      seg.key_row0 = seg.unit * P.max_seq_len;
+      seg.C = P.C[b];
+      seg.tile_begin = cls_tile_from(k, w);
+      seg.tile_end = cls_tile_from(k, w_end);
+      seg.next = min(w_end, k.begin + static_cast<int64_t>(n_tiles) * k.weight);
+      seg.index = static_cast<int>(blockIdx.x) - cls_cta_of(P, k.begin);
+      if (seg.tile_begin < seg.tile_end) break;
+      w = seg.next;   // the run begins inside the block's last tile, which is the previous CTA's
+    }
     return true;
   };
   auto q_row = [&](const ClsSeg& seg, int row) -> const __nv_bfloat16* {
@@ -425,15 +501,14 @@ __global__ void __launch_bounds__(256, 3)
   const int idx = blockIdx.x * (blockDim.x >> 5) + warp;
   const int unit = idx / P.row_block, row = idx - unit * P.row_block, b = min(unit / P.n_kv_heads, P.n_batch - 1);
   const bool exists = idx < total_rows && row < cls_rows(P, b);
-  const int n_tiles = cls_tiles(P, b), blk = row / tc::kQRows;
-  const int64_t w0 = P.w_prefix[b] + (static_cast<int64_t>(unit - b * P.n_kv_heads) * cls_blocks(P, b) + blk) * n_tiles;
-  const int i0 = cls_cta_of(P, w0), n_rec = 2 * (cls_cta_of(P, w0 + n_tiles - 1) - i0 + 1);
+  const ClsBlock k = cls_block(P, b, unit - b * P.n_kv_heads, min(row / tc::kQRows, cls_blocks(P, b) - 1));
+  const int i0 = cls_cta_of(P, k.begin), n_rec = 2 * (cls_cta_of(P, k.begin + static_cast<int64_t>(k.n_tiles - 1) * k.weight) - i0 + 1);
   const size_t rg = static_cast<size_t>(unit) * P.row_block + row;
   const float4* part = partial + rg * P.seg_max * 2;
   // offset of a record's entries, in float4s
   auto rec_at = [&](int rec) {
     const int sg = rec >> 1;
-    const int tile0 = sg == 0 ? 0 : static_cast<int>(cls_cta_begin(P, i0 + sg) - w0);
+    const int tile0 = sg == 0 ? 0 : cls_tile_from(k, cls_cta_begin(P, i0 + sg));
     return ((rec & 1) * P.list_stride + cls_list_at(P, tile0, sg)) >> 2;
   };
   const float4* row_list = reinterpret_cast<const float4*>(list + rg * 2 * P.list_stride);
@@ -465,22 +540,20 @@ __global__ void __launch_bounds__(256, 3)
     const int to = n4 + incl - cnt4;
     n4 += __shfl_sync(0xffffffffu, incl, 31);
     if (n4 <= cap) {
-      // eight lanes per record, four records at a time; what the last float4 holds behind the end becomes -inf, which
-      // no comparison below takes
+      // eight lanes per record, four records at a time, all copies in flight together (loads waited for record by record
+      // took a third of a row's time); what the last float4 holds behind the end becomes -inf, which no comparison below takes
       for (int r = lane >> 3; r < 32 && r0 + (r & ~3) < n_rec; r += 4) {
         const int c = __shfl_sync(0xffffffffu, cnt, r), o = __shfl_sync(0xffffffffu, to, r), at = __shfl_sync(0xffffffffu, my_at, r);
-#pragma unroll 4
-        for (int e = lane & 7; 4 * e < c; e += 8) {
-          float4 v = __ldcg(row_list + at + e);
-          if (4 * e + 4 > c) {
-            if (4 * e + 1 >= c) v.y = -INFINITY;
-            if (4 * e + 2 >= c) v.z = -INFINITY;
-            v.w = -INFINITY;
-          }
-          buf[o + e] = v;
-        }
-        __syncwarp();
+        for (int e = lane & 7; 4 * e < c; e += 8)
+          asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(buf + o + e)), "l"(row_list + at + e) : "memory");
       }
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      __syncwarp();
+      if (cnt & 3) {
+        float* end = reinterpret_cast<float*>(buf + to) + cnt;
+        for (int e = cnt & 3; e < 4; ++e) *end++ = -INFINITY;
+      }
+      __syncwarp();
     }
   }
 #pragma unroll
@@ -937,17 +1010,22 @@ cudaError_t cls_configure(int* n_sm) {
 // One launch; `dependent`: it may be set up while its predecessor on the stream still runs (every kernel here that is
 // launched so waits for the predecessor before it touches memory).
 template <class... Params, class... Args>
-cudaError_t launch_cls(void (*kernel)(Params...), int grid, int threads, size_t smem, cudaStream_t stream, bool dependent, Args... args) {
+cudaError_t launch_cls(void (*kernel)(Params...), int grid, int cluster, int threads, size_t smem, cudaStream_t stream, bool dependent, Args... args) {
   cudaLaunchConfig_t cfg{};
-  cudaLaunchAttribute attr{};
+  cudaLaunchAttribute attr[2] = {};
   cfg.gridDim = dim3(static_cast<unsigned>(grid));
   cfg.blockDim = dim3(static_cast<unsigned>(threads));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
-  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr.val.programmaticStreamSerializationAllowed = 1;
-  cfg.attrs = &attr;
-  cfg.numAttrs = dependent ? 1 : 0;
+  cfg.attrs = attr;
+  if (dependent) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (cluster > 1) {
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs++].val.clusterDim = {static_cast<unsigned>(cluster), 1u, 1u};
+  }
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
 }
 
@@ -1030,7 +1108,6 @@ extern "C" hkv_status hkv_classify_heads(const hkv_config* cfg, const void* k, c
   cudaStream_t cs = static_cast<cudaStream_t>(stream);
   int32_t* err = static_cast<int32_t*>(workspace);   // [0] error word, [1] flagged rows of the pass
   float* rowsum = reinterpret_cast<float*>(static_cast<char*>(workspace) + kAlign);
-  if (cudaMemsetAsync(err, 0, kAlign, cs) != cudaSuccess) return HKV_ERR_CUDA;
   const float scale =
       cfg->softmax_scale > 0.f ? cfg->softmax_scale : 1.0f / std::sqrt(static_cast<float>(cfg->head_dim));
   for (int b0 = 0; b0 < cfg->batch; b0 += s.group_batch) {
@@ -1080,30 +1157,52 @@ extern "C" hkv_status hkv_classify_heads(const hkv_config* cfg, const void* k, c
     // least 1.3 times their (generously) expected length, and up to six times where the workspace allows it in one pass:
     // keys of a video frame are correlated, so a stretch of the context may hold several times its share.
     const int n_tiles = (cg_max + tc::kKeysPerTile - 1) / tc::kKeysPerTile;
-    auto tiles_of = [&](int rows) {
-      int64_t w = 0;
-      for (int i = 0; i < nb; ++i)
-        w += static_cast<int64_t>(cfg->n_kv_heads) * ((std::min(rows, P.T[i] * G) + tc::kQRows - 1) / tc::kQRows) *
-             ((P.C[i] + tc::kKeysPerTile - 1) / tc::kKeysPerTile);
-      return w;
+    // the work of rows [begin, begin + rows) of every head: w_prefix and weight of P, the number of row blocks
+    auto work_of = [&](int begin, int rows) {
+      int blocks = 0, full = 0;
+      for (int i = 0; i < nb; ++i) {
+        const int r = std::max(0, std::min(rows, P.T[i] * G - begin)), last = (r + tc::kQRows - 1) % tc::kQRows + 1;
+        const int n = (r + tc::kQRows - 1) / tc::kQRows;
+        blocks += n;
+        full += n - (n > 0 && last <= tc::kQRows / 2 ? 1 : 0);
+      }
+      const bool mixed = full > 0 && full < blocks;
+      P.weight = mixed ? 3 : 1;
+      P.weight_half = mixed ? 2 : 1;
+      P.w_prefix[0] = 0;
+      for (int i = 0; i < nb; ++i) {
+        const int r = std::max(0, std::min(rows, P.T[i] * G - begin)), last = (r + tc::kQRows - 1) % tc::kQRows + 1;
+        const int n = (r + tc::kQRows - 1) / tc::kQRows;
+        const int64_t w = n == 0 ? 0 : (n - 1) * P.weight + (last > tc::kQRows / 2 ? P.weight : P.weight_half);
+        P.w_prefix[i + 1] = P.w_prefix[i] + w * cfg->n_kv_heads * ((P.C[i] + tc::kKeysPerTile - 1) / tc::kKeysPerTile);
+      }
+      return blocks * cfg->n_kv_heads;
     };
-    auto ctas_of = [&](int64_t w) { return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(n_sm, w / 2))); };
-    auto segs_of = [&](int64_t w) { return static_cast<int>(std::min<int64_t>(n_tiles, n_tiles / std::max<int64_t>(1, w / ctas_of(w)) + 2)); };
+    // CTAs of the scan (each holds the start of a pair of either weight) and the most that share a row block
+    auto ctas_of = [&]() { return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(n_sm, P.w_prefix[nb] / std::max(2, P.weight)))); };
+    auto segs_of = [&](int n_cta) { return static_cast<int>(std::min<int64_t>(n_tiles, static_cast<int64_t>(n_tiles) * P.weight / std::max<int64_t>(1, P.w_prefix[nb] / n_cta) + 2)); };
     auto bytes_of = [&](int seg_max, int per_tile) {
       return static_cast<size_t>(8) * (static_cast<size_t>(n_tiles) * per_tile + static_cast<size_t>(seg_max) * kClsSlack) + 32u * seg_max + 20u;
     };
     auto per_tile_of = [&](double times) { return std::min(64, static_cast<int>(std::ceil(times * share * 64.0))); };
-    P.sample_stride = static_cast<int32_t>(round_up(n_sample_max, tc::kKeysPerTile) + tc::kKeysPerTile);
+    // CTAs per row block of the sample: as many as leave a quarter of the SMs free (a cluster's CTAs need one GPC)
+    const int all_blocks = work_of(0, r_max), sample_tiles = static_cast<int>(round_up(n_sample_max, tc::kKeysPerTile) / tc::kKeysPerTile);
+    P.split = 8;
+    while (P.split > 1 && all_blocks * P.split > n_sm * 3 / 4) P.split /= 2;
+    auto sample_rows = [&]() { return P.split * ((sample_tiles + P.split - 1) / P.split + 1) * tc::kKeysPerTile; };
+    while (P.split > 1 && static_cast<size_t>(units) * sample_rows() * kRowBytes > room / 4) P.split /= 2;
+    P.sample_stride = static_cast<int32_t>(sample_rows());
     size_t sample_bytes = static_cast<size_t>(units) * P.sample_stride * kRowBytes;
     const bool sampled = sample_bytes <= room / 2;   // no room (the smallest workspace of a short context): list every entry
     if (!sampled) { sample_bytes = 0; share = 1.0; }
     const size_t fixed = 4 * kAlign + sample_bytes;
-    int row_block = r_max, seg_max = segs_of(tiles_of(r_max)), per_tile = per_tile_of(1.3);
+    int row_block = r_max, seg_max = segs_of(ctas_of()), per_tile = per_tile_of(1.3);
     while (row_block > 1 && bytes_of(seg_max, per_tile) * row_block * units + fixed > room) {
       const size_t fit = (room - fixed) / units / bytes_of(seg_max, per_tile);
       row_block = static_cast<int>(std::max<size_t>(1, std::min<size_t>(row_block - 1, fit)));
       if (row_block > tc::kQRows) row_block = row_block / tc::kQRows * tc::kQRows;
-      seg_max = segs_of(tiles_of(row_block));
+      work_of(0, row_block);
+      seg_max = segs_of(ctas_of());
     }
     if (row_block == r_max)
       while (per_tile < per_tile_of(6.0) && bytes_of(seg_max, per_tile + 1) * row_block * units + fixed <= room) ++per_tile;
@@ -1138,37 +1237,30 @@ extern "C" hkv_status hkv_classify_heads(const hkv_config* cfg, const void* k, c
     if (e == cudaSuccess && sampled) e = tc::key_map(&sample_map, samples, static_cast<uint64_t>(units) * P.sample_stride);
     if (e == cudaSuccess && sampled) {
       cls_gather_kernel<<<dim3(static_cast<unsigned>(P.sample_stride / 16), static_cast<unsigned>(units)), 256, 0, cs>>>(
-          P, reinterpret_cast<const uint4*>(kg), reinterpret_cast<uint4*>(samples));
+          P, reinterpret_cast<const uint4*>(kg), reinterpret_cast<uint4*>(samples), err, b0 == 0);
       e = cudaGetLastError();
+    } else if (e == cudaSuccess) {
+      e = cudaMemsetAsync(err + (b0 == 0 ? 0 : 1), 0, b0 == 0 ? 2 * sizeof(int32_t) : sizeof(int32_t), cs);
     }
     for (int rb = 0; rb < r_max && e == cudaSuccess; rb += row_block) {
       P.row_begin = rb;
-      int blocks = 0;
-      P.w_prefix[0] = 0;
-      for (int i = 0; i < nb; ++i) {
-        const int rows = std::max(0, std::min(row_block, P.T[i] * G - rb)), blk = (rows + tc::kQRows - 1) / tc::kQRows;
-        blocks += blk * cfg->n_kv_heads;
-        P.w_prefix[i + 1] = P.w_prefix[i] + static_cast<int64_t>(cfg->n_kv_heads) * blk * ((P.C[i] + tc::kKeysPerTile - 1) / tc::kKeysPerTile);
-      }
-      // fewer pairs than in the first pass never mean more CTAs per block than it was sized for
-      P.n_cta = ctas_of(P.w_prefix[nb]);
-      if (rb > 0) {
-        while (P.n_cta > 1 && segs_of(P.w_prefix[nb]) > seg_max && n_tiles / std::max<int64_t>(1, P.w_prefix[nb] / P.n_cta) + 2 > seg_max) --P.n_cta;
-      }
+      const int blocks = work_of(rb, row_block);
+      P.n_cta = ctas_of();
+      while (P.n_cta > 1 && segs_of(P.n_cta) > seg_max) --P.n_cta;   // a later pass: no more CTAs per block than there are records for
       P.small = (P.w_prefix[nb] + 1) * P.n_cta < (1ll << 31);
       if (rb > 0 && cudaMemsetAsync(err + 1, 0, sizeof(int32_t), cs) != cudaSuccess) return HKV_ERR_CUDA;
-      if (sampled) e = launch_cls(sample_kernel, blocks, tc::kSegThreads, kClsSampleSmem, cs, rb == 0, P, sample_map, qg, bounds, err);
-      if (e == cudaSuccess) e = launch_cls(cls_scan_kernel, P.n_cta, tc::kSegThreads, kClsScanSmem, cs, sampled, P, map, qg,
+      if (sampled) e = launch_cls(sample_kernel, blocks * P.split, P.split, tc::kSegThreads, kClsSampleSmem, cs, rb == 0, P, sample_map, qg, bounds, err);
+      if (e == cudaSuccess) e = launch_cls(cls_scan_kernel, P.n_cta, 1, tc::kSegThreads, kClsScanSmem, cs, sampled, P, map, qg,
                                            static_cast<const float4*>(bounds), partial, list, err);
-      if (e == cudaSuccess) e = launch_cls(cls_select_kernel, static_cast<int>((rows_all + sel_warps - 1) / sel_warps), sel_warps * 32,
+      if (e == cudaSuccess) e = launch_cls(cls_select_kernel, static_cast<int>((rows_all + sel_warps - 1) / sel_warps), 1, sel_warps * 32,
                                            static_cast<size_t>(sel_warps) * sel_cap * sizeof(float4), cs, true, P, static_cast<const float4*>(bounds),
                                            static_cast<const float4*>(partial), static_cast<const float*>(list), rowsum, err + 1, flagged,
                                            static_cast<int>(rows_all), sel_cap);
-      if (e == cudaSuccess) e = launch_cls(cls_fix_kernel, fix_ctas, kClsFixThreads, kClsFixScratch + static_cast<size_t>(smem_cols) * sizeof(float), cs, true,
+      if (e == cudaSuccess) e = launch_cls(cls_fix_kernel, fix_ctas, 1, kClsFixThreads, kClsFixScratch + static_cast<size_t>(smem_cols) * sizeof(float), cs, true,
                                            P, kg, qg, rowsum, static_cast<const int32_t*>(err + 1), static_cast<const int32_t*>(flagged), list,
                                            static_cast<int>(c_stride), smem_cols);
     }
-    if (e == cudaSuccess) e = launch_cls(cls_finish_kernel, units, 256, 0, cs, true, P, static_cast<const float*>(rowsum), static_cast<const int32_t*>(err),
+    if (e == cudaSuccess) e = launch_cls(cls_finish_kernel, units, 1, 256, 0, cs, true, P, static_cast<const float*>(rowsum), static_cast<const int32_t*>(err),
                                          theta, scores_out, head_type_out, b0 * cfg->n_kv_heads);
     if (e != cudaSuccess) { cudaGetLastError(); return HKV_ERR_CUDA; }
   }

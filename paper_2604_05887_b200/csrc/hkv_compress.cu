@@ -102,7 +102,7 @@ struct WindowParams {
   int32_t early;         // let the next kernel of a short chain start (see launch_window_scores)
 };
 struct WindowSeg {
-  int key_row0, tile_begin, tile_end;
+  int key_row0, tile_begin, tile_end, n_rows;
   int C, ordinal, ub, uh;
   int64_t ws_scores_off;
   int first, next;       // tiles of the launch before the unit, and behind the segment
@@ -162,6 +162,7 @@ __global__ void __maxnreg__(kWindowRegs)
     seg.uh = u->h;
     seg.ws_scores_off = u->ws_scores_off;
     seg.key_row0 = (u->b * hdr->n_kv_heads + u->h) * hdr->max_seq_len;
+    seg.n_rows = min(tc::kQRows, R - row0);
     seg.first = P.tile_prefix[o];
     seg.next = min(w_end, P.tile_prefix[o + 1]);
     seg.tile_begin = at - seg.first;

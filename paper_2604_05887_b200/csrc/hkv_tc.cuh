@@ -117,7 +117,8 @@ __device__ __forceinline__ void add_compensated(float& sum, float& comp, float x
 // accumulator buffer or a stage is a named barrier (arrive / sync): a warp that polls an mbarrier meanwhile took half
 // of its scheduler's issue slots from the draining warps.
 //   map               tensor map over all keys as rows of 128 bf16, boxes of 64 x 128 (key_map below)
-//   segment(s, seg)   the CTA's s-th segment; false behind the last.  Seg has tile_begin, tile_end and key_row0, the row
+//   segment(s, seg)   the CTA's s-th segment; false behind the last.  Seg has n_rows (query rows that exist: at most 128
+//                     need only half of the instructions), tile_begin, tile_end and key_row0, the row
 //                     of tile 0's first key in the map.  Rows behind the head's last key hold whatever the tensor holds
 //                     there (zero behind its end): the caller masks them
 //   q_row(seg, row)   pointer to a query row's 128 bf16, or nullptr for a zero row
@@ -217,6 +218,7 @@ __device__ bool segments_cta(uint8_t* smem_raw, const CUtensorMap* map, SegmentF
     int i = 0;
     for (int sg = 0; segment(sg, seg); ++sg) {
       named_sync(kBarDrainIssue, (kDrainWarps + 1) * 32);   // the segment's query rows are in place
+      const bool both = seg.n_rows > 128;
       fence_after_sync();
       for (int tile = seg.tile_begin; tile < seg.tile_end; ++tile, ++i) {
         const int s = i % kRing, buf = i & 1;
@@ -234,7 +236,7 @@ __device__ bool segments_cta(uint8_t* smem_raw, const CUtensorMap* map, SegmentF
               umma_bf16(d, smem_desc(k_addr + koff), smem_desc(q_addr + qoff), idesc, kk != 0);
             } else {
               umma_bf16(d, smem_desc(q_addr + qoff), smem_desc(k_addr + koff), idesc, kk != 0);
-              umma_bf16(d + 128u, smem_desc(q_addr + qoff + 128u * 128u), smem_desc(k_addr + koff), idesc, kk != 0);
+              if (both) umma_bf16(d + 128u, smem_desc(q_addr + qoff + 128u * 128u), smem_desc(k_addr + koff), idesc, kk != 0);
             }
           }
           umma_commit(acc_full + buf);   // the accumulator is complete, the stage may be refilled

@@ -233,3 +233,13 @@ def test_gpu_classify_edges_of_the_sampled_bounds(C, T, G, fraction, kind):
     L.k[0, 1, 4321] = 0x7FC0   # the head without it must not notice; the other one still answers
     got, _ = _gpu_scores(L, q_text, counts, fraction, 0.9)
     assert abs(got[0, 0] - ref[0, 0]) <= SCORE_TOL and 0.0 < got[0, 1] <= 1.0 + 1e-6
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("B,C,T,G,Hkv", [(1, 300, 32, 4, 1), (1, 20000, 33, 4, 2), (1, 9000, 48, 7, 4), (3, 3000, 37, 7, 4), (2, 2500, 64, 8, 8),
+                                         (4, 700, 256, 7, 4)])
+def test_gpu_classify_shared_samples_and_weighted_blocks(B, C, T, G, Hkv):
+    """Row blocks whose samples eight, four, two and one CTAs share (some without a tile of their own), and full blocks
+    beside blocks of at most 128 rows, which count half when the work is cut up."""
+    L = hi.tiny(seed=61, B=B, C=C, chunk_size=32, w=8, Hq=G * Hkv, Hkv=Hkv, d=128)
+    _check_case(L, T, 0.05)
