@@ -132,7 +132,7 @@ hkv_status hkv_plan(const hkv_config* cfg, const int32_t* seq_lens, const uint8_
  * to nearest-even bf16; the last chunk may be shorter.
  * k, v, q_obs, token_scores and is_text may be released once the stream has passed this call.
  * The window-score kernels (and hkv_classify_heads) run on the tcgen05 tensor cores: while they run,
- * each of their thread blocks holds all tensor memory and nearly all shared memory of its SM, so
+ * each of their thread blocks holds all tensor memory and most of the shared memory of its SM, so
  * kernels of other streams that need tensor memory wait for them.
  * On success *out receives a handle to free with hkv_cache_destroy. */
 hkv_status hkv_compress(const hkv_config* cfg, const void* k, const void* v, const void* q_obs,
