@@ -94,7 +94,8 @@ __device__ __forceinline__ ClsBlock cls_block(const ClsParams& P, int b, int h, 
 }
 // the first tile of a block that starts at or behind `w`
 __device__ __forceinline__ int cls_tile_from(const ClsBlock& k, int64_t w) {
-  return static_cast<int>(min(static_cast<int64_t>(k.n_tiles), (w - k.begin + k.weight - 1) / k.weight));
+  const uint32_t d = static_cast<uint32_t>(min(w - k.begin + k.weight - 1, static_cast<int64_t>(k.n_tiles * k.weight)));
+  return static_cast<int>(k.weight == 1 ? d : k.weight == 2 ? d / 2u : d / 3u);
 }
 // where CTA i begins, and the CTA that holds what starts at w
 __device__ __forceinline__ int64_t cls_cta_begin(const ClsParams& P, int i) {
@@ -491,6 +492,22 @@ __device__ __forceinline__ float cls_key_float(uint32_t key) {   // inverse of f
   return __uint_as_float((key & 0x80000000u) ? (key ^ 0x80000000u) : ~key);
 }
 
+// cls_take without the count
+__device__ __forceinline__ void cls_keep(float v, float p, float lo, float hi, float& sum, uint32_t& at) {
+  asm volatile(
+      "{\n"
+      ".reg .pred up, in;\n"
+      "setp.gt.f32 up, %2, %5;\n"
+      "@up add.f32 %0, %0, %3;\n"
+      "setp.ge.and.f32 in, %2, %4, !up;\n"
+      "@in st.shared.f32 [%1], %2;\n"
+      "@in add.u32 %1, %1, 128;\n"
+      "}\n"
+      : "+f"(sum), "+r"(at)
+      : "f"(v), "f"(p), "f"(lo), "f"(hi)
+      : "memory");
+}
+
 __global__ void __launch_bounds__(256, 3)
     cls_select_kernel(const __grid_constant__ ClsParams P, const float4* bounds, const float4* partial, const float* list, float* rowsum,
                       int32_t* n_flag, int32_t* flagged, int total_rows, int cap) {
@@ -650,14 +667,13 @@ __global__ void __launch_bounds__(256, 3)
   } else {
     const uint32_t column = smem_u32(buf) + lane * 4;
     uint32_t at = column;
-    int unused = 0;
     for (int e = 0; e < n4; e += 32) {
       const float4 v = e + lane < n4 ? buf[e + lane] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
       __syncwarp();
-      cls_take(v.x, weight(v.x), a, bb, s, unused, at);
-      cls_take(v.y, weight(v.y), a, bb, s, unused, at);
-      cls_take(v.z, weight(v.z), a, bb, s, unused, at);
-      cls_take(v.w, weight(v.w), a, bb, s, unused, at);
+      cls_keep(v.x, weight(v.x), a, bb, s, at);
+      cls_keep(v.y, weight(v.y), a, bb, s, at);
+      cls_keep(v.z, weight(v.z), a, bb, s, at);
+      cls_keep(v.w, weight(v.w), a, bb, s, at);
     }
     const int mine = static_cast<int>((at - column) / 128u), base = cb;
     float own[8];                    // the usual number in registers, more stay where they are
