@@ -650,8 +650,12 @@ __global__ void __launch_bounds__(256, 3)
     return cls_key_float(ka + kd / 4u * num + (num < 4u ? 1u : kd % 4u));
   };
   for (int it = 0; need > 0 && ca != need && a < bb && (!in_smem || ca - cb > kClsUndecided); ++it) {
-    const float x = place(), w = bb - a;
-    if (it < 3) count2(x - 0.07f * w, x + 0.07f * w);
+    const float w = bb - a;
+    // first by the logarithm of the rank, which is nearly linear in the tail of a row (the rank itself bends by a tenth of
+    // the bracket, and the window had to be twice as wide: 28672 rows 557 -> 549 us)
+    const float la = __log2f(static_cast<float>(above + n)), lb = __log2f(fmaxf(static_cast<float>(above), 0.5f));
+    const float x = it == 0 ? a + w * ((la - __log2f(static_cast<float>(P.k[b]))) / (la - lb)) : place();
+    if (it < 3) count2(x - 0.04f * w, x + 0.04f * w);
     else count2(middle(2), x);
   }
   // everything above the bracket; its own entries, if they still have to be ranked, move to the front of the buffer, a
