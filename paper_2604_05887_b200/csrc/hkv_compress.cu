@@ -88,8 +88,9 @@ __global__ void __launch_bounds__(kSetupThreads)
 //         to by later ones).
 // Bound: 2^x (16 per clock and SM; a scheduler whose four warps all have rows spends 2048 cycles per tile on them) at 85 %:
 // 2350 cycles per tile, 31 us a pass for ten units of 24-32 K tokens.  A quarter or half of the powers as polynomials on the
-// FMA pipes, and reading the accumulator ahead, changed nothing.  MODE 1 takes max and sum as one exponent, max + log2 sum: with
-// two constants per row its reads of shared memory took as long as the powers (2950 cycles per tile).  grid: CTAs; one launch per block of 256 window rows.
+// FMA pipes, and reading the accumulator ahead, changed nothing.  One exponent max + log2 sum instead of two constants per
+// row took 2 us off a second pass, but rounds a row's weight ten times as coarsely.
+// grid: CTAs; one launch per block of 256 window rows.
 // ---------------------------------------------------------------------------------------------
 struct WindowParams {
   char* cache;
@@ -107,8 +108,8 @@ struct WindowSeg {
   int64_t ws_scores_off;
   int first, next;       // tiles of the launch before the unit, and behind the segment
 };
-// the caller's shared memory of MODE 1: two buffers of the four quarters' sums; the rows' bias and last visible key
-constexpr int kWindowUser1 = 2 * 4 * 128 * 4 + tc::kQRows * 8;
+// the caller's shared memory of MODE 1: two buffers of the four quarters' sums; the rows' (max, 1 / sum), last visible keys
+constexpr int kWindowUser1 = 2 * 4 * 128 * 4 + tc::kQRows * 12;
 constexpr int kWindowRing0 = 3, kWindowRing1 = 3;   // key tiles in shared memory (more left less to the other stream's blocks and gained nothing)
 constexpr int kWindowSmem0 = tc::seg_smem_fixed(kWindowRing0), kWindowSmem1 = tc::seg_smem_fixed(kWindowRing1) + kWindowUser1;
 static_assert(kWindowSmem0 <= 232448 && kWindowSmem1 <= 232448, "one CTA's shared memory");
@@ -233,14 +234,14 @@ __global__ void __maxnreg__(kWindowRegs)
     ok = tc::segments_cta<false, kWindowRing0, WindowSeg>(tc_smem, &keys, segment, q_row, begin, tile_fn, end, &user);
   } else {
     const float inv_R = 1.f / static_cast<float>(R);
-    float* bias = nullptr;      // per row: -(max + log2 sum), so that 2^(logit + bias) is the row's probability
+    float4* info = nullptr;     // per pair of rows: (-max, -max, 1 / sum, 1 / sum)
     float* last = nullptr;      // per row: last visible key
     float* sums = nullptr;      // [2][4 quarters of the rows][128 keys]
     int n_done = 0;
     auto begin = [&](const WindowSeg& seg, int, int) {
       sums = reinterpret_cast<float*>(user);
-      bias = sums + 2 * 4 * 128;
-      last = bias + tc::kQRows;
+      info = reinterpret_cast<float4*>(sums + 2 * 4 * 128);
+      last = reinterpret_cast<float*>(info + tc::kQRows / 2);
       if (P.early) asm volatile("griddepcontrol.wait;" ::: "memory");   // for the first pass's statistics
       // the rows' statistics: two threads per row take every other partial
       const int dtid = threadIdx.x - 32, row = dtid >> 1, r = row0 + row;
@@ -270,7 +271,9 @@ __global__ void __maxnreg__(kWindowRegs)
       }
       tc::named_sync(tc::kBarDrain, tc::kDrainWarps * 32);   // (the previous segment's readers are done)
       if ((dtid & 1) == 0) {
-        bias[row] = r < R ? -(M + log2f(Z)) : -INFINITY;      // a padding row adds nothing
+        float* pair = reinterpret_cast<float*>(info + (row >> 1)) + (row & 1);
+        pair[0] = r < R ? -M : 0.f;
+        pair[2] = r < R ? 1.f / Z : 0.f;                      // a padding row adds nothing
         last[row] = r < R ? static_cast<float>(causal ? (seg.C - w + r / G) : (seg.C - 1)) : -1.f;
       }
       tc::named_sync(tc::kBarDrain, tc::kDrainWarps * 32);
@@ -285,21 +288,21 @@ __global__ void __maxnreg__(kWindowRegs)
         tc::drain_raw(taddr, [&](int g, uint32_t (&v)[16]) {
           const int rb = 64 * part + 16 * g;
           if (row0 + rb >= R) return;   // 16 padding rows: nothing to add (same for the whole warp)
-          const float4* bi = reinterpret_cast<const float4*>(bias + rb);
+          const float4* ri = info + rb / 2;
 #pragma unroll
           for (int c = 0; c < 16; c += 4) {
-            const float4 p = bi[c / 4];
+            const float4 p = ri[c / 2], q = ri[c / 2 + 1];
             float e0, e1, e2, e3;
             tc::unpack_f32x2(tc::fma_f32x2(tc::pack_f32x2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc2, tc::pack_f32x2(p.x, p.y)), e0, e1);
-            tc::unpack_f32x2(tc::fma_f32x2(tc::pack_f32x2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3])), sc2, tc::pack_f32x2(p.z, p.w)), e2, e3);
+            tc::unpack_f32x2(tc::fma_f32x2(tc::pack_f32x2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3])), sc2, tc::pack_f32x2(q.x, q.y)), e2, e3);
             if (!all_visible) {
               if (jf > last[rb + c]) e0 = -INFINITY;
               if (jf > last[rb + c + 1]) e1 = -INFINITY;
               if (jf > last[rb + c + 2]) e2 = -INFINITY;
               if (jf > last[rb + c + 3]) e3 = -INFINITY;
             }
-            a = tc::add_f32x2(a, tc::pack_f32x2(fast_exp2(e0), fast_exp2(e1)));
-            b = tc::add_f32x2(b, tc::pack_f32x2(fast_exp2(e2), fast_exp2(e3)));
+            a = tc::fma_f32x2(tc::pack_f32x2(fast_exp2(e0), fast_exp2(e1)), tc::pack_f32x2(p.z, p.w), a);
+            b = tc::fma_f32x2(tc::pack_f32x2(fast_exp2(e2), fast_exp2(e3)), tc::pack_f32x2(q.z, q.w), b);
           }
         });
       }
