@@ -356,6 +356,19 @@ hkv_status hkv_selftest_wait_timeout(hkv_cache* c, void* stream) {
   }
   return HKV_OK;
 }
+// The same for the tensor-core engine under the window scores and the classification: a few thread blocks stream twelve tiles of
+// `keys` (dev bf16 [512, 128], 16-byte aligned) while one role -- 0 the copies, 1 the tensor-core instructions, 2 the draining
+// warps, -1 none -- stops after `upto` tiles.  It must return by itself, leave HKV_ERR_TIMEOUT / detail 6 if a role waited in
+// vain and nothing otherwise, and free its tensor memory.  (For the tests alone: not in hkv.h.)
+hkv_status hkv_selftest_engine_timeout(hkv_cache* c, const void* keys, int32_t role, int32_t upto, void* stream) {
+  if (!c || !keys || (reinterpret_cast<uintptr_t>(keys) & 15) || role < -1 || role > 2 || upto < 0) return HKV_ERR_INVALID_ARG;
+  if (launch_selftest_engine(keys, role, upto, reinterpret_cast<int32_t*>(c->dev_base + c->hdr.err_off),
+                             static_cast<cudaStream_t>(stream)) != cudaSuccess) {
+    cudaGetLastError();
+    return HKV_ERR_CUDA;
+  }
+  return HKV_OK;
+}
 hkv_status hkv_clear_device_error(hkv_cache* c, void* stream) {
   if (!c) return HKV_ERR_INVALID_ARG;
   if (cudaMemsetAsync(c->dev_base + c->hdr.err_off, 0, 8, static_cast<cudaStream_t>(stream)) != cudaSuccess) {

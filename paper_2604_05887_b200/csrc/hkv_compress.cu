@@ -1043,6 +1043,49 @@ cudaError_t launch_build_dynamic(char* cache, const void* k, const void* v, cons
                           static_cast<const uint4*>(v), k_blocks);
 }
 
+#ifdef HKV_CHECKED
+namespace {
+// Self-test of the segment engine's bounded waits: kSelfSegments segments of kSelfTiles tiles over the same 512 keys, of which one role
+// (0 copies, 1 instructions, 2 drain; -1 none) sees only the first `upto` tiles, so that what the others wait for never comes.
+// The draining warps meet at named barriers as in the window scores.
+constexpr int kSelfSegments = 3, kSelfTiles = 4, kSelfRing = 3;
+struct SelfSeg { int key_row0, tile_begin, tile_end, n_rows; };
+__global__ void __launch_bounds__(tc::kSegThreads, 1)
+    engine_selftest_kernel(const __grid_constant__ CUtensorMap keys, const __nv_bfloat16* q, int role, int upto, int32_t* err) {
+  extern __shared__ __align__(16) uint8_t tc_smem[];
+  const int warp = threadIdx.x >> 5, mine = warp == 0 ? 1 : warp == tc::kDrainWarps + 1 ? 0 : 2;
+  auto segment = [&](int s, SelfSeg& seg) {
+    seg = SelfSeg{0, 0, kSelfTiles, tc::kQRows};
+    if (mine == role) seg.tile_end = max(0, min(kSelfTiles, upto - s * kSelfTiles));
+    return s < kSelfSegments;
+  };
+  auto q_row = [&](const SelfSeg&, int row) { return q + (row & 127) * kHeadDim; };
+  auto begin = [](const SelfSeg&, int, int) { tc::named_sync(tc::kBarDrain, tc::kDrainWarps * 32); };
+  float sum = 0.f;
+  auto tile_fn = [&](const SelfSeg&, int, int lane_row, int, uint32_t taddr) {
+    tc::drain_raw(taddr, [&](int, uint32_t (&r)[16]) { sum += __uint_as_float(r[0]); });
+    tc::named_sync(tc::kBarUser + (lane_row >> 5), 128);
+  };
+  bool drained = true;
+  auto end = [&](const SelfSeg&, int, int, bool so_far) { drained = so_far; };
+  uint8_t* user = nullptr;
+  const bool ok = tc::segments_cta<true, kSelfRing, SelfSeg>(tc_smem, &keys, segment, q_row, begin, tile_fn, end, &user);
+  if (!ok && threadIdx.x == 0) { atomicCAS(&err[0], 0, HKV_ERR_TIMEOUT); err[1] = kErrSelfTest; }
+  if (ok && (!drained || sum == 1.25e-30f)) err[1] = kErrIndex;   // (keeps the sums; a role that gave up must show in the result)
+}
+}  // namespace
+
+cudaError_t launch_selftest_engine(const void* keys, int role, int upto, int32_t* err_word, cudaStream_t stream) {
+  constexpr int smem = tc::seg_smem_fixed(kSelfRing);
+  CUtensorMap map;
+  cudaError_t e = tc::key_map(&map, keys, kSelfTiles * tc::kKeysPerTile);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(engine_selftest_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  engine_selftest_kernel<<<4, tc::kSegThreads, smem, stream>>>(map, static_cast<const __nv_bfloat16*>(keys), role, upto, err_word);
+  return cudaGetLastError();
+}
+#endif
+
 cudaError_t launch_append(char* cache, const void* k_new, const void* v_new, const Header& hdr, cudaStream_t stream) {
   return launch_dependent(append_kernel, dim3(hdr.n_units), kHeadDim, 0, stream, true, cache,
                           static_cast<const __nv_bfloat16*>(k_new), static_cast<const __nv_bfloat16*>(v_new));

@@ -129,6 +129,7 @@ cudaError_t launch_append(char* cache, const void* k_new, const void* v_new, con
 size_t decode_smem_bytes();
 #ifdef HKV_CHECKED
 cudaError_t launch_selftest_wait(int32_t* err_word, cudaStream_t stream);
+cudaError_t launch_selftest_engine(const void* keys, int role, int upto, int32_t* err_word, cudaStream_t stream);
 #endif
 
 }  // namespace hkv

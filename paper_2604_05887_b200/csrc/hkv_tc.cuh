@@ -113,9 +113,14 @@ __device__ __forceinline__ void add_compensated(float& sum, float& comp, float x
 // segments (by the draining warps, behind a named barrier they share with the issuer).
 // The last warp brings in key tiles (TMA, two boxes of 64 elements x 128 keys in the operands' swizzled layout), warp 0
 // feeds the tensor core; sixteen warps drain.  (With one warp for both, a tile's instructions held it for 1250 cycles and
-// the next tile's copies for 500 more: 2050 cycles per tile with a light drain, 1500 so.)  The hand-back of an
-// accumulator buffer or a stage is a named barrier (arrive / sync): a warp that polls an mbarrier meanwhile took half
-// of its scheduler's issue slots from the draining warps.
+// the next tile's copies for 500 more: 2050 cycles per tile with a light drain, 1500 so.)
+// Hand-overs.  What one role passes on to another travels over an mbarrier: a landed tile (full), a tile's completed
+// instructions (acc_full for the draining warps, stage_free for the copies), a drained accumulator (acc_free).  Every
+// wait on one is bounded.  A role whose wait runs out, or that sees that another's has, signals nothing more and waits for
+// none of these any more, so that nobody is told of something that did not happen.  Named barriers are only used where
+// every participant both arrives and waits, and are met the same number of times by all of them whether they have given up
+// or not: by the draining warps among themselves (the caller's) and once per segment by them and warp 0.  So every role
+// gets to the end, where each waits (bounded) for the copies or instructions it has started before the CTA may leave.
 //   map               tensor map over all keys as rows of 128 bf16, boxes of 64 x 128 (key_map below)
 //   segment(s, seg)   the CTA's s-th segment; false behind the last.  Seg has n_rows (query rows that exist: at most 128
 //                     need only half of the instructions), tile_begin, tile_end and key_row0, the row
@@ -131,14 +136,30 @@ __device__ __forceinline__ void add_compensated(float& sum, float& comp, float x
 // kRing: key tiles of shared memory.  *user: shared memory behind the barriers' page, the caller's.  kSegThreads threads.
 // ---------------------------------------------------------------------------------------------
 constexpr int kSegThreads = (2 + kDrainWarps) * 32;
-// named barriers: kBarAcc + accumulator buffer, kBarLoad + stage; kBarUser and above are the caller's
-constexpr int kBarDrainIssue = 1, kBarDrain = 2, kBarAcc = 3, kBarLoad = 5, kBarUser = 9;
+// named barriers; kBarDrain, kBarUser and above are the caller's
+constexpr int kBarDrainIssue = 1, kBarDrain = 2, kBarUser = 3;
 __device__ __forceinline__ void named_sync(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
-__device__ __forceinline__ void named_arrive(int id, int threads) {
-  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(threads) : "memory");
+__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+// mbar_try_wait that may sleep for up to `ns` before it answers no: a warp that asks again and again takes issue slots from
+// the draining warps of its scheduler
+__device__ __forceinline__ bool mbar_try_wait_ns(uint64_t* bar, uint32_t parity, uint32_t ns) {
+  uint32_t ok;
+  asm volatile(
+      "{\n"
+      ".reg .pred p;\n"
+      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
+      "selp.u32 %0, 1, 0, p;\n"
+      "}\n"
+      : "=r"(ok)
+      : "r"(smem_u32(bar)), "r"(parity), "r"(ns)
+      : "memory");
+  return ok != 0;
+}
+constexpr uint32_t kWaitNs = 20000;
 constexpr int seg_smem_fixed(int stages) { return kQBytes + stages * kStageBytes + kBarBytes + 1024; }   // + the caller's bytes
 
 // 32 lanes x 16 columns, waited for: the four warps of a scheduler hide each other's latency, and the values need no copy
@@ -178,16 +199,24 @@ __device__ bool segments_cta(uint8_t* smem_raw, const CUtensorMap* map, SegmentF
   uint8_t* qs = smem;
   uint8_t* ks = smem + kQBytes;
   uint64_t* full = reinterpret_cast<uint64_t*>(ks + kRing * kStageBytes);
-  uint64_t* acc_full = full + kRing;
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 2);
+  uint64_t* stage_free = full + kRing;
+  uint64_t* acc_full = stage_free + kRing;
+  uint64_t* acc_free = acc_full + 2;
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_free + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
   *user = ks + kRing * kStageBytes + kBarBytes;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  static_assert(kRing <= kBarUser - kBarLoad, "a named barrier per stage");
+  static_assert((2 * kRing + 4) * 8 + 8 <= kBarBytes, "the barriers' page");
 
   if (tid == 0) {
-    for (int s = 0; s < kRing; ++s) mbar_init(full + s, 1);
-    for (int b = 0; b < 2; ++b) mbar_init(acc_full + b, 1);
+    for (int s = 0; s < kRing; ++s) {
+      mbar_init(full + s, 1);
+      mbar_init(stage_free + s, 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(acc_full + b, 1);
+      mbar_init(acc_free + b, kDrainWarps);
+    }
     mbar_fence_init();
     *abort_flag = 0;
   }
@@ -199,15 +228,26 @@ __device__ bool segments_cta(uint8_t* smem_raw, const CUtensorMap* map, SegmentF
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem_base = *tmem_slot;
-  // a wait that runs out makes every role go on without waiting or working, so that all still meet at the barriers
-  bool ok = true;
+  bool ok = true;   // no wait of this warp has run out, and it has not seen that another's has; the same in all its lanes
   auto wait = [&](uint64_t* bar, uint32_t parity) {
-    if (ok && !mbar_try_wait(bar, parity)) {
-      const long long start = clock64();
-      for (uint32_t it = 1; ok && !mbar_try_wait(bar, parity); ++it) {
-        if ((it & 255u) == 0u && (*abort_flag || clock64() - start > HKV_WAIT_CYCLES)) ok = false;
+    if (!ok || __all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return;
+    const long long start = clock64();
+    for (uint32_t it = 1; !__all_sync(0xffffffffu, mbar_try_wait_ns(bar, parity, kWaitNs)); ++it) {
+      if ((it & 15u) == 0u && __any_sync(0xffffffffu, *abort_flag || clock64() - start > HKV_WAIT_CYCLES)) {
+        *abort_flag = 1;
+        ok = false;
+        return;
       }
-      if (!ok) *abort_flag = 1;
+    }
+  };
+  // what this warp has started itself, waited for whatever has become of the rest
+  auto settle = [&](uint64_t* bar, uint32_t parity) {
+    const long long start = clock64();
+    while (!__all_sync(0xffffffffu, mbar_try_wait_ns(bar, parity, kWaitNs))) {
+      if (__any_sync(0xffffffffu, clock64() - start > HKV_WAIT_CYCLES)) {
+        ok = false;
+        return;
+      }
     }
   };
 
@@ -220,12 +260,13 @@ __device__ bool segments_cta(uint8_t* smem_raw, const CUtensorMap* map, SegmentF
       named_sync(kBarDrainIssue, (kDrainWarps + 1) * 32);   // the segment's query rows are in place
       const bool both = seg.n_rows > 128;
       fence_after_sync();
-      for (int tile = seg.tile_begin; tile < seg.tile_end; ++tile, ++i) {
+      for (int tile = seg.tile_begin; ok && tile < seg.tile_end; ++tile) {
         const int s = i % kRing, buf = i & 1;
-        if (i >= 2) named_sync(kBarAcc + buf, (kDrainWarps + 1) * 32);   // tile i - 2 has been drained
+        if (i >= 2) wait(acc_free + buf, ((i >> 1) - 1) & 1);   // tile i - 2 has been drained
         wait(full + s, (i / kRing) & 1);
+        if (!ok) break;
         fence_after_sync();
-        if (ok && lane == 0) {
+        if (lane == 0) {
           const uint32_t k_addr = k_addr0 + static_cast<uint32_t>(s * kStageBytes);
           const uint32_t d = tmem_base + static_cast<uint32_t>(buf * 256);
 #pragma unroll
@@ -239,43 +280,34 @@ __device__ bool segments_cta(uint8_t* smem_raw, const CUtensorMap* map, SegmentF
               if (both) umma_bf16(d + 128u, smem_desc(q_addr + qoff + 128u * 128u), smem_desc(k_addr + koff), idesc, kk != 0);
             }
           }
-          umma_commit(acc_full + buf);   // the accumulator is complete, the stage may be refilled
+          umma_commit(stage_free + s);   // the stage may be refilled
+          umma_commit(acc_full + buf);   // the accumulator is complete
         }
         __syncwarp();
+        ++i;
       }
     }
-    // arrivals on the barriers of the last tiles must land before the CTA may leave
-    for (int t = max(0, i - 2); t < i; ++t) named_sync(kBarAcc + (t & 1), (kDrainWarps + 1) * 32);
+    for (int t = max(0, i - 2); t < i; ++t) settle(acc_full + (t & 1), (t >> 1) & 1);
   } else if (warp == kDrainWarps + 1) {
-    // ---- loads, kRing tiles ahead of the tensor core; the first draining warp passes on that a tile's instructions
-    // have completed, so that this warp never polls
-    Seg seg, done;
-    int n = 0, sg_ld = 0, tile = 0;
-    bool more = segment(0, seg);
-    if (more) tile = seg.tile_begin;
-    auto load_next = [&]() {
-      if (!more) return;
-      const int s = n++ % kRing;
-      if (ok && lane == 0) {
-        const uint32_t dst = smem_u32(ks) + static_cast<uint32_t>(s * kStageBytes);
-        mbar_arrive_expect_tx(full + s, kStageBytes);
-        tma_load_2d(dst, map, 0, seg.key_row0 + tile * kKeysPerTile, full + s);
-        tma_load_2d(dst + kPlaneBytesK, map, 64, seg.key_row0 + tile * kKeysPerTile, full + s);
+    // ---- loads, kRing tiles ahead of the tensor core ----
+    Seg seg;
+    int n = 0;
+    for (int sg = 0; ok && segment(sg, seg); ++sg) {
+      for (int tile = seg.tile_begin; ok && tile < seg.tile_end; ++tile) {
+        const int s = n % kRing;
+        if (n >= kRing) wait(stage_free + s, (n / kRing - 1) & 1);   // the instructions of tile n - kRing have completed
+        if (!ok) break;
+        if (lane == 0) {
+          const uint32_t dst = smem_u32(ks) + static_cast<uint32_t>(s * kStageBytes);
+          mbar_arrive_expect_tx(full + s, kStageBytes);
+          tma_load_2d(dst, map, 0, seg.key_row0 + tile * kKeysPerTile, full + s);
+          tma_load_2d(dst + kPlaneBytesK, map, 64, seg.key_row0 + tile * kKeysPerTile, full + s);
+        }
+        __syncwarp();
+        ++n;
       }
-      __syncwarp();
-      if (++tile == seg.tile_end) {
-        more = segment(++sg_ld, seg);
-        if (more) tile = seg.tile_begin;
-      }
-    };
-    for (int j = 0; j < kRing; ++j) load_next();
-    int i = 0;
-    for (int sg = 0; segment(sg, done); ++sg)
-      for (int t = done.tile_begin; t < done.tile_end; ++t, ++i) {
-        named_sync(kBarLoad + i % kRing, 64);
-        if (*abort_flag) ok = false;   // no copy may start once the others have given up
-        load_next();
-      }
+    }
+    for (int t = max(0, n - kRing); t < n; ++t) settle(full + t % kRing, (t / kRing) & 1);
   } else {
     // ---- drain: warp w owns lane quarter w % 4 (the hardware's rule) and column part (w - 1) / 4 ----
     const int quarter = warp & 3, part = (warp - 1) >> 2;
@@ -308,13 +340,13 @@ __device__ bool segments_cta(uint8_t* smem_raw, const CUtensorMap* map, SegmentF
       for (int tile = seg.tile_begin; tile < seg.tile_end; ++tile, ++i) {
         const int buf = i & 1;
         wait(acc_full + buf, (i >> 1) & 1);
-        if (warp == 1) named_arrive(kBarLoad + i % kRing, 64);   // its stage is free
         fence_after_sync();
         const uint32_t taddr =
             tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) + static_cast<uint32_t>(buf * 256 + part * 64);
         tile_fn(seg, tile, row, part, taddr);
         fence_before_sync();
-        named_arrive(kBarAcc + buf, (kDrainWarps + 1) * 32);
+        __syncwarp();
+        if (ok && lane == 0) mbar_arrive(acc_free + buf);
       }
       end(seg, row, part, ok);
     }

@@ -71,3 +71,26 @@ def test_a_wait_that_cannot_end_gives_up_and_the_device_stays_usable(checked):
     lc.close()
     # and a fresh cache on the same device still matches the oracle
     P.compare_layer(hi.cfg0(n_steps=1))
+
+
+@pytest.mark.parametrize("role", [-1, 0, 1, 2])
+def test_an_engine_role_that_stops_ends_the_launch_with_a_timeout(checked, role):
+    """The tensor-core engine with its copies, its instructions or its draining warps stopping early, at the first tiles, at
+    a segment's end and in mid-ring: every other role must give up at the cycle limit and still meet the others, so that
+    the launch ends, the error word tells of it and the tensor memory is free for the next launch.  (A role that stops
+    after the last tile, or two tiles before it while draining, leaves nobody waiting.)"""
+    from paper_2604_05887_b200.layer import LayerCache
+    hkv = checked
+    fn = hkv.lib.hkv_selftest_engine_timeout
+    fn.argtypes, fn.restype = [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int32, ctypes.c_int32, ctypes.c_void_p], ctypes.c_int
+    lc = LayerCache(hi.cfg0(n_steps=1))
+    keys = torch.randn(512, 128, device="cuda").bfloat16()
+    tiles, waits = 12, {-1: 0, 0: 12, 1: 12, 2: 10}[role]      # tiles somebody waits for
+    for upto in (0, 1, 2, 3, 4, 5, 7, 8, 9, 10, 11, tiles):
+        assert fn(lc.handle, keys.data_ptr(), role, upto, None) == 0
+        torch.cuda.synchronize()                                # returns: the waits gave up at their cycle limit
+        assert hkv.hkv_last_device_error(lc.handle) == ((7, 6) if upto < waits else (0, 0)), upto
+        assert hkv.lib.hkv_clear_device_error(lc.handle, None) == 0
+    lc.close()
+    import parity_util as P
+    P.compare_layer(hi.cfg0(n_steps=1))                         # window scores on every SM: tensor memory is all there
