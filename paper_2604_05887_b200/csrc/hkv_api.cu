@@ -291,9 +291,11 @@ static hkv_status compress_common(const hkv_config* cfg, const void* k, const vo
                            static_cast<int>(H.err_off + 8 - H.n_valid_off), tile_prefix, s) == cudaSuccess;
     int64_t build_bytes = 0;
     for (const auto& u : c->units) build_bytes += u.type == 0 ? 0 : 4ll * kRowBytes * u.C;
+    int n_sm = 1;
+    ok = ok && compress_configure(&n_sm) == cudaSuccess;
     // A short prompt: few key tiles (they leave half of the SMs free) and copies of a few microseconds.  All kernels go on one
     // stream, each set up beside its predecessors, the dynamic heads' last: it runs beside the selection and the gather.
-    const bool chain = window && total_tiles <= 74 && build_bytes <= (24ll << 20) && !c->host_bytes;
+    const bool chain = window && total_tiles <= n_sm / 2 && build_bytes <= (24ll << 20) && !c->host_bytes;
     // Else the static heads run beside the dynamic ones, on the library's second stream (forked from and joined to `s`): it has
     // the higher priority, so that the long chain of the static heads' kernels never queues behind the dynamic heads' blocks.
     StepSide* side = (H.n_static > 0 && H.n_dynamic > 0 && !chain) ? step_side() : nullptr;
@@ -307,7 +309,7 @@ static hkv_status compress_common(const hkv_config* cfg, const void* k, const vo
     // that got onto the SMs before a pass's held it up by the length of one: 5 to 8 us.  10 static + 6 dynamic units of 24-32 K
     // tokens: 131 us against 141; 13 + 19 of 50 K: 277 against 291.)
     bool later = false;
-    if (side && window) later = static_cast<double>(build_bytes) / 6.0e6 < 2.1 * static_cast<double>(total_tiles) / 148.0 + 30.0;
+    if (side && window) later = static_cast<double>(build_bytes) / 6.0e6 < 2.1 * static_cast<double>(total_tiles) / n_sm + 30.0;
     if (ok && H.n_static > 0) {
       if (window)
         ok = launch_window_scores(c->dev_base, static_cast<char*>(workspace), k, q_obs, H, total_tiles, ws_rowstat_off,

@@ -900,8 +900,6 @@ __global__ void __launch_bounds__(kHeadDim)
 
 }  // namespace
 
-namespace {
-
 // Shared-memory limits of the compression kernels and the number of SMs, once per device.
 cudaError_t compress_configure(int* n_sm) {
   constexpr int kMaxDevices = 64;
@@ -926,6 +924,8 @@ cudaError_t compress_configure(int* n_sm) {
   *n_sm = sms[dev];
   return cudaSuccess;
 }
+
+namespace {
 
 // One launch; `dependent`: it may be set up while its predecessor on the stream still runs (the kernel waits for it itself).
 template <class... Params, class... Args>

@@ -110,6 +110,8 @@ cudaError_t launch_decode(const DecodeParams<kMaxMulti>& params, int total_units
 // whether they take it.
 bool decode_step_instance(const DecodeParams<1>& params, int max_chunks, int max_tiles);
 cudaError_t launch_decode_step(const DecodeParams<1>& params, int max_chunks, int total_units, cudaStream_t stream);
+// Sets the compression kernels' shared-memory limits (once per device) and gives the current device's number of SMs.
+cudaError_t compress_configure(int* n_sm);
 // Writes the cache's tables (a host image of table_bytes), clears [zero_begin, zero_begin + zero_bytes) of the cache and, unless
 // null, fills tile_prefix with the static units' running tile counts.
 // chain (launch_window_scores .. launch_build_dynamic): the compression's kernels follow one another on one stream, each set up
