@@ -1104,8 +1104,6 @@ cudaError_t launch_nt(const DecodeParams<N>& params, int total_units, cudaStream
 
 }  // namespace
 
-size_t decode_smem_bytes() { return kSmemBytes; }
-
 constexpr int kLatencyCluster = 10;
 
 int choose_cluster(int total_units, int max_tiles, const int* max_active) {

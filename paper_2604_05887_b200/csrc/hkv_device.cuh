@@ -153,16 +153,6 @@ __device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
   return r;
 }
-__device__ __forceinline__ void st_cluster_f32(uint32_t addr, float v) {
-  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
-}
-__device__ __forceinline__ void st_cluster_f32x2(uint32_t addr, float x, float y) {
-  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(x), "f"(y) : "memory");
-}
-__device__ __forceinline__ void st_cluster_f32x4(uint32_t addr, float4 v) {
-  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
-               : "memory");
-}
 // Asynchronous stores into the shared memory of a CTA of the cluster (addr, bar: shared::cluster addresses
 // of the SAME destination CTA, from mapa): the value is written and its byte count is credited to the
 // destination's mbarrier, whose waiters then see the data.  No cluster barrier is involved.
@@ -191,9 +181,8 @@ __device__ __forceinline__ float2 ld_cluster_f32x2(uint32_t addr) {
   return v;
 }
 
-// ---- division by a divisor that is fixed for the whole kernel (chunk size, cluster size): the multiplier is
-// computed once, off the critical path, and x / d becomes one multiply-high.  Exact while x * d < 2^32, d > 1.
-__device__ __forceinline__ uint32_t fastdiv_magic(uint32_t d) { return 0xFFFFFFFFu / d + 1u; }
+// ---- division by a divisor that is fixed for the whole launch (chunk size, cluster size): the host computes the multiplier
+// 0xFFFFFFFF / d + 1, and x / d becomes one multiply-high.  Exact while x * d < 2^32, d > 1.
 __device__ __forceinline__ int fastdiv(int x, uint32_t magic) { return static_cast<int>(__umulhi(static_cast<uint32_t>(x), magic)); }
 
 // ---- order-preserving key of a finite float: larger float <=> larger key; every key > 0 ----

@@ -128,7 +128,6 @@ cudaError_t launch_gather_static(char* cache, const void* k, const void* v, cons
 cudaError_t launch_build_dynamic(char* cache, const void* k, const void* v, const Header& hdr,
                                  int max_rows, int max_chunks, bool chain, cudaStream_t stream);
 cudaError_t launch_append(char* cache, const void* k_new, const void* v_new, const Header& hdr, cudaStream_t stream);
-size_t decode_smem_bytes();
 #ifdef HKV_CHECKED
 cudaError_t launch_selftest_wait(int32_t* err_word, cudaStream_t stream);
 cudaError_t launch_selftest_engine(const void* keys, int role, int upto, int32_t* err_word, cudaStream_t stream);
