@@ -80,9 +80,9 @@ __global__ void __launch_bounds__(kSetupThreads)
 // (row r = window position r / G, query head r % G of the group).  The logits run on the tcgen05
 // tensor cores, in base 2, through the segment engine: the static units' 128-key tiles, one after the other, are cut
 // into one equal run per CTA (ranges set by the longest unit left the last CTAs of every shorter one idle).
-// MODE 0: accumulator rows = window rows; a draining thread owns one row and keeps its running
-//         (max, exp-sum) over its half of the segment's keys; stats: float2 [n_static][2 segments][Rpad].
-// MODE 1: the rows' final (max, sum) are put together from those at the start of a segment; accumulator rows = keys; a
+// MODE 0: accumulator rows = window rows; a draining thread owns one row and keeps a running reference (the maximum rounded
+//         up to an integer) and the sum of powers over its half of the segment's keys; stats: float2 [n_static][2 segments][Rpad].
+// MODE 1: the rows' final (reference, sum) are put together from those at the start of a segment; accumulator rows = keys; a
 //         draining thread owns one key and sums the normalised probabilities of its quarter of the rows, the four
 //         quarters meet in shared memory, and s_w[key] (+)= sum / R (written by the first row block, added
 //         to by later ones).
@@ -116,7 +116,8 @@ static_assert(kWindowSmem0 <= 232448 && kWindowSmem1 <= 232448, "one CTA's share
 // Leaves room for four blocks of build_dynamic_kernel beside a CTA (with the 96 registers it takes otherwise there were two, and
 // 19 dynamic units of 50 K tokens took 25 us longer).
 constexpr int kWindowRegs = 72;
-constexpr float kNoKey = -1.0e30f;   // running maximum of a row that has seen no key
+constexpr float kNoKey = -1.0e30f;   // reference of a row that has seen no key
+constexpr float kCeil = 12582912.f;  // 1.5 x 2^23: x + kCeil has no bits behind the point
 
 __device__ __forceinline__ int window_cta_begin(int i, int total, int n_cta) {
   return static_cast<int>(static_cast<int64_t>(i) * total / n_cta);
@@ -204,7 +205,9 @@ __global__ void __maxnreg__(kWindowRegs)
         float top = __uint_as_float(v[0]);
 #pragma unroll
         for (int c = 1; c < 16; ++c) top = fmaxf(top, __uint_as_float(v[c]));
-        top *= sc;   // the scale is positive
+        // (the scale is positive.)  Rounded up to an integer, so that every change of reference, here and when the
+        // segments' parts are put together, is an exact power of two
+        top = __fadd_ru(top * sc, kCeil) - kCeil;
         if (__any_sync(0xffffffffu, top > m_run)) {
           const float m_new = fmaxf(m_run, top);
           z *= fast_exp2(m_run - m_new);
@@ -234,7 +237,7 @@ __global__ void __maxnreg__(kWindowRegs)
     ok = tc::segments_cta<false, kWindowRing0, WindowSeg>(tc_smem, &keys, segment, q_row, begin, tile_fn, end, &user);
   } else {
     const float inv_R = 1.f / static_cast<float>(R);
-    float4* info = nullptr;     // per pair of rows: (-max, -max, 1 / sum, 1 / sum)
+    float4* info = nullptr;     // per pair of rows: (-reference, -reference, 1 / sum, 1 / sum)
     float* last = nullptr;      // per row: last visible key
     float* sums = nullptr;      // [2][4 quarters of the rows][128 keys]
     int n_done = 0;

@@ -38,3 +38,17 @@ def test_keep_set_with_a_crowded_threshold(kind):
     elif kind == "equal_text":
         L.is_text[0, :7000] = 1
     P.compare_layer(L, token_scores=ts)
+
+
+@pytest.mark.parametrize("C,G", [(2001, 4), (20000, 7), (48000, 1)])
+def test_window_scores_sum_to_one(C, G):
+    """The probabilities of a window row sum to one, so a head's scores do, whatever the logits: what is left is the
+    rounding of the row's normaliser.  Bound: two float32 roundings, 2^-23, in the mean of a head's rows; the errors of
+    single powers (mean -5e-8) are in both sums and cancel as long as no change of a running reference adds its own.
+    (Summed in float64 from the float32 scores; each is the sum of many probabilities, rounded without a bias.)"""
+    from paper_2604_05887_b200.layer import LayerCache
+    L = _layer(1, C, [[0, 0]], w=32, Hq=2 * G, ragged=False)
+    lc = LayerCache(L, keep_workspace=True)
+    err = [float(lc.window_scores(0, h, C).astype(np.float64).sum()) - 1.0 for h in range(2)]
+    lc.close()
+    assert max(abs(e) for e in err) <= 2.0 ** -23, err
