@@ -534,7 +534,7 @@ __global__ void __launch_bounds__(256, 3)
   if (!exists) return;
 
   const float4 bd = cls_bounds(bounds, rg);
-  float z = 0.f, s = 0.f;
+  float z = 0.f, top = 0.f, s = 0.f;   // normaliser; sum above hi; sum of listed entries (small beside the other two: kept apart)
   int above = 0, n = 0, n4 = 0;
   bool bad = false;
   for (int r0 = 0; r0 < n_rec; r0 += 32) {
@@ -542,7 +542,7 @@ __global__ void __launch_bounds__(256, 3)
     if (r0 + lane < n_rec) rec = __ldcg(part + r0 + lane);
     if (r0 > 0) my_at = rec_at(min(r0 + lane, n_rec - 1));
     z += rec.x;
-    s += rec.y;
+    top += rec.y;
     above += __float_as_int(rec.z);
     const uint32_t m = __float_as_uint(rec.w);
     bad = bad || (m >> 31);
@@ -702,8 +702,11 @@ __global__ void __launch_bounds__(256, 3)
   }
   if (need > 0 && ca != need && lane == 0) s += static_cast<float>(need - cb) * weight(a);   // copies of one value: need - cb of them count
 #pragma unroll
-  for (int off = 16; off >= 1; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-  if (lane == 0) rowsum[static_cast<size_t>(unit) * P.r_stride + P.row_begin + row] = s / z;
+  for (int off = 16; off >= 1; off >>= 1) {
+    s += __shfl_xor_sync(0xffffffffu, s, off);
+    top += __shfl_xor_sync(0xffffffffu, top, off);
+  }
+  if (lane == 0) rowsum[static_cast<size_t>(unit) * P.r_stride + P.row_begin + row] = (top + s) / z;
 }
 
 // Whole block (kClsFixThreads threads, every one calls): the highest bin b of hist[0, nbins) with

@@ -243,3 +243,24 @@ def test_gpu_classify_shared_samples_and_weighted_blocks(B, C, T, G, Hkv):
     beside blocks of at most 128 rows, which count half when the work is cut up."""
     L = hi.tiny(seed=61, B=B, C=C, chunk_size=32, w=8, Hq=G * Hkv, Hkv=Hkv, d=128)
     _check_case(L, T, 0.05)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("C,fraction", [(9000, 0.05), (32768, 0.05), (32768, 0.2)])
+def test_gpu_classify_many_small_entries_beside_a_large_one(C, fraction):
+    """One key takes nearly all of every row and each of the others about 2^-25 of it, less than half a unit in the last
+    place: added one by one to a sum that holds the large entry they would all be lost.  Bound: the roundings of the
+    row's two sums, of their quotient and of the powers' mean error, 2^-23 in all."""
+    L = hi.tiny(seed=71, B=1, C=C, chunk_size=32, w=8, Hq=8, Hkv=2, d=128, ragged=False)
+    rng = np.random.default_rng(11)
+    u = rng.standard_normal((2, 128))
+    u /= np.linalg.norm(u, axis=1, keepdims=True)
+    k = 0.05 * rng.standard_normal((2, C, 128))
+    k[:, C // 3] = 10.0 * u
+    L.k[0] = bits(k)
+    q_text = bits(20.0 * np.repeat(u, 4, axis=0)[None, None] + rng.standard_normal((1, 8, 8, 128)))
+    counts = np.array([8], np.int32)
+    ref = _oracle_scores(L, q_text, counts, fraction)
+    got, _ = _gpu_scores(L, q_text, counts, fraction, 0.9)
+    assert 0.99 < ref.min() < 0.99999
+    assert np.abs(got - ref).max() <= 2.0 ** -23, (got - ref)
