@@ -21,8 +21,9 @@
  *     helper stream with a few events per device (hkv_compress builds the dynamic heads on it beside
  *     the static ones, hkv_decode_step_host runs its copies on it; both fork it from and join it to
  *     the caller's stream, so the caller sees one ordered stream) and the fixed scratch of
- *     hkv_topk_chunks_noalloc.  hkv_compress uploads its plan from ordinary host memory that it frees
- *     on return, so it is not a call to capture in a CUDA graph; the decode calls are.
+ *     hkv_topk_chunks_noalloc.  hkv_compress is not a call to capture in a CUDA graph; the decode
+ *     calls are.  (It uploads a plan of more than 16 KB, some 150 heads, from ordinary host memory
+ *     that it frees on return; while the stream is being captured that is refused, HKV_ERR_CUDA.)
  *   - "dev" pointers are device (HBM) addresses on the current CUDA device, "host" pointers are
  *     ordinary host memory.  bf16 tensors are passed as void*.
  *   - the caller owns every device buffer, including cache_mem and workspace.  The library never

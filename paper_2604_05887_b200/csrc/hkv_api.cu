@@ -298,7 +298,7 @@ static hkv_status compress_common(const hkv_config* cfg, const void* k, const vo
     const bool chain = window && total_tiles <= n_sm / 2 && build_bytes <= (24ll << 20) && !c->host_bytes;
     // Else the static heads run beside the dynamic ones, on the library's second stream (forked from and joined to `s`): it has
     // the higher priority, so that the long chain of the static heads' kernels never queues behind the dynamic heads' blocks.
-    StepSide* side = (H.n_static > 0 && H.n_dynamic > 0 && !chain) ? step_side() : nullptr;
+    StepSide* side = (ok && H.n_static > 0 && H.n_dynamic > 0 && !chain) ? step_side() : nullptr;
     std::unique_lock<std::mutex> side_lock;
     if (side) side_lock = std::unique_lock<std::mutex>(side->enqueue);
     cudaStream_t ss = side ? side->stream : s;

@@ -973,7 +973,11 @@ cudaError_t launch_setup(char* cache, const void* image, int table_bytes, int ze
                          cudaStream_t stream) {
   if (table_bytes <= 3584) return launch_setup_n<3584>(cache, image, table_bytes, zero_begin, zero_bytes, tile_prefix, stream);
   if (table_bytes <= 16384) return launch_setup_n<16384>(cache, image, table_bytes, zero_begin, zero_bytes, tile_prefix, stream);
-  const cudaError_t e = cudaMemcpyAsync(cache, image, static_cast<size_t>(table_bytes), cudaMemcpyHostToDevice, stream);
+  // a captured copy would read the image when the graph is launched, long after it has been freed
+  cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+  cudaError_t e = cudaStreamIsCapturing(stream, &capture);
+  if (e == cudaSuccess && capture != cudaStreamCaptureStatusNone) e = cudaErrorStreamCaptureUnsupported;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(cache, image, static_cast<size_t>(table_bytes), cudaMemcpyHostToDevice, stream);
   return e == cudaSuccess ? launch_setup_n<0>(cache, image, table_bytes, zero_begin, zero_bytes, tile_prefix, stream) : e;
 }
 

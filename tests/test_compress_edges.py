@@ -52,3 +52,27 @@ def test_window_scores_sum_to_one(C, G):
     err = [float(lc.window_scores(0, h, C).astype(np.float64).sum()) - 1.0 for h in range(2)]
     lc.close()
     assert max(abs(e) for e in err) <= 2.0 ** -23, err
+
+
+def test_tables_copied_from_the_host_are_refused_while_the_stream_is_captured():
+    """Tables beyond 16 KB are copied from a host image that does not outlive the call: captured, the copy would read freed
+    memory at every replay.  The call says so, leaves the capture intact and works outside one."""
+    import torch
+    import parity_util as P
+    from paper_2604_05887_b200 import binding as hkv
+    L = _layer(80, 300, np.tile([[0, 1]], (80, 1)), ragged=False)      # 160 units of 104 bytes
+    cfg = hkv.make_config(80, 8, 2, 128, L.max_seq_len, 32, 8)
+    dev = [torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (L.k, L.v, L.q_obs, L.is_text)]
+    cache_bytes, ws_bytes = hkv.hkv_plan(cfg, L.seq_lens, L.head_type, L.budgets)
+    cache, ws = (torch.empty(n, dtype=torch.uint8, device="cuda") for n in (cache_bytes, ws_bytes))
+    mark = torch.zeros(1, device="cuda")
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        with pytest.raises(hkv.HkvError) as e:
+            hkv.hkv_compress(cfg, *dev[:3], None, dev[3], L.seq_lens, L.head_type, L.budgets, cache, ws)
+        mark += 1
+    assert e.value.status == 6                                         # HKV_ERR_CUDA
+    g.replay()
+    torch.cuda.synchronize()
+    assert mark.item() == 1
+    P.compare_layer(L, units=[(0, 0), (79, 1)])
