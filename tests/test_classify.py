@@ -92,6 +92,7 @@ def _gpu_scores(L, q_text, counts, fraction, theta, workspace="preferred"):
     hkv.hkv_classify_heads(cfg, to_device_bf16(L.k), to_device_bf16(q_text), L.seq_lens, counts, fraction, theta,
                            ws, scores, types)
     torch.cuda.synchronize()
+    _gpu_scores.flagged = int(ws[4:8].view(torch.int32))      # rows (of the last pass) that were done again one by one
     return scores.cpu().numpy(), types.cpu().numpy()
 
 
@@ -141,9 +142,8 @@ def test_gpu_classify_several_row_blocks_in_one_pass():
 @pytest.mark.gpu
 @pytest.mark.parametrize("C", [32768, 32765, 31745, 1023, 5])
 def test_gpu_classify_rows_kept_in_registers(C):
-    """Rows of up to 32768 entries take the pipelined kernel (the row in registers, the next row's copy in flight):
-    the longest such row, lengths that are no multiple of four, a last piece of one vector, rows shorter than one
-    piece, and rows of a handful of entries."""
+    """Contexts of a whole number of tiles, a few keys less, one key in the last tile, one less than a whole number, and
+    fewer keys than a warp has lanes."""
     L = hi.tiny(seed=41, B=2 if C < 2000 else 1, C=C, chunk_size=32 if C >= 64 else 1, w=8 if C >= 64 else 2, Hq=8, Hkv=2,
                 d=128, ragged=False)
     _check_case(L, 5, 0.05)
@@ -152,13 +152,14 @@ def test_gpu_classify_rows_kept_in_registers(C):
 @pytest.mark.gpu
 @pytest.mark.parametrize("C", [32769, 49152])
 def test_gpu_classify_rows_kept_in_shared_memory(C):
-    """Between 32769 and 49152 entries a row stays in shared memory (the general kernel), beyond that in the workspace."""
+    """The longest contexts whose rows, were they done again, would stay in shared memory."""
     L = hi.tiny(seed=42, B=1, C=C, chunk_size=32, w=8, Hq=4, Hkv=2, d=128, ragged=False)
     _check_case(L, 3, 0.05)
 
 
 @pytest.mark.gpu
 def test_gpu_classify_rows_longer_than_shared_memory():
+    """A context longer than shared memory holds, and few rows (rows done again there: the packed case below)."""
     L = hi.tiny(seed=33, B=1, C=50021, chunk_size=32, w=8, Hq=8, Hkv=2, d=128)
     _check_case(L, 3, 0.05)
 
@@ -213,11 +214,14 @@ def test_gpu_classify_random_shapes(case):
 @pytest.mark.gpu
 @pytest.mark.parametrize("C,T,G,fraction,kind", [
     (127, 9, 4, 0.05, ""), (129, 64, 4, 0.05, ""), (4096, 37, 7, 0.05, ""), (4097, 65, 4, 0.2, ""), (8200, 256, 1, 0.05, ""),
-    (9000, 40, 7, 0.05, "ties"), (9000, 40, 7, 0.3, "ties"), (6000, 33, 8, 0.05, "clustered"), (5000, 7, 4, 0.001, "nan")])
+    (9000, 40, 7, 0.05, "ties"), (9000, 40, 7, 0.3, "ties"), (6000, 33, 8, 0.05, "clustered"), (5000, 7, 4, 0.001, "nan"),
+    (6000, 512, 8, 0.05, "packed"), (50021, 150, 4, 0.05, "packed")])
 def test_gpu_classify_edges_of_the_sampled_bounds(C, T, G, fraction, kind):
     """Contexts around the sample's and a tile's size, row blocks of 256 rows and one more, and inputs whose threshold the
     sample cannot bound closely: a value shared by a third of the keys at the threshold, keys near the threshold
-    packed into one stretch of the context (the list of that stretch overflows), keys that are not finite."""
+    in one stretch of the context, a stretch of keys so alike that the lists of the segments it fills overflow for the rows
+    whose threshold lies among them (these and the rows with a key that is not finite are done again one by one, at
+    50021 keys in the workspace)."""
     L = hi.tiny(seed=51, B=1, C=C, chunk_size=32, w=8, Hq=2 * G, Hkv=2, d=128, ragged=False)
     rng = np.random.default_rng(C)
     if kind == "ties":        # one key repeated: its logit lies at or near the threshold for many rows
@@ -225,13 +229,19 @@ def test_gpu_classify_edges_of_the_sampled_bounds(C, T, G, fraction, kind):
     elif kind == "clustered":
         L.k[0, :, 1000:1900] = hi.f32_to_bf16_bits(hi.bf16_bits_to_f32(L.k[0, :, 1000:1001]) +
                                                    0.2 * rng.standard_normal((2, 900, 128)).astype(np.float32))
+    elif kind == "packed":
+        n = C // 5
+        L.k[0, :, 1000:1000 + n] = hi.f32_to_bf16_bits(hi.bf16_bits_to_f32(L.k[0, :, 1000:1001]) +
+                                                       0.02 * rng.standard_normal((2, n, 128)).astype(np.float32))
     if kind != "nan":
         _check_case(L, T, fraction)
+        assert (_gpu_scores.flagged > 0) == (kind == "packed"), _gpu_scores.flagged
         return
     q_text, counts = hi.text_queries(L, T, seed=5)
     ref = _oracle_scores(L, q_text, counts, fraction)
     L.k[0, 1, 4321] = 0x7FC0   # the head without it must not notice; the other one still answers
     got, _ = _gpu_scores(L, q_text, counts, fraction, 0.9)
+    assert _gpu_scores.flagged > 0
     assert abs(got[0, 0] - ref[0, 0]) <= SCORE_TOL and 0.0 < got[0, 1] <= 1.0 + 1e-6
 
 
@@ -240,7 +250,7 @@ def test_gpu_classify_edges_of_the_sampled_bounds(C, T, G, fraction, kind):
                                          (4, 700, 256, 7, 4)])
 def test_gpu_classify_shared_samples_and_weighted_blocks(B, C, T, G, Hkv):
     """Row blocks whose samples eight, four, two and one CTAs share (some without a tile of their own), and full blocks
-    beside blocks of at most 128 rows, which count half when the work is cut up."""
+    beside blocks of at most 128 rows, which count two against their three when the work is cut up."""
     L = hi.tiny(seed=61, B=B, C=C, chunk_size=32, w=8, Hq=G * Hkv, Hkv=Hkv, d=128)
     _check_case(L, T, 0.05)
 
