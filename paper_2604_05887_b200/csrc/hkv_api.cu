@@ -303,13 +303,18 @@ static hkv_status compress_common(const hkv_config* cfg, const void* k, const vo
     if (side) side_lock = std::unique_lock<std::mutex>(side->enqueue);
     cudaStream_t ss = side ? side->stream : s;
     if (ok && side) ok = cudaEventRecord(side->fork, s) == cudaSuccess && cudaStreamWaitEvent(ss, side->fork, 0) == cudaSuccess;
-    // The dynamic heads' copies slow the window scores down where both run (HBM).  If they are short enough to be done
-    // while the second pass, the selection and the gather run (~2.1 us per tile of a CTA + 30 us; the copies at about
-    // 6 TB/s), they start once the second pass's blocks are running; else once the first one's are.  (Blocks of the copies
-    // that got onto the SMs before a pass's held it up by the length of one: 5 to 8 us.  10 static + 6 dynamic units of 24-32 K
-    // tokens: 131 us against 141; 13 + 19 of 50 K: 277 against 291.)
+    // When the dynamic heads' copies start: once the first pass's blocks are running, or once the second one's are.  Blocks of
+    // the copies that take an SM's room between the passes hold up the second one by their length, which is that of a
+    // chunk: with chunks of up to 32 tokens it hardly shows.  Starting later avoids it but leaves HBM idle in the first pass, which pays
+    // only if the copies (about 6 TB/s) still end within the selection and the gather, and the passes are not long themselves;
+    // beyond 64 tokens a chunk the copies' few long blocks no longer do.  Mean loss against the better of the two over 139 shapes each
+    // (28 / 4 heads, 5 to 50 K tokens, batch 1 to 8, 25 to 75 % static), chunks of 16 / 32 / 48 / 64 / 128: this line
+    // 0.1 / 0.6 / 0.4 / 0.4 / 1.1 %, always the first pass 0.1 / 0.6 / 1.1 / 1.9 / 1.1, always the second 5.5 / 5.0 / 4.3 / 3.9 / 4.8.
+    // (Four sequences of 24-32 K tokens, 10 + 6 heads, chunk 64: 126.4 us behind the second pass, 128.8 behind the first; chunk 32:
+    // 125.8 and 123.2; eight of 50 K, 19 + 13 heads: 316 and 263.)
     bool later = false;
-    if (side && window) later = static_cast<double>(build_bytes) / 6.0e6 < 2.1 * static_cast<double>(total_tiles) / n_sm + 30.0;
+    if (side && window)
+      later = H.chunk_size > 32 && H.chunk_size <= 64 && static_cast<double>(build_bytes) / 6.0e6 < 30.0 && total_tiles < 20ll * n_sm;
     if (ok && H.n_static > 0) {
       if (window)
         ok = launch_window_scores(c->dev_base, static_cast<char*>(workspace), k, q_obs, H, total_tiles, ws_rowstat_off,
