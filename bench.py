@@ -633,7 +633,7 @@ def main():
     ap.add_argument("--no-extra", action="store_true",
                     help="skip the other workloads (cfg4 cell, cfg1, cfg3 reduced, cfg0) and the next rows")
     ap.add_argument("--sweep", action="store_true", help="run the 100-cell single-layer sweep (cfg4) instead of the step benchmark")
-    ap.add_argument("--sweep-quick", action="store_true", help="with --sweep: only budgets 10 % and 100 % at static fraction 0.5")
+    ap.add_argument("--sweep-quick", action="store_true", help="with --sweep: only budgets 10 %% and 100 %% at static fraction 0.5")
     ap.add_argument("--next-rows", action="store_true",
                     help="time hkv_classify_heads and the host-offload variant on layer 0 even in a reduced (--layers) run")
     ap.add_argument("--timeline", action="store_true",
