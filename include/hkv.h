@@ -267,7 +267,7 @@ hkv_status hkv_allocate_budgets(int32_t n_heads, const uint8_t* head_type, const
  *   seq_lens     host int32 [B]  C_b in 1..max_seq_len;   n_text  host int32 [B]  in 1..n_text_max
  *   topk_fraction in (0, 1] (the paper's focus fraction is 0.05);  theta finite (the paper settles on 0.9)
  *   workspace    dev, 256-B aligned, >= min_bytes of hkv_classify_workspace; with less than
- *                preferred_bytes the rows are processed in several passes (same result)
+ *                preferred_bytes the rows may take several passes (the same sums up to rounding)
  *   scores_out   dev f64 [B, Hkv]  S (float32 softmax arithmetic, rows averaged in double, fixed order)
  *   head_type_out dev u8 [B, Hkv]  the array hkv_plan / hkv_compress take, once copied to the host
  * Enqueued on `stream`, no synchronisation; deterministic.  Errors: HKV_ERR_SHAPE (lengths),

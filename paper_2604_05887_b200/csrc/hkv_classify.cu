@@ -152,7 +152,8 @@ __global__ void __launch_bounds__(256)
   const int per = cls_sample_per(P, b), slot = j / tc::kKeysPerTile, rank = slot / (per + 1), at = slot - rank * (per + 1);
   const int tile = at == 0 ? 0 : rank * per + at;
   if (rank >= P.split || tile > cls_sample_tiles(P, b)) return;
-  uint32_t x = static_cast<uint32_t>(tile * tc::kKeysPerTile + j % tc::kKeysPerTile) * 0x9E3779B1u + 0x7F4A7C15u;   // any mixing will do
+  // (mixed by the 32-bit finaliser of MurmurHash3)
+  uint32_t x = static_cast<uint32_t>(tile * tc::kKeysPerTile + j % tc::kKeysPerTile) * 0x9E3779B1u + 0x7F4A7C15u;
   x ^= x >> 16; x *= 0x85EBCA6Bu; x ^= x >> 13; x *= 0xC2B2AE35u; x ^= x >> 16;
   const size_t key = static_cast<size_t>(unit) * P.max_seq_len + __umulhi(x, static_cast<uint32_t>(P.C[b]));
   samples[(static_cast<size_t>(unit) * P.sample_stride + j) * 16 + piece] = __ldg(kin + key * 16 + piece);
@@ -166,7 +167,7 @@ __global__ void __launch_bounds__(256)
 // as single samples do with an eighth of the shared-memory atomics (one atomic per sample: 5 us per tile).
 // Bound: a chain of copy, instructions and drain per tile, 33 tiles one after the other (37 us whatever the number of row
 // blocks).  Where SMs would stay empty a cluster of P.split CTAs shares a block's tiles, each with its own copy of tile 0
-// in front, and adds the histograms up over distributed shared memory: with eight, 8 row blocks take 15 us.
+// in front, and adds the histograms up over distributed shared memory: with eight, 8 row blocks take 18 us.
 // grid: row blocks of the pass x P.split.  bounds: float4 [unit][row_block] = (lo, hi, scaled reference, -).
 // ---------------------------------------------------------------------------------------------
 constexpr int kClsHistBytes = kClsSampleBins * tc::kQRows * 2;
@@ -321,9 +322,9 @@ __global__ void __launch_bounds__(tc::kSegThreads, 1)
 // sums and list position in registers.  An entry above the upper bound joins sum and count; one between the bounds is
 // appended, by predicated instructions, to the thread's own column of shared memory, which goes to the row's list in
 // groups of four.
-// Bound: issue slots (ten per warp and entry at 72 % of the scheduler's cycles; four warps per scheduler is all the
-// registers allow).  One context of 32768 keys against 7168 rows: 132 us = 2.8 us per 256 x 128 tile; with only the lower
-// bound tested here 133 us and lists twice as long, with slots advanced by sign arithmetic instead of predicates 158 us.
+// Bound: issue slots (13 instructions per warp and entry, 75 % of the scheduler's cycles; four warps per scheduler is all the
+// registers allow).  One context of 32768 keys against 7168 rows: 127 us = 2.6 us per 256 x 128 tile.  With only the lower
+// bound tested here lists are twice as long and the time the same; slots advanced by sign arithmetic instead of predicates: + 20 %.
 // grid: P.n_cta.  partial: float4 [unit][row_block][seg_max][2] = (normaliser, sum above hi, number above hi, listed
 // entries; the sign bit of the last = the list was full), list: float [unit][row_block][2][list_stride].
 // ---------------------------------------------------------------------------------------------
@@ -484,7 +485,7 @@ __global__ void __launch_bounds__(tc::kSegThreads, 1)
 // thresholds around the place where the k-th largest should lie (interpolated between the bounds), which leaves about a
 // hundred entries undecided; pass 2 adds up what lies above and moves the undecided to the front of each lane's part,
 // where the threshold is closed in on exactly, interpolating and halving the order-preserving keys in turn.
-// Bound: instructions, about 1500 per warp and row.  cap: float4s of shared memory per warp (a longer list is walked in
+// Bound: instructions, about 2400 per warp and row (7168 rows of 32768 keys: 28 us).  cap: float4s of shared memory per warp (a longer list is walked in
 // global memory).
 // ---------------------------------------------------------------------------------------------
 constexpr int kClsUndecided = 256;   // entries the last stage takes over (eight per lane)
@@ -1063,7 +1064,7 @@ hkv_status cls_check(const hkv_config* cfg, int32_t n_text_max) {
   return HKV_OK;
 }
 
-// sequences per group of launches, units of a group, bytes of the row-sum array in front of the logits
+// sequences per group of launches, units of a group, bytes of the row-sum array in front of the rest
 struct ClsShape {
   int group_batch, group_units, r_max;
   size_t head_bytes;   // error word (kAlign bytes) + row sums
@@ -1092,7 +1093,8 @@ extern "C" hkv_status hkv_classify_workspace(const hkv_config* cfg, int32_t n_te
   const size_t row_bytes = round_up(cfg->max_seq_len, tc::kKeysPerTile) * sizeof(float) * s.group_units;
   if (min_bytes) *min_bytes = s.head_bytes + 16 * row_bytes;
   if (preferred_bytes) {
-    // every row at once, up to half a gigabyte of logits
+    // A float per key of every row, up to half a gigabyte (the size this call has always asked for): what a pass keeps is a fraction of
+    // it, so all rows fit one pass and their lists get up to six times their expected length.
     size_t rows = round_up(s.r_max, 16);
     const size_t cap = std::max<size_t>(16, (static_cast<size_t>(512) << 20) / row_bytes / 16 * 16);
     rows = std::min(rows, cap);
@@ -1178,7 +1180,9 @@ extern "C" hkv_status hkv_classify_heads(const hkv_config* cfg, const void* k, c
     // Rows per pass and list room.  A row takes its bounds, two partial records per CTA that shares its block, its entry
     // in the flag list and two lists of `per_tile` entries per key tile plus kClsSlack per segment.  The lists get at
     // least 1.3 times their (generously) expected length, and up to six times where the workspace allows it in one pass:
-    // keys of a video frame are correlated, so a stretch of the context may hold several times its share.
+    // keys of a video frame are correlated, so a stretch of the context may hold several times its share.  28168 rows of
+    // 24-32 K keys get 1.6 times: no row overflows with keys of frame means plus noise, 259 do when a direction that all queries share
+    // rises by three standard deviations over the context (560 -> 835 us: such a row keeps its SM 140 us at 32 K keys, 200 at 50 K).
     const int n_tiles = (cg_max + tc::kKeysPerTile - 1) / tc::kKeysPerTile;
     // the work of rows [begin, begin + rows) of every head: w_prefix and weight of P, the number of row blocks
     auto work_of = [&](int begin, int rows) {

@@ -86,8 +86,10 @@ __global__ void __launch_bounds__(kSetupThreads)
 //         draining thread owns one key and sums the normalised probabilities of its quarter of the rows, the four
 //         quarters meet in shared memory, and s_w[key] (+)= sum / R (written by the first row block, added
 //         to by later ones).
-// Bound: 2^x (16 per clock and SM; a scheduler whose four warps all have rows spends 2048 cycles per tile on them) at 85 %:
-// 2350 cycles per tile, 31 us a pass for ten units of 24-32 K tokens.  A quarter or half of the powers as polynomials on the
+// Bound: the tensor core's instructions and the drain of a tile overlap only in part, and a pass is short.  Ten units of 24-32 K
+// tokens (15 tiles per CTA): 38.7 and 39.1 us; without the powers (16 per clock and SM, 2048 cycles per tile) 32.9 and 31.0, without
+// the drain 28.1 and 23.3, without the copies 35.0 and 40.1, without copies and drain 24.0 and 21.4.  A tile takes 1.41 and 1.75 us, the
+// launch, the query block and the first tiles' way 16 and 11.  A quarter or half of the powers as polynomials on the
 // FMA pipes, and reading the accumulator ahead, changed nothing.  One exponent max + log2 sum instead of two constants per
 // row took 2 us off a second pass, but rounds a row's weight ten times as coarsely.
 // grid: CTAs; one launch per block of 256 window rows.

@@ -149,7 +149,9 @@ __device__ __noinline__ int select_global(const float* gscores, int n_chunks, in
 // NT: 8-wide column tiles of query heads (1 for groups up to 8, 2 up to 16); W: warps; N: caches the arguments have room for.
 // IPT > 0: a whole step of one cache (selection and attention) whose units have at most 256 IPT chunks of a multiple of eight
 // tokens (of kTile, if ONE); IPT = 0: anything.  The general kernel has 160 KB of instructions, more than an SM caches, of which
-// a step executes a fifth: an instance for what nearly every step is made the 28-layer step of four sequences 287 -> 255 us.
+// a step executes a fifth: an instance for what nearly every step is makes the 28-layer step of four sequences of 24-32 K tokens 278 ->
+// 256 us (graph, L2 flushed) and that of one of 16 K 209 -> 188.  IPT follows from the chunks the cache has room for, not from those it
+// holds: a recorded launch may be replayed after appends.
 template <int NT, int W, int N, int IPT, bool ONE>
 __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __grid_constant__ DecodeParams<N> P) {
   constexpr bool FULL = IPT > 0;
@@ -1112,8 +1114,10 @@ int choose_cluster(int total_units, int max_tiles, const int* max_active) {
   // Even sizes only: two CTAs share an SM, and an odd cluster leaves half an SM idle (measured: 13 CTAs
   // per unit are slower than 12).  Sizes need not be powers of two.
   // Short lists (at most 16 tiles per CTA at ten CTAs per unit) are bound by the step's chain of latencies,
-  // not by bandwidth; there ten CTAs per unit measured best at every batch size tried (1 .. 6 sequences of
-  // four KV heads), larger clusters paying more for their barriers and exchanges than they gain.
+  // not by bandwidth.  What the size changes there is the number of rounds in which a CTA's eight warps and six stages take its
+  // tiles, and how many CTAs of the next launch find room.  Over 45 shapes (1 .. 12 sequences of four KV heads, 52 to 205
+  // tiles) this choice is within 4 % of the best even size in 36; more than ten CTAs are better (up to 21 %, 79 tiles) where
+  // they bring a CTA's tiles to the six that fit the ring and ten do not, fewer (3 to 9 %) where the rounds stay the same.
   int c = 1;
   for (int t = 2; t <= kMaxCluster; t += 2)
     if (max_active[t] >= total_units && t * 2 <= max_tiles) c = t;
