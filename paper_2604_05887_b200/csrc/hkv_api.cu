@@ -489,7 +489,16 @@ static hkv_status decode_stages_n(hkv_cache* const* caches, const void* const* q
     cudaGetLastError();
     return HKV_ERR_CUDA;
   }
-  for (int i = 0; i < n; ++i) caches[i]->fresh = false;
+  if (fresh) {
+    // a recorded launch has not run: the next one may still be the first to follow the compression or the append (the
+    // legacy default stream cannot be recorded, and asking costs a short request 1 %)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (stream && cudaStreamIsCapturing(static_cast<cudaStream_t>(stream), &capture) != cudaSuccess) {
+      cudaGetLastError();   // not known: as if recorded
+    } else if (capture == cudaStreamCaptureStatusNone) {
+      for (int i = 0; i < n; ++i) caches[i]->fresh = false;
+    }
+  }
   return HKV_OK;
 }
 

@@ -143,6 +143,6 @@ struct hkv_cache {
   size_t cache_bytes, workspace_bytes, host_bytes;
   int64_t kv_bytes, summary_bytes, algo_bytes, retained;
   int max_static_rows, max_dyn_rows, max_chunks, max_tiles;
-  bool fresh;   // no decode launch has followed the last compression / append yet
+  bool fresh;   // no decode launch has followed the last compression / append yet (one that was only recorded does not count)
   int appended; // tokens added by hkv_append so far
 };

@@ -51,3 +51,41 @@ def test_append_and_decode_interleaved_over_layers():
     want = run(True)
     for _ in range(3):
         assert all(np.array_equal(a, b) for a, b in zip(run(False), want))
+
+
+def test_a_recorded_step_does_not_stand_for_the_first_after_an_append():
+    """A decode call recorded between an append and the next step has not run: the step must still wait for the append (a
+    launch that need not may read the cache's tables and rows while the append writes them).  The recording itself
+    waits for nothing, so the append may still be on its way when the step is launched."""
+    from paper_2604_05887_b200.layer import LayerCache, to_device_bf16
+    L = hi.cfg1(layer=0, C=2048, block=256, n_steps=1)
+    q = to_device_bf16(L.q[0])
+    g = torch.Generator(device="cuda").manual_seed(9)
+    new = torch.randn(12, 2, 1, 4, 128, device="cuda", generator=g).bfloat16().contiguous()
+    ballast = torch.randn(4096, 4096, device="cuda")
+
+    def run(recorded):
+        lc = LayerCache(L, append_capacity=12)
+        spare, side, outs, graphs = lc.new_out(), torch.cuda.Stream(), [], []
+        lc.decode(q, spare)
+        torch.cuda.synchronize()
+        for t in range(12):
+            if recorded:
+                ballast @ ballast                      # keeps the append waiting while the step is recorded
+            lc.append(new[t, 0], new[t, 1])
+            if recorded:
+                with torch.cuda.stream(side):
+                    graphs.append(torch.cuda.CUDAGraph())
+                    graphs[-1].capture_begin(capture_error_mode="relaxed")
+                    lc.decode(q, spare)
+                    graphs[-1].capture_end()
+            else:
+                torch.cuda.synchronize()
+            outs.append(lc.new_out())
+            lc.decode(q, outs[-1])
+        torch.cuda.synchronize()
+        res = [o.view(torch.int16).cpu().numpy() for o in outs]
+        lc.close()
+        return res
+
+    assert all(np.array_equal(a, b) for a, b in zip(run(True), run(False)))
