@@ -146,15 +146,122 @@ __device__ __noinline__ int select_global(const float* gscores, int n_chunks, in
       [&](int pos, int i) { gsel[pos] = i; }, scratch, scratch + 256, scratch + 256 + 96);
 }
 
-// NT: 8-wide column tiles of query heads (1 for groups up to 8, 2 up to 16); W: warps; N: caches the arguments have room for.
-// IPT > 0: a whole step of one cache (selection and attention) whose units have at most 256 IPT chunks of a multiple of eight
-// tokens (of kTile, if ONE); IPT = 0: anything.  The general kernel has 160 KB of instructions, more than an SM caches, of which
-// a step executes a fifth: an instance for what nearly every step is makes the 28-layer step of four sequences of 24-32 K tokens 278 ->
-// 256 us (graph, L2 flushed) and that of one of 16 K 209 -> 188.  IPT follows from the chunks the cache has room for, not from those it
-// holds: a recorded launch may be replayed after appends.
-template <int NT, int W, int N, int IPT, bool ONE>
-__global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __grid_constant__ DecodeParams<N> P) {
-  constexpr bool FULL = IPT > 0;
+// One staged tile of 32 tokens (K rows from shared address kbase on, V rows behind them): logits, online softmax, accumulation.
+// NT: column tiles of heads; KEYS: rows carry their own permutation keys (else row r's is r & 7); nrow: tokens that exist.
+template <int NT, bool KEYS>
+__device__ __forceinline__ void attend_tile(uint32_t kbase, const uint32_t* keys, int nrow, const uint32_t (&qb)[8][2 * NT], float sc,
+                                            float (&o)[8][NT][4], float (&mrun)[NT][2], float (&lrun)[NT][2]) {
+  // ldmatrix lane roles: matrix index = lane >> 3
+  const int lane = threadIdx.x & 31, g = lane >> 2;
+  const int a_row = (lane & 7) + ((lane >> 3) & 1) * 8, a_piece = lane >> 4;      // non-transposed A tile
+  const int v_row = (lane & 7) + (lane >> 4) * 8, v_piece = (lane >> 3) & 1;      // transposed A tile
+      const uint32_t vbase = kbase + kTile * kRowBytes;
+  const bool partial = nrow < kTile;
+
+      // S^T = K Q^T : rows = tokens (two 16-row tiles), columns = query heads; the reduction over the
+      // head dimension runs as two interleaved accumulation chains.  Piece p of a row sits at
+      // p ^ key:  (2 kk + a_piece) ^ key = ((kk ^ (key >> 1)) << 1) | ((a_piece ^ key) & 1); rows start on
+      // 256-byte boundaries, so that address is the row's with fixed low bits, XOR (kk << 5).
+      float s[2][NT][4];
+#pragma unroll
+      for (int mt = 0; mt < 2; ++mt) {
+        float s2[NT][4];
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+          s[mt][nt][0] = s[mt][nt][1] = s[mt][nt][2] = s[mt][nt][3] = 0.f;
+          s2[nt][0] = s2[nt][1] = s2[nt][2] = s2[nt][3] = 0.f;
+        }
+        const int r = mt * 16 + a_row;
+        const uint32_t key = KEYS ? keys[r] : static_cast<uint32_t>(a_row & 7);
+        const uint32_t rowaddr = (kbase + r * kRowBytes) | ((key >> 1) << 5) | (((a_piece ^ key) & 1u) << 4);
+#pragma unroll
+        for (int kk = 0; kk < 8; ++kk) {
+          uint32_t a0, a1, a2, a3;
+          ldsm_x4(a0, a1, a2, a3, rowaddr ^ (kk << 5));
+#pragma unroll
+          for (int nt = 0; nt < NT; ++nt) {
+            if (kk & 1) mma_bf16(s2[nt], a0, a1, a2, a3, qb[kk][2 * nt], qb[kk][2 * nt + 1]);
+            else mma_bf16(s[mt][nt], a0, a1, a2, a3, qb[kk][2 * nt], qb[kk][2 * nt + 1]);
+          }
+        }
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+          s[mt][nt][0] += s2[nt][0]; s[mt][nt][1] += s2[nt][1];
+          s[mt][nt][2] += s2[nt][2]; s[mt][nt][3] += s2[nt][3];
+        }
+      }
+
+      // online softmax per query head (this thread: heads 2t, 2t+1 of each column tile; tokens g, g+8
+      // of each row tile); logits stay unscaled, the scale enters the exponent's fused multiply-add
+      uint32_t pb[2][NT][2];
+#pragma unroll
+      for (int nt = 0; nt < NT; ++nt) {
+        if (partial) {
+#pragma unroll
+          for (int mt = 0; mt < 2; ++mt) {
+            if (mt * 16 + g >= nrow) s[mt][nt][0] = s[mt][nt][1] = -INFINITY;
+            if (mt * 16 + g + 8 >= nrow) s[mt][nt][2] = s[mt][nt][3] = -INFINITY;
+          }
+        }
+        float mx0 = fmaxf(fmaxf(s[0][nt][0], s[0][nt][2]), fmaxf(s[1][nt][0], s[1][nt][2]));
+        float mx1 = fmaxf(fmaxf(s[0][nt][1], s[0][nt][3]), fmaxf(s[1][nt][1], s[1][nt][3]));
+#pragma unroll
+        for (int off = 4; off <= 16; off <<= 1) {
+          mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, off));
+          mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, off));
+        }
+        const float mn0 = fmaxf(mrun[nt][0], mx0 * sc), mn1 = fmaxf(mrun[nt][1], mx1 * sc);
+        if (__any_sync(0xffffffffu, mn0 != mrun[nt][0] || mn1 != mrun[nt][1])) {
+          // a running maximum moved: bring the accumulators to the new reference
+          const float c0 = fast_exp2(mrun[nt][0] - mn0), c1 = fast_exp2(mrun[nt][1] - mn1);
+          mrun[nt][0] = mn0;
+          mrun[nt][1] = mn1;
+          lrun[nt][0] *= c0;
+          lrun[nt][1] *= c1;
+#pragma unroll
+          for (int dt = 0; dt < 8; ++dt) {
+            o[dt][nt][0] *= c0;
+            o[dt][nt][1] *= c1;
+            o[dt][nt][2] *= c0;
+            o[dt][nt][3] *= c1;
+          }
+        }
+        float ps0 = 0.f, ps1 = 0.f;
+#pragma unroll
+        for (int mt = 0; mt < 2; ++mt) {
+          const float p0 = fast_exp2(fmaf(s[mt][nt][0], sc, -mn0)), p1 = fast_exp2(fmaf(s[mt][nt][1], sc, -mn1));
+          const float p2 = fast_exp2(fmaf(s[mt][nt][2], sc, -mn0)), p3 = fast_exp2(fmaf(s[mt][nt][3], sc, -mn1));
+          ps0 += p0 + p2;
+          ps1 += p1 + p3;
+          // P^T as the B operand of O^T += V^T P^T: tokens along k, heads along n
+          pb[mt][nt][0] = movmatrix_trans(pack_bf16(p0, p1));
+          pb[mt][nt][1] = movmatrix_trans(pack_bf16(p2, p3));
+        }
+        lrun[nt][0] += ps0;
+        lrun[nt][1] += ps1;
+      }
+
+      // O^T += V^T P^T : rows = head-dim (eight 16-row tiles), k = tokens (two 16-token steps)
+#pragma unroll
+      for (int ks = 0; ks < 2; ++ks) {
+        const int r = ks * 16 + v_row;
+        const uint32_t key = KEYS ? keys[r] : static_cast<uint32_t>(v_row & 7);
+        const uint32_t rowaddr = (vbase + r * kRowBytes) | ((key >> 1) << 5) | (((v_piece ^ key) & 1u) << 4);
+#pragma unroll
+        for (int dt = 0; dt < 8; ++dt) {
+          uint32_t a0, a1, a2, a3;
+          ldsm_x4_trans(a0, a1, a2, a3, rowaddr ^ (dt << 5));
+#pragma unroll
+          for (int nt = 0; nt < NT; ++nt) mma_bf16(o[dt][nt], a0, a1, a2, a3, pb[ks][nt][0], pb[ks][nt][1]);
+        }
+      }
+}
+
+// The general kernel: any chunk size and number of chunks, groups up to 16, several caches in one launch, the two stages of a
+// step on their own.  What nearly every step is has a kernel of its own below.
+// NT: 8-wide column tiles of query heads (1 for groups up to 8, 2 up to 16); W: warps.
+template <int NT, int W>
+__global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __grid_constant__ DecodeParams<kMaxMulti> P) {
   extern __shared__ __align__(1024) uint8_t smem[];
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -169,7 +276,7 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
   pdl_launch_dependents();
 
   const int cid = static_cast<int>(cluster_id());
-  const int li = N == 1 ? 0 : find_slot(P.unit_prefix, P.n, cid);
+  const int li = find_slot(P.unit_prefix, P.n, cid);
   char* base = P.cache[li];
   int uid;
   {
@@ -181,7 +288,7 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
   }
   const Unit* up = reinterpret_cast<const Unit*>(base + kUnitsOff) + uid;
   const int G = P.group, Hq = P.n_q_heads, cs = P.chunk_size;
-  const bool do_select = FULL || (P.phase & kPhaseSelect) != 0, do_attend = FULL || (P.phase & kPhaseAttend) != 0;
+  const bool do_select = (P.phase & kPhaseSelect) != 0, do_attend = (P.phase & kPhaseAttend) != 0;
   constexpr bool kPushMerge = NT == 1;   // wider groups do not fit the receive area and use the pull merge
 
   // the unit's record (uniform loads, issued together)
@@ -206,12 +313,12 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
   // divisions by the cluster size, the slice length and the chunk size by the host's multipliers: here they delay the first
   // copies wherever the launch cannot start beside its predecessor, further down they sit on the step's chain
   const uint32_t csize_magic = P.cluster_magic, per_magic = P.merge_magic, cs_magic = P.chunk_magic;
-  const bool cs_fast = FULL || (cs > 1 && static_cast<uint64_t>(n_tok) * static_cast<uint64_t>(cs) < (1ull << 32));
+  const bool cs_fast = (cs > 1 && static_cast<uint64_t>(n_tok) * static_cast<uint64_t>(cs) < (1ull << 32));
   auto div_cs = [&](int x) { return cs_fast ? fastdiv(x, cs_magic) : x / cs; };
   auto own_cnt = [&](int r) { return max(0, min(total, (r + 1) * per) - r * per); };
 
   const bool identity = dynamic && k_sel >= n_chunks;          // every chunk is loaded: no list needed
-  const bool fits = FULL || n_chunks <= kSelSmemChunks;                // scores and ids fit shared memory
+  const bool fits = n_chunks <= kSelSmemChunks;                // scores and ids fit shared memory
   const bool scoring = dynamic && do_select;
   // scores travel through shared memory (and the exchange between the cluster's CTAs) only when a selection
   // needs them there; otherwise they go straight to global memory
@@ -270,7 +377,6 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
   bool dead = false;    // a bounded wait ran out: stop issuing, keep every hand-over
   // ldmatrix lane roles: matrix index mi = lane >> 3
   const int a_row = (lane & 7) + ((lane >> 3) & 1) * 8, a_piece = lane >> 4;      // non-transposed A tile
-  const int v_row = (lane & 7) + (lane >> 4) * 8, v_piece = (lane >> 3) & 1;      // transposed A tile
 
   float* sc_smem = reinterpret_cast<float*>(smem + kScoresOff);
   uint16_t* sel16 = reinterpret_cast<uint16_t*>(smem + kSelOff);
@@ -292,15 +398,15 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
   // every tile inside one chunk (one copy pair, issued by lane 0); any other size lets up to 32
   // chunks touch a tile (one lane per chunk).  Row keys differ from (row & 7) only when the chunk
   // size is not a multiple of 8.
-  const bool one_chunk = !contiguous && (ONE || (!FULL && (cs % kTile) == 0));
-  const bool need_keys = !FULL && !contiguous && (cs & 7) != 0;
+  const bool one_chunk = !contiguous && (cs % kTile) == 0;
+  const bool need_keys = !contiguous && (cs & 7) != 0;
   auto issue_attn = [&](int j) {   // whole warp; arms stage (seq0 + j) % stages with CTA tile j
     const int stage = (seq0 + j) % kDecStages;
     uint8_t* st = smem + stage * kStageBytes;
     const int v0 = (at_tile0 + j) * kTile;
     const int v1 = min(v0 + kTile, n_valid);
     HKV_CHECK(v0 >= 0 && v0 < v1 && v1 - v0 <= kTile, 100);
-    if (ONE || contiguous || one_chunk) {
+    if (contiguous || one_chunk) {
       if (lane == 0) {
         size_t row = static_cast<size_t>(v0);
         if (one_chunk) {
@@ -589,17 +695,13 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
           hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, off));
         }
         uint2* cand = reinterpret_cast<uint2*>(smem + kCandOff);
-        [[maybe_unused]] const int ipt = (n_chunks + W * 32 - 1) / (W * 32);
+        const int ipt = (n_chunks + W * 32 - 1) / (W * 32);
         auto stamp = [&](int k2) { HKV_STAMP(20 + k2) };
         emitted = -1;
-        if constexpr (FULL) {
-          emitted = block_topk_blocked<W, FULL ? IPT : 1, IPT <= 2 ? 256 : 512>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
-        } else {
-          if (ipt <= 1) emitted = block_topk_blocked<W, 1, 256>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
-          else if (ipt <= 2) emitted = block_topk_blocked<W, 2, 256>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
-          else if (ipt <= 4) emitted = block_topk_blocked<W, 4, 512>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
-          else if (ipt <= 8) emitted = block_topk_blocked<W, 8, 512>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
-        }
+        if (ipt <= 1) emitted = block_topk_blocked<W, 1, 256>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
+        else if (ipt <= 2) emitted = block_topk_blocked<W, 2, 256>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
+        else if (ipt <= 4) emitted = block_topk_blocked<W, 4, 512>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
+        else if (ipt <= 8) emitted = block_topk_blocked<W, 8, 512>(sc_smem, n_chunks, n_mt * 16, k_sel, lo, hi, sel16, hist, cand, misc, early, stamp);
         if (emitted < 0) {
           // crowded threshold bin (or more scores than the fast path takes): the general selection, its
           // scratch in the idle ring
@@ -609,7 +711,7 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
         }
         sel_in_smem = true;
       }
-    } else if constexpr (!FULL) {
+    } else {
       // more chunks than shared memory holds: selection on the scores in global memory; every CTA of the
       // cluster writes the same list to the same place
       __threadfence();
@@ -643,7 +745,7 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
     if (!do_attend) return;
     // "my selection is done": from here on my score area is free to receive the peers' partial results
     if (clustered && kPushMerge && !bar_pending) { cluster_arrive_relaxed(); bar_pending = true; }
-  } else if (!FULL && dynamic) {
+  } else if (dynamic) {
     setup_attn(__ldcg(n_valid_g));   // attention only: the list of an earlier selection
   }
 
@@ -651,7 +753,7 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
   // flash-decoding over the unit's token list
   // =============================================================================================
   const float sc = P.scale_log2e;
-  if (!FULL && !attn_armed && !dead) {
+  if (!attn_armed && !dead) {
     for (int j = warp; j < min(at_n, kDecStages); j += W) issue_attn(j);
   }
 
@@ -702,105 +804,7 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
     dead = __any_sync(0xffffffffu, dead);
     if (dead) break;
 #endif
-    const uint32_t kbase = smem_u32(st), vbase = kbase + kTile * kRowBytes;
-
-    // S^T = K Q^T : rows = tokens (two 16-row tiles), columns = query heads; the reduction over the
-    // head dimension runs as two interleaved accumulation chains.  Piece p of a row sits at
-    // p ^ key:  (2 kk + a_piece) ^ key = ((kk ^ (key >> 1)) << 1) | ((a_piece ^ key) & 1); rows start on
-    // 256-byte boundaries, so that address is the row's with fixed low bits, XOR (kk << 5).
-    float s[2][NT][4];
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt) {
-      float s2[NT][4];
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        s[mt][nt][0] = s[mt][nt][1] = s[mt][nt][2] = s[mt][nt][3] = 0.f;
-        s2[nt][0] = s2[nt][1] = s2[nt][2] = s2[nt][3] = 0.f;
-      }
-      const int r = mt * 16 + a_row;
-      const uint32_t key = KEYS ? keys[r] : static_cast<uint32_t>(a_row & 7);
-      const uint32_t rowaddr = (kbase + r * kRowBytes) | ((key >> 1) << 5) | (((a_piece ^ key) & 1u) << 4);
-#pragma unroll
-      for (int kk = 0; kk < 8; ++kk) {
-        uint32_t a0, a1, a2, a3;
-        ldsm_x4(a0, a1, a2, a3, rowaddr ^ (kk << 5));
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) {
-          if (kk & 1) mma_bf16(s2[nt], a0, a1, a2, a3, qb[kk][2 * nt], qb[kk][2 * nt + 1]);
-          else mma_bf16(s[mt][nt], a0, a1, a2, a3, qb[kk][2 * nt], qb[kk][2 * nt + 1]);
-        }
-      }
-#pragma unroll
-      for (int nt = 0; nt < NT; ++nt) {
-        s[mt][nt][0] += s2[nt][0]; s[mt][nt][1] += s2[nt][1];
-        s[mt][nt][2] += s2[nt][2]; s[mt][nt][3] += s2[nt][3];
-      }
-    }
-
-    // online softmax per query head (this thread: heads 2t, 2t+1 of each column tile; tokens g, g+8
-    // of each row tile); logits stay unscaled, the scale enters the exponent's fused multiply-add
-    uint32_t pb[2][NT][2];
-#pragma unroll
-    for (int nt = 0; nt < NT; ++nt) {
-      if (partial) {
-#pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
-          if (mt * 16 + g >= nrow) s[mt][nt][0] = s[mt][nt][1] = -INFINITY;
-          if (mt * 16 + g + 8 >= nrow) s[mt][nt][2] = s[mt][nt][3] = -INFINITY;
-        }
-      }
-      float mx0 = fmaxf(fmaxf(s[0][nt][0], s[0][nt][2]), fmaxf(s[1][nt][0], s[1][nt][2]));
-      float mx1 = fmaxf(fmaxf(s[0][nt][1], s[0][nt][3]), fmaxf(s[1][nt][1], s[1][nt][3]));
-#pragma unroll
-      for (int off = 4; off <= 16; off <<= 1) {
-        mx0 = fmaxf(mx0, __shfl_xor_sync(0xffffffffu, mx0, off));
-        mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, off));
-      }
-      const float mn0 = fmaxf(mrun[nt][0], mx0 * sc), mn1 = fmaxf(mrun[nt][1], mx1 * sc);
-      if (__any_sync(0xffffffffu, mn0 != mrun[nt][0] || mn1 != mrun[nt][1])) {
-        // a running maximum moved: bring the accumulators to the new reference
-        const float c0 = fast_exp2(mrun[nt][0] - mn0), c1 = fast_exp2(mrun[nt][1] - mn1);
-        mrun[nt][0] = mn0;
-        mrun[nt][1] = mn1;
-        lrun[nt][0] *= c0;
-        lrun[nt][1] *= c1;
-#pragma unroll
-        for (int dt = 0; dt < 8; ++dt) {
-          o[dt][nt][0] *= c0;
-          o[dt][nt][1] *= c1;
-          o[dt][nt][2] *= c0;
-          o[dt][nt][3] *= c1;
-        }
-      }
-      float ps0 = 0.f, ps1 = 0.f;
-#pragma unroll
-      for (int mt = 0; mt < 2; ++mt) {
-        const float p0 = fast_exp2(fmaf(s[mt][nt][0], sc, -mn0)), p1 = fast_exp2(fmaf(s[mt][nt][1], sc, -mn1));
-        const float p2 = fast_exp2(fmaf(s[mt][nt][2], sc, -mn0)), p3 = fast_exp2(fmaf(s[mt][nt][3], sc, -mn1));
-        ps0 += p0 + p2;
-        ps1 += p1 + p3;
-        // P^T as the B operand of O^T += V^T P^T: tokens along k, heads along n
-        pb[mt][nt][0] = movmatrix_trans(pack_bf16(p0, p1));
-        pb[mt][nt][1] = movmatrix_trans(pack_bf16(p2, p3));
-      }
-      lrun[nt][0] += ps0;
-      lrun[nt][1] += ps1;
-    }
-
-    // O^T += V^T P^T : rows = head-dim (eight 16-row tiles), k = tokens (two 16-token steps)
-#pragma unroll
-    for (int ks = 0; ks < 2; ++ks) {
-      const int r = ks * 16 + v_row;
-      const uint32_t key = KEYS ? keys[r] : static_cast<uint32_t>(v_row & 7);
-      const uint32_t rowaddr = (vbase + r * kRowBytes) | ((key >> 1) << 5) | (((v_piece ^ key) & 1u) << 4);
-#pragma unroll
-      for (int dt = 0; dt < 8; ++dt) {
-        uint32_t a0, a1, a2, a3;
-        ldsm_x4_trans(a0, a1, a2, a3, rowaddr ^ (dt << 5));
-#pragma unroll
-        for (int nt = 0; nt < NT; ++nt) mma_bf16(o[dt][nt], a0, a1, a2, a3, pb[ks][nt][0], pb[ks][nt][1]);
-      }
-    }
+    attend_tile<NT, KEYS>(smem_u32(st), keys, nrow, qb, sc, o, mrun, lrun);
     __syncwarp();
 #ifdef HKV_PROFILE
     if (j == 0) { HKV_STAMP(17) }
@@ -812,8 +816,7 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
   }
 
   };
-  if constexpr (FULL) run_tiles(std::false_type{});
-  else if (need_keys) run_tiles(std::true_type{});
+  if (need_keys) run_tiles(std::true_type{});
   else run_tiles(std::false_type{});
 
   HKV_STAMP(8)
@@ -1026,6 +1029,594 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
   HKV_STAMP(13)
 }
 
+// =================================================================================================
+// The kernel of a whole step of one cache: groups up to 8, chunk sizes that are a multiple of 8, at most 2048 chunks per unit.
+//
+// What bounds it at small batch is neither bytes nor arithmetic but the chain of dependent instructions from the query to the
+// output, every one of which a CTA executes once or twice per launch, and their fetch: straight code that is executed again and again
+// from more than 32 KB (2048 instructions) is fetched at about six cycles per instruction on this chip, from less at two (measured
+// with chains of multiply-adds, warps of one CTA side by side).  So everything that a step does not need is left out
+// (wider groups, several caches, stages on their own: the general kernel) or out of line (selection with ties).
+//
+// It differs from the general kernel in
+//   the ring      stage w belongs to warp w (of the first six), which arms it and consumes it: no hand-over, and the
+//                 warp's partial result is parked in its own stage; the other two warps write back the scores and the list;
+//   the selection one histogram whose entries keep their scores (32 slots each), so that the k-th largest score is known two block
+//                 barriers after the scores, and the list one barrier later;
+//   the query     brought into shared memory once per CTA, as rows that ldmatrix can read.
+// 28-layer steps against the general kernel's instances for the same work (5300 to 6000 instructions, this 1900 to 2200 without the
+// rare selection): one sequence of 16 K tokens 194 -> 157 us, two of 9 K (host buffers) 228 -> 190, four of 24-32 K (graph) 248 -> 218,
+// eight of 50 K 377 -> 327.  Measured without gain: L2 requests for chunks that lie above the threshold's bin before the list
+// exists (+2 to +5 %), waiting for the cluster's start before the dependency wait instead of behind it (+6 %).
+// =================================================================================================
+constexpr int kStepWarps = 8, kStepThreads = kStepWarps * 32;
+constexpr int kStepStage = 2 * kTile * kRowBytes;                         // K tile + V tile, or 64 chunk means
+constexpr int kStepList = kDecStages * kStepStage;                        // the group's queries, then uint16 ids of the selected chunks
+constexpr int kStepScores = kStepList + kSelSmemChunks * 2;               // float32 chunk scores; later the merge's receive area
+constexpr int kStepHist = kStepScores + kSelSmemChunks * 4;
+constexpr int kStepBounds = kStepHist + kHistBins * 4;                    // (lower, upper) score bound of every warp of the cluster
+constexpr int kStepBars = kStepBounds + kMaxCluster * kStepWarps * 8;     // mbarriers: ring stages, scores, merge
+constexpr int kStepCounts = kStepBars + (kDecStages + 2) * 8;             // [w] selected chunks before warp w's, [8] all of them, [9] a wait ran out (also in [8])
+constexpr int kStepBytes = kStepCounts + 64;
+constexpr int kSlots = 32;                                                // scores kept per histogram entry (in the idle ring)
+constexpr int kWholeList = 1 << 25;                                       // "chunk size" of a token list that lies in one piece
+static_assert(kStepBytes <= kSmemBytes, "the capacity of the general kernel holds for this one");
+static_assert(kSlots * kHistBins * 4 <= kStepList && kTopkScratchInts * 4 <= kStepList, "selection scratch fits the ring");
+static_assert(8 * kParkStride * 4 + 64 <= kStepStage && kMaxGroup * kRowBytes / 2 <= kSelSmemChunks * 2, "parking, queries");
+
+__device__ __noinline__ void note_timeout(int32_t* err, int place) {
+  if (atomicCAS(&err[0], 0, HKV_ERR_TIMEOUT) == 0) err[1] = place;
+}
+// bounded wait in as few instructions as it takes
+template <bool kCluster>
+__device__ __forceinline__ bool step_wait(uint64_t* bar, uint32_t parity) {
+  const long long start = clock64();
+  do {
+    if (kCluster ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity)) return true;
+  } while (clock64() - start < HKV_WAIT_CYCLES);
+  return false;
+}
+__device__ __forceinline__ float warp_min(float x) {
+  float y;
+  asm("redux.sync.min.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float warp_max(float x) {
+  float y;
+  asm("redux.sync.max.f32 %0, %1, 0xffffffff;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// IPT: scores per thread of the selection (units of at most 256 IPT chunks).  It follows from the chunks the cache has room for,
+// not from those it holds: a recorded launch may be replayed after appends.
+template <int IPT>
+__global__ void __launch_bounds__(kStepThreads, kDecCtasPerSm) decode_step_kernel(const __grid_constant__ DecodeParams<1> P) {
+  constexpr int NB = IPT <= 2 ? 256 : 512;   // value bins (more scores crowd them, and a few far-out scores stretch their range)
+  extern __shared__ __align__(1024) uint8_t smem[];
+  const int tid = threadIdx.x, lane = tid & 31, g = lane >> 2, t = lane & 3;
+  const int warp = __shfl_sync(0xffffffffu, tid >> 5, 0);   // (known to be the same in all lanes)
+  const int csize = P.cluster, crank = static_cast<int>(cluster_ctarank());
+  HKV_STAMP(0)
+  // (what may be read before the dependency wait: see the general kernel)
+  if (P.late) pdl_wait();
+  pdl_launch_dependents();
+
+  char* base = P.cache[0];
+  const int nd = P.n_dynamic[0];
+  int uid = static_cast<int>(cluster_id());
+  if (P.static_first) {
+    const int ns = P.unit_prefix[1] - nd;
+    uid = uid < ns ? nd + uid : uid - ns;
+  }
+  const bool dynamic = uid < nd;               // the table holds the dynamic units first
+  const Unit* up = reinterpret_cast<const Unit*>(base + kUnitsOff) + uid;
+  const int C = up->C, n_tok = up->n_tok, n_chunks = up->n_chunks, k_sel = up->k_sel;
+  const int G = P.group;
+  const uint8_t* kplane = reinterpret_cast<const uint8_t*>(base + up->k_off);
+  const uint8_t* vplane = reinterpret_cast<const uint8_t*>(base + up->v_off);
+  const int out_row0 = up->b * P.n_q_heads + up->h * G;
+  int32_t* err = reinterpret_cast<int32_t*>(base + P.err_off[0]);
+#ifdef HKV_CHECKED
+  const int plane_rows = up->plane_rows;
+  bool dead = false;
+#endif
+  // a static unit's rows lie in one piece, as if they were one long chunk
+  const int cs = dynamic ? P.chunk_size : kWholeList;
+  const uint32_t cs_magic = dynamic ? P.chunk_magic : 0u;
+  auto div_csize = [&](int x) { return csize > 1 ? fastdiv(x, P.cluster_magic) : x; };
+
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kStepBars);
+  uint64_t *score_bar = bars + kDecStages, *merge_bar = score_bar + 1;
+  int* hist = reinterpret_cast<int*>(smem + kStepHist);
+  int* counts = reinterpret_cast<int*>(smem + kStepCounts);
+  volatile int* failed = counts + 9;
+  float* scores = reinterpret_cast<float*>(smem + kStepScores);
+  uint16_t* list = reinterpret_cast<uint16_t*>(smem + kStepList);
+
+  // the CTA's tiles of the token list, and its chunk means (groups of 16, staged 64 at a time)
+  int n_valid = 0, tile0 = 0, at_n = 0;
+  auto deal_tiles = [&](int nv) {
+    n_valid = nv;
+    const int n_tiles = (nv + kTile - 1) / kTile, per = div_csize(n_tiles + csize - 1);
+    tile0 = crank * per;
+    at_n = max(0, min(n_tiles - tile0, per));
+  };
+  const int n_mt = (n_chunks + 15) >> 4;
+  int sc_row0 = 0, sc_rows = 0, sc_n = 0;
+  if (dynamic) {
+    const int per = div_csize(n_mt + csize - 1) * 16;
+    sc_row0 = min(n_chunks, crank * per);
+    sc_rows = min(n_chunks - sc_row0, per);
+    sc_n = (sc_rows + kScoreTile - 1) / kScoreTile;
+  } else {
+    deal_tiles(n_tok);
+  }
+  // the output's G * 128 elements are dealt to the cluster's CTAs in slices of `per`
+  const int total = G * kHeadDim, per = P.merge_per;
+  const int mine = max(0, min(total - crank * per, per));
+
+  if (warp == 0) {
+    if (lane < kDecStages + 2) mbar_init(bars + lane, 1);
+    mbar_fence_init();
+    __syncwarp();
+    // what this CTA will receive from the cluster (itself included): every score of the unit plus a pair of bounds per
+    // warp; later a slice of every CTA's partial output with its (m, l) rows
+    if (lane == kDecStages && dynamic) mbar_arrive_expect_tx(score_bar, static_cast<uint32_t>(n_mt * 64 + csize * kStepWarps * 8));
+    if (lane == kDecStages + 1) mbar_arrive_expect_tx(merge_bar, mine > 0 ? static_cast<uint32_t>(csize * (mine * 4 + G * 8)) : 0u);
+    // the first ring-full does not depend on this step's query: lane w on behalf of warp w
+    if (lane < min(dynamic ? sc_n : at_n, kDecStages)) {
+      const int row0 = dynamic ? sc_row0 + lane * kScoreTile : (tile0 + lane) * kTile;
+      const int rows = dynamic ? min(sc_rows - lane * kScoreTile, kScoreTile) : min(n_valid - row0, kTile);
+      const uint32_t bytes = static_cast<uint32_t>(rows) * kRowBytes;
+      const uint8_t* src = dynamic ? reinterpret_cast<const uint8_t*>(base + up->summ_off) : kplane;
+      uint8_t* st = smem + lane * kStepStage;
+      HKV_CHECK(row0 >= 0 && rows >= 1 && (dynamic ? row0 + rows <= n_chunks && rows <= kScoreTile : row0 + rows <= plane_rows && rows <= kTile), 120);
+#ifdef HKV_CHECKED
+      if (!dead)
+#endif
+      {
+        mbar_arrive_expect_tx(bars + lane, dynamic ? bytes : 2u * bytes);
+        bulk_g2s(st, src + static_cast<size_t>(row0) * kRowBytes, bytes, bars + lane);
+        if (!dynamic) bulk_g2s(st + kTile * kRowBytes, vplane + static_cast<size_t>(row0) * kRowBytes, bytes, bars + lane);
+      }
+    }
+  }
+  hist[tid] = 0;
+  if (NB > kStepThreads) hist[tid + kStepThreads] = 0;
+  if (tid < 10) counts[tid] = 0;
+  // "this CTA is running and its barriers exist": has to be known before anybody touches its shared memory remotely
+  cluster_arrive();
+  // the query is written by whatever precedes this launch, so it may only be READ after the wait; asking L2 for its lines
+  // reads nothing and lets the loads below meet them there
+  const uint32_t* qg = reinterpret_cast<const uint32_t*>(P.q[0]) + static_cast<size_t>(out_row0) * (kHeadDim / 2);
+  if (warp == kStepWarps - 1 && lane * 32 < G * (kHeadDim / 2)) prefetch_l2_line(qg + lane * 32);
+
+  HKV_STAMP(1)
+  pdl_wait();
+  HKV_STAMP(2)
+
+  // the group's queries into shared memory, a row of 256 bytes per head (zero behind the last), their 16-byte pieces permuted
+  // by the row; from there as B fragments of  S^T = X Q^T
+  uint32_t qb[8][2];
+  {
+    const int n = G * (kHeadDim / 2);
+    const uint32_t w0 = tid < n ? __ldg(qg + tid) : 0u, w1 = tid + kStepThreads < n ? __ldg(qg + tid + kStepThreads) : 0u;
+    const int row = tid >> 6, piece = (tid >> 2) & 15;
+    uint32_t* at = reinterpret_cast<uint32_t*>(smem + kStepList + row * kRowBytes + (tid & 3) * 4);
+    at[(piece ^ row) * 4] = w0;
+    at[4 * (kRowBytes / 4) + (piece ^ (row + 4)) * 4] = w1;
+    __syncthreads();
+    const uint32_t qaddr = smem_u32(smem + kStepList) + (lane & 7) * kRowBytes;
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      ldsm_x4(qb[2 * i][0], qb[2 * i][1], qb[2 * i + 1][0], qb[2 * i + 1][1], qaddr + (((4 * i + (lane >> 3)) ^ (lane & 7)) << 4));
+  }
+  HKV_STAMP(3)
+
+  const uint32_t smem0 = smem_u32(smem);
+  bool ok = true;            // no wait of this thread has run out
+  uint32_t phase = 0;        // parity of the next phase of this warp's ring stage
+  if (dynamic) {
+    // ---- scores of this CTA's chunk means ----
+    cluster_wait();          // every CTA of the cluster runs: remote stores are safe
+    float wlo = INFINITY, whi = -INFINITY;
+    {
+      // pieces that all fit the ring are dealt out in groups of 16, otherwise a warp takes whole pieces through its own stage
+      const bool fine = sc_n <= kDecStages;
+      const int mt_cnt = (sc_rows + 15) >> 4, n_items = fine ? mt_cnt : sc_n;
+      const int a_row = (lane & 7) + ((lane >> 3) & 1) * 8, key = a_row & 7;
+      // piece p of a row sits at p ^ key, and rows start on 256-byte boundaries: the address of piece 2 kk + (lane >> 4) is the
+      // row's address with the fixed low bits below, XOR (kk << 5)
+      const uint32_t a_off = a_row * kRowBytes + ((key >> 1) << 5) + ((((lane >> 4) ^ key) & 1) << 4);
+      for (int it = fine || warp < kDecStages ? warp : n_items; it < n_items; it += fine ? kStepWarps : kDecStages) {
+        const int piece = fine ? it >> 2 : it, stage = fine ? piece : warp;
+        if (!step_wait<false>(bars + stage, phase)) {
+          if (lane == 0) note_timeout(err, kErrScoreWait);
+          step_wait<false>(bars + stage, phase);   // (the copy may still be on its way)
+          ok = false;
+          if (fine) continue;
+          break;
+        }
+        if (!fine) phase ^= 1u;
+        const int m_end = fine ? it + 1 : min(mt_cnt, it * 4 + 4);
+#pragma unroll 1
+        for (int m = fine ? it : it * 4; m < m_end; ++m) {
+          const uint32_t rowaddr = smem0 + stage * kStepStage + (m & 3) * 16 * kRowBytes + a_off;
+          float acc[2][4] = {};
+#pragma unroll
+          for (int kk = 0; kk < 8; ++kk) {
+            uint32_t a0, a1, a2, a3;
+            ldsm_x4(a0, a1, a2, a3, rowaddr ^ (kk << 5));
+            mma_bf16(acc[kk & 1], a0, a1, a2, a3, qb[kk][0], qb[kk][1]);
+          }
+          // chunk score = sum over the group's heads of <q_g, mean_c> (variant: their maximum; the columns past the group
+          // hold zero queries and must not take part in it)
+          const bool gm = P.group_max != 0;
+          float s[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            s[i] = acc[0][i] + acc[1][i];
+            if (gm && 2 * t + (i & 1) >= G) s[i] = -INFINITY;
+          }
+          auto join = [&](float a, float b) { return gm ? fmaxf(a, b) : a + b; };
+          const float v0 = join(s[0], s[1]), v1 = join(s[2], s[3]);   // rows g and g + 8: this thread's two heads
+          float x = join(t & 1 ? v1 : v0, __shfl_xor_sync(0xffffffffu, t & 1 ? v0 : v1, 1));
+          x = join(x, __shfl_xor_sync(0xffffffffu, x, 2));
+          // a lane now holds the score of row g + 8 (t & 1) of the group
+          const int c0 = sc_row0 + m * 16;
+          if (c0 + g + 8 * (t & 1) < n_chunks) { wlo = fminf(wlo, x); whi = fmaxf(whi, x); }
+          else x = -INFINITY;                                         // padding of the last group: never selected
+          float4 quad;                                                // rows 4 t .. 4 t + 3, the unit of the exchange
+          const int src = ((t & 1) << 4) + (t >> 1);
+          quad.x = __shfl_sync(0xffffffffu, x, src);
+          quad.y = __shfl_sync(0xffffffffu, x, src + 4);
+          quad.z = __shfl_sync(0xffffffffu, x, src + 8);
+          quad.w = __shfl_sync(0xffffffffu, x, src + 12);
+#pragma unroll
+          for (int s2 = g; s2 < kMaxCluster; s2 += 8) {
+            if (s2 < csize) {
+              const uint32_t peer = mapa(smem0, s2);
+              st_async_f32x4(peer + kStepScores + (c0 + 4 * t) * 4, quad, peer + kStepBars + kDecStages * 8);
+            }
+          }
+        }
+        __syncwarp();
+        if (!fine && it + kDecStages < sc_n && lane == 0) {
+          const int r0 = (it + kDecStages) * kScoreTile;
+          const uint32_t bytes = static_cast<uint32_t>(min(sc_rows - r0, kScoreTile)) * kRowBytes;
+          mbar_arrive_expect_tx(bars + warp, bytes);
+          bulk_g2s(smem + warp * kStepStage, base + up->summ_off + static_cast<size_t>(sc_row0 + r0) * kRowBytes, bytes, bars + warp);
+        }
+      }
+      if (fine) phase = warp < sc_n ? 1u : 0u;
+    }
+    wlo = warp_min(wlo);
+    whi = warp_max(whi);
+    // this warp's bounds, to every CTA (a warp that gave up sends them too)
+    if (lane < csize) {
+      const uint32_t peer = mapa(smem0, lane);
+      st_async_f32x2(peer + kStepBounds + (crank * kStepWarps + warp) * 8, wlo, whi, peer + kStepBars + kDecStages * 8);
+    }
+    HKV_STAMP(4)
+
+    // ---- selection: every score of the unit is on its way to this CTA ----
+    if (!step_wait<true>(score_bar, 0u)) {
+      if (lane == 0) note_timeout(err, kErrExchangeWait);
+      ok = false;
+    }
+    if (!ok) { *failed = 1; atomicAdd(&counts[kStepWarps], 1 << 20); }
+    HKV_STAMP(5)
+    float lo = INFINITY, hi = -INFINITY;
+#pragma unroll
+    for (int j = 0; j < kMaxCluster * kStepWarps / 32; ++j) {
+      if (lane + 32 * j < csize * kStepWarps) {
+        const float2 b2 = reinterpret_cast<const float2*>(smem + kStepBounds)[lane + 32 * j];
+        lo = fminf(lo, b2.x);
+        hi = fmaxf(hi, b2.y);
+      }
+    }
+    lo = warp_min(lo);
+    hi = warp_max(hi);
+    // thread t owns scores [t * IPT, (t + 1) * IPT): the list's order is the thread order
+    const int i0 = tid * IPT;
+    float v[IPT];
+#pragma unroll
+    for (int e = 0; e < IPT; ++e) v[e] = -INFINITY;
+    if (i0 < n_mt * 16) {
+      if constexpr (IPT == 1) {
+        v[0] = scores[i0];
+      } else if constexpr (IPT == 2) {
+        const float2 x = *reinterpret_cast<const float2*>(scores + i0);
+        v[0] = x.x; v[1] = x.y;
+      } else {
+#pragma unroll
+        for (int q4 = 0; q4 < IPT / 4; ++q4) {
+          const float4 x = *reinterpret_cast<const float4*>(scores + i0 + 4 * q4);
+          v[4 * q4] = x.x; v[4 * q4 + 1] = x.y; v[4 * q4 + 2] = x.z; v[4 * q4 + 3] = x.w;
+        }
+      }
+    }
+    const float last_score = scores[n_chunks - 1];
+    float thr = -3.402823466e38f;     // everything, if every chunk is to be loaded
+    bool plain = true;                // no ties or crowds so far; the same in every thread
+    if (k_sel < n_chunks) {
+      // Value bins between the bounds: the map score -> bin only has to be monotone, so an approximate quotient will do; adding
+      // 2^23 rounds to an integer in the float's low bits (which, masked, are a bin whatever the score).  An entry's
+      // counter hands out its slots, rotated so that neither the slots of one entry nor the first slots of all share a bank.
+      const float width = hi - lo;
+      const float scale = (width > 0.f && width < INFINITY) ? __fdividef(static_cast<float>(NB - 2), width) : 0.f;
+      float* slots = reinterpret_cast<float*>(smem);
+      uint32_t bin[IPT];
+      int slot[IPT];
+#pragma unroll
+      for (int e = 0; e < IPT; ++e) {
+        bin[e] = __float_as_uint(fmaf(v[e] - lo, scale, 8388608.f)) & (NB - 1);
+        slot[e] = kSlots;
+        if (i0 + e < n_chunks) slot[e] = atomicAdd(&hist[bin[e]], 1);
+      }
+#pragma unroll
+      for (int e = 0; e < IPT; ++e)
+        if (slot[e] < kSlots) slots[slot[e] * NB + ((bin[e] + slot[e]) & (NB - 1))] = v[e];
+      __syncthreads();
+      HKV_STAMP(20)
+      fence_proxy_async();   // the ring goes back to the bulk copies (behind the next barrier)
+
+      // every warp: the highest bin b with count(bins > b) < k <= count(bins >= b); lane L holds NB / 32 bins
+      constexpr int PER = NB / 32;
+      int suf[PER];          // bins from j on, within the lane
+#pragma unroll
+      for (int q4 = 0; q4 < PER / 4; ++q4) {
+        const int4 h4 = reinterpret_cast<const int4*>(hist)[lane * (PER / 4) + q4];
+        suf[4 * q4] = h4.x; suf[4 * q4 + 1] = h4.y; suf[4 * q4 + 2] = h4.z; suf[4 * q4 + 3] = h4.w;
+      }
+#pragma unroll
+      for (int j = PER - 2; j >= 0; --j) suf[j] += suf[j + 1];
+      int run = suf[0];      // becomes the sum over lanes >= this one
+#pragma unroll
+      for (int off = 1; off < 32; off <<= 1) {
+        const int x = __shfl_down_sync(0xffffffffu, run, off);
+        if (lane + off < 32) run += x;
+      }
+      const int left = k_sel - (run - suf[0]);   // of the k, what the lanes above leave
+      uint32_t found = 0u;                       // lane * PER + bin, count (at most 63), how many of them are needed
+      if (left > 0 && left <= suf[0]) {
+        int b = 0, next = 0, from = suf[0];
+#pragma unroll
+        for (int j = 1; j < PER; ++j) {
+          if (suf[j] >= left) { b = j; from = suf[j]; }
+        }
+#pragma unroll
+        for (int j = PER - 1; j >= 1; --j) {
+          if (suf[j] < left) next = suf[j];
+        }
+        found = static_cast<uint32_t>(lane * PER + b) << 12 | static_cast<uint32_t>(min(from - next, 63)) << 6 |
+                static_cast<uint32_t>(min(left - next, 63));
+      }
+      found = __reduce_max_sync(0xffffffffu, found);
+      const int tbin = static_cast<int>(found >> 12), cnt = static_cast<int>(found >> 6) & 63, need = static_cast<int>(found) & 63;
+      HKV_STAMP(21)
+      plain = cnt >= 1 && cnt <= kSlots;
+      if (plain) {
+        // the need-th largest of the bin's scores, lane j holding one of them
+        const float own = lane < cnt ? slots[lane * NB + ((tbin + lane) & (NB - 1))] : -INFINITY;
+        int above = 0;
+#pragma unroll 4
+        for (int j = 0; j < cnt; ++j) above += __shfl_sync(0xffffffffu, own, j) > own;
+        thr = __shfl_sync(0xffffffffu, own, __ffs(__ballot_sync(0xffffffffu, lane < cnt && above == need - 1)) - 1);
+      }
+      HKV_STAMP(22)
+    } else {
+      __syncthreads();
+    }
+
+    // the list: scores from thr on, in order; the sequence's last chunk may be short
+    deal_tiles(k_sel * cs - (last_score >= thr ? n_chunks * cs - C : 0));
+    if (plain) {
+      const uint32_t below = (1u << lane) - 1u;
+      int before = 0, all = 0;      // in this warp: before this thread's, in total
+#pragma unroll
+      for (int e = 0; e < IPT; ++e) {
+        const uint32_t b = __ballot_sync(0xffffffffu, v[e] >= thr);
+        before += __popc(b & below);
+        all += __popc(b);
+      }
+      if (lane > warp && lane <= kStepWarps) atomicAdd(&counts[lane], all);
+      __syncthreads();
+      HKV_STAMP(23)
+      plain = counts[kStepWarps] == k_sel;   // (not so with ties at the threshold, or if a wait has run out)
+      uint16_t* at = list + counts[warp] + before;
+      if (plain) {
+#pragma unroll
+        for (int e = 0; e < IPT; ++e)
+          if (v[e] >= thr) *at++ = static_cast<uint16_t>(i0 + e);
+      }
+    }
+    if (!plain) {
+      int emitted = 0;
+      if (!*failed) {   // the general selection, its scratch in the idle ring
+        emitted = min(k_sel, select_crowded<kStepWarps>(scores, n_chunks, k_sel, list, reinterpret_cast<int*>(smem)));
+        fence_proxy_async();
+        __syncthreads();
+      }
+      deal_tiles(emitted * cs - (emitted > 0 && static_cast<int>(list[max(emitted, 1) - 1]) == n_chunks - 1 ? n_chunks * cs - C : 0));
+    }
+    __syncthreads();
+    HKV_STAMP(6)
+  }
+
+  // ---- attention: tile j of the CTA goes through stage j % 6 of warp j % 6 ----
+  auto issue = [&](int j) {   // whole warp, into its stage: a copy of K and of V rows per chunk that the tile touches
+    const int v0 = (tile0 + j) * kTile, v1 = min(v0 + kTile, n_valid);
+    if (lane == 0) mbar_arrive_expect_tx(bars + warp, static_cast<uint32_t>(v1 - v0) * 2u * kRowBytes);
+    __syncwarp();
+#pragma unroll 1
+    for (int p0 = v0; p0 < v1;) {
+      const int ci = fastdiv(p0, cs_magic), p1 = min(v1, ci * cs + cs);
+      const int row = p0 + (dynamic ? (static_cast<int>(list[ci]) - ci) * cs : 0);
+      const uint32_t bytes = static_cast<uint32_t>(p1 - p0) * kRowBytes;
+      HKV_CHECK(v0 >= 0 && p1 > p0 && p1 - v0 <= kTile, 104);
+      HKV_CHECK(row >= 0 && row + (p1 - p0) <= plane_rows, 103);
+#ifdef HKV_CHECKED
+      if (!dead)
+#endif
+      if (lane == 0) {
+        uint8_t* st = smem + warp * kStepStage + (p0 - v0) * kRowBytes;
+        bulk_g2s(st, kplane + static_cast<size_t>(row) * kRowBytes, bytes, bars + warp);
+        bulk_g2s(st + kTile * kRowBytes, vplane + static_cast<size_t>(row) * kRowBytes, bytes, bars + warp);
+      }
+      p0 = p1;
+    }
+  };
+  if (dynamic) {
+    if (warp < kDecStages) {
+      if (warp < at_n) issue(warp);
+    } else if (!*failed) {
+      // what later calls may ask for: scores, selected ids, attended tokens
+      const int k = tid - kDecStages * 32;
+      constexpr int kStride = (kStepWarps - kDecStages) * 32;
+      float* gscores = reinterpret_cast<float*>(base + up->scores_off) + sc_row0;
+      int32_t* gsel = reinterpret_cast<int32_t*>(base + up->idx_off);
+#pragma unroll 1
+      for (int i = k; i < sc_rows; i += kStride) gscores[i] = scores[sc_row0 + i];
+      if (crank == 0) {
+        const int n = min(k_sel, (n_valid + cs - 1) / cs);
+#pragma unroll 1
+        for (int i = k; i < n; i += kStride) gsel[i] = list[i];
+        if (k == 0) reinterpret_cast<int32_t*>(base + P.n_valid_off[0])[uid] = n_valid;
+      }
+    }
+    // "my selection is done": from here on the score area is free to receive the peers' partial results
+    cluster_arrive_relaxed();
+  }
+
+  HKV_STAMP(7)
+  float o[8][1][4] = {}, mrun[1][2] = {{-INFINITY, -INFINITY}}, lrun[1][2] = {};
+  if (warp < kDecStages) {
+    uint8_t* st = smem + warp * kStepStage;
+#pragma unroll 1
+    for (int j = warp; j < at_n; j += kDecStages) {
+      const int nrow = min(kTile, n_valid - (tile0 + j) * kTile);
+      // V rows past the end are not copied: cleared, while the others are still on their way, so that stale bits cannot
+      // poison P*V (their logits are masked, so stale K rows do no harm)
+#pragma unroll 1
+      for (int r = nrow + (lane >> 4); r < kTile; r += 2)
+        reinterpret_cast<uint4*>(st + (kTile + r) * kRowBytes)[lane & 15] = make_uint4(0u, 0u, 0u, 0u);
+      if (!step_wait<false>(bars + warp, phase)) {
+        if (lane == 0) note_timeout(err, kErrDecodeWait);
+        step_wait<false>(bars + warp, phase);      // (the copies may still be on their way)
+        break;
+      }
+      phase ^= 1u;
+      __syncwarp();
+#ifdef HKV_PROFILE
+      if (j == 0) { HKV_STAMP(14) }
+      if (warp == 0 && j == kDecStages) { HKV_STAMP(19) }
+#endif
+      attend_tile<1, false>(smem_u32(st), nullptr, nrow, qb, P.scale_log2e, o, mrun, lrun);
+      __syncwarp();
+#ifdef HKV_PROFILE
+      if (j == 0) { HKV_STAMP(17) }
+#endif
+      if (j + kDecStages < at_n) issue(j + kDecStages);
+#ifdef HKV_PROFILE
+      if (j == 0) { HKV_STAMP(18) }
+#endif
+    }
+    HKV_STAMP(8)
+    // the warp parks (O, m, l) in its own stage: O as [8 heads][kParkStride] floats
+    float l0 = lrun[0][0], l1 = lrun[0][1];
+#pragma unroll
+    for (int off = 4; off <= 16; off <<= 1) {
+      l0 += __shfl_xor_sync(0xffffffffu, l0, off);
+      l1 += __shfl_xor_sync(0xffffffffu, l1, off);
+    }
+    float* wo = reinterpret_cast<float*>(st) + 2 * t * kParkStride + g;
+#pragma unroll
+    for (int dt = 0; dt < 8; ++dt) {
+      wo[dt * 16] = o[dt][0][0];
+      wo[dt * 16 + kParkStride] = o[dt][0][1];
+      wo[dt * 16 + 8] = o[dt][0][2];
+      wo[dt * 16 + 8 + kParkStride] = o[dt][0][3];
+    }
+    if (g == 0)
+      *reinterpret_cast<float4*>(st + 8 * kParkStride * 4 + t * 16) = make_float4(mrun[0][0], l0, mrun[0][1], l1);
+  }
+  __syncthreads();
+  HKV_STAMP(16)
+
+  // ---- merge: the CTA's warps, a warp per head and a lane per four columns; then every owner gets its share ----
+  cluster_wait();            // static units: every CTA of the cluster runs; dynamic ones: the peers' score areas are free
+  if (warp < G) {
+    float2 ml[kDecStages];
+    float M = -1e30f;        // (finite, so that a warp without tiles weighs nothing)
+#pragma unroll
+    for (int w = 0; w < kDecStages; ++w) {
+      ml[w] = reinterpret_cast<const float2*>(smem + w * kStepStage + 8 * kParkStride * 4)[warp];
+      M = fmaxf(M, ml[w].x);
+    }
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    float L = 0.f;
+#pragma unroll
+    for (int w = 0; w < kDecStages; ++w) {
+      const float f = fast_exp2(ml[w].x - M);
+      const float4 x = reinterpret_cast<const float4*>(smem + w * kStepStage + warp * kParkStride * 4)[lane];
+      acc.x += x.x * f; acc.y += x.y * f; acc.z += x.z * f; acc.w += x.w * f;
+      L += ml[w].y * f;
+    }
+    const int e0 = warp * kHeadDim + lane * 4, owner = fastdiv(e0, P.merge_magic);
+    uint32_t peer = mapa(smem0, owner);
+    st_async_f32x4(peer + kStepScores + (crank * per + (e0 - owner * per)) * 4, acc, peer + kStepBars + (kDecStages + 1) * 8);
+    // the row's (m, l) goes to every owner: lane s sends to owner s
+    if (lane < csize && lane * per < total) {
+      peer = mapa(smem0, lane);
+      st_async_f32x2(peer + kStepScores + kRecvMlOff + (crank * G + warp) * 8, M, L, peer + kStepBars + (kDecStages + 1) * 8);
+    }
+  }
+  HKV_STAMP(10)
+
+  if (tid >= mine) return;    // nothing of this thread's is left; peers only write to this CTA, which stays until its reducers leave
+  if (!step_wait<true>(merge_bar, 0u)) {
+    note_timeout(err, kErrMergeWait);
+    return;
+  }
+  HKV_STAMP(11)
+  const float* racc = scores;
+  const float2* rml = reinterpret_cast<const float2*>(smem + kStepScores + kRecvMlOff);
+#pragma unroll 1
+  for (int le = tid; le < mine; le += kStepThreads) {
+    const int e = crank * per + le, row = e >> 7;
+    float M = -1e30f, acc = 0.f, L = 0.f;
+#pragma unroll 1
+    for (int s0 = 0; s0 < csize; s0 += 8) {   // senders in groups of eight, in order
+      float2 ml[8];
+      float av[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        ml[i] = make_float2(-INFINITY, 0.f);
+        av[i] = 0.f;
+        if (s0 + i < csize) { ml[i] = rml[(s0 + i) * G + row]; av[i] = racc[(s0 + i) * per + le]; }
+      }
+      const float m0 = M;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) M = fmaxf(M, ml[i].x);
+      const float c = fast_exp2(m0 - M);
+      acc *= c;
+      L *= c;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float f = fast_exp2(ml[i].x - M);
+        acc += av[i] * f;
+        L += ml[i].y * f;
+      }
+    }
+    const float r = L > 0.f ? __fdividef(acc, L) : 0.f;
+    const size_t off = static_cast<size_t>(out_row0) * kHeadDim + e;
+    if (P.out_f32) reinterpret_cast<float*>(P.out[0])[off] = r;
+    else reinterpret_cast<__nv_bfloat16*>(P.out[0])[off] = __float2bfloat16_rn(r);
+  }
+  HKV_STAMP(13)
+}
+
 // warps per CTA of each instance: the wide-group kernel needs twice the registers per thread
 constexpr int warps_of(int nt) { return nt == 1 ? kMaxWarps : 4; }
 
@@ -1074,12 +1665,9 @@ cudaError_t configure(const ClusterCaps** out) {
       if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
       if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
     };
-    allow(decode_kernel<NT, warps_of(NT), kMaxMulti, 0, false>);
+    allow(decode_kernel<NT, warps_of(NT)>);
     if constexpr (NT == 1) {
-      allow(decode_kernel<1, warps_of(1), 1, 1, false>); allow(decode_kernel<1, warps_of(1), 1, 1, true>);
-      allow(decode_kernel<1, warps_of(1), 1, 2, false>); allow(decode_kernel<1, warps_of(1), 1, 2, true>);
-      allow(decode_kernel<1, warps_of(1), 1, 4, false>); allow(decode_kernel<1, warps_of(1), 1, 4, true>);
-      allow(decode_kernel<1, warps_of(1), 1, 8, false>); allow(decode_kernel<1, warps_of(1), 1, 8, true>);
+      allow(decode_step_kernel<1>); allow(decode_step_kernel<2>); allow(decode_step_kernel<4>); allow(decode_step_kernel<8>);
     }
     if (e != cudaSuccess) return e;
     for (int c = 1; c <= kMaxCluster; ++c) {
@@ -1087,7 +1675,7 @@ cudaError_t configure(const ClusterCaps** out) {
       cudaLaunchAttribute attr[2];
       fill_config<NT>(cfg, attr, 1, c, false, nullptr);
       int n = 0;
-      if (cudaOccupancyMaxActiveClusters(&n, decode_kernel<NT, warps_of(NT), kMaxMulti, 0, false>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+      if (cudaOccupancyMaxActiveClusters(&n, decode_kernel<NT, warps_of(NT)>, &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
       caps.max_active[c] = n;
     }
     caps.ready = true;
@@ -1096,12 +1684,13 @@ cudaError_t configure(const ClusterCaps** out) {
   return cudaSuccess;
 }
 
-template <int NT, int N, int IPT, bool ONE>
-cudaError_t launch_nt(const DecodeParams<N>& params, int total_units, cudaStream_t stream) {
+template <int NT, class Kernel, class Params>
+cudaError_t launch_nt(Kernel kernel, const Params& params, int total_units, int smem, cudaStream_t stream) {
   cudaLaunchConfig_t cfg;
   cudaLaunchAttribute attr[2];
   fill_config<NT>(cfg, attr, total_units, params.cluster, true, stream);
-  return cudaLaunchKernelEx(&cfg, decode_kernel<NT, warps_of(NT), N, IPT, ONE>, params);
+  cfg.dynamicSmemBytes = smem;
+  return cudaLaunchKernelEx(&cfg, kernel, params);
 }
 
 }  // namespace
@@ -1154,26 +1743,22 @@ cudaError_t launch_selftest_wait(int32_t* err_word, cudaStream_t stream) {
 
 cudaError_t launch_decode(const DecodeParams<kMaxMulti>& params, int total_units, cudaStream_t stream) {
   if (total_units <= 0) return cudaSuccess;
-  return params.group > 8 ? launch_nt<2, kMaxMulti, 0, false>(params, total_units, stream)
-                          : launch_nt<1, kMaxMulti, 0, false>(params, total_units, stream);
+  return params.group > 8 ? launch_nt<2>(decode_kernel<2, warps_of(2)>, params, total_units, kSmemBytes, stream)
+                          : launch_nt<1>(decode_kernel<1, warps_of(1)>, params, total_units, kSmemBytes, stream);
 }
 
 bool decode_step_instance(const DecodeParams<1>& P, int max_chunks, int max_tiles) {
   return P.phase == (kPhaseSelect | kPhaseAttend) && P.group <= 8 && P.chunk_size % 8 == 0 && max_chunks <= kSelSmemChunks &&
-         static_cast<uint64_t>(max_tiles + 1) * kTile * static_cast<uint64_t>(P.chunk_size) < (1ull << 32);
+         max_tiles < kWholeList / kTile && static_cast<uint64_t>(max_tiles + 1) * kTile * static_cast<uint64_t>(P.chunk_size) < (1ull << 32);
 }
 
 cudaError_t launch_decode_step(const DecodeParams<1>& params, int max_chunks, int total_units, cudaStream_t stream) {
   if (total_units <= 0) return cudaSuccess;
-  const bool one = params.chunk_size % kTile == 0;
-  auto go = [&](auto ipt) {
-    return one ? launch_nt<1, 1, decltype(ipt)::value, true>(params, total_units, stream)
-               : launch_nt<1, 1, decltype(ipt)::value, false>(params, total_units, stream);
-  };
-  if (max_chunks <= 256) return go(std::integral_constant<int, 1>{});
-  if (max_chunks <= 512) return go(std::integral_constant<int, 2>{});
-  if (max_chunks <= 1024) return go(std::integral_constant<int, 4>{});
-  return go(std::integral_constant<int, 8>{});
+  auto go = [&](auto kernel) { return launch_nt<1>(kernel, params, total_units, kStepBytes, stream); };
+  if (max_chunks <= 256) return go(decode_step_kernel<1>);
+  if (max_chunks <= 512) return go(decode_step_kernel<2>);
+  if (max_chunks <= 1024) return go(decode_step_kernel<4>);
+  return go(decode_step_kernel<8>);
 }
 
 }  // namespace hkv

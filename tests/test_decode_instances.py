@@ -89,3 +89,76 @@ def test_a_recorded_step_does_not_stand_for_the_first_after_an_append():
         return res
 
     assert all(np.array_equal(a, b) for a, b in zip(run(True), run(False)))
+
+
+def _one_layer(C, cs, budget_fraction, head_type, edit=None, n_steps=1, **kw):
+    L = hi.tiny(seed=72, B=kw.pop("B", 1), C=C, chunk_size=cs, w=4, Hq=kw.pop("Hq", 7), Hkv=kw.pop("Hkv", 1), d=128,
+                budget_fraction=budget_fraction, n_steps=n_steps, ragged=False, head_type=head_type, **kw)
+    if edit:
+        edit(L)
+    return L
+
+
+def _repeat(first, count, cs):
+    """Chunks first .. first + count - 1 get the keys of chunk `first`: equal means, equal scores."""
+    def edit(L):
+        for b, h in [(b, h) for b in range(L.batch) for h in range(L.n_kv_heads)]:
+            k = L.k[b, h]
+            for c in range(first + 1, first + count):
+                k[c * cs:(c + 1) * cs] = k[first * cs:(first + 1) * cs]
+    return edit
+
+
+@pytest.mark.parametrize("n_chunks,cs,k,first,count", [(200, 8, 20, 0, 200),     # every score equal
+                                                       (300, 16, 40, 100, 60),   # a crowd beyond what a value bin keeps
+                                                       (64, 8, 33, 0, 64), (700, 8, 5, 3, 690), (1500, 8, 1499, 10, 3)])
+def test_equal_scores_at_the_threshold(n_chunks, cs, k, first, count):
+    """Ties go to the lower chunk, whatever path selects: the whole list is known from the oracle's scores."""
+    from oracle import hkv_oracle as o
+    from paper_2604_05887_b200 import binding as hkv
+    from paper_2604_05887_b200.layer import LayerCache, to_device_bf16
+    L = _one_layer(n_chunks * cs, cs, k / n_chunks, [[1]], _repeat(first, count, cs))
+    lc = LayerCache(L)
+    lc.decode(to_device_bf16(L.q[0]))
+    torch.cuda.synchronize()
+    assert hkv.hkv_last_device_error(lc.handle) == (0, 0)
+    s = hkv.hkv_get_chunk_scores(lc.handle, 0, 0, n_chunks)
+    assert len(set(s[first:first + count].tolist())) == 1       # equal means give equal bits
+    want = np.sort(np.lexsort((np.arange(n_chunks), -s.astype(np.float64)))[:k])
+    assert np.array_equal(hkv.hkv_get_selected_chunks(lc.handle, 0, 0), want)
+    lc.close()
+    import parity_util as P
+    P.compare_layer(L)
+
+
+@pytest.mark.parametrize("n_chunks,cs", [(5, 8), (256, 8), (400, 24), (2048, 8)])
+def test_every_chunk_selected(n_chunks, cs):
+    import parity_util as P
+    P.compare_layer(_one_layer(n_chunks * cs - 3, cs, 1.0, [[1]]))
+
+
+def test_one_cta_per_unit_with_more_chunk_means_than_its_ring_holds():
+    import parity_util as P
+    L = _one_layer(4000, 8, 0.05, [[1, 1, 0, 1]] * 40, B=40, Hq=4, Hkv=4)
+    P.compare_layer(L, units=[(0, 0), (0, 2), (17, 1), (39, 3)])
+
+
+def test_scores_that_are_not_numbers_leave_lists_in_range():
+    """A query of NaN or infinities has no meaningful selection, but what is selected must exist."""
+    from paper_2604_05887_b200 import binding as hkv
+    from paper_2604_05887_b200.layer import LayerCache, to_device_bf16
+    for n_chunks, cs in ((300, 16), (1800, 8), (100, 32)):
+        L = _one_layer(n_chunks * cs, cs, 0.1, [[1]])
+        lc = LayerCache(L)
+        q = to_device_bf16(L.q[0])
+        good = lc.decode(q).clone()
+        for value in (float("nan"), float("inf"), float("-inf")):
+            for dims in (slice(0, 128), slice(3, 4)):
+                bad = q.clone()
+                bad[..., dims] = value
+                lc.decode(bad)
+                torch.cuda.synchronize()
+                ids = hkv.hkv_get_selected_chunks(lc.handle, 0, 0)
+                assert np.all((ids >= 0) & (ids < n_chunks)) and np.all(np.diff(ids) > 0)
+        assert torch.equal(lc.decode(q), good)
+        lc.close()
