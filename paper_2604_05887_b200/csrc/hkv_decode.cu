@@ -1695,22 +1695,24 @@ cudaError_t launch_nt(Kernel kernel, const Params& params, int total_units, int 
 
 }  // namespace
 
-constexpr int kLatencyCluster = 10;
-
 int choose_cluster(int total_units, int max_tiles, const int* max_active) {
-  // The largest even size (or 1) that (a) the device can hold in ONE wave of clusters, (b) leaves every
-  // CTA at least two tiles of the longest unit.  max_active[c] = clusters of size c resident at once.
-  // Even sizes only: two CTAs share an SM, and an odd cluster leaves half an SM idle (measured: 13 CTAs
-  // per unit are slower than 12).  Sizes need not be powers of two.
-  // Short lists (at most 16 tiles per CTA at ten CTAs per unit) are bound by the step's chain of latencies,
-  // not by bandwidth.  What the size changes there is the number of rounds in which a CTA's eight warps and six stages take its
-  // tiles, and how many CTAs of the next launch find room.  Over 45 shapes (1 .. 12 sequences of four KV heads, 52 to 205
-  // tiles) this choice is within 4 % of the best even size in 36; more than ten CTAs are better (up to 21 %, 79 tiles) where
-  // they bring a CTA's tiles to the six that fit the ring and ten do not, fewer (3 to 9 %) where the rounds stay the same.
+  // max_active[c] = clusters of size c the device holds at once: a launch has to fit in ONE wave.  Even sizes only (or 1): two
+  // CTAs share an SM, and an odd cluster leaves half an SM idle (13 CTAs per unit are slower than 12).
+  // What decides is the number of rounds in which a CTA's ring takes its tiles; a larger cluster with as many rounds only makes
+  // the exchange and the merge wait for more CTAs.  Up to eight CTAs that costs nothing that one tile less per CTA does not
+  // bring in (two sequences, 32 tiles per unit: 4 CTAs 6.17 us, 6 5.21, 8 4.81, 10 5.14, 16 5.50), so lists of 16 tiles and more get
+  // eight, and more than eight only where that saves a round (52 tiles: 8 CTAs of 7 tiles 5.90 us, 10 of 6 5.58, 12 5.83;
+  // 94 tiles, one sequence: 8 6.17, 14 6.17, 16 of 6 5.49; four sequences, 79 tiles: 8 9.72, 10 10.12) or leaves four tiles
+  // instead of five (40 tiles: one sequence 8 5.13, 10 4.81; two sequences level, four 2 % slower).  Measured over 130 shapes of 2 to 256
+  // tiles and 1 to 16 sequences of four KV heads: within 4 % of the best even size in all but a few.
+  auto per = [&](int c) { return (max_tiles + c - 1) / c; };
+  auto rounds = [&](int c) { return (per(c) + kDecStages - 1) / kDecStages; };
   int c = 1;
-  for (int t = 2; t <= kMaxCluster; t += 2)
-    if (max_active[t] >= total_units && t * 2 <= max_tiles) c = t;
-  if (c > kLatencyCluster && max_tiles <= kLatencyCluster * 16) c = kLatencyCluster;
+  for (int t = 2; t <= 8; t += 2)
+    if (max_active[t] >= total_units && (t > 4 ? 2 * t : t) <= max_tiles) c = t;
+  const bool five = per(c) == 5;
+  for (int t = 10; t <= kMaxCluster; t += 2)
+    if (max_active[t] >= total_units && 2 * t <= max_tiles && (rounds(t) < rounds(c) || (five && t == 10))) c = t;
   return c;
 }
 
