@@ -149,7 +149,7 @@ __device__ __noinline__ int select_global(const float* gscores, int n_chunks, in
 // One staged tile of 32 tokens (K rows from shared address kbase on, V rows behind them): logits, online softmax, accumulation.
 // NT: column tiles of heads; KEYS: rows carry their own permutation keys (else row r's is r & 7); nrow: tokens that exist.
 template <int NT, bool KEYS>
-__device__ __forceinline__ void attend_tile(uint32_t kbase, const uint32_t* keys, int nrow, const uint32_t (&qb)[8][2 * NT], float sc,
+__device__ __forceinline__ void attend_tile(uint32_t kbase, const uint32_t* keys, int nrow, bool first, const uint32_t (&qb)[8][2 * NT], float sc,
                                             float (&o)[8][NT][4], float (&mrun)[NT][2], float (&lrun)[NT][2]) {
   // ldmatrix lane roles: matrix index = lane >> 3
   const int lane = threadIdx.x & 31, g = lane >> 2;
@@ -211,7 +211,10 @@ __device__ __forceinline__ void attend_tile(uint32_t kbase, const uint32_t* keys
           mx1 = fmaxf(mx1, __shfl_xor_sync(0xffffffffu, mx1, off));
         }
         const float mn0 = fmaxf(mrun[nt][0], mx0 * sc), mn1 = fmaxf(mrun[nt][1], mx1 * sc);
-        if (__any_sync(0xffffffffu, mn0 != mrun[nt][0] || mn1 != mrun[nt][1])) {
+        if (first) {
+      mrun[nt][0] = mn0;
+      mrun[nt][1] = mn1;
+    } else if (__any_sync(0xffffffffu, mn0 != mrun[nt][0] || mn1 != mrun[nt][1])) {
           // a running maximum moved: bring the accumulators to the new reference
           const float c0 = fast_exp2(mrun[nt][0] - mn0), c1 = fast_exp2(mrun[nt][1] - mn1);
           mrun[nt][0] = mn0;
@@ -804,7 +807,7 @@ __global__ void __launch_bounds__(W * 32, kDecCtasPerSm) decode_kernel(const __g
     dead = __any_sync(0xffffffffu, dead);
     if (dead) break;
 #endif
-    attend_tile<NT, KEYS>(smem_u32(st), keys, nrow, qb, sc, o, mrun, lrun);
+    attend_tile<NT, KEYS>(smem_u32(st), keys, nrow, j == warp, qb, sc, o, mrun, lrun);
     __syncwarp();
 #ifdef HKV_PROFILE
     if (j == 0) { HKV_STAMP(17) }
@@ -1064,9 +1067,6 @@ static_assert(kStepBytes <= kSmemBytes, "the capacity of the general kernel hold
 static_assert(kSlots * kHistBins * 4 <= kStepList && kTopkScratchInts * 4 <= kStepList, "selection scratch fits the ring");
 static_assert(8 * kParkStride * 4 + 64 <= kStepStage && kMaxGroup * kRowBytes / 2 <= kSelSmemChunks * 2, "parking, queries");
 
-__device__ __noinline__ void note_timeout(int32_t* err, int place) {
-  if (atomicCAS(&err[0], 0, HKV_ERR_TIMEOUT) == 0) err[1] = place;
-}
 // bounded wait in as few instructions as it takes
 template <bool kCluster>
 __device__ __forceinline__ bool step_wait(uint64_t* bar, uint32_t parity) {
@@ -1075,6 +1075,12 @@ __device__ __forceinline__ bool step_wait(uint64_t* bar, uint32_t parity) {
     if (kCluster ? mbar_try_wait_cluster(bar, parity) : mbar_try_wait(bar, parity)) return true;
   } while (clock64() - start < HKV_WAIT_CYCLES);
   return false;
+}
+// A wait has run out: the error word says so; `bar`, if given, gets another bounded chance, because its copies may still be on
+// their way into memory that is used for something else next.
+__device__ __noinline__ void gave_up(int32_t* err, int place, uint64_t* bar, uint32_t parity) {
+  if (atomicCAS(&err[0], 0, HKV_ERR_TIMEOUT) == 0) err[1] = place;
+  if (bar) step_wait<false>(bar, parity);
 }
 __device__ __forceinline__ float warp_min(float x) {
   float y;
@@ -1231,8 +1237,7 @@ __global__ void __launch_bounds__(kStepThreads, kDecCtasPerSm) decode_step_kerne
       for (int it = fine || warp < kDecStages ? warp : n_items; it < n_items; it += fine ? kStepWarps : kDecStages) {
         const int piece = fine ? it >> 2 : it, stage = fine ? piece : warp;
         if (!step_wait<false>(bars + stage, phase)) {
-          if (lane == 0) note_timeout(err, kErrScoreWait);
-          step_wait<false>(bars + stage, phase);   // (the copy may still be on its way)
+          gave_up(err, kErrScoreWait, bars + stage, phase);
           ok = false;
           if (fine) continue;
           break;
@@ -1251,17 +1256,22 @@ __global__ void __launch_bounds__(kStepThreads, kDecCtasPerSm) decode_step_kerne
           }
           // chunk score = sum over the group's heads of <q_g, mean_c> (variant: their maximum; the columns past the group
           // hold zero queries and must not take part in it)
-          const bool gm = P.group_max != 0;
-          float s[4];
+          float x;
+          auto fold = [&](auto join) {
+            const float v0 = join(acc[0][0], acc[0][1]), v1 = join(acc[0][2], acc[0][3]);   // rows g and g + 8: this thread's two heads
+            x = join(t & 1 ? v1 : v0, __shfl_xor_sync(0xffffffffu, t & 1 ? v0 : v1, 1));
+            x = join(x, __shfl_xor_sync(0xffffffffu, x, 2));
+          };
 #pragma unroll
-          for (int i = 0; i < 4; ++i) {
-            s[i] = acc[0][i] + acc[1][i];
-            if (gm && 2 * t + (i & 1) >= G) s[i] = -INFINITY;
+          for (int i = 0; i < 4; ++i) acc[0][i] += acc[1][i];
+          if (P.group_max) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (2 * t + (i & 1) >= G) acc[0][i] = -INFINITY;
+            fold([](float a, float b) { return fmaxf(a, b); });
+          } else {
+            fold([](float a, float b) { return a + b; });
           }
-          auto join = [&](float a, float b) { return gm ? fmaxf(a, b) : a + b; };
-          const float v0 = join(s[0], s[1]), v1 = join(s[2], s[3]);   // rows g and g + 8: this thread's two heads
-          float x = join(t & 1 ? v1 : v0, __shfl_xor_sync(0xffffffffu, t & 1 ? v0 : v1, 1));
-          x = join(x, __shfl_xor_sync(0xffffffffu, x, 2));
           // a lane now holds the score of row g + 8 (t & 1) of the group
           const int c0 = sc_row0 + m * 16;
           if (c0 + g + 8 * (t & 1) < n_chunks) { wlo = fminf(wlo, x); whi = fmaxf(whi, x); }
@@ -1301,7 +1311,7 @@ __global__ void __launch_bounds__(kStepThreads, kDecCtasPerSm) decode_step_kerne
 
     // ---- selection: every score of the unit is on its way to this CTA ----
     if (!step_wait<true>(score_bar, 0u)) {
-      if (lane == 0) note_timeout(err, kErrExchangeWait);
+      gave_up(err, kErrExchangeWait, nullptr, 0u);
       ok = false;
     }
     if (!ok) { *failed = 1; atomicAdd(&counts[kStepWarps], 1 << 20); }
@@ -1502,8 +1512,7 @@ __global__ void __launch_bounds__(kStepThreads, kDecCtasPerSm) decode_step_kerne
       for (int r = nrow + (lane >> 4); r < kTile; r += 2)
         reinterpret_cast<uint4*>(st + (kTile + r) * kRowBytes)[lane & 15] = make_uint4(0u, 0u, 0u, 0u);
       if (!step_wait<false>(bars + warp, phase)) {
-        if (lane == 0) note_timeout(err, kErrDecodeWait);
-        step_wait<false>(bars + warp, phase);      // (the copies may still be on their way)
+        gave_up(err, kErrDecodeWait, bars + warp, phase);
         break;
       }
       phase ^= 1u;
@@ -1512,7 +1521,7 @@ __global__ void __launch_bounds__(kStepThreads, kDecCtasPerSm) decode_step_kerne
       if (j == 0) { HKV_STAMP(14) }
       if (warp == 0 && j == kDecStages) { HKV_STAMP(19) }
 #endif
-      attend_tile<1, false>(smem_u32(st), nullptr, nrow, qb, P.scale_log2e, o, mrun, lrun);
+      attend_tile<1, false>(smem_u32(st), nullptr, nrow, j == warp, qb, P.scale_log2e, o, mrun, lrun);
       __syncwarp();
 #ifdef HKV_PROFILE
       if (j == 0) { HKV_STAMP(17) }
@@ -1576,7 +1585,7 @@ __global__ void __launch_bounds__(kStepThreads, kDecCtasPerSm) decode_step_kerne
 
   if (tid >= mine) return;    // nothing of this thread's is left; peers only write to this CTA, which stays until its reducers leave
   if (!step_wait<true>(merge_bar, 0u)) {
-    note_timeout(err, kErrMergeWait);
+    gave_up(err, kErrMergeWait, nullptr, 0u);
     return;
   }
   HKV_STAMP(11)
@@ -1587,23 +1596,23 @@ __global__ void __launch_bounds__(kStepThreads, kDecCtasPerSm) decode_step_kerne
     const int e = crank * per + le, row = e >> 7;
     float M = -1e30f, acc = 0.f, L = 0.f;
 #pragma unroll 1
-    for (int s0 = 0; s0 < csize; s0 += 8) {   // senders in groups of eight, in order
-      float2 ml[8];
-      float av[8];
+    for (int s0 = 0; s0 < csize; s0 += 4) {   // senders in groups of four, in order
+      float2 ml[4];
+      float av[4];
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
+      for (int i = 0; i < 4; ++i) {
         ml[i] = make_float2(-INFINITY, 0.f);
         av[i] = 0.f;
         if (s0 + i < csize) { ml[i] = rml[(s0 + i) * G + row]; av[i] = racc[(s0 + i) * per + le]; }
       }
       const float m0 = M;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) M = fmaxf(M, ml[i].x);
+      for (int i = 0; i < 4; ++i) M = fmaxf(M, ml[i].x);
       const float c = fast_exp2(m0 - M);
       acc *= c;
       L *= c;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
+      for (int i = 0; i < 4; ++i) {
         const float f = fast_exp2(ml[i].x - M);
         acc += av[i] * f;
         L += ml[i].y * f;
