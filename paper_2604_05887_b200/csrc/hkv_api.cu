@@ -165,7 +165,7 @@ namespace {
 constexpr int kStepGroups = 4;
 struct StepSide {
   cudaStream_t stream = nullptr;
-  cudaEvent_t fork = nullptr, q_done = nullptr, q_done2 = nullptr, join = nullptr, out[kStepGroups] = {};
+  cudaEvent_t fork = nullptr, tables = nullptr, q_done = nullptr, q_done2 = nullptr, join = nullptr, out[kStepGroups] = {};
   bool ready = false;
   std::mutex enqueue;   // held while a call records and waits on these events, so that host threads do not interleave
 };
@@ -182,6 +182,7 @@ StepSide* step_side() {
     bool ok = cudaDeviceGetStreamPriorityRange(&least, &greatest) == cudaSuccess &&
               cudaStreamCreateWithPriority(&s.stream, cudaStreamNonBlocking, greatest) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&s.fork, cudaEventDisableTiming) == cudaSuccess;
+    ok = ok && cudaEventCreateWithFlags(&s.tables, cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&s.q_done, cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&s.q_done2, cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaEventCreateWithFlags(&s.join, cudaEventDisableTiming) == cudaSuccess;
@@ -279,20 +280,18 @@ static hkv_status compress_common(const hkv_config* cfg, const void* k, const vo
       Unit* sta = dyn + H.n_dynamic;
       for (const auto& u : c->units) *(u.type ? dyn++ : sta++) = u;
     }
-    // the running tile counts lie behind the row statistics (see build_plan)
+    // the static units' running work lies behind the row statistics (see build_plan)
     const bool window = H.n_static > 0 && !token_scores;
     const int R_pad = (H.obs_window * H.group + 15) / 16 * 16;
-    int32_t* tile_prefix = window ? reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + ws_rowstat_off +
-                                                               8ll * H.n_static * tiles_max * R_pad)
-                                  : nullptr;
+    int32_t* prefix = window ? reinterpret_cast<int32_t*>(static_cast<char*>(workspace) + ws_rowstat_off +
+                                                          8ll * H.n_static * tiles_max * R_pad)
+                             : nullptr;
     int64_t total_tiles = 0;
     for (const auto& u : c->units) total_tiles += u.type == 0 ? (u.C + 127) / 128 : 0;
-    bool ok = launch_setup(c->dev_base, img.data(), static_cast<int>(tables), static_cast<int>(H.n_valid_off),
-                           static_cast<int>(H.err_off + 8 - H.n_valid_off), tile_prefix, s) == cudaSuccess;
     int64_t build_bytes = 0;
     for (const auto& u : c->units) build_bytes += u.type == 0 ? 0 : 4ll * kRowBytes * u.C;
     int n_sm = 1;
-    ok = ok && compress_configure(&n_sm) == cudaSuccess;
+    bool ok = compress_configure(&n_sm) == cudaSuccess;
     // A short prompt: few key tiles (they leave half of the SMs free) and copies of a few microseconds.  All kernels go on one
     // stream, each set up beside its predecessors, the dynamic heads' last: it runs beside the selection and the gather.
     const bool chain = window && total_tiles <= n_sm / 2 && build_bytes <= (24ll << 20) && !c->host_bytes;
@@ -302,7 +301,14 @@ static hkv_status compress_common(const hkv_config* cfg, const void* k, const vo
     std::unique_lock<std::mutex> side_lock;
     if (side) side_lock = std::unique_lock<std::mutex>(side->enqueue);
     cudaStream_t ss = side ? side->stream : s;
+    // The first window pass runs beside the set-up of the tables if it needs none of them (4 us of a compression).
+    WindowLaunch L{c->dev_base, static_cast<char*>(workspace), k, q_obs, &H, &c->units, total_tiles, ws_rowstat_off, tiles_max, prefix,
+                   chain, !window_scores_inline(H, c->workspace_bytes)};
     if (ok && side) ok = cudaEventRecord(side->fork, s) == cudaSuccess && cudaStreamWaitEvent(ss, side->fork, 0) == cudaSuccess;
+    ok = ok && launch_setup(c->dev_base, img.data(), static_cast<int>(tables), static_cast<int>(H.n_valid_off),
+                            static_cast<int>(H.err_off + 8 - H.n_valid_off), prefix, window_unit_cost(total_tiles, n_sm), s) == cudaSuccess;
+    if (ok && side) ok = cudaEventRecord(side->tables, s) == cudaSuccess;
+    auto wait_tables = [&] { return !side || cudaStreamWaitEvent(ss, side->tables, 0) == cudaSuccess; };
     // When the dynamic heads' copies start: once the first pass's blocks are running, or once the second one's are.  Blocks of
     // the copies that take an SM's room between the passes hold up the second one by their length, which is that of a
     // chunk: with chunks of up to 32 tokens it hardly shows.  Starting later avoids it but leaves HBM idle in the first pass, which pays
@@ -316,9 +322,14 @@ static hkv_status compress_common(const hkv_config* cfg, const void* k, const vo
     if (side && window)
       later = H.chunk_size > 32 && H.chunk_size <= 64 && static_cast<double>(build_bytes) / 6.0e6 < 30.0 && total_tiles < 20ll * n_sm;
     if (ok && H.n_static > 0) {
-      if (window)
-        ok = launch_window_scores(c->dev_base, static_cast<char*>(workspace), k, q_obs, H, total_tiles, ws_rowstat_off,
-                                  tiles_max, tile_prefix, side ? side->q_done : nullptr, later ? 1 : 0, chain, ss) == cudaSuccess;
+      if (window) {
+        if (L.tables_first) ok = wait_tables();
+        ok = ok && launch_window_scores(L, 0, side && !later ? side->q_done : nullptr, ss) == cudaSuccess;
+        if (!L.tables_first) ok = ok && wait_tables();
+        ok = ok && launch_window_scores(L, 1, side && later ? side->q_done : nullptr, ss) == cudaSuccess;
+      } else {
+        ok = wait_tables();
+      }
       ok = ok && launch_static_select(c->dev_base, static_cast<char*>(workspace), token_scores, is_text, H, chain, ss) == cudaSuccess;
       ok = ok && launch_gather_static(c->dev_base, k, v, H, c->max_static_rows, chain, ss) == cudaSuccess;
       if (side) ok = ok && cudaEventRecord(side->join, ss) == cudaSuccess;

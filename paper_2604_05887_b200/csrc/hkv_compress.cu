@@ -26,7 +26,7 @@ __device__ __forceinline__ const Unit* unit_of(const char* cache, const Header* 
 
 // ---------------------------------------------------------------------------------------------
 // The cache's tables (header, unit records) written, the counters behind them cleared, and the running sum
-// of the static units' key tiles, by which the window-score kernels share out their work, left in the workspace.
+// of the static units' work (key tiles + unit_cost), by which the window-score kernels share it out, left in the workspace.
 // Tables of up to N bytes travel in the launch itself (one launch instead of a staged copy and a fill: 4 us less before
 // the first kernel may start); larger ones have been copied before (N = 0).  One block.
 // ---------------------------------------------------------------------------------------------
@@ -38,7 +38,9 @@ constexpr int kSetupThreads = 512;
 template <int N>
 __global__ void __launch_bounds__(kSetupThreads)
     setup_kernel(const __grid_constant__ TableImage<N> image, char* cache, int table_bytes, int zero_begin, int zero_bytes,
-                 int32_t* tile_prefix) {
+                 int32_t* tile_prefix, int unit_cost) {
+  // (the window scores of a few units need none of this and run beside it)
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   __shared__ int warp_sum[kSetupThreads / 32];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const char* src = cache;
@@ -54,7 +56,7 @@ __global__ void __launch_bounds__(kSetupThreads)
   int before = 0;
   for (int base = 0; base < hdr->n_static; base += kSetupThreads) {
     const int i = base + tid;
-    const int mine = i < hdr->n_static ? (units[i].C + tc::kKeysPerTile - 1) / tc::kKeysPerTile : 0;
+    const int mine = i < hdr->n_static ? (units[i].C + tc::kKeysPerTile - 1) / tc::kKeysPerTile + unit_cost : 0;
     int incl = mine;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
@@ -78,8 +80,8 @@ __global__ void __launch_bounds__(kSetupThreads)
 // ---------------------------------------------------------------------------------------------
 // Window scores.  S_w = softmax over ALL tokens of the w*G window rows' logits, s_w = mean of rows
 // (row r = window position r / G, query head r % G of the group).  The logits run on the tcgen05
-// tensor cores, in base 2, through the segment engine: the static units' 128-key tiles, one after the other, are cut
-// into one equal run per CTA (ranges set by the longest unit left the last CTAs of every shorter one idle).
+// tensor cores, in base 2, through the segment engine: the static units' 128-key tiles, one after the other and each unit with a
+// fixed cost in front, are cut into one equal run per CTA (ranges set by the longest unit left the last CTAs of every shorter one idle).
 // MODE 0: accumulator rows = window rows; a draining thread owns one row and keeps a running reference (the maximum rounded
 //         up to an integer) and the sum of powers over its half of the segment's keys; stats: float2 [n_static][2 segments][Rpad].
 // MODE 1: the rows' final (reference, sum) are put together from those at the start of a segment; accumulator rows = keys; a
@@ -94,21 +96,40 @@ __global__ void __launch_bounds__(kSetupThreads)
 // row took 2 us off a second pass, but rounds a row's weight ten times as coarsely.
 // grid: CTAs; one launch per block of 256 window rows.
 // ---------------------------------------------------------------------------------------------
+// A static unit as these kernels see it.  Its work is its key tiles plus a fixed cost at its beginning, in units of tiles:
+// the place of a piece of work in the launch is counted over both.
+struct WindowUnit {
+  int32_t begin, next;        // work of the launch before the unit, and with it
+  int32_t C, b, h;
+  int32_t first_cta, n_cta;   // CTAs that hold tiles of it
+  int32_t scores_at;          // of s_w in the workspace, in kAlign bytes
+};
+// Units that travel in the launch itself.  Found through header, prefix and record in memory, one after the other, a
+// CTA's first query row was asked for 3 us after its start.
+constexpr int kWindowInline = 96;
 struct WindowParams {
   char* cache;
   char* workspace;
   const __nv_bfloat16* q_obs;
   float2* stats;
-  const int32_t* tile_prefix;
+  const int32_t* prefix; // work before every static unit (units that did not fit)
+  int32_t* err;
   int32_t n_static, n_cta, n_partials;   // partial statistics a row may have (stats' second dimension)
+  int32_t total, unit_cost;   // work of the launch; fixed cost of a unit, or of a CTA's further segments
   int32_t Rpad, row_block;
   int32_t early;         // let the next kernel of a short chain start (see launch_window_scores)
+  int32_t group, obs_window, n_q_heads, n_kv_heads, max_seq_len, causal;
+  uint32_t group_magic;
+  float scale_log2e;
+  int32_t n_inline;      // 0: the units are read from memory
+  WindowUnit unit[kWindowInline];
 };
 struct WindowSeg {
   int key_row0, tile_begin, tile_end, n_rows;
   int C, ordinal, ub, uh;
-  int64_t ws_scores_off;
-  int first, next;       // tiles of the launch before the unit, and behind the segment
+  int first_cta, unit_ctas;
+  int scores_at;
+  int next;              // place in the launch's work behind the segment
 };
 // the caller's shared memory of MODE 1: two buffers of the four quarters' sums; the rows' (max, 1 / sum), last visible keys
 constexpr int kWindowUser1 = 2 * 4 * 128 * 4 + tc::kQRows * 12;
@@ -118,68 +139,101 @@ static_assert(kWindowSmem0 <= 232448 && kWindowSmem1 <= 232448, "one CTA's share
 // Leaves room for four blocks of build_dynamic_kernel beside a CTA (with the 96 registers it takes otherwise there were two, and
 // 19 dynamic units of 50 K tokens took 25 us longer).
 constexpr int kWindowRegs = 72;
+// Fixed cost of a segment in tiles: a CTA whose run goes over the end of a unit exchanges its query rows and puts the statistics of
+// another unit together; with the tiles alone shared out equally it was done 3.4 (first pass) and 4.6 us (second) after the others.
+// Compression and one step of ten static and six dynamic units of 24-32 K tokens with a cost of 0 / 1 / 2 / 3 tiles: 115.7 / 112.9 /
+// 109.2 / 109.1 us.  (No cost where a CTA has a single tile.)
+constexpr int kWindowUnitCost = 2;
 constexpr float kNoKey = -1.0e30f;   // reference of a row that has seen no key
 constexpr float kCeil = 12582912.f;  // 1.5 x 2^23: x + kCeil has no bits behind the point
 
-__device__ __forceinline__ int window_cta_begin(int i, int total, int n_cta) {
+__host__ __device__ __forceinline__ int window_cta_begin(int i, int total, int n_cta) {
   return static_cast<int>(static_cast<int64_t>(i) * total / n_cta);
 }
-__device__ __forceinline__ int window_cta_of(int w, int total, int n_cta) {
+__host__ __device__ __forceinline__ int window_cta_of(int w, int total, int n_cta) {
   return static_cast<int>((static_cast<int64_t>(w + 1) * n_cta - 1) / total);
+}
+// 2^x of an integer x <= 0 (0 below the normal range)
+__device__ __forceinline__ float pow2_int(float x) {
+  return x < -126.f ? 0.f : __int_as_float((static_cast<int>(x) + 127) << 23);
 }
 
 template <int MODE>
 __global__ void __maxnreg__(kWindowRegs)
     window_scores_tc_kernel(const __grid_constant__ WindowParams P, const __grid_constant__ CUtensorMap keys) {
   extern __shared__ __align__(16) uint8_t tc_smem[];
-  // (in a short chain the tables are complete when the first pass has passed its wait, and the second one starts after that)
-  if (MODE == 0 || !P.early) asm volatile("griddepcontrol.wait;" ::: "memory");
+  // The first pass needs nothing of the launch before it (the tables) if its units came with it; it then waits at its end, so
+  // that whoever waits for it has waited for the tables too.  In a short chain the second pass waits where it needs the statistics.
+  const bool wait_first = MODE == 0 ? P.n_inline == 0 : !P.early;
+  if (wait_first) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (P.early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const Header* hdr = reinterpret_cast<const Header*>(P.cache);
-  const int G = hdr->group, w = hdr->obs_window, Hq = hdr->n_q_heads;
+  const int G = P.group, w = P.obs_window, Hq = P.n_q_heads;
   const int R = w * G, row0 = P.row_block * tc::kQRows;
-  const bool causal = (hdr->flags & HKV_CAUSAL_WINDOW) != 0;
-  const float sc = hdr->scale * kLog2e;
+  const bool causal = P.causal != 0;
+  const float sc = P.scale_log2e;
   const uint64_t sc2 = tc::pack_f32x2(sc, sc);
-  const int total = P.tile_prefix[P.n_static];
-  const int w_begin = window_cta_begin(blockIdx.x, total, P.n_cta), w_end = window_cta_begin(blockIdx.x + 1, total, P.n_cta);
+  const int w_begin = window_cta_begin(blockIdx.x, P.total, P.n_cta), w_end = window_cta_begin(blockIdx.x + 1, P.total, P.n_cta);
 
   auto segment = [&](int s, WindowSeg& seg) {   // whole warps call it
-    const int at = s == 0 ? w_begin : seg.next;
+    int at = s == 0 ? w_begin : seg.next;
     if (at >= w_end) return false;
     int o;
     if (s == 0) {   // the last unit that starts at or before `at`
       o = -1;
       for (int base = 0; base < P.n_static; base += 32) {
         const int i = base + static_cast<int>(threadIdx.x & 31);
-        const uint32_t in = __ballot_sync(0xffffffffu, i < P.n_static && P.tile_prefix[i] <= at);
+        const uint32_t in = __ballot_sync(0xffffffffu, i < P.n_static && (P.n_inline ? P.unit[i].begin : P.prefix[i]) <= at);
         o += __popc(in);
         if (in != 0xffffffffu) break;
       }
     } else {
       o = seg.ordinal + 1;    // segments end with their unit or with the CTA's run
     }
-    const Unit* u = unit_of(P.cache, hdr, false, o, nullptr);
+    for (;; ++o) {
+      int begin;
+      if (P.n_inline) {
+        const WindowUnit& u = P.unit[o];
+        begin = u.begin;
+        seg.next = min(w_end, u.next);
+        seg.C = u.C;
+        seg.ub = u.b;
+        seg.uh = u.h;
+        seg.first_cta = u.first_cta;
+        seg.unit_ctas = u.n_cta;
+        seg.scores_at = u.scores_at;
+      } else {
+        const Header* hdr = reinterpret_cast<const Header*>(P.cache);
+        const Unit* u = unit_of(P.cache, hdr, false, o, nullptr);
+        const int next = P.prefix[o + 1];
+        begin = P.prefix[o];
+        seg.next = min(w_end, next);
+        seg.C = u->C;
+        seg.ub = u->b;
+        seg.uh = u->h;
+        seg.first_cta = window_cta_of(begin + P.unit_cost, P.total, P.n_cta);
+        seg.unit_ctas = window_cta_of(next - 1, P.total, P.n_cta) - seg.first_cta + 1;
+        seg.scores_at = static_cast<int>(u->ws_scores_off / kAlign);
+      }
+      begin += P.unit_cost;
+      seg.tile_begin = max(0, at - begin);
+      seg.tile_end = max(0, seg.next - begin);
+      if (seg.tile_begin < seg.tile_end) break;
+      if (seg.next >= w_end) return false;   // nothing but the fixed cost
+      at = seg.next;
+    }
     seg.ordinal = o;
-    seg.C = u->C;
-    seg.ub = u->b;
-    seg.uh = u->h;
-    seg.ws_scores_off = u->ws_scores_off;
-    seg.key_row0 = (u->b * hdr->n_kv_heads + u->h) * hdr->max_seq_len;
+    seg.key_row0 = (seg.ub * P.n_kv_heads + seg.uh) * P.max_seq_len;
     seg.n_rows = min(tc::kQRows, R - row0);
-    seg.first = P.tile_prefix[o];
-    seg.next = min(w_end, P.tile_prefix[o + 1]);
-    seg.tile_begin = at - seg.first;
-    seg.tile_end = seg.next - seg.first;
     return true;
   };
+  auto window_of = [&](int r) { return G > 1 ? fastdiv(r, P.group_magic) : r; };   // position of row r in the window
   auto q_row = [&](const WindowSeg& seg, int row) -> const __nv_bfloat16* {
     const int r = row0 + row;
     if (r >= R) return nullptr;
-    const int i = r / G;
+    const int i = window_of(r);
     return P.q_obs + ((static_cast<size_t>(seg.ub) * w + i) * Hq + seg.uh * G + (r - i * G)) * kHeadDim;
   };
-  int32_t* err = reinterpret_cast<int32_t*>(P.cache + hdr->err_off);
+  int32_t* err = P.err;
   uint8_t* user = nullptr;
   bool ok;
 
@@ -196,7 +250,7 @@ __global__ void __maxnreg__(kWindowRegs)
       const int r = row0 + 128 * (part >> 1) + lane_row;
       if (row0 + 128 * (part >> 1) + (lane_row & ~31) >= R) return;   // the warp's rows are all padding
       const int C = seg.C, j0 = tile * tc::kKeysPerTile + 64 * (part & 1);
-      const int lim = causal ? (C - w + r / G) : (C - 1);      // last key the row sees
+      const int lim = causal ? (C - w + window_of(r)) : (C - 1);      // last key the row sees
       const bool all_visible = j0 + 63 <= (causal ? C - w : C - 1);   // to every row
       tc::drain_raw(taddr, [&](int g, uint32_t (&v)[16]) {
         if (!all_visible) {
@@ -233,7 +287,7 @@ __global__ void __maxnreg__(kWindowRegs)
     auto end = [&](const WindowSeg& seg, int lane_row, int part, bool) {
       // two threads share a row (one per half of every tile): two partial statistics per segment
       const int r = row0 + 128 * (part >> 1) + lane_row;
-      const int index = static_cast<int>(blockIdx.x) - window_cta_of(seg.first, total, P.n_cta);
+      const int index = static_cast<int>(blockIdx.x) - seg.first_cta;
       if (r < R) P.stats[(static_cast<size_t>(seg.ordinal) * P.n_partials + 2 * index + (part & 1)) * P.Rpad + r] = make_float2(m_run, z);
     };
     ok = tc::segments_cta<false, kWindowRing0, WindowSeg>(tc_smem, &keys, segment, q_row, begin, tile_fn, end, &user);
@@ -250,7 +304,7 @@ __global__ void __maxnreg__(kWindowRegs)
       if (P.early) asm volatile("griddepcontrol.wait;" ::: "memory");   // for the first pass's statistics
       // the rows' statistics: two threads per row take every other partial
       const int dtid = threadIdx.x - 32, row = dtid >> 1, r = row0 + row;
-      const int n_part = 2 * (window_cta_of(P.tile_prefix[seg.ordinal + 1] - 1, total, P.n_cta) - window_cta_of(seg.first, total, P.n_cta) + 1);
+      const int n_part = 2 * seg.unit_ctas;
       const float2* st = P.stats + static_cast<size_t>(seg.ordinal) * P.n_partials * P.Rpad + r;
       // (sixteen loads in flight: one after the other they took 5 us before the first tile)
       float M = kNoKey, Z = 0.f;
@@ -262,14 +316,14 @@ __global__ void __maxnreg__(kWindowRegs)
         float top = M;
 #pragma unroll
         for (int e = 0; e < 16; ++e) top = fmaxf(top, v[e].x);
-        Z *= exp2f(M - top);
+        Z *= pow2_int(M - top);
         M = top;
 #pragma unroll
-        for (int e = 0; e < 16; ++e) Z += v[e].y * exp2f(v[e].x - M);
+        for (int e = 0; e < 16; ++e) Z += v[e].y * pow2_int(v[e].x - M);
       }
       {
         const float other = __shfl_xor_sync(0xffffffffu, M, 1), top = fmaxf(M, other);
-        Z *= exp2f(M - top);
+        Z *= pow2_int(M - top);
         M = top;
         const float z0 = __shfl_sync(0xffffffffu, Z, (threadIdx.x & 31) & ~1), z1 = __shfl_sync(0xffffffffu, Z, (threadIdx.x & 31) | 1);
         Z = z0 + z1;
@@ -279,7 +333,7 @@ __global__ void __maxnreg__(kWindowRegs)
         float* pair = reinterpret_cast<float*>(info + (row >> 1)) + (row & 1);
         pair[0] = r < R ? -M : 0.f;
         pair[2] = r < R ? 1.f / Z : 0.f;                      // a padding row adds nothing
-        last[row] = r < R ? static_cast<float>(causal ? (seg.C - w + r / G) : (seg.C - 1)) : -1.f;
+        last[row] = r < R ? static_cast<float>(causal ? (seg.C - w + window_of(r)) : (seg.C - 1)) : -1.f;
       }
       tc::named_sync(tc::kBarDrain, tc::kDrainWarps * 32);
     };
@@ -319,7 +373,7 @@ __global__ void __maxnreg__(kWindowRegs)
       tc::named_sync(tc::kBarUser + (lane_row >> 5), 128);   // the four warps of these lanes
       if (part == 0 && j < C) {
         const float tot = ((buf[lane_row] + buf[128 + lane_row]) + (buf[256 + lane_row] + buf[384 + lane_row])) * inv_R;
-        float* sw = reinterpret_cast<float*>(P.workspace + seg.ws_scores_off);
+        float* sw = reinterpret_cast<float*>(P.workspace + static_cast<int64_t>(seg.scores_at) * kAlign);
         sw[j] = P.row_block == 0 ? tot : sw[j] + tot;
       }
       ++n_done;
@@ -327,6 +381,7 @@ __global__ void __maxnreg__(kWindowRegs)
     auto end = [](const WindowSeg&, int, int, bool) {};
     ok = tc::segments_cta<true, kWindowRing1, WindowSeg>(tc_smem, &keys, segment, q_row, begin, tile_fn, end, &user);
   }
+  if (!wait_first) asm volatile("griddepcontrol.wait;" ::: "memory");
   if (!ok && threadIdx.x == 0) { atomicCAS(&err[0], 0, HKV_ERR_TIMEOUT); err[1] = kErrScoreWait; }
 }
 
@@ -962,56 +1017,89 @@ cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, int threads, 
 
 template <int N>
 cudaError_t launch_setup_n(char* cache, const void* image, int table_bytes, int zero_begin, int zero_bytes, int32_t* prefix,
-                           cudaStream_t stream) {
+                           int unit_cost, cudaStream_t stream) {
   TableImage<N> img;
   if constexpr (N > 0) std::memcpy(img.bytes, image, static_cast<size_t>(table_bytes));
-  setup_kernel<N><<<1, kSetupThreads, 0, stream>>>(img, cache, table_bytes, zero_begin, zero_bytes, prefix);
+  setup_kernel<N><<<1, kSetupThreads, 0, stream>>>(img, cache, table_bytes, zero_begin, zero_bytes, prefix, unit_cost);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_setup(char* cache, const void* image, int table_bytes, int zero_begin, int zero_bytes, int32_t* tile_prefix,
-                         cudaStream_t stream) {
-  if (table_bytes <= 3584) return launch_setup_n<3584>(cache, image, table_bytes, zero_begin, zero_bytes, tile_prefix, stream);
-  if (table_bytes <= 16384) return launch_setup_n<16384>(cache, image, table_bytes, zero_begin, zero_bytes, tile_prefix, stream);
+cudaError_t launch_setup(char* cache, const void* image, int table_bytes, int zero_begin, int zero_bytes, int32_t* prefix,
+                         int unit_cost, cudaStream_t stream) {
+  if (table_bytes <= 3584) return launch_setup_n<3584>(cache, image, table_bytes, zero_begin, zero_bytes, prefix, unit_cost, stream);
+  if (table_bytes <= 16384) return launch_setup_n<16384>(cache, image, table_bytes, zero_begin, zero_bytes, prefix, unit_cost, stream);
   // a captured copy would read the image when the graph is launched, long after it has been freed
   cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
   cudaError_t e = cudaStreamIsCapturing(stream, &capture);
   if (e == cudaSuccess && capture != cudaStreamCaptureStatusNone) e = cudaErrorStreamCaptureUnsupported;
   if (e == cudaSuccess) e = cudaMemcpyAsync(cache, image, static_cast<size_t>(table_bytes), cudaMemcpyHostToDevice, stream);
-  return e == cudaSuccess ? launch_setup_n<0>(cache, image, table_bytes, zero_begin, zero_bytes, tile_prefix, stream) : e;
+  return e == cudaSuccess ? launch_setup_n<0>(cache, image, table_bytes, zero_begin, zero_bytes, prefix, unit_cost, stream) : e;
 }
 
-cudaError_t launch_window_scores(char* cache, char* workspace, const void* k, const void* q_obs, const Header& hdr,
-                                 int64_t total_tiles, int64_t ws_rowstat_off, int n_partials, const int32_t* tile_prefix,
-                                 cudaEvent_t started, int started_pass, bool chain, cudaStream_t stream) {
+int window_unit_cost(int64_t total_tiles, int n_sm) { return total_tiles > n_sm ? kWindowUnitCost : 0; }
+
+cudaError_t launch_window_scores(WindowLaunch& L, int mode, cudaEvent_t started, cudaStream_t stream) {
+  const Header& hdr = *L.hdr;
   if (hdr.n_static == 0) return cudaSuccess;
-  if (total_tiles > 0x7FFFFFFF) return cudaErrorInvalidValue;
   const int R = hdr.obs_window * hdr.group;
   int n_sm = 0;
   cudaError_t e = compress_configure(&n_sm);
   CUtensorMap map;
-  if (e == cudaSuccess) e = tc::key_map(&map, k, static_cast<uint64_t>(hdr.batch) * hdr.n_kv_heads * hdr.max_seq_len);
-  WindowParams P{};
-  P.cache = cache;
-  P.workspace = workspace;
-  P.q_obs = static_cast<const __nv_bfloat16*>(q_obs);
-  P.stats = reinterpret_cast<float2*>(workspace + ws_rowstat_off);
-  P.tile_prefix = tile_prefix;
+  if (e == cudaSuccess) e = tc::key_map(&map, L.k, static_cast<uint64_t>(hdr.batch) * hdr.n_kv_heads * hdr.max_seq_len);
+  if (e != cudaSuccess) return e;
+  WindowParams P;
+  P.cache = L.cache;
+  P.workspace = L.workspace;
+  P.q_obs = static_cast<const __nv_bfloat16*>(L.q_obs);
+  P.stats = reinterpret_cast<float2*>(L.workspace + L.ws_rowstat_off);
+  P.prefix = L.prefix;
+  P.err = reinterpret_cast<int32_t*>(L.cache + hdr.err_off);
   P.n_static = hdr.n_static;
-  P.n_cta = static_cast<int>(std::min<int64_t>(n_sm, total_tiles));
-  P.n_partials = n_partials;
-  P.early = chain ? 1 : 0;
+  P.n_cta = static_cast<int>(std::min<int64_t>(n_sm, L.total_tiles));
+  P.unit_cost = window_unit_cost(L.total_tiles, n_sm);
+  const int64_t total = L.total_tiles + static_cast<int64_t>(P.unit_cost) * hdr.n_static;
+  if (total > 0x7FFFFFFF) return cudaErrorInvalidValue;
+  P.total = static_cast<int>(total);
+  P.n_partials = L.n_partials;
+  P.early = L.chain ? 1 : 0;
   P.Rpad = (R + 15) / 16 * 16;
-  const int n_row_blocks = (R + tc::kQRows - 1) / tc::kQRows;
-  for (int mode = 0; mode < 2; ++mode) {
-    for (P.row_block = 0; P.row_block < n_row_blocks && e == cudaSuccess; ++P.row_block)
-      e = launch_compress(mode == 0 ? window_scores_tc_kernel<0> : window_scores_tc_kernel<1>, dim3(P.n_cta), tc::kSegThreads,
-                          mode == 0 ? kWindowSmem0 : kWindowSmem1, stream, chain || P.row_block > 0 || mode > 0,
-                          mode == started_pass && P.row_block == 0 ? started : nullptr, P, map);
+  P.group = hdr.group;
+  P.obs_window = hdr.obs_window;
+  P.n_q_heads = hdr.n_q_heads;
+  P.n_kv_heads = hdr.n_kv_heads;
+  P.max_seq_len = hdr.max_seq_len;
+  P.causal = (hdr.flags & HKV_CAUSAL_WINDOW) != 0;
+  P.group_magic = hdr.group > 1 ? 0xFFFFFFFFu / static_cast<uint32_t>(hdr.group) + 1u : 0u;
+  P.scale_log2e = hdr.scale * kLog2e;
+  P.n_inline = L.tables_first ? 0 : hdr.n_static;
+  if (P.n_inline) {
+    int64_t before = 0;
+    int o = 0;
+    for (const Unit& u : *L.units) {
+      if (u.type != 0) continue;
+      WindowUnit& x = P.unit[o++];
+      x.begin = static_cast<int>(before);
+      before += (u.C + tc::kKeysPerTile - 1) / tc::kKeysPerTile + P.unit_cost;
+      x.next = static_cast<int>(before);
+      x.C = u.C;
+      x.b = u.b;
+      x.h = u.h;
+      x.first_cta = window_cta_of(x.begin + P.unit_cost, P.total, P.n_cta);
+      x.n_cta = window_cta_of(x.next - 1, P.total, P.n_cta) - x.first_cta + 1;
+      x.scores_at = static_cast<int>(u.ws_scores_off / kAlign);
+    }
   }
+  const int n_row_blocks = (R + tc::kQRows - 1) / tc::kQRows;
+  for (P.row_block = 0; P.row_block < n_row_blocks && e == cudaSuccess; ++P.row_block)
+    e = launch_compress(mode == 0 ? window_scores_tc_kernel<0> : window_scores_tc_kernel<1>, dim3(P.n_cta), tc::kSegThreads,
+                        mode == 0 ? kWindowSmem0 : kWindowSmem1, stream, L.chain || P.row_block > 0 || mode > 0,
+                        P.row_block == 0 ? started : nullptr, P, map);
   return e;
+}
+bool window_scores_inline(const Header& hdr, size_t workspace_bytes) {
+  return hdr.n_static <= kWindowInline && workspace_bytes / kAlign < 0x7FFFFFFFull;
 }
 
 cudaError_t launch_static_select(char* cache, char* workspace, const float* token_scores, const uint8_t* is_text,

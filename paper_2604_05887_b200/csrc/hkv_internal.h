@@ -113,14 +113,27 @@ cudaError_t launch_decode_step(const DecodeParams<1>& params, int max_chunks, in
 // Sets the compression kernels' shared-memory limits (once per device) and gives the current device's number of SMs.
 cudaError_t compress_configure(int* n_sm);
 // Writes the cache's tables (a host image of table_bytes), clears [zero_begin, zero_begin + zero_bytes) of the cache and, unless
-// null, fills tile_prefix with the static units' running tile counts.
+// null, fills prefix with the static units' running work: key tiles, and unit_cost for each.
 // chain (launch_window_scores .. launch_build_dynamic): the compression's kernels follow one another on one stream, each set up
 // beside its predecessors.
-cudaError_t launch_setup(char* cache, const void* image, int table_bytes, int zero_begin, int zero_bytes, int32_t* tile_prefix,
-                         cudaStream_t stream);
-cudaError_t launch_window_scores(char* cache, char* workspace, const void* k, const void* q_obs, const Header& hdr,
-                                 int64_t total_tiles, int64_t ws_rowstat_off, int n_partials, const int32_t* tile_prefix,
-                                 cudaEvent_t started, int started_pass, bool chain, cudaStream_t stream);   // `started` (or null): recorded once that pass's blocks run
+cudaError_t launch_setup(char* cache, const void* image, int table_bytes, int zero_begin, int zero_bytes, int32_t* prefix,
+                         int unit_cost, cudaStream_t stream);
+// The two passes of the window scores.
+struct WindowLaunch {
+  char *cache, *workspace;
+  const void *k, *q_obs;
+  const Header* hdr;
+  const std::vector<Unit>* units;
+  int64_t total_tiles, ws_rowstat_off;
+  int n_partials;
+  const int32_t* prefix;   // the static units' running work, left by launch_setup
+  bool chain;
+  bool tables_first;       // the passes read the cache's tables: they have to follow launch_setup on the stream
+};
+cudaError_t launch_window_scores(WindowLaunch& launch, int mode, cudaEvent_t started, cudaStream_t stream);   // `started` (or null): recorded once the pass's blocks run
+// whether the units' records fit the launches, so that the first pass may run beside launch_setup
+bool window_scores_inline(const Header& hdr, size_t workspace_bytes);
+int window_unit_cost(int64_t total_tiles, int n_sm);   // what a unit counts beyond its tiles
 cudaError_t launch_static_select(char* cache, char* workspace, const float* token_scores,
                                  const uint8_t* is_text, const Header& hdr, bool chain, cudaStream_t stream);
 cudaError_t launch_gather_static(char* cache, const void* k, const void* v, const Header& hdr,
