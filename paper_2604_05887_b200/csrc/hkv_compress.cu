@@ -532,8 +532,10 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThrea
   __shared__ int wtot[32];
   extern __shared__ __align__(16) uint32_t skey[];          // slice_slots keys, then slice_slots text flags (bytes)
   uint8_t* stxt = reinterpret_cast<uint8_t*>(skey + slice_slots);
-  if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  // (not before the wait: the dynamic heads' copies at the end of a short chain read the tables without waiting, and the
+  // window passes may have begun before those were complete)
+  if (early) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 
   const Header* hdr = reinterpret_cast<const Header*>(cache);
   const uint32_t rank = cluster_ctarank();
