@@ -301,14 +301,10 @@ static hkv_status compress_common(const hkv_config* cfg, const void* k, const vo
     std::unique_lock<std::mutex> side_lock;
     if (side) side_lock = std::unique_lock<std::mutex>(side->enqueue);
     cudaStream_t ss = side ? side->stream : s;
-    // The first window pass runs beside the set-up of the tables if it needs none of them (4 us of a compression).
-    WindowLaunch L{c->dev_base, static_cast<char*>(workspace), k, q_obs, &H, &c->units, total_tiles, ws_rowstat_off, tiles_max, prefix,
-                   chain, !window_scores_inline(H, c->workspace_bytes)};
     if (ok && side) ok = cudaEventRecord(side->fork, s) == cudaSuccess && cudaStreamWaitEvent(ss, side->fork, 0) == cudaSuccess;
     ok = ok && launch_setup(c->dev_base, img.data(), static_cast<int>(tables), static_cast<int>(H.n_valid_off),
                             static_cast<int>(H.err_off + 8 - H.n_valid_off), prefix, window_unit_cost(total_tiles, n_sm), s) == cudaSuccess;
     if (ok && side) ok = cudaEventRecord(side->tables, s) == cudaSuccess;
-    auto wait_tables = [&] { return !side || cudaStreamWaitEvent(ss, side->tables, 0) == cudaSuccess; };
     // When the dynamic heads' copies start: once the first pass's blocks are running, or once the second one's are.  Blocks of
     // the copies that take an SM's room between the passes hold up the second one by their length, which is that of a
     // chunk: with chunks of up to 32 tokens it hardly shows.  Starting later avoids it but leaves HBM idle in the first pass, which pays
@@ -322,14 +318,12 @@ static hkv_status compress_common(const hkv_config* cfg, const void* k, const vo
     if (side && window)
       later = H.chunk_size > 32 && H.chunk_size <= 64 && static_cast<double>(build_bytes) / 6.0e6 < 30.0 && total_tiles < 20ll * n_sm;
     if (ok && H.n_static > 0) {
-      if (window) {
-        if (L.tables_first) ok = wait_tables();
-        ok = ok && launch_window_scores(L, 0, side && !later ? side->q_done : nullptr, ss) == cudaSuccess;
-        if (!L.tables_first) ok = ok && wait_tables();
-        ok = ok && launch_window_scores(L, 1, side && later ? side->q_done : nullptr, ss) == cudaSuccess;
-      } else {
-        ok = wait_tables();
-      }
+      if (window)
+        ok = launch_window_scores({c->dev_base, static_cast<char*>(workspace), k, q_obs, &H, &c->units, total_tiles, ws_rowstat_off, tiles_max,
+                                   prefix, chain, c->workspace_bytes},
+                                  side ? side->tables : nullptr, side ? side->q_done : nullptr, later ? 1 : 0, ss) == cudaSuccess;
+      else if (side)
+        ok = cudaStreamWaitEvent(ss, side->tables, 0) == cudaSuccess;
       ok = ok && launch_static_select(c->dev_base, static_cast<char*>(workspace), token_scores, is_text, H, chain, ss) == cudaSuccess;
       ok = ok && launch_gather_static(c->dev_base, k, v, H, c->max_static_rows, chain, ss) == cudaSuccess;
       if (side) ok = ok && cudaEventRecord(side->join, ss) == cudaSuccess;

@@ -6,6 +6,7 @@
 #include <algorithm>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 
 #include "hkv_device.cuh"
 #include "hkv_internal.h"
@@ -106,7 +107,7 @@ struct WindowUnit {
 };
 // Units that travel in the launch itself.  Found through header, prefix and record in memory, one after the other, a
 // CTA's first query row was asked for 3 us after its start.
-constexpr int kWindowInline = 96;
+constexpr int kWindowInline = 48;
 struct WindowParams {
   char* cache;
   char* workspace;
@@ -344,26 +345,30 @@ __global__ void __maxnreg__(kWindowRegs)
       const bool all_visible = j0 + tc::kKeysPerTile - 1 <= (causal ? C - w : C - 1);   // to every row
       uint64_t a = 0, b = 0;
       if (row0 + 64 * part < R) {                      // same for the whole warp
-        tc::drain_raw(taddr, [&](int g, uint32_t (&v)[16]) {
-          const int rb = 64 * part + 16 * g;
-          if (row0 + rb >= R) return;   // 16 padding rows: nothing to add (same for the whole warp)
-          const float4* ri = info + rb / 2;
+        auto go = [&](auto visible) {   // (a tile of its own for the keys at the end: a test per four powers cost 11 % of the pass)
+          tc::drain_raw(taddr, [&](int g, uint32_t (&v)[16]) {
+            const int rb = 64 * part + 16 * g;
+            if (row0 + rb >= R) return;   // 16 padding rows: nothing to add (same for the whole warp)
+            const float4* ri = info + rb / 2;
 #pragma unroll
-          for (int c = 0; c < 16; c += 4) {
-            const float4 p = ri[c / 2], q = ri[c / 2 + 1];
-            float e0, e1, e2, e3;
-            tc::unpack_f32x2(tc::fma_f32x2(tc::pack_f32x2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc2, tc::pack_f32x2(p.x, p.y)), e0, e1);
-            tc::unpack_f32x2(tc::fma_f32x2(tc::pack_f32x2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3])), sc2, tc::pack_f32x2(q.x, q.y)), e2, e3);
-            if (!all_visible) {
-              if (jf > last[rb + c]) e0 = -INFINITY;
-              if (jf > last[rb + c + 1]) e1 = -INFINITY;
-              if (jf > last[rb + c + 2]) e2 = -INFINITY;
-              if (jf > last[rb + c + 3]) e3 = -INFINITY;
+            for (int c = 0; c < 16; c += 4) {
+              const float4 p = ri[c / 2], q = ri[c / 2 + 1];
+              float e0, e1, e2, e3;
+              tc::unpack_f32x2(tc::fma_f32x2(tc::pack_f32x2(__uint_as_float(v[c]), __uint_as_float(v[c + 1])), sc2, tc::pack_f32x2(p.x, p.y)), e0, e1);
+              tc::unpack_f32x2(tc::fma_f32x2(tc::pack_f32x2(__uint_as_float(v[c + 2]), __uint_as_float(v[c + 3])), sc2, tc::pack_f32x2(q.x, q.y)), e2, e3);
+              if constexpr (!decltype(visible)::value) {
+                if (jf > last[rb + c]) e0 = -INFINITY;
+                if (jf > last[rb + c + 1]) e1 = -INFINITY;
+                if (jf > last[rb + c + 2]) e2 = -INFINITY;
+                if (jf > last[rb + c + 3]) e3 = -INFINITY;
+              }
+              a = tc::fma_f32x2(tc::pack_f32x2(fast_exp2(e0), fast_exp2(e1)), tc::pack_f32x2(p.z, p.w), a);
+              b = tc::fma_f32x2(tc::pack_f32x2(fast_exp2(e2), fast_exp2(e3)), tc::pack_f32x2(q.z, q.w), b);
             }
-            a = tc::fma_f32x2(tc::pack_f32x2(fast_exp2(e0), fast_exp2(e1)), tc::pack_f32x2(p.z, p.w), a);
-            b = tc::fma_f32x2(tc::pack_f32x2(fast_exp2(e2), fast_exp2(e3)), tc::pack_f32x2(q.z, q.w), b);
-          }
-        });
+          });
+        };
+        if (all_visible) go(std::true_type{});
+        else go(std::false_type{});
       }
       float x, y;
       tc::unpack_f32x2(tc::add_f32x2(a, b), x, y);
@@ -1042,7 +1047,7 @@ cudaError_t launch_setup(char* cache, const void* image, int table_bytes, int ze
 
 int window_unit_cost(int64_t total_tiles, int n_sm) { return total_tiles > n_sm ? kWindowUnitCost : 0; }
 
-cudaError_t launch_window_scores(WindowLaunch& L, int mode, cudaEvent_t started, cudaStream_t stream) {
+cudaError_t launch_window_scores(const WindowLaunch& L, cudaEvent_t tables, cudaEvent_t started, int started_pass, cudaStream_t stream) {
   const Header& hdr = *L.hdr;
   if (hdr.n_static == 0) return cudaSuccess;
   const int R = hdr.obs_window * hdr.group;
@@ -1075,7 +1080,7 @@ cudaError_t launch_window_scores(WindowLaunch& L, int mode, cudaEvent_t started,
   P.causal = (hdr.flags & HKV_CAUSAL_WINDOW) != 0;
   P.group_magic = hdr.group > 1 ? 0xFFFFFFFFu / static_cast<uint32_t>(hdr.group) + 1u : 0u;
   P.scale_log2e = hdr.scale * kLog2e;
-  P.n_inline = L.tables_first ? 0 : hdr.n_static;
+  P.n_inline = hdr.n_static <= kWindowInline && L.workspace_bytes / kAlign < 0x7FFFFFFFull ? hdr.n_static : 0;
   if (P.n_inline) {
     int64_t before = 0;
     int o = 0;
@@ -1094,16 +1099,15 @@ cudaError_t launch_window_scores(WindowLaunch& L, int mode, cudaEvent_t started,
     }
   }
   const int n_row_blocks = (R + tc::kQRows - 1) / tc::kQRows;
-  for (P.row_block = 0; P.row_block < n_row_blocks && e == cudaSuccess; ++P.row_block)
-    e = launch_compress(mode == 0 ? window_scores_tc_kernel<0> : window_scores_tc_kernel<1>, dim3(P.n_cta), tc::kSegThreads,
-                        mode == 0 ? kWindowSmem0 : kWindowSmem1, stream, L.chain || P.row_block > 0 || mode > 0,
-                        P.row_block == 0 ? started : nullptr, P, map);
+  for (int mode = 0; mode < 2; ++mode) {
+    if (tables && e == cudaSuccess && mode == (P.n_inline ? 1 : 0)) e = cudaStreamWaitEvent(stream, tables, 0);
+    for (P.row_block = 0; P.row_block < n_row_blocks && e == cudaSuccess; ++P.row_block)
+      e = launch_compress(mode == 0 ? window_scores_tc_kernel<0> : window_scores_tc_kernel<1>, dim3(P.n_cta), tc::kSegThreads,
+                          mode == 0 ? kWindowSmem0 : kWindowSmem1, stream, L.chain || P.row_block > 0 || mode > 0,
+                          mode == started_pass && P.row_block == 0 ? started : nullptr, P, map);
+  }
   return e;
 }
-bool window_scores_inline(const Header& hdr, size_t workspace_bytes) {
-  return hdr.n_static <= kWindowInline && workspace_bytes / kAlign < 0x7FFFFFFFull;
-}
-
 cudaError_t launch_static_select(char* cache, char* workspace, const float* token_scores, const uint8_t* is_text,
                                  const Header& hdr, bool chain, cudaStream_t stream) {
   if (hdr.n_static == 0) return cudaSuccess;

@@ -128,11 +128,11 @@ struct WindowLaunch {
   int n_partials;
   const int32_t* prefix;   // the static units' running work, left by launch_setup
   bool chain;
-  bool tables_first;       // the passes read the cache's tables: they have to follow launch_setup on the stream
+  size_t workspace_bytes;
 };
-cudaError_t launch_window_scores(WindowLaunch& launch, int mode, cudaEvent_t started, cudaStream_t stream);   // `started` (or null): recorded once the pass's blocks run
-// whether the units' records fit the launches, so that the first pass may run beside launch_setup
-bool window_scores_inline(const Header& hdr, size_t workspace_bytes);
+// `tables` (or null): launch_setup's end, if that is on another stream.  The first pass runs beside it where the units' records fit
+// the launch.  `started` (or null): recorded once the blocks of pass `started_pass` run.
+cudaError_t launch_window_scores(const WindowLaunch& launch, cudaEvent_t tables, cudaEvent_t started, int started_pass, cudaStream_t stream);
 int window_unit_cost(int64_t total_tiles, int n_sm);   // what a unit counts beyond its tiles
 cudaError_t launch_static_select(char* cache, char* workspace, const float* token_scores,
                                  const uint8_t* is_text, const Header& hdr, bool chain, cudaStream_t stream);
