@@ -1,4 +1,4 @@
-"""Builds libhkv.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a."""
+"""Builds libhkv.so (the C-ABI CUDA library) in-tree with nvcc for sm_100a, and the binding's small extension."""
 from __future__ import annotations
 
 import os
@@ -64,5 +64,33 @@ def build_profile(force: bool = False) -> str:
     return build_library(force, extra_flags=["-DHKV_PROFILE"], out=PROFILE_LIB_PATH)
 
 
+CALLS_PATH = os.path.join(PKG_DIR, "_calls.so")    # Python extension: the calls of every layer and token
+
+
+def build_calls(force: bool = False) -> str:
+    src = os.path.join(CSRC, "hkv_calls.cpp")
+    if not force and os.path.exists(CALLS_PATH) and os.path.getmtime(CALLS_PATH) >= os.path.getmtime(src):
+        return CALLS_PATH
+    import sysconfig
+
+    import torch
+    from torch.utils.cpp_extension import include_paths, library_paths
+    cuda = os.path.dirname(os.path.dirname(os.path.realpath(_nvcc())))
+    cmd = [os.environ.get("CXX", "g++"), "-std=c++17", "-O2", "-fPIC", "-shared", "-o", CALLS_PATH, src,
+           f"-D_GLIBCXX_USE_CXX11_ABI={int(torch._C._GLIBCXX_USE_CXX11_ABI)}",
+           "-isystem", sysconfig.get_paths()["include"], "-isystem", os.path.join(cuda, "include")]
+    for d in include_paths():
+        cmd += ["-isystem", d]
+    for d in library_paths():
+        cmd += ["-L" + d, "-Wl,-rpath," + d]
+    cmd += ["-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_python"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        sys.stderr.write(r.stdout + r.stderr)
+        raise RuntimeError("building _calls.so failed")
+    return CALLS_PATH
+
+
 if __name__ == "__main__":
     print(build_library(force=True, verbose="-v" in sys.argv))
+    print(build_calls(force=True))

@@ -1,0 +1,153 @@
+// The two calls that a program issues once per layer and token, hkv_decode_attn and hkv_append, straight from the interpreter:
+// tensors' addresses and the current stream taken in C++, no argument conversion by ctypes.
+//
+// What bounds a short prompt's steps is the host: a layer's call took 3.1 us, 1.1 of them between the caller and the library.
+//
+// Call(general, error, name): a callable (cache, tensor, tensor) for a C function (handle, addresses ..., stream).
+// Plain forms -- an integer handle, contiguous CUDA tensors of torch's own classes, no stream given -- are called directly; every
+// other form goes to `general`, the Python function, which takes or refuses it.
+#include <Python.h>
+
+#include <c10/cuda/CUDAStream.h>
+#include <torch/csrc/autograd/python_variable.h>
+
+namespace {
+
+struct Call {
+  PyObject_HEAD
+  vectorcallfunc vectorcall;
+  void* fn;             // the C function, or null: everything goes to `general`
+  PyObject *general, *error, *name;
+};
+
+// The address of a tensor that `general` would take too; anything that might answer differently from Python is left to it.
+bool plain(PyObject* o, void** address) {
+  if (!THPVariable_CheckExact(o)) return false;
+  const at::Tensor& t = THPVariable_Unpack(o);
+  c10::TensorImpl* impl = t.unsafeGetTensorImpl();
+  constexpr c10::DispatchKeySet special({c10::DispatchKey::Python, c10::DispatchKey::FuncTorchGradWrapper,
+                                         c10::DispatchKey::FuncTorchBatched, c10::DispatchKey::Functionalize});
+  if (!impl->has_storage() || impl->key_set().has_any(special) || !impl->is_cuda() || !impl->is_contiguous()) return false;
+  *address = t.data_ptr();
+  return true;
+}
+
+PyObject* invoke(PyObject* self, PyObject* const* args, size_t nargsf, PyObject* kwnames) {
+  Call* c = reinterpret_cast<Call*>(self);
+  void *handle = nullptr, *p[2] = {}, *stream = nullptr;
+  bool direct = c->fn && !kwnames && PyVectorcall_NARGS(nargsf) == 3 && PyLong_CheckExact(args[0]);
+  if (direct) {
+    handle = PyLong_AsVoidPtr(args[0]);
+    if (!handle && PyErr_Occurred()) {
+      PyErr_Clear();
+      direct = false;
+    }
+  }
+  if (direct) {
+    try {
+      direct = plain(args[1], &p[0]) && plain(args[2], &p[1]);
+      if (direct) stream = c10::cuda::getCurrentCUDAStream().stream();
+    } catch (...) {
+      direct = false;
+    }
+  }
+  if (!direct) return PyObject_Vectorcall(c->general, args, nargsf, kwnames);
+  int status;
+  PyThreadState* thread = PyEval_SaveThread();
+  status = reinterpret_cast<int (*)(void*, const void*, void*, void*)>(c->fn)(handle, p[0], p[1], stream);
+  PyEval_RestoreThread(thread);
+  if (status == 0) Py_RETURN_NONE;
+  if (PyObject* e = PyObject_CallFunction(c->error, "iO", status, c->name)) {
+    PyErr_SetObject(c->error, e);
+    Py_DECREF(e);
+  }
+  return nullptr;
+}
+
+PyObject* call_new(PyTypeObject* type, PyObject* args, PyObject*) {
+  PyObject *general, *error, *name;
+  if (!PyArg_ParseTuple(args, "OOU", &general, &error, &name)) return nullptr;
+  Call* c = reinterpret_cast<Call*>(type->tp_alloc(type, 0));
+  if (!c) return nullptr;
+  c->vectorcall = invoke;
+  c->fn = nullptr;
+  Py_INCREF(general);
+  Py_INCREF(error);
+  Py_INCREF(name);
+  c->general = general;
+  c->error = error;
+  c->name = name;
+  return reinterpret_cast<PyObject*>(c);
+}
+
+int call_traverse(PyObject* self, visitproc visit, void* arg) {
+  Call* c = reinterpret_cast<Call*>(self);
+  Py_VISIT(c->general);
+  Py_VISIT(c->error);
+  return 0;
+}
+int call_clear(PyObject* self) {
+  Call* c = reinterpret_cast<Call*>(self);
+  Py_CLEAR(c->general);
+  Py_CLEAR(c->error);
+  return 0;
+}
+void call_dealloc(PyObject* self) {
+  PyObject_GC_UnTrack(self);
+  call_clear(self);
+  Py_CLEAR(reinterpret_cast<Call*>(self)->name);
+  Py_TYPE(self)->tp_free(self);
+}
+
+// name, documentation, signature: the Python function's
+PyObject* call_getattro(PyObject* self, PyObject* name) {
+  if (PyUnicode_CompareWithASCIIString(name, "__doc__") != 0) {
+    if (PyObject* own = PyObject_GenericGetAttr(self, name)) return own;
+    if (!PyErr_ExceptionMatches(PyExc_AttributeError)) return nullptr;
+    PyErr_Clear();
+  }
+  if (PyUnicode_CompareWithASCIIString(name, "__wrapped__") == 0) {
+    Py_INCREF(reinterpret_cast<Call*>(self)->general);
+    return reinterpret_cast<Call*>(self)->general;
+  }
+  return PyObject_GetAttr(reinterpret_cast<Call*>(self)->general, name);
+}
+
+// the address of the C function (0: none)
+PyObject* call_bind(PyObject* self, PyObject* address) {
+  void* fn = PyLong_AsVoidPtr(address);
+  if (!fn && PyErr_Occurred()) return nullptr;
+  reinterpret_cast<Call*>(self)->fn = fn;
+  Py_RETURN_NONE;
+}
+
+PyMethodDef call_methods[] = {{"bind", call_bind, METH_O, "bind(address): the C function to call"}, {nullptr, nullptr, 0, nullptr}};
+
+PyTypeObject call_type = {PyVarObject_HEAD_INIT(nullptr, 0)};
+PyModuleDef module = {PyModuleDef_HEAD_INIT, "_calls", "Direct calls into libhkv.", -1, nullptr, nullptr, nullptr, nullptr, nullptr};
+
+}  // namespace
+
+PyMODINIT_FUNC PyInit__calls() {
+  call_type.tp_name = "paper_2604_05887_b200._calls.Call";
+  call_type.tp_basicsize = sizeof(Call);
+  call_type.tp_flags = Py_TPFLAGS_DEFAULT | Py_TPFLAGS_HAVE_GC | Py_TPFLAGS_HAVE_VECTORCALL;
+  call_type.tp_vectorcall_offset = offsetof(Call, vectorcall);
+  call_type.tp_call = PyVectorcall_Call;
+  call_type.tp_new = call_new;
+  call_type.tp_traverse = call_traverse;
+  call_type.tp_clear = call_clear;
+  call_type.tp_dealloc = call_dealloc;
+  call_type.tp_getattro = call_getattro;
+  call_type.tp_methods = call_methods;
+  if (PyType_Ready(&call_type) < 0) return nullptr;
+  PyObject* m = PyModule_Create(&module);
+  if (!m) return nullptr;
+  Py_INCREF(&call_type);
+  if (PyModule_AddObject(m, "Call", reinterpret_cast<PyObject*>(&call_type)) < 0) {
+    Py_DECREF(&call_type);
+    Py_DECREF(m);
+    return nullptr;
+  }
+  return m;
+}

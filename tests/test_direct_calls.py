@@ -1,0 +1,69 @@
+"""The extension through which hkv_decode_attn and hkv_append are called: the usual form goes straight to the C function, every
+other form to the Python function behind it, with that function's name, signature and errors."""
+import ctypes as C
+import inspect
+
+import pytest
+import torch
+
+from paper_2604_05887_b200 import _calls, binding
+
+
+def test_name_and_signature_are_the_functions():
+    for call, params in ((binding.hkv_decode_attn, ["cache", "q", "out", "stream"]), (binding.hkv_append, ["cache", "k_new", "v_new", "stream"])):
+        assert list(inspect.signature(call).parameters) == params
+        assert inspect.signature(call).parameters["stream"].default is None
+        assert call.__name__ == getattr(call.__wrapped__, "__name__") and call.__doc__ == call.__wrapped__.__doc__
+
+
+def test_other_forms_go_to_the_python_function():
+    seen = []
+
+    def general(cache, a, b, stream=None):
+        seen.append((cache, a, b, stream))
+        return "general"
+
+    def never(*_):
+        raise AssertionError("called")
+
+    fn = C.CFUNCTYPE(C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p)(never)
+    call = _calls.Call(general, binding.HkvError, "x")
+    t = torch.zeros(4)
+    assert call(1, t, t) == "general"                      # not bound yet
+    call.bind(C.cast(fn, C.c_void_p).value)
+    for args, kw in (((1, t, t), {}), ((1, t), {"b": t}), ((1, t, t, 5), {}), ((None, t, t), {}), ((1 << 70, t, t), {}),
+                     ((1, object(), t), {}), ((1, t.as_subclass(type("Sub", (torch.Tensor,), {})), t), {})):
+        assert call(*args, **kw) == "general"
+    assert len(seen) == 8
+    with pytest.raises(TypeError):
+        call(1)
+    with pytest.raises(ValueError, match="contiguous CUDA tensor"):
+        binding.hkv_decode_attn(1, t, t)
+    with pytest.raises(ValueError, match="contiguous CUDA tensor"):
+        binding.hkv_append(1, t, t)
+
+
+@pytest.mark.gpu
+def test_usual_form_is_called_directly():
+    got = []
+    fn = C.CFUNCTYPE(C.c_int, C.c_void_p, C.c_void_p, C.c_void_p, C.c_void_p)(lambda *a: got.append(a) or (0 if len(got) < 4 else 2))
+
+    def general(cache, a, b, stream=None):
+        return "general"
+
+    call = _calls.Call(general, binding.HkvError, "x")
+    call.bind(C.cast(fn, C.c_void_p).value)
+    a, b = torch.zeros(4, 8, device="cuda"), torch.nn.Parameter(torch.zeros(8, device="cuda"))
+    assert call(7, a, b) is None and got[-1] == (7, a.data_ptr(), b.data_ptr(), None)
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        assert call(7, a[1], b) is None and got[-1] == (7, a[1].data_ptr(), b.data_ptr(), side.cuda_stream)
+    assert call(0, a, b) is None and got[-1][0] is None
+    assert call(7, a.t(), b) == "general" and call(7, a.cpu(), b) == "general" and call(7, a, b, stream=None) == "general"
+    assert len(got) == 3
+    with pytest.raises(binding.HkvError) as e:
+        call(7, a, b)
+    assert e.value.status == 2 and "x: HKV_ERR_SHAPE" in str(e.value)
+    # a tensor that stands for others has no address
+    with pytest.raises(RuntimeError):
+        torch.vmap(lambda x: binding.hkv_decode_attn(1, x, x))(a)
