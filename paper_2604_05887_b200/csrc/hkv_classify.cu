@@ -19,6 +19,7 @@
 #include <algorithm>
 #include <cmath>
 #include <mutex>
+#include <type_traits>
 
 #include "hkv_device.cuh"
 #include "hkv_internal.h"
@@ -436,30 +437,35 @@ __global__ void __launch_bounds__(tc::kSegThreads, 1)
   auto tile_fn = [&](const ClsSeg& seg, int tile, int, int part, uint32_t taddr) {
     if (idle) return;
     const int left = seg.C - (tile * tc::kKeysPerTile + 64 * (part & 1));   // keys of the thread's 64 columns that exist
-    tc::drain_raw<1>(taddr, [&](int g, uint32_t (&r)[16]) {
-      if (left < 64) {
+    // (a tile that ends with the context in a loop of its own: with the test in one loop 28168 rows of 24-32 K keys took 546 us, not 531)
+    auto go = [&](auto whole) {
+      tc::drain_raw<1>(taddr, [&](int g, uint32_t (&r)[16]) {
+        if constexpr (!decltype(whole)::value) {
 #pragma unroll
-        for (int c = 0; c < 16; ++c)
-          if (16 * g + c >= left) r[c] = 0xFF800000u;   // -inf: no weight, below every bound
-      }
-      if (__any_sync(0xffffffffu, at - slots > (kClsSlots - 16) * 128u)) flush();   // room for 16 more in every lane
-      uint64_t z2 = 0;
-      float t0 = 0.f, t1 = 0.f;
+          for (int c = 0; c < 16; ++c)
+            if (16 * g + c >= left) r[c] = 0xFF800000u;   // -inf: no weight, below every bound
+        }
+        if (__any_sync(0xffffffffu, at - slots > (kClsSlots - 16) * 128u)) flush();   // room for 16 more in every lane
+        uint64_t z2 = 0;
+        float t0 = 0.f, t1 = 0.f;
 #pragma unroll
-      for (int c = 0; c < 16; c += 2) {
-        const float v0 = __uint_as_float(r[c]), v1 = __uint_as_float(r[c + 1]);
-        float e0, e1;
-        tc::unpack_f32x2(tc::fma_f32x2(tc::pack_f32x2(v0, v1), sc2, nref2), e0, e1);
-        const float p0 = fast_exp2(e0), p1 = fast_exp2(e1);
-        z2 = tc::add_f32x2(z2, tc::pack_f32x2(p0, p1));
-        cls_take(v0, p0, lo, hi, t0, cnt, at);
-        cls_take(v1, p1, lo, hi, t1, cnt, at);
-      }
-      float a, b2;
-      tc::unpack_f32x2(z2, a, b2);
-      tc::add_compensated(z, zc, a + b2);
-      tc::add_compensated(top, topc, t0 + t1);
-    });
+        for (int c = 0; c < 16; c += 2) {
+          const float v0 = __uint_as_float(r[c]), v1 = __uint_as_float(r[c + 1]);
+          float e0, e1;
+          tc::unpack_f32x2(tc::fma_f32x2(tc::pack_f32x2(v0, v1), sc2, nref2), e0, e1);
+          const float p0 = fast_exp2(e0), p1 = fast_exp2(e1);
+          z2 = tc::add_f32x2(z2, tc::pack_f32x2(p0, p1));
+          cls_take(v0, p0, lo, hi, t0, cnt, at);
+          cls_take(v1, p1, lo, hi, t1, cnt, at);
+        }
+        float a, b2;
+        tc::unpack_f32x2(z2, a, b2);
+        tc::add_compensated(z, zc, a + b2);
+        tc::add_compensated(top, topc, t0 + t1);
+      });
+    };
+    if (left >= 64) go(std::true_type{});
+    else go(std::false_type{});
   };
   auto end = [&](const ClsSeg& seg, int lane_row, int part, bool) {
     const int row = 128 * (part >> 1) + lane_row;
