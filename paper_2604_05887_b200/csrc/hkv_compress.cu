@@ -510,14 +510,15 @@ __global__ void __launch_bounds__(kKeepThreads)
 
 // ---------------------------------------------------------------------------------------------
 // The same keep-set with one thread-block CLUSTER per static unit: the unit's tokens are cut into kSelCluster
-// contiguous slices, one per CTA, so that no SM walks a whole 32 K-token sequence alone.  Four cluster barriers:
+// contiguous slices, one per CTA, so that no SM walks a whole 32 K-token sequence alone.  Three cluster barriers:
 //   1. every CTA publishes its slice's statistics (text tokens before the window; smallest / largest score key
 //      among the text and among the visual tokens) -> all know which class is ranked, k, and the key range;
 //   2. local 1024-bin histograms of the ranked keys are complete -> every CTA adds up all eight (thread b reads
 //      bin b of every peer through distributed shared memory) and finds the threshold bin on its own copy;
 //   3. the threshold bin's items, (key, index), have been stored into every CTA's candidate list at slots that
 //      follow from the peers' counts of that bin -> every CTA ranks them exactly and knows the threshold element;
-//   4. the per-CTA numbers of selected tokens are known -> each CTA emits its ascending run at its offset.
+// The numbers of tokens that lower slices take (always kept, above the threshold bin, taken from it) are known to every CTA by
+// then, so that each emits its ascending run at its offset, and nobody reads a peer's shared memory any more.
 // A threshold bin with more than 1024 items (many near-equal scores) is taken apart by another histogram over its own
 // key range, and so on; if all of them have the same key, the lower positions win.
 // ---------------------------------------------------------------------------------------------
@@ -531,10 +532,9 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThrea
   __shared__ __align__(16) int hist[kKeyedBins];
   __shared__ __align__(16) uint2 cand[kKeepThreads];
   __shared__ SelStats stats[kSelCluster];
-  __shared__ int counts[kSelCluster];
   __shared__ int cnt_by_rank[kSelCluster];
   __shared__ __align__(8) int ctl[8];
-  __shared__ int wtot[32];
+  __shared__ int2 wtot[32];
   extern __shared__ __align__(16) uint32_t skey[];          // slice_slots keys, then slice_slots text flags (bytes)
   uint8_t* stxt = reinterpret_cast<uint8_t*>(skey + slice_slots);
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -601,11 +601,12 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThrea
   }
   cluster_arrive(); cluster_wait();   // 1
 
-  int n_text = 0;
+  int n_text = 0, text_below = 0;   // text tokens of all slices, of the lower ones
   uint32_t kmin_t = 0xFFFFFFFFu, kmax_t = 0u, kmin_v = 0xFFFFFFFFu, kmax_v = 0u;
 #pragma unroll
   for (int r = 0; r < kSelCluster; ++r) {
     n_text += stats[r].n_text;
+    text_below += r < static_cast<int>(rank) ? stats[r].n_text : 0;
     kmin_t = min(kmin_t, stats[r].tmin); kmax_t = max(kmax_t, stats[r].tmax);
     kmin_v = min(kmin_v, stats[r].vmin); kmax_v = max(kmax_v, stats[r].vmax);
   }
@@ -620,6 +621,7 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThrea
 
   uint32_t tkey = 0xFFFFFFFFu;   // nothing ranked is taken unless the selection below says so
   int tidx = -1;
+  int below = max(0, lo - hist_end) + (rank_text ? 0 : text_below);   // tokens that lower slices take: those always kept, ...
   if (k > 0) {
     uint32_t bin0 = kmin;        // the bins cover keys bin0 + [b, b + 1) << shift, `span` keys in all
     uint64_t span = 1ull << 32;
@@ -634,35 +636,36 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThrea
         if (is_cand(j) && skey[j] >= bin0 && static_cast<uint64_t>(skey[j] - bin0) < span) atomicAdd(&hist[(skey[j] - bin0) >> shift], 1);
       __syncthreads();
       cluster_arrive(); cluster_wait();   // 2
-      int hr[kSelCluster], mine_tot = 0;
+      int hr[kSelCluster], mine_tot = 0, low_tot = 0;   // all slices', the lower ones' scores in this thread's bin
       {
         const uint32_t a = smem_u32(&hist[tid]);
 #pragma unroll
         for (int r = 0; r < kSelCluster; ++r) {
           asm volatile("ld.shared::cluster.u32 %0, [%1];" : "=r"(hr[r]) : "r"(mapa(a, r)) : "memory");
           mine_tot += hr[r];
+          low_tot += r < static_cast<int>(rank) ? hr[r] : 0;
         }
       }
       // the highest bin b with count(bins > b) < need <= count(bins >= b): thread t owns bin t
       {
-        int run = mine_tot;
+        int2 run = make_int2(mine_tot, low_tot);
+        auto suffix = [&](int2& x) {
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-          const int v = __shfl_down_sync(0xffffffffu, run, off);
-          if (lane + off < 32) run += v;
-        }
+          for (int off = 1; off < 32; off <<= 1) {
+            const int v = __shfl_down_sync(0xffffffffu, x.x, off), v2 = __shfl_down_sync(0xffffffffu, x.y, off);
+            if (lane + off < 32) { x.x += v; x.y += v2; }
+          }
+        };
+        suffix(run);
         if (lane == 0) wtot[warp] = run;
         __syncthreads();
-        const int wt = wtot[lane];
-        int wrun = wt;
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) {
-          const int v = __shfl_down_sync(0xffffffffu, wrun, off);
-          if (lane + off < 32) wrun += v;
-        }
-        const int above = __shfl_sync(0xffffffffu, wrun - wt, warp) + run - mine_tot;
+        const int2 wt = wtot[lane];
+        int2 wrun = wt;
+        suffix(wrun);
+        const int above = __shfl_sync(0xffffffffu, wrun.x - wt.x, warp) + run.x - mine_tot;
+        const int above_low = __shfl_sync(0xffffffffu, wrun.y - wt.y, warp) + run.y - low_tot;
         if (above < need && need <= above + mine_tot) {
-          ctl[1] = tid; ctl[2] = need - above; ctl[3] = mine_tot;
+          ctl[1] = tid; ctl[2] = need - above; ctl[3] = mine_tot; ctl[6] = above_low;
 #pragma unroll
           for (int r = 0; r < kSelCluster; ++r) cnt_by_rank[r] = hr[r];
         }
@@ -671,6 +674,7 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThrea
       tbin = ctl[1];
       need = ctl[2];
       cnt = ctl[3];
+      below += ctl[6];             // ... those above the threshold bin, ...
       if (cnt <= kKeepThreads || shift == 0) break;
       cluster_arrive(); cluster_wait();   // peers may still be reading my histogram; all have read the control words
       bin0 += static_cast<uint32_t>(tbin) << shift;
@@ -703,6 +707,7 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThrea
           seen += __popc(m);
         }
       }
+      below += min(need, base);
       cluster_arrive(); cluster_wait();   // 3
     } else {
       // ---- the threshold bin's items into every CTA's candidate list ----
@@ -717,6 +722,7 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThrea
         }
       }
       cluster_arrive(); cluster_wait();   // 3
+      bool low = false;
       if (tid < cnt) {
         const uint2 me = cand[tid];
         int rk = 0;
@@ -725,8 +731,9 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThrea
           rk += (o.x > me.x) || (o.x == me.x && o.y < me.y);
         }
         if (rk == need - 1) { ctl[4] = static_cast<int>(me.x); ctl[5] = static_cast<int>(me.y); }
+        low = rk < need && static_cast<int>(me.y) < lo;
       }
-      __syncthreads();
+      below += __syncthreads_count(low);   // ... and those taken from it
     }
     tkey = static_cast<uint32_t>(ctl[4]);
     tidx = ctl[5];
@@ -748,41 +755,31 @@ __global__ void __cluster_dims__(kSelCluster, 1, 1) __launch_bounds__(kKeepThrea
     mine_n += __popc(__ballot_sync(0xffffffffu, j < end && taken(j)));
   }
   __syncthreads();   // wtot is free again
-  if (lane == 0) wtot[warp] = mine_n;
+  if (lane == 0) wtot[warp].x = mine_n;
   __syncthreads();
   int before = 0, total = 0;
   {
-    const int wt = wtot[lane];
+    const int wt = wtot[lane].x;
     int incl = wt;
 #pragma unroll
     for (int off = 1; off < 32; off <<= 1) {
       const int v = __shfl_up_sync(0xffffffffu, incl, off);
       if (lane >= off) incl += v;
     }
-    before = __shfl_sync(0xffffffffu, incl - wt, warp);
-    total = __shfl_sync(0xffffffffu, incl, 31);
+    before = below + __shfl_sync(0xffffffffu, incl - wt, warp);
+    total = below + __shfl_sync(0xffffffffu, incl, 31);
   }
-  if (tid < kSelCluster)
-    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(mapa(smem_u32(&counts[rank]), tid)), "r"(total) : "memory");
-  cluster_arrive(); cluster_wait();   // 4
-  int off0 = 0, all = 0;
-#pragma unroll
-  for (int r = 0; r < kSelCluster; ++r) {
-    if (r < static_cast<int>(rank)) off0 += counts[r];
-    all += counts[r];
-  }
-  before += off0;
-  const uint32_t below = (1u << lane) - 1u;
+  const uint32_t lanes_below = (1u << lane) - 1u;
   for (int j0 = beg; j0 < end; j0 += 32) {
     const int j = j0 + lane;
     const bool sel = j < end && taken(j);
     const uint32_t b = __ballot_sync(0xffffffffu, sel);
-    if (sel) out[before + __popc(b & below)] = lo + j;
+    if (sel) out[before + __popc(b & lanes_below)] = lo + j;
     before += __popc(b);
   }
-  if (rank == 0 && tid == 0) {
-    *n_valid = all;
-    if (all != budget) {
+  if (rank == kSelCluster - 1 && tid == 0) {
+    *n_valid = total;
+    if (total != budget) {
       int32_t* err = reinterpret_cast<int32_t*>(cache + hdr->err_off);
       atomicCAS(&err[0], 0, HKV_ERR_INDEX);
       err[1] = kErrIndex;
