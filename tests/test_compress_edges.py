@@ -76,3 +76,64 @@ def test_tables_copied_from_the_host_are_refused_while_the_stream_is_captured():
     torch.cuda.synchronize()
     assert mark.item() == 1
     P.compare_layer(L, units=[(0, 0), (79, 1)])
+
+
+@pytest.mark.parametrize("B,C,w,Hq", [(24, 700, 8, 8), (25, 700, 8, 8), (25, 700, 40, 16), (1, 9600, 40, 16)])
+def test_units_that_travel_in_the_launch_and_units_read_from_memory(B, C, w, Hq):
+    """48 static units are the most that come as launch parameters, 50 are read from the cache's tables; more key tiles than
+    SMs, so that every unit counts a fixed cost beside its tiles; one and two blocks of window rows."""
+    import parity_util as P
+    L = _layer(B, C, np.zeros((B, 2), np.uint8), w=w, Hq=Hq, ragged=B > 1)
+    P.compare_layer(L, units=[(b, h) for b in sorted({0, B // 2, B - 1}) for h in range(2)])
+
+
+@pytest.mark.parametrize("kind", ["text_fills_budget", "text_ranked", "kept_in_last_slices"])
+def test_keep_set_over_slices(kind):
+    """Eight thread blocks share a unit; where a block's run of kept positions begins follows from what the lower ones take:
+    text only (nothing is ranked), ranked text, scores that rise with the position."""
+    import parity_util as P
+    L = _layer(1, 6001, [[0, 1]], budget_fraction=0.25)
+    rng = np.random.default_rng(9)
+    ts = rng.random((1, 2, 6001)).astype(np.float32)
+    room = int(L.budgets[0, 0]) - 8
+    L.is_text[0] = 0
+    if kind == "text_fills_budget":
+        L.is_text[0, rng.choice(6001 - 8, room, replace=False)] = 1
+    elif kind == "text_ranked":
+        L.is_text[0, rng.choice(6001 - 8, 2 * room, replace=False)] = 1
+    else:
+        L.is_text[0, :40] = 1
+        ts[0, 0] = np.arange(6001) + 1.0
+    P.compare_layer(L, token_scores=ts)
+
+
+@pytest.mark.parametrize("C", [900, 12000])
+def test_recorded_compression_writes_everything_a_step_reads(C):
+    """A compression and a step recorded in one graph and replayed over a cache whose tables and planes have been cleared:
+    they are written before anything reads them, on one stream (short prompts) and on two."""
+    import torch
+    from paper_2604_05887_b200 import binding as hkv
+    L = _layer(1, C, [[0, 1]], ragged=False)
+    cfg = hkv.make_config(1, 8, 2, 128, L.max_seq_len, 32, 8)
+    k, v, q_obs, is_text = (torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (L.k, L.v, L.q_obs, L.is_text))
+    g = torch.Generator(device="cuda").manual_seed(1)
+    q = torch.randn(1, 8, 128, device="cuda", generator=g).bfloat16()
+    cache, ws = (torch.empty(n, dtype=torch.uint8, device="cuda") for n in hkv.hkv_plan(cfg, L.seq_lens, L.head_type, L.budgets))
+    out = torch.empty(1, 8, 128, device="cuda", dtype=torch.bfloat16)
+
+    def once():
+        h = hkv.hkv_compress(cfg, k, v, q_obs, None, is_text, L.seq_lens, L.head_type, L.budgets, cache, ws)
+        hkv.hkv_decode_attn(h, q, out)
+        hkv.hkv_cache_destroy(h)
+    once()
+    torch.cuda.synchronize()
+    want = out.clone()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        once()
+    for _ in range(20):
+        cache[256:].zero_()     # (a record of zeroes read too early leads nowhere outside the buffers)
+        ws.fill_(255)
+        out.zero_()
+        graph.replay()
+        assert torch.equal(out, want)
