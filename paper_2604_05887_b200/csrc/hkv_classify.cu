@@ -36,6 +36,7 @@ constexpr int kClsGroupMax = 8;        // most sampled keys that share a histogr
 constexpr int kClsSampleBins = 112;    // histogram of the sample, six standard deviations wide
 constexpr double kClsSigmas = 4.75;    // margin of the bounds in standard deviations of the sample's rank
 constexpr int kClsSlack = 256;         // list entries per segment beyond its share: half of a video frame whose keys all lie between the bounds
+constexpr int kClsSlackTight = 16;     // the same where segments of a tile or two get several times their share instead
 constexpr int kClsFixThreads = 1024;
 constexpr int kClsSmemCols = 49152;    // longest row the fix kernel keeps in shared memory
 constexpr int kClsRank = 256;          // largest threshold bin that is sorted directly
@@ -59,7 +60,7 @@ struct ClsParams {
   int32_t weight, weight_half;    // of a pair with more than 128 rows, of any other
   int32_t small;                  // W * n_cta fits 31 bits: 32-bit divisions
   int32_t seg_max;                // most CTAs that share one row block
-  int32_t per_tile;               // list entries per half tile
+  int32_t per_tile, slack;        // list entries per half tile and per segment
   int32_t list_stride;            // entries of one half row's list
   int32_t sample_stride;          // rows of a unit in the sample buffer
   int32_t split;                  // CTAs (a cluster) that share a row block's samples
@@ -110,7 +111,7 @@ __device__ __forceinline__ int cls_cta_of(const ClsParams& P, int64_t w) {
 
 // Where a segment's entries lie in a half row's list: a share for every tile before it, slack for every segment.
 __device__ __forceinline__ int cls_list_at(const ClsParams& P, int tile_begin, int index) {
-  return (tile_begin * P.per_tile & ~3) + index * kClsSlack;
+  return (tile_begin * P.per_tile & ~3) + index * P.slack;
 }
 
 // A row's bounds; without a sample (a workspace too small for one) every entry is listed.
@@ -323,9 +324,12 @@ __global__ void __launch_bounds__(tc::kSegThreads, 1)
 // sums and list position in registers.  An entry above the upper bound joins sum and count; one between the bounds is
 // appended, by predicated instructions, to the thread's own column of shared memory, which goes to the row's list in
 // groups of four.
-// Bound: issue slots (13 instructions per warp and entry, 75 % of the scheduler's cycles; four warps per scheduler is all the
-// registers allow).  One context of 32768 keys against 7168 rows: 127 us = 2.6 us per 256 x 128 tile.  With only the lower
-// bound tested here lists are twice as long and the time the same; slots advanced by sign arithmetic instead of predicates: + 20 %.
+// Bound: issue slots (13 instructions per warp and entry, 8 of them for the comparison with the bounds, 75 % of the scheduler's
+// cycles; four warps per scheduler is all the registers allow).  28168 rows of 24-32 K keys: 396 us.  With only the lower
+// bound tested here lists are twice as long and the time the same; with the staged entries compared with the upper one when they are
+// flushed + 22 % (a flush lasts as long as the fullest lane's entries, and rows peak in different frames); slots advanced by sign
+// arithmetic instead of predicates + 20 %; sum and number as one packed addition + 14 %; set-to-float masks instead of
+// predicates + 3 %; two groups of columns unrolled + 2 %.
 // grid: P.n_cta.  partial: float4 [unit][row_block][seg_max][2] = (normaliser, sum above hi, number above hi, listed
 // entries; the sign bit of the last = the list was full), list: float [unit][row_block][2][list_stride].
 // ---------------------------------------------------------------------------------------------
@@ -417,7 +421,7 @@ __global__ void __launch_bounds__(tc::kSegThreads, 1)
     cnt = 0;
     full = false;
     first = ptr = reinterpret_cast<float4*>(list + (rg * 2 + (part & 1)) * P.list_stride + cls_list_at(P, seg.tile_begin, seg.index));
-    limit = first + ((seg.tile_end - seg.tile_begin) * P.per_tile + kClsSlack) / 4 - 2;
+    limit = first + ((seg.tile_end - seg.tile_begin) * P.per_tile + P.slack) / 4 - 2;
     at = slots = smem_u32(user) + ((threadIdx.x >> 5) - 1) * (kClsSlots * 128) + (threadIdx.x & 31) * 4;
   };
   // whole groups of four staged entries go to the row's list, the newest first; up to three stay
@@ -1184,7 +1188,7 @@ extern "C" hkv_status hkv_classify_heads(const hkv_config* cfg, const void* k, c
     P.bins_at = static_cast<float>(at_sigma);
     P.scale_log2e = scale * kLog2e;
     // Rows per pass and list room.  A row takes its bounds, two partial records per CTA that shares its block, its entry
-    // in the flag list and two lists of `per_tile` entries per key tile plus kClsSlack per segment.  The lists get at
+    // in the flag list and two lists of `per_tile` entries per key tile plus a slack per segment.  The lists get at
     // least 1.3 times their (generously) expected length, and up to six times where the workspace allows it in one pass:
     // keys of a video frame are correlated, so a stretch of the context may hold several times its share.  28168 rows of
     // 24-32 K keys get 1.6 times: no row overflows with keys of frame means plus noise, 259 do when a direction that all queries share
@@ -1215,7 +1219,7 @@ extern "C" hkv_status hkv_classify_heads(const hkv_config* cfg, const void* k, c
     auto ctas_of = [&]() { return static_cast<int>(std::max<int64_t>(1, std::min<int64_t>(n_sm, P.w_prefix[nb] / std::max(2, P.weight)))); };
     auto segs_of = [&](int n_cta) { return static_cast<int>(std::min<int64_t>(n_tiles, static_cast<int64_t>(n_tiles) * P.weight / std::max<int64_t>(1, P.w_prefix[nb] / n_cta) + 2)); };
     auto bytes_of = [&](int seg_max, int per_tile) {
-      return static_cast<size_t>(8) * (static_cast<size_t>(n_tiles) * per_tile + static_cast<size_t>(seg_max) * kClsSlack) + 32u * seg_max + 20u;
+      return static_cast<size_t>(8) * (static_cast<size_t>(n_tiles) * per_tile + static_cast<size_t>(seg_max) * P.slack) + 32u * seg_max + 20u;
     };
     auto per_tile_of = [&](double times) { return std::min(64, static_cast<int>(std::ceil(times * share * 64.0))); };
     // CTAs per row block of the sample: as many as leave a quarter of the SMs free (a cluster's CTAs need one GPC)
@@ -1230,6 +1234,18 @@ extern "C" hkv_status hkv_classify_heads(const hkv_config* cfg, const void* k, c
     if (!sampled) { sample_bytes = 0; share = 1.0; }
     const size_t fixed = 4 * kAlign + sample_bytes;
     int row_block = r_max, seg_max = segs_of(ctas_of()), per_tile = per_tile_of(1.3);
+    auto all_rows_fit = [&](int entries) { return bytes_of(seg_max, entries) * r_max * units + fixed <= room; };
+    P.slack = kClsSlack;
+    if (!all_rows_fit(per_tile)) {
+      // Short contexts cut into segments of a tile or two: the slack alone is more than their keys, and the rows went through in
+      // three or four passes of 40 us each (944 rows of 1562 keys, two heads: 176 us).  With a share that takes
+      // three times what is expected, and hardly any slack, they mostly fit one.
+      P.slack = kClsSlackTight;
+      int entries = 64;
+      while (entries > 0 && !all_rows_fit(entries)) --entries;
+      if (entries > 0 && entries >= per_tile_of(3.0)) per_tile = entries;
+      else P.slack = kClsSlack;
+    }
     while (row_block > 1 && bytes_of(seg_max, per_tile) * row_block * units + fixed > room) {
       const size_t fit = (room - fixed) / units / bytes_of(seg_max, per_tile);
       row_block = static_cast<int>(std::max<size_t>(1, std::min<size_t>(row_block - 1, fit)));
@@ -1244,7 +1260,7 @@ extern "C" hkv_status hkv_classify_heads(const hkv_config* cfg, const void* k, c
     P.row_block = row_block;
     P.seg_max = seg_max;
     P.per_tile = per_tile;
-    P.list_stride = (n_tiles * per_tile & ~3) + seg_max * kClsSlack;
+    P.list_stride = (n_tiles * per_tile & ~3) + seg_max * P.slack;
     char* at = static_cast<char*>(workspace) + s.head_bytes;
     char* samples = at;                               at += sample_bytes;
     float4* bounds = reinterpret_cast<float4*>(at);   at += round_up(rows_all * sizeof(float4), kAlign);

@@ -89,12 +89,15 @@ __global__ void __launch_bounds__(kSetupThreads)
 //         draining thread owns one key and sums the normalised probabilities of its quarter of the rows, the four
 //         quarters meet in shared memory, and s_w[key] (+)= sum / R (written by the first row block, added
 //         to by later ones).
-// Bound: the tensor core's instructions and the drain of a tile overlap only in part, and a pass is short.  Ten units of 24-32 K
-// tokens (15 tiles per CTA): 38.7 and 39.1 us; without the powers (16 per clock and SM, 2048 cycles per tile) 32.9 and 31.0, without
-// the drain 28.1 and 23.3, without the copies 35.0 and 40.1, without copies and drain 24.0 and 21.4.  A tile takes 1.41 and 1.75 us, the
-// launch, the query block and the first tiles' way 16 and 11.  A quarter or half of the powers as polynomials on the
-// FMA pipes, and reading the accumulator ahead, changed nothing.  One exponent max + log2 sum instead of two constants per
-// row took 2 us off a second pass, but rounds a row's weight ten times as coarsely.
+// Bound: the drain of a tile (dependent loads, powers and sums of four warps per scheduler; the powers alone, 16 per clock and
+// SM, are 2048 cycles) and the start of a pass.  Ten units of 24-32 K tokens, 15 tiles per CTA: 30.8 and 31.2 us from the first CTA's
+// start to the last one's end (34.8 and 36.4 with units found through memory, without a unit's fixed cost and with the
+// test for keys behind a row's end in every step of the second pass).  1.6 and 1.55 us per tile; query rows in place after 3.3 and 2.4 us,
+// beside the first tiles of all CTAs in the same queues, statistics put together after another 2.0.  Without gain: a quarter or half of
+// the powers as polynomials on the FMA pipes, reading the accumulator ahead, powers taken against a reference that is
+// checked afterwards (first pass + 18 %), no barrier between the four quarters (second pass level), the second pass's tiles backwards or
+// with L2 eviction hints (level), tiles behind the first held back until it has landed (level).  One exponent max + log2 sum instead of two
+// constants per row took 2 us off a second pass, but rounds a row's weight ten times as coarsely.
 // grid: CTAs; one launch per block of 256 window rows.
 // ---------------------------------------------------------------------------------------------
 // A static unit as these kernels see it.  Its work is its key tiles plus a fixed cost at its beginning, in units of tiles:
