@@ -19,7 +19,6 @@
 #include <algorithm>
 #include <cmath>
 #include <mutex>
-#include <type_traits>
 
 #include "hkv_device.cuh"
 #include "hkv_internal.h"
@@ -361,6 +360,13 @@ __device__ __forceinline__ void cls_take(float v, float p, float lo, float hi, f
       : "memory");
 }
 
+// kApart: a tile that ends with the context goes through a loop of its own, without the test for keys behind it in the others': 28168
+// rows of 24-32 K keys 531 us instead of 546, but a CTA with few tiles pays for fetching both (600 rows of 11 K keys, 7 tiles per CTA: 70.1
+// and 69.1; 1344 of 50 K, 21 tiles: 99.5 and 100.2).
+template <bool kValue>
+struct ClsFlag { __device__ constexpr operator bool() const { return kValue; } };
+constexpr int kClsApartTiles = 12;       // tiles per CTA from which it pays
+template <bool kApart>
 __global__ void __launch_bounds__(tc::kSegThreads, 1)
     cls_scan_kernel(const __grid_constant__ ClsParams P, const __grid_constant__ CUtensorMap keys, const __nv_bfloat16* q_text, const float4* bounds,
                     float4* partial, float* list, int32_t* err) {
@@ -441,10 +447,9 @@ __global__ void __launch_bounds__(tc::kSegThreads, 1)
   auto tile_fn = [&](const ClsSeg& seg, int tile, int, int part, uint32_t taddr) {
     if (idle) return;
     const int left = seg.C - (tile * tc::kKeysPerTile + 64 * (part & 1));   // keys of the thread's 64 columns that exist
-    // (a tile that ends with the context in a loop of its own: with the test in one loop 28168 rows of 24-32 K keys took 546 us, not 531)
     auto go = [&](auto whole) {
       tc::drain_raw<1>(taddr, [&](int g, uint32_t (&r)[16]) {
-        if constexpr (!decltype(whole)::value) {
+        if (!whole) {
 #pragma unroll
           for (int c = 0; c < 16; ++c)
             if (16 * g + c >= left) r[c] = 0xFF800000u;   // -inf: no weight, below every bound
@@ -468,8 +473,12 @@ __global__ void __launch_bounds__(tc::kSegThreads, 1)
         tc::add_compensated(top, topc, t0 + t1);
       });
     };
-    if (left >= 64) go(std::true_type{});
-    else go(std::false_type{});
+    if constexpr (kApart) {
+      if (left >= 64) go(ClsFlag<true>());
+      else go(ClsFlag<false>());
+    } else {
+      go(left >= 64);
+    }
   };
   auto end = [&](const ClsSeg& seg, int lane_row, int part, bool) {
     const int row = 128 * (part >> 1) + lane_row;
@@ -1030,7 +1039,8 @@ cudaError_t cls_configure(int* n_sm) {
         (e = cudaFuncSetAttribute(cls_sample_kernel<4>, attr, kClsSampleSmem)) != cudaSuccess ||
         (e = cudaFuncSetAttribute(cls_sample_kernel<2>, attr, kClsSampleSmem)) != cudaSuccess ||
         (e = cudaFuncSetAttribute(cls_sample_kernel<1>, attr, kClsSampleSmem)) != cudaSuccess ||
-        (e = cudaFuncSetAttribute(cls_scan_kernel, attr, kClsScanSmem)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(cls_scan_kernel<true>, attr, kClsScanSmem)) != cudaSuccess ||
+        (e = cudaFuncSetAttribute(cls_scan_kernel<false>, attr, kClsScanSmem)) != cudaSuccess ||
         (e = cudaFuncSetAttribute(cls_select_kernel, attr, 200 * 1024)) != cudaSuccess ||
         (e = cudaFuncSetAttribute(cls_fix_kernel, attr, kClsFixScratch + kClsSmemCols * 4)) != cudaSuccess ||
         (e = cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess)
@@ -1299,7 +1309,8 @@ extern "C" hkv_status hkv_classify_heads(const hkv_config* cfg, const void* k, c
       P.small = (P.w_prefix[nb] + 1) * P.n_cta < (1ll << 31);
       if (rb > 0 && cudaMemsetAsync(err + 1, 0, sizeof(int32_t), cs) != cudaSuccess) return HKV_ERR_CUDA;
       if (sampled) e = launch_cls(sample_kernel, blocks * P.split, P.split, tc::kSegThreads, kClsSampleSmem, cs, rb == 0, P, sample_map, qg, bounds, err);
-      if (e == cudaSuccess) e = launch_cls(cls_scan_kernel, P.n_cta, 1, tc::kSegThreads, kClsScanSmem, cs, sampled, P, map, qg,
+      const bool apart = P.w_prefix[nb] >= static_cast<int64_t>(kClsApartTiles) * P.weight * P.n_cta;
+      if (e == cudaSuccess) e = launch_cls(apart ? cls_scan_kernel<true> : cls_scan_kernel<false>, P.n_cta, 1, tc::kSegThreads, kClsScanSmem, cs, sampled, P, map, qg,
                                            static_cast<const float4*>(bounds), partial, list, err);
       if (e == cudaSuccess) e = launch_cls(cls_select_kernel, static_cast<int>((rows_all + sel_warps - 1) / sel_warps), 1, sel_warps * 32,
                                            static_cast<size_t>(sel_warps) * sel_cap * sizeof(float4), cs, true, P, static_cast<const float4*>(bounds),
