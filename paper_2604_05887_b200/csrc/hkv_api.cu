@@ -292,9 +292,19 @@ static hkv_status compress_common(const hkv_config* cfg, const void* k, const vo
     for (const auto& u : c->units) build_bytes += u.type == 0 ? 0 : 4ll * kRowBytes * u.C;
     int n_sm = 1;
     bool ok = compress_configure(&n_sm) == cudaSuccess;
-    // A short prompt: few key tiles (they leave half of the SMs free) and copies of a few microseconds.  All kernels go on one
-    // stream, each set up beside its predecessors, the dynamic heads' last: it runs beside the selection and the gather.
-    const bool chain = window && total_tiles <= n_sm / 2 && build_bytes <= (24ll << 20) && !c->host_bytes;
+    // A short prompt: all kernels go on one stream, each set up beside its predecessors, the dynamic heads' last: it runs beside the
+    // selection and the gather.  With few key tiles (they leave half of the SMs free) and copies of a few microseconds that is
+    // faster in every case.  Beyond, it saves what two streams cost a compression that is launched as it comes, events and waits
+    // (16 K tokens, half of the heads static: 53.2 -> 47.6 us; four of 4 K 46.0 -> 42.2; two of 16 K 60.4 -> 56.5), as long as the copies are
+    // done by the gather's end (four of 4 K, 48 MB of copies: 41.2 -> 42.2; 50 K tokens, 1173 tiles: 78.7 -> 81.3).  A recorded one pays
+    // no such cost (16 K tokens: 43.5 and 44.1, 8 K 35.4 and 37.0) and keeps two streams.
+    const bool one_stream = window && !c->host_bytes;
+    bool chain = one_stream && total_tiles <= n_sm / 2 && build_bytes <= (24ll << 20);
+    if (one_stream && !chain && total_tiles <= 5ll * n_sm && build_bytes <= (24ll << 20) + (total_tiles * 48 << 10)) {
+      cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;   // (the legacy default stream cannot be recorded)
+      ok = ok && (!s || cudaStreamIsCapturing(s, &capture) == cudaSuccess);
+      chain = capture == cudaStreamCaptureStatusNone;
+    }
     // Else the static heads run beside the dynamic ones, on the library's second stream (forked from and joined to `s`): it has
     // the higher priority, so that the long chain of the static heads' kernels never queues behind the dynamic heads' blocks.
     StepSide* side = (ok && H.n_static > 0 && H.n_dynamic > 0 && !chain) ? step_side() : nullptr;
