@@ -301,19 +301,42 @@ __global__ void __launch_bounds__(tc::kSegThreads, 1)
   } else if (threadIdx.x < share) {
     top = fmaxf(stat[0][threadIdx.x].x, stat[1][threadIdx.x].x);
   }
-  const int row = first + threadIdx.x;
-  if (threadIdx.x >= share || row0 + row >= rows) return;
+  // The bounds: 512 threads, 2 P.split of them per row, each with its share of the entries (one thread per row walked all of
+  // them: 2.5 us).  `stat` has been read and holds the shares' sums and the places found.
+  __syncthreads();
+  int* sums = reinterpret_cast<int*>(&stat[0][0]);             // [shares][rows]
+  int *at_hi = reinterpret_cast<int*>(&stat[1][0]), *at_lo = at_hi + tc::kQRows;
+  const int tid = threadIdx.x, mine = tid & (share - 1), part = tid / share, n_part = 512 / share, per_part = kClsSampleBins / n_part;
+  const int row = first + mine;
+  auto entry = [&](int i) { return static_cast<int>((hist[i * (tc::kQRows / 2) + (row >> 1)] >> ((row & 1) * 16)) & 0xFFFFu); };
   int cum = 0;
-  float lo = kClsOpen, hi = INFINITY;
-  bool have_lo = false;
+  if (tid < 512) {
+    for (int i = part * per_part; i < (part + 1) * per_part; ++i) cum += entry(i);
+    sums[tid] = cum;
+  }
+  if (tid < share) {
+    at_hi[tid] = kClsSampleBins;
+    at_lo[tid] = 0;
+  }
+  __syncthreads();
+  if (tid < 512) {
+    cum = 0;
+    for (int p = part + 1; p < n_part; ++p) cum += sums[p * share + mine];
+    int hi_at = kClsSampleBins, lo_at = 0;   // lowest entry from which on at most rank_hi lie, highest from which on at least rank_lo
+    for (int i = (part + 1) * per_part - 1; i >= max(1, part * per_part); --i) {
+      cum += entry(i);
+      if (cum <= P.rank_hi[b]) hi_at = i;
+      if (lo_at == 0 && cum >= P.rank_lo[b]) lo_at = i;
+    }
+    if (hi_at < kClsSampleBins) atomicMin(&at_hi[mine], hi_at);
+    if (lo_at > 0) atomicMax(&at_lo[mine], lo_at);
+  }
+  __syncthreads();
+  if (tid >= share || row0 + row >= rows) return;
   a_bin = place[row].x;
   width = place[row].y;
-  for (int i = kClsSampleBins - 1; i >= 1; --i) {
-    cum += static_cast<int>((hist[i * (tc::kQRows / 2) + (row >> 1)] >> ((row & 1) * 16)) & 0xFFFFu);
-    const float edge = a_bin + static_cast<float>(i) * width;
-    if (cum <= P.rank_hi[b]) hi = edge;
-    if (!have_lo && cum >= P.rank_lo[b]) { lo = edge; have_lo = true; }
-  }
+  const float hi = at_hi[tid] < kClsSampleBins ? a_bin + static_cast<float>(at_hi[tid]) * width : INFINITY;
+  const float lo = at_lo[tid] > 0 ? a_bin + static_cast<float>(at_lo[tid]) * width : kClsOpen;
   bounds[static_cast<size_t>(b * P.n_kv_heads + h) * P.row_block + row0 + row] = make_float4(lo, hi, top * P.scale_log2e, 0.f);
 }
 
