@@ -776,7 +776,7 @@ def main():
                    "compress_GBps_of_input_kv": sb.kv_in_bytes0 / (comp_ms * 1e-3) / 1e9,
                    "compress_how": "hkv_compress of layer 0 alone (inputs resident, buffers preallocated), CUDA events around the call, fastest of 5; GB/s = that layer's full K/V bytes / that time"},
         "frac_of_measured_peak": value / world / peak, "frac_of_8TBps": value / world / NOMINAL_HBM_GBS,
-        "roofline": {"bound": "hbm", "kernel": "decode_kernel (score + top-k + flash-decode + merge, one launch per layer)",
+        "roofline": {"bound": "hbm", "kernel": "decode_step_kernel (score + top-k + flash-decode + merge, one launch per layer)",
                      "achieved": achieved, "peak": peak, "peak_source": peak_src, "unit": "GB/s",
                      "frac": achieved / peak, "frac_of_8TBps": achieved / NOMINAL_HBM_GBS,
                      "avg_launch_us": fused_avg_s * 1e6, "median_launch_us": sp["median"] / n_layers,
