@@ -274,3 +274,19 @@ def test_gpu_classify_many_small_entries_beside_a_large_one(C, fraction):
     got, _ = _gpu_scores(L, q_text, counts, fraction, 0.9)
     assert 0.99 < ref.min() < 0.99999
     assert np.abs(got - ref).max() <= 2.0 ** -23, (got - ref)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("B,C,T,G,Hkv,fraction", [(1, 1562, 118, 8, 2, 0.05), (2, 1562, 40, 4, 2, 0.3), (1, 129, 64, 8, 2, 0.05),
+                                                  (1, 2100, 30, 7, 4, 0.05)])
+@pytest.mark.parametrize("frames", [False, True])
+def test_gpu_classify_short_contexts_with_tight_lists(B, C, T, G, Hkv, fraction, frames):
+    """Segments of a tile or two whose lists get several times their share instead of a fixed slack.  With `frames` keys of 256
+    tokens share a mean that dominates their noise, so whole tiles lie between a row's bounds and lists run full: such rows are
+    done again, with the same result."""
+    L = hi.tiny(seed=71, B=B, C=C, chunk_size=32, w=8, Hq=G * Hkv, Hkv=Hkv, d=128)
+    if frames:
+        rng = np.random.default_rng(4)
+        k = np.repeat(rng.standard_normal((B, Hkv, -(-C // 256), 128)), 256, axis=2)[:, :, :C] + 0.05 * hi.bf16_bits_to_f32(L.k)
+        L.k[:] = hi.f32_to_bf16_bits(k.astype(np.float32))
+    _check_case(L, T, fraction)
